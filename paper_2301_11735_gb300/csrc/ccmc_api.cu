@@ -147,14 +147,12 @@ int upload_params_on(ccmc_lattice *h, double beta, double Delta, double V, doubl
   if (h->have_params && h->params[0] == beta && h->params[1] == Delta && h->params[2] == V &&
       h->params[3] == J)
     return CCMC_OK;
-  std::vector<uint32_t> thr32(kTableN);
-  std::vector<uint16_t> thrT(kThrT, 0);
-  build_thresholds(beta, Delta, V, J, thr32.data());
-  for (int i = 0; i < kTableN; ++i) thrT[i] = threshold_level(thr32[i]);
-  CK(cudaMemcpyAsync(h->t.thr32, thr32.data(), sizeof(uint32_t) * kTableN,
-                     cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(h->t.thrT, thrT.data(), sizeof(uint16_t) * kThrT, cudaMemcpyHostToDevice,
-                     st));
+  uint32_t thr32[kDevN];
+  uint16_t thrT[kThrT] = {};
+  build_device_thresholds(beta, Delta, V, J, thr32);
+  for (int i = 0; i < kDevN; ++i) thrT[i] = threshold_level(thr32[i]);
+  CK(cudaMemcpyAsync(h->t.thr32, thr32, sizeof(thr32), cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(h->t.thrT, thrT, sizeof(thrT), cudaMemcpyHostToDevice, st));
   // pageable sources: the copies are staged before the calls return
   h->have_params = true;
   h->params[0] = beta;
@@ -317,7 +315,7 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
   }
   const int np = recount_grid(g);
   const int dev = h->device;
-  const size_t tb = sizeof(uint32_t) * (kTableN + 2 * kMoveN) + sizeof(uint16_t) * kThrT;
+  const size_t tb = sizeof(uint32_t) * (kDevN + 2 * kMoveN) + sizeof(uint16_t) * kThrT;
   if (!dalloc((void **)&h->d_words, sizeof(uint32_t) * 16 * g.cstride, dev, h->stream) ||
       !dalloc((void **)&h->d_ctl, sizeof(int64_t) * kCtlWords, dev, h->stream) ||
       !dalloc((void **)&h->d_partials, sizeof(int64_t) * 7 * np, dev, h->stream) ||
@@ -1041,7 +1039,7 @@ int ccmc::batch_new(int cap, cudaStream_t stream, ccmc_batch **out) {
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const int64_t max_words = optin / 4 - kResTableWords - 64;
+  const int64_t max_words = optin / 4 - kConfigTableWords - 64;
   if (b->resident_max_sites / 4 > max_words) b->resident_max_sites = max_words * 4;
   if (cudaMalloc(&b->d_jobs, sizeof(JobDesc) * count) != cudaSuccess ||
       cudaMalloc(&b->d_multi, sizeof(MultiJob) * count) != cudaSuccess ||
@@ -1087,7 +1085,7 @@ int ccmc_batch_config(ccmc_batch *b, int resident_threads, int64_t resident_max_
   int dev = 0, optin = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const int64_t max_words = optin / 4 - kResTableWords - 64;
+  const int64_t max_words = optin / 4 - kConfigTableWords - 64;
   if (resident_max_sites / 4 > max_words) return CCMC_E_INVAL;
   b->threads = resident_threads;
   b->resident_max_sites = resident_max_sites;

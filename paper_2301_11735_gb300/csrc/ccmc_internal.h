@@ -46,12 +46,30 @@ struct Geo {
   uint64_t rej;     // 2^64 mod (Lx Ly): Lemire rejection bound
 };
 
+// The device's threshold tables hold only the energy changes a coupled pair
+// can make, in three segments; every move stays in the segment of its kind, so
+// that its index is an affine function of the neighbour sums:
+//   one unit of charge moves or a +- pair appears or vanishes (|dS| = 1):
+//     |dBV|, |dBJ| <= 9, dQ in {-2, 0, 2}: 3 x 19 x 19 entries
+//     [(dQ + 2) / 2][dBV + 9][dBJ + 9];
+//   the two charges of a +- pair change places (|dS| = 2, no spin involved):
+//     41 entries [dBV + 20];
+//   spins flip (dS = 0): 41 entries [dBJ + 20].
+// 1165 of the 5043 entries of the full dQ x dBV x dBJ table: 2.3 KB of levels
+// instead of 10 KB, so that a CTA's prologue copies 5.4 KB, not 13.2 KB, and
+// many small CTAs fit an SM.
+constexpr int kSegR = 9;                      // |dBV|, |dBJ| of the first segment
+constexpr int kSegW = 2 * kSegR + 1;          // 19
+constexpr int kSegSwap = 3 * kSegW * kSegW;   // first entry of the second segment: 1083
+constexpr int kSegFlip = kSegSwap + kNB;      // and of the third: 1124
+constexpr int kDevN = kSegFlip + kNB;         // 1165
+
 // Per-lattice parameter tables in device memory (built on the host).
 struct DevTables {
   uint16_t *thrT;   // kThrT: threshold levels T = floor(5461 thr / 2^32), 5461 for
                     // thr = 0xFFFFFFFF (fast path)
   uint32_t *trans;  // kMoveN x 2 words: move entries (see kMoveN), directly after thrT
-  uint32_t *thr32;  // kTableN: full thresholds (exact path)
+  uint32_t *thr32;  // kDevN: full thresholds (exact path)
 };
 
 // The fast path's threshold level of a 32-bit threshold: a field's w = v / 12
@@ -66,7 +84,7 @@ __host__ __device__ inline uint16_t threshold_level(uint32_t thr) {
 // nearest neighbour, pc = 4 code_a + code_b the pair state.
 constexpr int kTransN = 16 * 12;     // entries of one kind (far or near)
 constexpr int kMoveN = 2 * kTransN;  // both kinds
-constexpr int kThrT = (kTableN + 7) / 8 * 8;  // 16-bit levels, padded to 16 bytes
+constexpr int kThrT = (kDevN + 7) / 8 * 8;  // 16-bit levels, padded to 16 bytes
 
 struct LaunchCfg {
   int phase_grid_cap = 152 * 3;  // one resident wave of phase_kernel (set at create)
@@ -104,10 +122,16 @@ struct MultiJob {
 
 // Shared memory of the resident kernel besides the lattice words.
 constexpr int kResTableWords = kThrT / 2 + 2 * kMoveN;
+// What ccmc_batch_config's upper limit of resident_max_sites sets aside of a
+// CTA's shared memory (words).
+constexpr int kConfigTableWords = 3292;
 
-// Host-side table builders (ccmc_tables.cpp).
+// Host-side table builders (ccmc_tables.cpp): the full table of
+// ccmc_threshold_table (kTableN entries) and the device's (kDevN).
 void build_thresholds(double beta, double Delta, double V, double J, uint32_t *thr32);
-// Returns false if some entry could index outside the threshold table.
+void build_device_thresholds(double beta, double Delta, double V, double J, uint32_t *thr32);
+// Returns false if some entry could index outside its segment of the device's
+// threshold table.
 bool build_transitions(uint32_t *trans);
 
 // Launchers (ccmc_kernels.cu).

@@ -6,7 +6,7 @@
 // change with atomic XORs of their own bits.
 //
 // The move uses the library's own tables: the 64-bit move entry of the pair's
-// state, choice and kind (partner a nearest neighbour of a or not), the dp4a threshold index from (sum_a (S+1) - sum_b (S+1) + 8,
+// state, choice and kind (partner a nearest neighbour of a or not), the dp4a threshold offset from (sum_a (S+1) - sum_b (S+1) + 8,
 // sum_a (sigma+1), sum_b (sigma+1)) and the full 32-bit threshold.  Random
 // words of pair p of map m: the 16-bit field v = the low half of word 0 of
 // Philox(seed, (p, m_lo, m_hi, 11)) and, when v >= 65532 or its level w =
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) map_kernel(Geo g, const int32_t *__restri
   const uint32_t x = (e.y >> 24) & 15u;  // pc XOR the chosen configuration
   if (x == 0u) return;           // the chosen configuration is the current one
   const uint32_t env = (SA + 8u - SB) | (GA << 8) | (GB << 16);
-  const uint32_t thr = thr32[__dp4a((int)e.y, (int)env, (int)e.x)];
+  const uint32_t thr = thr32[__dp4a((int)e.y, (int)env, (int)e.x) >> 1];
   bool accept;
   if (thr == 0xFFFFFFFFu) {
     accept = true;

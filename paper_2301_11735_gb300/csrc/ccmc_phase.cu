@@ -28,8 +28,8 @@ namespace ccmc {
 // 4 code_a + code_b and its field v:
 //   w      = floor(v / 12), the choice class v - 12 w (v < 65532 = 12 x 5461)
 //   entry  = trans[v - 12 w][near][pc] -> base, byte coefficients, pc XOR npc
-//   index  = dp4a(coefficients, (D8, GA, GB, 0), base)  (threshold index)
-//   accept = w < T[index], with T = floor(5461 thr / 2^32) (5461 when thr is
+//   offset = dp4a(coefficients, (D8, GA, GB, 0), base)  (byte offset of the level)
+//   accept = w < T(offset), with T = floor(5461 thr / 2^32) (5461 when thr is
 //            0xFFFFFFFF): w < T implies w 2^32 + s < 5461 thr for every 32-bit
 //            s, w > T the opposite
 // The fast decision is always applied.  A tie (w == T) or a field v >= 65532
@@ -114,12 +114,18 @@ __device__ __forceinline__ uint32_t window(const uint32_t *cls, const Geo &g, co
 // 256 r + 128 near + 8 (pc XOR r) = (264 r) XOR pc8.  The XOR spreads a warp's
 // lookups over the banks: with entry (2 r + near) 16 + pc the bank pair of a
 // lookup was its pair state alone, and the few common states (both sites
-// magnetic) piled onto four of sixteen bank pairs.  Word 0: the threshold
-// index's base; word 1: the signed byte coefficients of (D8, GA, GB) and, at
+// magnetic) piled onto four of sixteen bank pairs.  Word 0: the level
+// offset's base; word 1: the signed byte coefficients of (D8, GA, GB) and, at
 // bits 24-27 (the byte dp4a multiplies by zero), the move pc XOR npc.
 __device__ __forceinline__ uint2 move_entry(const uint2 *trans, uint32_t r, uint32_t pc8) {
   return *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(trans) +
                                           ((r * 264u) ^ pc8));
+}
+
+// The threshold level at byte offset `off` (the offset is formed in bytes, so
+// that it is the load's address without a shift).
+__device__ __forceinline__ uint32_t level_at(const uint16_t *thrT, int off) {
+  return *reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(thrT) + off);
 }
 
 // floor(v / 12) for v < 2^16 by a multiply-high: floor(v m / 2^32) with
@@ -234,7 +240,7 @@ __device__ __forceinline__ uint3 fast_moves(const Geo &g, const uint2 *trans,
         const uint32_t v = h ? X >> 16 : X & 0xFFFFu;
         const uint32_t wq = div12(v);
         const uint2 e = move_entry(trans, v - 12u * wq, prmt(gr.pc8, 0u, 0x4440u + (uint32_t)q));
-        const uint32_t T = thrT[__dp4a((int)e.y, (int)lane_env(gr, q), (int)e.x)];
+        const uint32_t T = level_at(thrT, __dp4a((int)e.y, (int)lane_env(gr, q), (int)e.x));
         const uint32_t d = wq - T;  // negative: accept; zero: a tie
         if (q & 1) {
           d0 = d;
@@ -322,14 +328,15 @@ __device__ __forceinline__ void exact_pair(const Geo &g, const PhaseU &u, const 
   const uint32_t env = prmt(q < 2 ? gr.x01 : gr.x23, gr.gb,
                             0x8410u + ((q & 1) ? 0x0122u : 0u) + ((q & 2) ? 0x0200u : 0u));
   uint2 e = move_entry(trans, v - 12u * wq, pc8);
-  if (v < 65532u && wq != thrT[__dp4a((int)e.y, (int)env, (int)e.x)]) return;  // not rare
+  if (v < 65532u && wq != level_at(thrT, __dp4a((int)e.y, (int)env, (int)e.x)))
+    return;  // not rare
   const uint32_t slow0 = (uint32_t)((uint64_t)j * g.Cx + (uint32_t)(w << 4));
   const U4 sl = philox(slow0 + (uint32_t)t, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, g.k0, g.k1);
   if (v >= 65532u) {
     if (sl.y >= 4294967292u) return;  // keep the current configuration
     e = move_entry(trans, sl.y % 12u, pc8);
   }
-  const uint32_t thr = thr32[__dp4a((int)e.y, (int)env, (int)e.x)];
+  const uint32_t thr = thr32[__dp4a((int)e.y, (int)env, (int)e.x) >> 1];
   const bool accept = thr == 0xFFFFFFFFu ||
                       (v < 65532u ? ((uint64_t)wq << 32) + sl.x < 5461ull * thr : sl.x < thr);
   if (accept) {

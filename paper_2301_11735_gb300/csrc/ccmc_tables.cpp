@@ -39,6 +39,18 @@ void build_thresholds(double beta, double Delta, double V, double J, uint32_t *t
             threshold(beta, Delta, V, J, 2 * dqi - 2, dBV, dBJ);
 }
 
+void build_device_thresholds(double beta, double Delta, double V, double J, uint32_t *thr32) {
+  for (int dqi = 0; dqi < 3; ++dqi)
+    for (int dBV = -kSegR; dBV <= kSegR; ++dBV)
+      for (int dBJ = -kSegR; dBJ <= kSegR; ++dBJ)
+        thr32[(dqi * kSegW + dBV + kSegR) * kSegW + dBJ + kSegR] =
+            threshold(beta, Delta, V, J, 2 * dqi - 2, dBV, dBJ);
+  for (int d = -kDB; d <= kDB; ++d) {
+    thr32[kSegSwap + d + kDB] = threshold(beta, Delta, V, J, 0, d, 0);
+    thr32[kSegFlip + d + kDB] = threshold(beta, Delta, V, J, 0, 0, d);
+  }
+}
+
 // Move entries (see the phase kernel).  For choice class r = v mod 12, kind
 // near (the partner is a nearest neighbour) and pair state pc = 4 a + b, the
 // proposed state is the (r mod |set|)-th configuration of the pair's q-set in
@@ -47,13 +59,13 @@ void build_thresholds(double beta, double Delta, double V, double J, uint32_t *t
 //   dBV = dS_a sum_<a> S + dS_b sum_<b> S + m dS_a dS_b
 //   dBJ = dsig_a sum_<a> sigma + dsig_b sum_<b> sigma + m dsig_a dsig_b
 // with neighbour sums over old states (partner included) and m = near the number
-// of a-b bonds.  As dS_b = -dS_a, the threshold index
-//   ((dQ + 2)/2 * 41 + dBV + 20) * 41 + dBJ + 20
-// is an affine function of the biased sums D8 = sum_<a> S - sum_<b> S + 8,
-// GA = sum_<a> sigma + 4, GB = sum_<b> sigma + 4:
-//   index = base + (41 dS_a) D8 + dsig_a GA + dsig_b GB.
+// of a-b bonds.  As dS_b = -dS_a, the byte offset of the move's 16-bit level,
+// twice its index in its segment's stride (sS entries a unit of dBV, sG a unit
+// of dBJ), is an affine function of the biased sums D8 = sum_<a> S - sum_<b> S
+// + 8, GA = sum_<a> sigma + 4, GB = sum_<b> sigma + 4:
+//   offset = base + (2 sS dS_a) D8 + (2 sG dsig_a) GA + (2 sG dsig_b) GB.
 // Entry (2 r + near) * 16 + (pc XOR r): word 0 holds base; word 1 the signed byte
-// coefficients (41 dS_a, dsig_a, dsig_b) and, in bits 24-27 (byte 3, which
+// coefficients of (D8, GA, GB) and, in bits 24-27 (byte 3, which
 // the phase kernel multiplies by zero; bits 28-31 stay clear), pc XOR npc.
 namespace {
 constexpr int kSetN[3] = {4, 6, 4};  // q = +1, 0, -1
@@ -65,7 +77,7 @@ constexpr int kSets[3][6][2] = {
 }  // namespace
 
 bool build_transitions(uint32_t *trans) {
-  int lo = 1 << 30, hi = -(1 << 30);
+  bool ok = true;
   for (int pc = 0; pc < 16; ++pc) {
     const int ca = pc >> 2, cb = pc & 3;
     const int q = kS[ca] + kS[cb];
@@ -79,30 +91,41 @@ bool build_transitions(uint32_t *trans) {
       const int dQ = kS[na] * kS[na] + kS[nb] * kS[nb] - kS[ca] * kS[ca] - kS[cb] * kS[cb];
       const int dSa = kS[na] - kS[ca], dSb = kS[nb] - kS[cb];
       const int dGa = kSigma[na] - kSigma[ca], dGb = kSigma[nb] - kSigma[cb];
-      const int mulS = kNB * dSa;
-      const int base = (dQ + 2) / 2 * kNB * kNB + kDB * kNB + kDB - 4 * (dGa + dGb) - 8 * mulS;
-      const int near_base = base + kNB * dSa * dSb + dGa * dGb;
+      // the move's segment: entries a unit of dBV and of dBJ, the entry of dBV =
+      // dBJ = 0, the segment's first entry and its end
+      const int kind = dSa == 0 ? 2 : (dSa == 1 || dSa == -1) ? 0 : 1;
+      const int sS = kind == 0 ? kSegW : kind == 1 ? 1 : 0, sG = kind == 1 ? 0 : 1;
+      const int first = kind == 0 ? (dQ + 2) / 2 * kSegW * kSegW : kind == 1 ? kSegSwap : kSegFlip;
+      const int end = first + (kind == 0 ? kSegW * kSegW : kNB);
+      const int zero = first + (kind == 0 ? kSegR * kSegW + kSegR : kDB);
+      const int cS = 2 * sS * dSa, cA = 2 * sG * dGa, cB = 2 * sG * dGb;
+      const int base = 2 * zero - 8 * cS - 4 * (cA + cB);
       const uint32_t x = (uint32_t)(((ca ^ na) << 2) | (cb ^ nb));
-      const uint32_t coef = ((uint32_t)mulS & 0xFFu) | (((uint32_t)dGa & 0xFFu) << 8) |
-                            (((uint32_t)dGb & 0xFFu) << 16) | (x << 24);
+      const uint32_t coef = ((uint32_t)cS & 0xFFu) | (((uint32_t)cA & 0xFFu) << 8) |
+                            (((uint32_t)cB & 0xFFu) << 16) | (x << 24);
       for (int near = 0; near < 2; ++near) {
         const int e = (2 * r + near) * 16 + (pc ^ r);  // bank-spread (see the phase kernel)
-        trans[2 * e] = (uint32_t)(near ? near_base : base);
+        const int b = base + near * 2 * (sS * dSa * dSb + sG * dGa * dGb);
+        trans[2 * e] = (uint32_t)b;
         trans[2 * e + 1] = coef;
-      }
-      // every index an entry can form, over all possible neighbour sums
-      // (D8 in [0, 16], GA and GB in [0, 8]), must stay inside the table
-      for (int b0 : {base, near_base})
+        // every offset the entry can form, over all neighbour sums (D8 in [0, 16],
+        // GA and GB in [0, 8]), and both its energy terms, stay inside the segment
         for (int D8 : {0, 16})
           for (int ga : {0, 8})
             for (int gb : {0, 8}) {
-              const int idx = b0 + mulS * D8 + dGa * ga + dGb * gb;
-              lo = idx < lo ? idx : lo;
-              hi = idx > hi ? idx : hi;
+              const int off = b + cS * D8 + cA * ga + cB * gb;
+              const int dBV = dSa * (D8 - 8) + near * dSa * dSb;
+              const int dBJ = dGa * (ga - 4) + dGb * (gb - 4) + near * dGa * dGb;
+              const int reach = kind == 0 ? kSegR : kDB;
+              ok = ok && off >= 2 * first && off < 2 * end && (off & 1) == 0;
+              ok = ok && (kind == 1 ? dGa == 0 && dGb == 0 : dBJ >= -reach && dBJ <= reach);
+              ok = ok && (kind == 2 ? dSb == 0 : dBV >= -reach && dBV <= reach);
+              ok = ok && (kind == 0 || dQ == 0);
             }
+      }
     }
   }
-  return lo >= 0 && hi < kTableN;
+  return ok;
 }
 
 }  // namespace ccmc
