@@ -17,9 +17,9 @@ __device__ __forceinline__ int64_t warp_sum(int64_t v) {
   return v;
 }
 
-// Bit planes of a class word X against its right and down neighbour windows
-// Yr, Yd, with every site's type bit (1 = charged) left in place at the odd
-// bit and its sign bit (1 = minus) at the even bit below it.  `vo` holds the
+// Bit planes of a class word X (linear code) against its right and down
+// neighbour windows Yr, Yd, a site's type (1 = charged, b1 XOR b0) at its odd
+// bit and its sign (b0, 1 = minus) at the even bit below it.  `vo` holds the
 // odd bits of the valid sites.  Bonds are laid out two to a site: the right
 // bond at the odd bit, the down bond at the even bit (the down masks shifted
 // down one place, which adds to the right ones without carries).
@@ -33,12 +33,13 @@ __device__ __forceinline__ WordPlanes word_planes(uint32_t X, uint32_t Yr, uint3
                                                   uint32_t vo) {
   constexpr uint32_t kEven = 0x55555555u, kOdd = 0xAAAAAAAAu;
   WordPlanes p;
-  const uint32_t Xs = X << 1;  // sign bits moved up to the type bits
-  p.k = X & vo;
-  p.kg = X & Xs & vo;
-  p.ug = ~X & Xs & vo;
-  p.kk = (X & Yr & vo) + ((X & Yd & vo) >> 1);
-  p.uu = (~(X | Yr) & vo) + ((~(X | Yd) & vo) >> 1);
+  const uint32_t Xs = X << 1;  // sign bits moved up to the odd bits
+  const uint32_t K = X ^ Xs, Kr = Yr ^ (Yr << 1), Kd = Yd ^ (Yd << 1);
+  p.k = K & vo;
+  p.kg = ~X & Xs & vo;
+  p.ug = X & Xs & vo;
+  p.kk = (K & Kr & vo) + ((K & Kd & vo) >> 1);
+  p.uu = (~(K | Kr) & vo) + ((~(K | Kd) & vo) >> 1);
   p.f = (((X ^ Yr) << 1) & kOdd) | ((X ^ Yd) & kEven);
   return p;
 }
@@ -120,16 +121,6 @@ struct QuadCounts {
   int nK = 0, nKG = 0, nUG = 0, nKK = 0, nKKd = 0, nUUd = 0, quads = 0;
 };
 
-// One three-input logic instruction: kLut is the function's truth table on
-// the canonical inputs a = 0xF0, b = 0xCC, c = 0xAA.
-template <uint32_t kLut>
-__device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  asm("lop3.b32 %0, %1, %2, %3, %4;" : "=r"(d) : "r"(a), "r"(b), "r"(c), "n"(kLut));
-  return d;
-}
-constexpr uint32_t kLutMux = 0xE4;      // c ? a : b, bit by bit
-constexpr uint32_t kLutAnd3 = 0x80;     // a & b & c
 constexpr uint32_t kLutNorAnd = 0x02;   // ~(a | b) & c
 constexpr uint32_t kLutAndNot = 0x0C;   // ~a & b
 
@@ -165,10 +156,10 @@ __device__ __forceinline__ void count_quads(const uint32_t *__restrict__ X0,
     for (int k = 0; k < 4; ++k) {
       const uint32_t X = xs[k], Yd = ds[k];
       const uint32_t Yr = kColR ? __funnelshift_r(rs[k], rs[k + 1], 2) : rs[k];
-      const uint32_t tX = lop3<kLutMux>(X, X >> 1, kOdd);  // type in both bits
-      const uint32_t gX = lop3<kLutMux>(X << 1, X, kOdd);  // sign in both bits
-      const uint32_t tY = lop3<kLutMux>(Yr, Yd >> 1, kOdd);
+      const uint32_t gX = lop3<kLutMux>(X << 1, X, kOdd);        // sign in both bits
+      const uint32_t tX = lop3<kLutMux>(X, X >> 1, kOdd) ^ gX;   // type in both bits
       const uint32_t gY = lop3<kLutMux>(Yr << 1, Yd, kOdd);
+      const uint32_t tY = lop3<kLutMux>(Yr, Yd >> 1, kOdd) ^ gY;
       const uint32_t f = gX ^ gY;
       n.nKK += __popc(tX & tY);
       n.nKKd += __popc(lop3<kLutAnd3>(tX, tY, f));
@@ -176,8 +167,8 @@ __device__ __forceinline__ void count_quads(const uint32_t *__restrict__ X0,
     }
 #pragma unroll
     for (int k = 0; k < 4; k += 2) {
-      const uint32_t T = lop3<kLutMux>(xs[k], xs[k + 1] >> 1, kOdd);
       const uint32_t S = lop3<kLutMux>(xs[k] << 1, xs[k + 1], kOdd);
+      const uint32_t T = lop3<kLutMux>(xs[k], xs[k + 1] >> 1, kOdd) ^ S;
       n.nK += __popc(T);
       n.nKG += __popc(T & S);
       n.nUG += __popc(lop3<kLutAndNot>(T, S, 0u));

@@ -7,7 +7,11 @@
 // (Cx = Lx / 4, Cy = Ly / 4).  Each class row is stored as W = ceil(Cx / 16)
 // 32-bit words, 16 sites per word, site i at bits 2 (i mod 16) .. +1 of word
 // i / 16; the 16 classes are stored one after another (class c = 4 (y mod 4) +
-// (x mod 4)).  A colour phase updates all pairs (a, a + r) with a in one class:
+// (x mod 4)).  A site's two bits are its code in linear form: bit 0 the sign,
+// bit 1 the type XOR the sign (site codes 1 and 3 of the host buffers change
+// places), in which S = b1 - b0 and sigma = 1 - b1 - b0 hold for all four states:
+// the phases sum neighbours and the recount multiplies bonds without decoding
+// them; only the host buffers' conversions do (linear_code).  A colour phase updates all pairs (a, a + r) with a in one class:
 // the a-sites of one word are 16 pairs whose partners, and all their
 // neighbours, are 16 consecutive sites of other class rows -- fetched as one
 // shifted word ("window").
@@ -198,48 +202,39 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   return d;
 }
 
-// Neighbour sums of 16 sites held in four neighbour windows, in 4-bit lanes:
-// lane u of *_e is site 2u, of *_o site 2u + 1; value = sum over the four
-// neighbours of (S + 1) (s*) or (sigma + 1) (g*), in [0, 8].
-struct Sums {
-  uint32_t se, so, ge, go;
-};
-
-// Each window is first rewritten in the linear code (bit 1 = charged XOR
-// sign, bit 0 = sign), in which S = b1 - b0 and sigma = 1 - b1 - b0 hold for all
-// four states.  Two lane sums over the neighbours, c = sum (2 b1 + b0) and
-// n1 = sum b1, then give sum (S + 1) = 3 n1 - c + 4 and sum (sigma + 1) =
-// n1 - c + 8.  (Lane values may overflow in between; the 32-bit results are
-// exact because every final lane value lies in [0, 8].)
+// Host site codes <-> the linear form of the lattice words (its own inverse).
 __device__ __forceinline__ uint32_t linear_code(uint32_t X) {
   return X ^ ((X << 1) & 0xAAAAAAAAu);
 }
 
-__device__ __forceinline__ Sums neighbour_sums(uint32_t X0, uint32_t X1, uint32_t X2,
-                                               uint32_t X3) {
-  const uint32_t Y0 = linear_code(X0), Y1 = linear_code(X1), Y2 = linear_code(X2),
-                 Y3 = linear_code(X3);
-  const uint32_t E0 = Y0 & 0x33333333u, E1 = Y1 & 0x33333333u, E2 = Y2 & 0x33333333u,
-                 E3 = Y3 & 0x33333333u;
-  const uint32_t O0 = (Y0 >> 2) & 0x33333333u, O1 = (Y1 >> 2) & 0x33333333u,
-                 O2 = (Y2 >> 2) & 0x33333333u, O3 = (Y3 >> 2) & 0x33333333u;
-  const uint32_t ce = E0 + E1 + E2 + E3, co = O0 + O1 + O2 + O3;
-  const uint32_t ne = ((E0 & 0x22222222u) + (E1 & 0x22222222u) + (E2 & 0x22222222u) +
-                       (E3 & 0x22222222u)) >> 1;
-  const uint32_t no = ((O0 & 0x22222222u) + (O1 & 0x22222222u) + (O2 & 0x22222222u) +
-                       (O3 & 0x22222222u)) >> 1;
-  Sums s;
-  s.se = 3u * ne + 0x44444444u - ce;
-  s.so = 3u * no + 0x44444444u - co;
-  s.ge = ne + 0x88888888u - ce;
-  s.go = no + 0x88888888u - co;
-  return s;
+// One three-input logic instruction: kLut is the function's truth table on
+// the canonical inputs a = 0xF0, b = 0xCC, c = 0xAA.
+template <uint32_t kLut>
+__device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t d;
+  asm("lop3.b32 %0, %1, %2, %3, %4;" : "=r"(d) : "r"(a), "r"(b), "r"(c), "n"(kLut));
+  return d;
 }
+constexpr uint32_t kLutMux = 0xE4;      // c ? a : b, bit by bit
+constexpr uint32_t kLutAnd3 = 0x80;     // a & b & c
+constexpr uint32_t kLutXor3 = 0x96;     // a ^ b ^ c
+constexpr uint32_t kLutMaj = 0xE8;      // at least two of a, b, c
+constexpr uint32_t kLutXorAnd = 0x78;   // a ^ (b & c)
+constexpr uint32_t kLutAndXor = 0x6A;   // (a & b) ^ c
 
-// Byte lanes of group k (sites k, k + 4, k + 8, k + 12) from 4-bit lanes.
-__device__ __forceinline__ uint32_t group_bytes(uint32_t e, uint32_t o, int k) {
-  const uint32_t src = (k & 1) ? o : e;
-  return ((k & 2) ? (src >> 4) : src) & 0x0F0F0F0Fu;
+// The four neighbour windows of 16 sites added up bit by bit, as the three
+// bit planes of the counts (0 to 4): at a site's bits b1 and b0, the number of
+// its neighbours with that bit set is O + 2 T + 4 F.  Five logic instructions
+// for both counts of all 16 sites; adding 4-bit lanes (two masked sums a side,
+// neighbours decoded first) took 44.
+struct Planes {
+  uint32_t O, T, F;
+};
+
+__device__ __forceinline__ Planes neighbour_planes(uint32_t X0, uint32_t X1, uint32_t X2,
+                                                   uint32_t X3) {
+  const uint32_t s = lop3<kLutXor3>(X0, X1, X2), m = lop3<kLutMaj>(X0, X1, X2);
+  return Planes{s ^ X3, lop3<kLutXorAnd>(m, s, X3), lop3<kLutAnd3>(m, s, X3)};
 }
 
 }  // namespace ccmc

@@ -64,7 +64,7 @@ __global__ void init_kernel(Geo g, int h, int64_t n_plus, int64_t n_minus) {
       }
       word |= code << (2 * t);
     }
-    g.words[wid] = word;
+    g.words[wid] = linear_code(word);
   }
 }
 
@@ -213,7 +213,7 @@ __global__ void unpack_kernel(Geo g, uint8_t *out) {
     const int64_t rem = wid - (int64_t)cls * g.cstride;
     const int j = (int)(rem / g.W), w = (int)(rem - (int64_t)j * g.W);
     const int s0 = w << 4, n = min(16, g.Cx - s0);
-    const uint32_t X = g.words[wid];
+    const uint32_t X = linear_code(g.words[wid]);
     for (int t = 0; t < n; ++t) {
       const int64_t x = 4 * (s0 + t) + (cls & 3), y = 4 * j + (cls >> 2);
       out[y * g.Lx + x] = (uint8_t)((X >> (2 * t)) & 3u);
@@ -236,7 +236,7 @@ __global__ void pack_kernel(Geo g, const uint8_t *in, int *bad) {
       if (c > 3u) *bad = 1;
       X |= (c & 3u) << (2 * t);
     }
-    g.words[wid] = X;
+    g.words[wid] = linear_code(X);
   }
 }
 
@@ -284,7 +284,7 @@ __global__ void pack2_kernel(Geo g, const uint8_t *in) {
       uint32_t word = 0u;
 #pragma unroll
       for (int k = 0; k < 4; ++k) word |= gather_field(q[k], cx) << (8 * k);
-      g.words[(int64_t)(cy * 4 + cx) * g.cstride + (int64_t)j * g.W + w] = word;
+      g.words[(int64_t)(cy * 4 + cx) * g.cstride + (int64_t)j * g.W + w] = linear_code(word);
     }
   }
 }
@@ -303,7 +303,8 @@ __global__ void unpack2_kernel(Geo g, uint8_t *out) {
     uint32_t q[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int cx = 0; cx < 4; ++cx) {
-      const uint32_t word = g.words[(int64_t)(cy * 4 + cx) * g.cstride + (int64_t)j * g.W + w];
+      const uint32_t word =
+          linear_code(g.words[(int64_t)(cy * 4 + cx) * g.cstride + (int64_t)j * g.W + w]);
 #pragma unroll
       for (int k = 0; k < 4; ++k) q[k] |= scatter_field((word >> (8 * k)) & 0xFFu, cx);
     }

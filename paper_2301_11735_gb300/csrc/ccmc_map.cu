@@ -6,8 +6,9 @@
 // change with atomic XORs of their own bits.
 //
 // The move uses the library's own tables: the 64-bit move entry of the pair's
-// state, choice and kind (partner a nearest neighbour of a or not), the dp4a threshold offset from (sum_a (S+1) - sum_b (S+1) + 8,
-// sum_a (sigma+1), sum_b (sigma+1)) and the full 32-bit threshold.  Random
+// state, choice and kind (partner a nearest neighbour of a or not), the dp4a
+// threshold offset from the neighbours' bit counts (2 n1, n0 of a and b) and the
+// full 32-bit threshold.  Random
 // words of pair p of map m: the 16-bit field v = the low half of word 0 of
 // Philox(seed, (p, m_lo, m_hi, 11)) and, when v >= 65532 or its level w =
 // v / 12 ties the threshold's level, the slow words of Philox(seed, (p, m_lo,
@@ -42,9 +43,8 @@ __device__ __forceinline__ uint32_t code_at(const Geo &g, int x, int y) {
   return (*r.word >> r.shift) & 3u;
 }
 
-// S + 1 and sigma + 1 of a site code (0: s=+1/2, 1: s=-1/2, 2: S=+1, 3: S=-1)
-__device__ __forceinline__ uint32_t s_plus1(uint32_t c) { return (0x0211u >> (4 * c)) & 3u; }
-__device__ __forceinline__ uint32_t g_plus1(uint32_t c) { return (0x1102u >> (4 * c)) & 3u; }
+// A neighbour's contribution to (2 n1, n0), in the two low bytes.
+__device__ __forceinline__ uint32_t counts_of(uint32_t c) { return (c & 2u) | ((c & 1u) << 8); }
 
 __global__ void __launch_bounds__(256) map_kernel(Geo g, const int32_t *__restrict__ pairs,
                                                   int64_t npairs, uint32_t m_lo, uint32_t m_hi,
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256) map_kernel(Geo g, const int32_t *__restri
   const SiteRef ra = site_ref(g, ax, ay), rb = site_ref(g, bx, by);
   const uint32_t ca = (*ra.word >> ra.shift) & 3u, cb = (*rb.word >> rb.shift) & 3u;
   // neighbour sums (old states, partner included)
-  uint32_t SA = 0, GA = 0, SB = 0, GB = 0;
+  uint32_t nA = 0, nB = 0;
   bool near = false;
   {
     const int nx[4] = {ax == 0 ? Lx - 1 : ax - 1, ax + 1 == Lx ? 0 : ax + 1, ax, ax};
@@ -66,8 +66,7 @@ __global__ void __launch_bounds__(256) map_kernel(Geo g, const int32_t *__restri
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const uint32_t c = code_at(g, nx[k], ny[k]);
-      SA += s_plus1(c);
-      GA += g_plus1(c);
+      nA += counts_of(c);
       near |= (nx[k] == bx && ny[k] == by);
     }
   }
@@ -77,8 +76,7 @@ __global__ void __launch_bounds__(256) map_kernel(Geo g, const int32_t *__restri
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const uint32_t c = code_at(g, nx[k], ny[k]);
-      SB += s_plus1(c);
-      GB += g_plus1(c);
+      nB += counts_of(c);
     }
   }
   const U4 rw = philox((uint32_t)p, m_lo, m_hi, kTagMapMove, g.k0, g.k1);
@@ -96,10 +94,10 @@ __global__ void __launch_bounds__(256) map_kernel(Geo g, const int32_t *__restri
   }
   const uint32_t pc = (ca << 2) | cb;
   const uint2 e = trans[(2u * r + (near ? 1u : 0u)) * 16u + (pc ^ r)];
-  const uint32_t x = (e.y >> 24) & 15u;  // pc XOR the chosen configuration
+  const uint32_t x = e.x >> 24;  // pc XOR the chosen configuration
   if (x == 0u) return;           // the chosen configuration is the current one
-  const uint32_t env = (SA + 8u - SB) | (GA << 8) | (GB << 16);
-  const uint32_t thr = thr32[__dp4a((int)e.y, (int)env, (int)e.x) >> 1];
+  const uint32_t off = (uint32_t)__dp4a((int)e.y, (int)(nA | (nB << 16)), (int)e.x) & 0xFFFFu;
+  const uint32_t thr = thr32[off >> 1];
   bool accept;
   if (thr == 0xFFFFFFFFu) {
     accept = true;

@@ -28,7 +28,8 @@ namespace ccmc {
 // 4 code_a + code_b and its field v:
 //   w      = floor(v / 12), the choice class v - 12 w (v < 65532 = 12 x 5461)
 //   entry  = trans[v - 12 w][near][pc] -> base, byte coefficients, pc XOR npc
-//   offset = dp4a(coefficients, (D8, GA, GB, 0), base)  (byte offset of the level)
+//   offset = dp4a(coefficients, (2 n1_a, n0_a, 2 n1_b, n0_b), base), n1 and n0 the
+//            neighbours with bit 1, bit 0 set (byte offset of the level)
 //   accept = w < T(offset), with T = floor(5461 thr / 2^32) (5461 when thr is
 //            0xFFFFFFFF): w < T implies w 2^32 + s < 5461 thr for every 32-bit
 //            s, w > T the opposite
@@ -109,22 +110,21 @@ __device__ __forceinline__ uint32_t window(const uint32_t *cls, const Geo &g, co
   }
 }
 
-// Move entry of choice class r (v mod 12) and pc8 = 8 pc + 128 near: entry
+// Move entry of choice class r (v mod 12) and r264 = 264 r + 128 near: entry
 // (2 r + near) 16 + (pc XOR r) of the move table, at byte offset
-// 256 r + 128 near + 8 (pc XOR r) = (264 r) XOR pc8.  The XOR spreads a warp's
+// 256 r + 128 near + 8 (pc XOR r) = r264 XOR 8 pc.  The XOR spreads a warp's
 // lookups over the banks: with entry (2 r + near) 16 + pc the bank pair of a
 // lookup was its pair state alone, and the few common states (both sites
 // magnetic) piled onto four of sixteen bank pairs.  Word 0: the level
-// offset's base; word 1: the signed byte coefficients of (D8, GA, GB) and, at
-// bits 24-27 (the byte dp4a multiplies by zero), the move pc XOR npc.
-__device__ __forceinline__ uint2 move_entry(const uint2 *trans, uint32_t r, uint32_t pc8) {
-  return *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(trans) +
-                                          ((r * 264u) ^ pc8));
+// offset's base and, at bits 24-27, the move pc XOR npc; word 1: the signed byte
+// coefficients of (2 n1_a, n0_a, 2 n1_b, n0_b).
+__device__ __forceinline__ uint2 move_entry(const uint2 *trans, uint32_t off) {
+  return *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(trans) + off);
 }
 
 // The threshold level at byte offset `off` (the offset is formed in bytes, so
 // that it is the load's address without a shift).
-__device__ __forceinline__ uint32_t level_at(const uint16_t *thrT, int off) {
+__device__ __forceinline__ uint32_t level_at(const uint16_t *thrT, uint32_t off) {
   return *reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(thrT) + off);
 }
 
@@ -132,42 +132,44 @@ __device__ __forceinline__ uint32_t level_at(const uint16_t *thrT, int off) {
 // m = ceil(2^32 / 12) is exact there.
 __device__ __forceinline__ uint32_t div12(uint32_t v) { return __umulhi(v, 357913942u); }
 
-// The pair's move nibble (a bits 2-3, b bits 0-1) in an entry's word 1.
-__device__ __forceinline__ uint32_t move_nibble(uint32_t ey) { return (ey >> 24) & 15u; }
+// A pair's neighbour counts as dp4a's byte operands.  A word's pairs form four
+// groups k (sites k, k + 4, k + 8, k + 12: one a byte); group k = 2 c + h is
+// half h of MOVE call c.
+constexpr uint32_t kEnvMask = 0x070E070Eu;  // 2 n1 at bits 1-3, n0 at bits 0-2 of a nibble
 
-// Byte lanes of one pair group (sites k, k + 4, k + 8, k + 12): x01/x23 hold
-// (D8, GA) of lanes 0, 1 / 2, 3, gb the GB of its four lanes, pc8 the
-// move-table offsets 8 pc + near128.
-struct Group {
-  uint32_t x01, x23, gb, pc8;
+// The counts of half h's pairs of both calls: byte q of ev[q] .. is lane q's
+// (2 n1_a, n0_a, 2 n1_b, n0_b), call 0 in the low nibbles, call 1 in the high
+// ones (bits outside kEnvMask are whatever the planes hold there).  Two
+// selections put a count's three bits side by side (its unwanted neighbours
+// are masked with the nibble), then eight byte permutes transpose the four
+// counts: 30 instructions for eight pairs, where masked additions, byte
+// extraction per group and a permute per pair took about 70.
+struct Env {
+  uint32_t ev[4];
 };
 
-__device__ __forceinline__ Group group_env(const Sums &sa, const Sums &sb, uint32_t pcE,
-                                           uint32_t pcO, uint32_t near128, int k) {
-  const uint32_t d8 = group_bytes(sa.se, sa.so, k) + 0x08080808u - group_bytes(sb.se, sb.so, k);
-  const uint32_t ga = group_bytes(sa.ge, sa.go, k);
-  Group gr;
-  gr.gb = group_bytes(sb.ge, sb.go, k);
-  gr.x01 = prmt(d8, ga, 0x5140u);
-  gr.x23 = prmt(d8, ga, 0x7362u);
-  gr.pc8 = group_bytes(pcE, pcO, k) * 8u + near128 * 0x01010101u;
-  return gr;
-}
-
-// dp4a operand (D8, GA, GB, 0) of lane q of a group (q a compile-time constant
-// in the unrolled loops).
-__device__ __forceinline__ uint32_t lane_env(const Group &gr, int q) {
-  return q == 0 ? prmt(gr.x01, gr.gb, 0x8410u)
-       : q == 1 ? prmt(gr.x01, gr.gb, 0x8532u)
-       : q == 2 ? prmt(gr.x23, gr.gb, 0x8610u)
-                : prmt(gr.x23, gr.gb, 0x8732u);
+__device__ __forceinline__ Env half_env(const Planes &a, const Planes &b, int h) {
+  // bits of half h's sites at the low two bits of every nibble
+  const uint32_t m1 = 0x22222222u, m2 = 0x88888888u, m3 = 0x11111111u, m4 = 0x44444444u;
+  const uint32_t aO = h ? a.O >> 2 : a.O, aT = h ? a.T >> 1 : a.T << 1,
+                 aF = h ? a.F : a.F << 2;
+  const uint32_t bO = h ? b.O >> 2 : b.O, bT = h ? b.T >> 1 : b.T << 1,
+                 bF = h ? b.F : b.F << 2;
+  const uint32_t a1 = lop3<kLutMux>(aF, lop3<kLutMux>(aO, aT, m1), m2);
+  const uint32_t a0 = lop3<kLutMux>(aF, lop3<kLutMux>(aO, aT, m3), m4);
+  const uint32_t b1 = lop3<kLutMux>(bF, lop3<kLutMux>(bO, bT, m1), m2);
+  const uint32_t b0 = lop3<kLutMux>(bF, lop3<kLutMux>(bO, bT, m3), m4);
+  const uint32_t x01 = prmt(a1, a0, 0x5140u), x23 = prmt(a1, a0, 0x7362u);
+  const uint32_t y01 = prmt(b1, b0, 0x5140u), y23 = prmt(b1, b0, 0x7362u);
+  return Env{{prmt(x01, y01, 0x5410u), prmt(x01, y01, 0x7632u), prmt(x23, y23, 0x5410u),
+              prmt(x23, y23, 0x7632u)}};
 }
 
 // The inputs of a word's pairs: its a word, its b window and the neighbour
-// sums of both sides.
+// counts of both sides.
 struct WordIn {
   uint32_t A, B;
-  Sums sa, sb;
+  Planes na, nb;
 };
 
 // Row jr + dy of a class (periodic in Cy); staged bands start at the right row.
@@ -183,22 +185,28 @@ __device__ __forceinline__ WordIn gather(const Geo &g, const PhaseU &u, int jr, 
   in.A = u.cA[jr * g.W + w];
   const int jb = band_row<kMode>(g, jr, u.qy);
   in.B = window<kMode>(u.cB, g, u, jb, w, u.offB, n);
-  in.sa = neighbour_sums(window<kMode>(u.cAL, g, u, jr, w, u.offAL, n),
+  in.na = neighbour_planes(window<kMode>(u.cAL, g, u, jr, w, u.offAL, n),
                          window<kMode>(u.cAR, g, u, jr, w, u.offAR, n),
                          u.cAU[band_row<kMode>(g, jr, u.dyAU) * g.W + w],
                          u.cAD[band_row<kMode>(g, jr, u.dyAD) * g.W + w]);
-  in.sb = neighbour_sums(window<kMode>(u.cBL, g, u, jb, w, u.offBL, n),
+  in.nb = neighbour_planes(window<kMode>(u.cBL, g, u, jb, w, u.offBL, n),
                          window<kMode>(u.cBR, g, u, jb, w, u.offBR, n),
                          window<kMode>(u.cBU, g, u, band_row<kMode>(g, jb, u.dyBU), w, u.offB, n),
                          window<kMode>(u.cBD, g, u, band_row<kMode>(g, jb, u.dyBD), w, u.offB, n));
   return in;
 }
 
-__device__ __forceinline__ uint32_t pcE_of(const WordIn &in) {
-  return ((in.A & 0x33333333u) << 2) | (in.B & 0x33333333u);
+// The pair states pc (a's code above b's) of half h's pairs: lane q of call c at
+// bits 8 q + 4 c .. + 3.
+__device__ __forceinline__ uint32_t half_pc(const WordIn &in, int h) {
+  return h ? lop3<kLutMux>(in.A, in.B >> 2, 0xCCCCCCCCu)
+           : lop3<kLutMux>(in.A << 2, in.B, 0xCCCCCCCCu);
 }
-__device__ __forceinline__ uint32_t pcO_of(const WordIn &in) {
-  return (in.A & 0xCCCCCCCCu) | ((in.B >> 2) & 0x33333333u);
+
+// 264 r + 128 near XOR 8 pc, the move entry's offset (pcs >> sh: the pair's pc
+// at bits 3-6; sh < 0 shifts left).
+__device__ __forceinline__ uint32_t entry_offset(uint32_t pcs, int sh, uint32_t r264) {
+  return lop3<kLutAndXor>(sh < 0 ? pcs << -sh : pcs >> sh, 0x78u, r264);
 }
 
 // The fast path of the pairs of a word one thread evaluates: kTPW threads
@@ -219,43 +227,48 @@ __device__ __forceinline__ uint3 fast_moves(const Geo &g, const uint2 *trans,
   constexpr int kHalves = kTPW == 4 ? 1 : 2;
   const int c0 = kTPW == 1 ? 0 : (kTPW == 2 ? sub : sub >> 1);
   const int h0 = kTPW == 4 ? (sub & 1) : 0;
-  const uint32_t pcE = pcE_of(in), pcO = pcO_of(in);
   const uint32_t gbase = (uint32_t)j * (uint32_t)(2 * g.W) + (uint32_t)(2 * w);
+  Env env[kHalves];
+  uint32_t pcs[kHalves];
+#pragma unroll
+  for (int hi = 0; hi < kHalves; ++hi) {
+    env[hi] = half_env(in.na, in.nb, h0 + hi);
+    pcs[hi] = half_pc(in, h0 + hi);
+  }
   uint32_t dA = 0u, dB = 0u, slow = 0u;
 #pragma unroll
   for (int ci = 0; ci < kCalls; ++ci) {
     const int c = c0 + ci;
     const U4 r = keys(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE);
-    uint32_t mn = 0xFFFFFFFFu, mx = 0u;  // smallest w - T, largest v of the call
+    uint32_t mn = 0xFFFFFFFFu;  // smallest w - T of the call
 #pragma unroll
     for (int hi = 0; hi < kHalves; ++hi) {
       const int h = h0 + hi;
       const int k = 2 * c + h;
-      const Group gr = group_env(in.sa, in.sb, pcE, pcO, near128, k);
-      uint32_t acc = 0u;  // byte q: the accepted move of lane q
-      uint32_t d0 = 0xFFFFFFFFu, v0 = 0u;
+      uint32_t d[4], t[4];
 #pragma unroll
-      for (int q = 3; q >= 0; --q) {
+      for (int q = 0; q < 4; ++q) {
         const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
         const uint32_t v = h ? X >> 16 : X & 0xFFFFu;
         const uint32_t wq = div12(v);
-        const uint2 e = move_entry(trans, v - 12u * wq, prmt(gr.pc8, 0u, 0x4440u + (uint32_t)q));
-        const uint32_t T = level_at(thrT, __dp4a((int)e.y, (int)lane_env(gr, q), (int)e.x));
-        const uint32_t d = wq - T;  // negative: accept; zero: a tie
-        if (q & 1) {
-          d0 = d;
-          v0 = v;
-        } else {
-          mn = __vimin3_u32(mn, d0, d);
-          mx = __vimax3_u32(mx, v0, v);
-        }
-        acc = __funnelshift_l((int)d < 0 ? e.y : 0u, acc, 8);
+        const uint2 e = move_entry(
+            trans, entry_offset(pcs[hi], 8 * q + 4 * c - 3, (v - 12u * wq) * 264u + near128));
+        t[q] = (uint32_t)__dp4a((int)e.y, (int)((env[hi].ev[q] >> (4 * c)) & kEnvMask), (int)e.x);
+        d[q] = wq - level_at(thrT, t[q] & 0xFFFFu);  // negative: accept; zero: a tie
       }
+      mn = __vimin3_u32(mn, d[0], d[1]);
+      mn = __vimin3_u32(mn, d[2], d[3]);
+      // byte q: the accepted move of lane q, i.e. byte 3 of t[q] under the sign
+      // of d[q] (byte permutes: bit 3 of a selector replicates a byte's sign)
+      const uint32_t acc = prmt(prmt(d[0], d[1], 0x00FBu), prmt(d[2], d[3], 0x00FBu), 0x5410u) &
+                           prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
       // byte q of acc -> site k + 4 q: b bits to 2 (k + 4 q) of dB, a bits of dA
       dB |= (acc & 0x03030303u) << (2 * k);
       dA |= ((acc >> 2) & 0x03030303u) << (2 * k);
     }
-    if (mn == 0u || mx >= 65532u) slow |= 1u << c;
+    // a rare pair: a tie, or a field >= 65532 in either half of the call's words
+    const uint32_t mx = __vmaxu2(__vimax3_u16x2(r.x, r.y, r.z), r.w);
+    if (mn == 0u || mx >= 0xFFFC0000u || (mx & 0xFFFFu) >= 0xFFFCu) slow |= 1u << c;
   }
   return make_uint3(dA, dB, slow);
 }
@@ -323,24 +336,28 @@ __device__ __forceinline__ void exact_pair(const Geo &g, const PhaseU &u, const 
   const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
   const uint32_t v = h ? X >> 16 : X & 0xFFFFu;
   const uint32_t wq = div12(v);
-  const Group gr = group_env(in.sa, in.sb, pcE_of(in), pcO_of(in), near128, k);
-  const uint32_t pc8 = prmt(gr.pc8, 0u, 0x4440u + (uint32_t)q);
-  const uint32_t env = prmt(q < 2 ? gr.x01 : gr.x23, gr.gb,
-                            0x8410u + ((q & 1) ? 0x0122u : 0u) + ((q & 2) ? 0x0200u : 0u));
-  uint2 e = move_entry(trans, v - 12u * wq, pc8);
-  if (v < 65532u && wq != level_at(thrT, __dp4a((int)e.y, (int)env, (int)e.x)))
+  // the pair's own counts and state, from bits 2 t and 2 t + 1 of the planes
+  auto counts = [&](const Planes &p) {
+    const uint32_t O = p.O >> (2 * t), T = p.T >> (2 * t), F = p.F >> (2 * t);
+    return ((O & 2u) + 2u * (T & 2u) + 4u * (F & 2u)) |
+           (((O & 1u) + 2u * (T & 1u) + 4u * (F & 1u)) << 8);
+  };
+  const uint32_t env = counts(in.na) | (counts(in.nb) << 16);
+  const uint32_t pc8 = ((((in.A >> (2 * t)) & 3u) << 2) | ((in.B >> (2 * t)) & 3u)) << 3;
+  uint2 e = move_entry(trans, ((v - 12u * wq) * 264u + near128) ^ pc8);
+  if (v < 65532u && wq != level_at(thrT, (uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu))
     return;  // not rare
   const uint32_t slow0 = (uint32_t)((uint64_t)j * g.Cx + (uint32_t)(w << 4));
   const U4 sl = philox(slow0 + (uint32_t)t, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, g.k0, g.k1);
   if (v >= 65532u) {
     if (sl.y >= 4294967292u) return;  // keep the current configuration
-    e = move_entry(trans, sl.y % 12u, pc8);
+    e = move_entry(trans, ((sl.y % 12u) * 264u + near128) ^ pc8);
   }
-  const uint32_t thr = thr32[__dp4a((int)e.y, (int)env, (int)e.x) >> 1];
+  const uint32_t thr = thr32[((uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu) >> 1];
   const bool accept = thr == 0xFFFFFFFFu ||
                       (v < 65532u ? ((uint64_t)wq << 32) + sl.x < 5461ull * thr : sl.x < thr);
   if (accept) {
-    const uint32_t x = move_nibble(e.y);
+    const uint32_t x = e.x >> 24;
     apply_moves<kMode, false>(g, u, jr, w, n, (x >> 2) << (2 * t), (x & 3u) << (2 * t));
   }
 }
@@ -383,14 +400,12 @@ __device__ __forceinline__ void warp_word(const Geo &g, const PhaseU &u, const u
       WordIn o;
       o.A = __shfl_sync(0xFFFFFFFFu, in.A, src);
       o.B = __shfl_sync(0xFFFFFFFFu, in.B, src);
-      o.sa.se = __shfl_sync(0xFFFFFFFFu, in.sa.se, src);
-      o.sa.so = __shfl_sync(0xFFFFFFFFu, in.sa.so, src);
-      o.sa.ge = __shfl_sync(0xFFFFFFFFu, in.sa.ge, src);
-      o.sa.go = __shfl_sync(0xFFFFFFFFu, in.sa.go, src);
-      o.sb.se = __shfl_sync(0xFFFFFFFFu, in.sb.se, src);
-      o.sb.so = __shfl_sync(0xFFFFFFFFu, in.sb.so, src);
-      o.sb.ge = __shfl_sync(0xFFFFFFFFu, in.sb.ge, src);
-      o.sb.go = __shfl_sync(0xFFFFFFFFu, in.sb.go, src);
+      o.na.O = __shfl_sync(0xFFFFFFFFu, in.na.O, src);
+      o.na.T = __shfl_sync(0xFFFFFFFFu, in.na.T, src);
+      o.na.F = __shfl_sync(0xFFFFFFFFu, in.na.F, src);
+      o.nb.O = __shfl_sync(0xFFFFFFFFu, in.nb.O, src);
+      o.nb.T = __shfl_sync(0xFFFFFFFFu, in.nb.T, src);
+      o.nb.F = __shfl_sync(0xFFFFFFFFu, in.nb.F, src);
       const int oj = __shfl_sync(0xFFFFFFFFu, j, src), ojr = __shfl_sync(0xFFFFFFFFu, jr, src),
                 ow = __shfl_sync(0xFFFFFFFFu, w, src), on = __shfl_sync(0xFFFFFFFFu, n, src);
       // the owner's pairs, one a lane: 16 (both calls), 8 (one call) or 4

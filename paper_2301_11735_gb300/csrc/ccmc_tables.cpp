@@ -59,15 +59,19 @@ void build_device_thresholds(double beta, double Delta, double V, double J, uint
 //   dBV = dS_a sum_<a> S + dS_b sum_<b> S + m dS_a dS_b
 //   dBJ = dsig_a sum_<a> sigma + dsig_b sum_<b> sigma + m dsig_a dsig_b
 // with neighbour sums over old states (partner included) and m = near the number
-// of a-b bonds.  As dS_b = -dS_a, the byte offset of the move's 16-bit level,
-// twice its index in its segment's stride (sS entries a unit of dBV, sG a unit
-// of dBJ), is an affine function of the biased sums D8 = sum_<a> S - sum_<b> S
-// + 8, GA = sum_<a> sigma + 4, GB = sum_<b> sigma + 4:
-//   offset = base + (2 sS dS_a) D8 + (2 sG dsig_a) GA + (2 sG dsig_b) GB.
-// Entry (2 r + near) * 16 + (pc XOR r): word 0 holds base; word 1 the signed byte
-// coefficients of (D8, GA, GB) and, in bits 24-27 (byte 3, which
-// the phase kernel multiplies by zero; bits 28-31 stay clear), pc XOR npc.
+// of a-b bonds.  With n1, n0 the numbers of a site's neighbours whose linear
+// code has bit 1, bit 0 set, sum S = n1 - n0 and sum sigma = 4 - n1 - n0.  As
+// dS_b = -dS_a, the byte offset of the move's 16-bit level, twice its index in
+// its segment's strides (sS entries a unit of dBV, sG a unit of dBJ), is an
+// affine function of 2 n1 and n0 of both sides:
+//   offset = base + (sS dS_a - sG dsig_a) 2 n1_a - 2 (sS dS_a + sG dsig_a) n0_a
+//                 + (sS dS_b - sG dsig_b) 2 n1_b - 2 (sS dS_b + sG dsig_b) n0_b.
+// Entry (2 r + near) * 16 + (pc XOR r), pc the pair's two linear codes: word 0
+// holds base in its low half and, in bits 24-27, the move pc XOR npc (both
+// survive the sum, whose value stays below 2^16); word 1 the four signed byte
+// coefficients.
 namespace {
+constexpr int kLinear[4] = {0, 3, 2, 1};  // a site code's linear form (ccmc_device.cuh)
 constexpr int kSetN[3] = {4, 6, 4};  // q = +1, 0, -1
 constexpr int kSets[3][6][2] = {
     {{2, 0}, {2, 1}, {0, 2}, {1, 2}, {0, 0}, {0, 0}},  // q = +1
@@ -78,8 +82,9 @@ constexpr int kSets[3][6][2] = {
 
 bool build_transitions(uint32_t *trans) {
   bool ok = true;
-  for (int pc = 0; pc < 16; ++pc) {
-    const int ca = pc >> 2, cb = pc & 3;
+  for (int codes = 0; codes < 16; ++codes) {
+    const int ca = codes >> 2, cb = codes & 3;
+    const int pc = (kLinear[ca] << 2) | kLinear[cb];
     const int q = kS[ca] + kS[cb];
     for (int r = 0; r < 12; ++r) {
       int na = ca, nb = cb;
@@ -98,30 +103,30 @@ bool build_transitions(uint32_t *trans) {
       const int first = kind == 0 ? (dQ + 2) / 2 * kSegW * kSegW : kind == 1 ? kSegSwap : kSegFlip;
       const int end = first + (kind == 0 ? kSegW * kSegW : kNB);
       const int zero = first + (kind == 0 ? kSegR * kSegW + kSegR : kDB);
-      const int cS = 2 * sS * dSa, cA = 2 * sG * dGa, cB = 2 * sG * dGb;
-      const int base = 2 * zero - 8 * cS - 4 * (cA + cB);
-      const uint32_t x = (uint32_t)(((ca ^ na) << 2) | (cb ^ nb));
-      const uint32_t coef = ((uint32_t)cS & 0xFFu) | (((uint32_t)cA & 0xFFu) << 8) |
-                            (((uint32_t)cB & 0xFFu) << 16) | (x << 24);
+      const int cA1 = sS * dSa - sG * dGa, cA0 = -2 * (sS * dSa + sG * dGa);
+      const int cB1 = sS * dSb - sG * dGb, cB0 = -2 * (sS * dSb + sG * dGb);
+      const int base = 2 * zero + 8 * sG * (dGa + dGb);
+      const uint32_t x = (uint32_t)(pc ^ ((kLinear[na] << 2) | kLinear[nb]));
+      const uint32_t coef = ((uint32_t)cA1 & 0xFFu) | (((uint32_t)cA0 & 0xFFu) << 8) |
+                            (((uint32_t)cB1 & 0xFFu) << 16) | ((uint32_t)cB0 << 24);
       for (int near = 0; near < 2; ++near) {
         const int e = (2 * r + near) * 16 + (pc ^ r);  // bank-spread (see the phase kernel)
         const int b = base + near * 2 * (sS * dSa * dSb + sG * dGa * dGb);
-        trans[2 * e] = (uint32_t)b;
+        trans[2 * e] = (uint32_t)b + (x << 24);
         trans[2 * e + 1] = coef;
-        // every offset the entry can form, over all neighbour sums (D8 in [0, 16],
-        // GA and GB in [0, 8]), and both its energy terms, stay inside the segment
-        for (int D8 : {0, 16})
-          for (int ga : {0, 8})
-            for (int gb : {0, 8}) {
-              const int off = b + cS * D8 + cA * ga + cB * gb;
-              const int dBV = dSa * (D8 - 8) + near * dSa * dSb;
-              const int dBJ = dGa * (ga - 4) + dGb * (gb - 4) + near * dGa * dGb;
-              const int reach = kind == 0 ? kSegR : kDB;
-              ok = ok && off >= 2 * first && off < 2 * end && (off & 1) == 0;
-              ok = ok && (kind == 1 ? dGa == 0 && dGb == 0 : dBJ >= -reach && dBJ <= reach);
-              ok = ok && (kind == 2 ? dSb == 0 : dBV >= -reach && dBV <= reach);
-              ok = ok && (kind == 0 || dQ == 0);
-            }
+        // every offset the entry can form, over all neighbour counts (linear in
+        // them: the corners), and both its energy terms, stay inside the segment
+        for (int c = 0; c < 16; ++c) {
+          const int a1 = c & 1 ? 4 : 0, a0 = c & 2 ? 4 : 0, b1 = c & 4 ? 4 : 0, b0 = c & 8 ? 4 : 0;
+          const int off = b + 2 * cA1 * a1 + cA0 * a0 + 2 * cB1 * b1 + cB0 * b0;
+          const int dBV = dSa * (a1 - a0) + dSb * (b1 - b0) + near * dSa * dSb;
+          const int dBJ = dGa * (4 - a1 - a0) + dGb * (4 - b1 - b0) + near * dGa * dGb;
+          const int reach = kind == 0 ? kSegR : kDB;
+          ok = ok && off == 2 * (zero + sS * dBV + sG * dBJ);
+          ok = ok && off >= 2 * first && off < 2 * end && (kind == 0 || dQ == 0);
+          ok = ok && (kind == 1 ? dGa == 0 && dGb == 0 : dBJ >= -reach && dBJ <= reach);
+          ok = ok && (kind == 2 ? dSb == 0 : dBV >= -reach && dBV <= reach);
+        }
       }
     }
   }
