@@ -1,9 +1,10 @@
 """Build ``libccmc.so`` in-tree (``paper_2301_11735_gb300/_build``) for sm_103a.
 
-Nine translation units are compiled in parallel and linked into one shared
+Ten translation units are compiled in parallel and linked into one shared
 library that exports the C ABI of ``include/ccmc.h``:
 
 * ``csrc/ccmc_phase.cu``   -- the colour-phase kernels (nvcc, sm_103a only);
+* ``csrc/ccmc_resident.cu`` -- whole sweeps of lattices held in shared memory;
 * ``csrc/ccmc_map.cu``     -- the paper-faithful map mode's kernel;
 * ``csrc/ccmc_maps.cpp``   -- host map generation (g++, host threads);
 * ``csrc/ccmc_kernels.cu`` -- the other CUDA kernels (init, recount, packing);
@@ -66,6 +67,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_verbose: bool = Fals
         common += ["-Xptxas", "-v"]
     jobs = {
         "ccmc_phase.o": [nvcc, "-c", *common, os.path.join(CSRC, "ccmc_phase.cu")],
+        "ccmc_resident.o": [nvcc, "-c", *common, os.path.join(CSRC, "ccmc_resident.cu")],
         "ccmc_map.o": [nvcc, "-c", *common, os.path.join(CSRC, "ccmc_map.cu")],
         "ccmc_kernels.o": [nvcc, "-c", *common, os.path.join(CSRC, "ccmc_kernels.cu")],
         "ccmc_api.o": [nvcc, "-c", *common, os.path.join(CSRC, "ccmc_api.cu")],

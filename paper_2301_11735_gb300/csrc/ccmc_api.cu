@@ -116,6 +116,7 @@ struct ccmc_lattice {
   bool have_params = false;
   double params[4] = {0, 0, 0, 0};  // beta, Delta, V, J
   LaunchCfg cfg{};
+  bool resident = false;  // may be swept by the resident kernel
   std::vector<GraphEntry> graphs;
   int32_t *d_maps = nullptr;  // paper-map mode: uploaded pairs
   int64_t map_cap = 0;        // int32 entries held by d_maps
@@ -123,6 +124,13 @@ struct ccmc_lattice {
 };
 
 namespace {
+
+// Lattices that the resident kernel sweeps unless the caller says otherwise: up
+// to 4608 a-words a phase (1024^2 has 4096), 288 a CTA of a cluster of 16, where
+// a launch of a phase's own begins to be as fast (1024^2: 3.2 us a phase
+// resident, 3.7 us a launch; 1000^2, ragged: 3.4 against 4.6; 256^2: 1.4 against
+// 3.3; 64^2: 0.7 against 3.3).
+bool resident_default(const Geo &g) { return g.cstride <= 4608; }
 
 int validate_shape(int Lx, int Ly) {
   if (Lx < 4 || Ly < 4 || (Lx & 3) || (Ly & 3)) return CCMC_E_INVAL;
@@ -202,6 +210,32 @@ int run_graph(ccmc_lattice *h, int sweeps, int obs_every) {
     hit = &h->graphs.back();
   }
   CK(cudaGraphLaunch(hit->exec, h->stream));
+  return CCMC_OK;
+}
+
+ResJob resident_job(const ccmc_lattice *h, int64_t nsweeps, int obs_every, int rows) {
+  ResJob j{};
+  j.g = h->g;
+  j.thrT = h->t.thrT;
+  j.thr32 = h->t.thr32;
+  j.nsweeps = (int)nsweeps;
+  j.ring = h->d_ring;
+  j.ring_cap = h->ring_cap;
+  j.hist = h->d_hist;
+  j.nbins = h->nbins;
+  j.obs_every = obs_every;
+  j.rows = rows;
+  return j;
+}
+
+// Sweep one lattice by the resident kernel, a bounded number of sweeps a launch.
+int resident_sweeps(ccmc_lattice *h, int64_t nsweeps, int obs_every) {
+  const ResShape sh = resident_shape(h->g, kResMaxCluster, 0.0, 512, 4);
+  for (int64_t s = 0; s < nsweeps; s += kResMaxSweeps) {
+    const ResJob j =
+        resident_job(h, std::min<int64_t>(nsweeps - s, kResMaxSweeps), obs_every, sh.rows);
+    CK(launch_resident_sweep(&j, nullptr, 1, sh, (h->g.Cx & 15) == 0, h->stream));
+  }
   return CCMC_OK;
 }
 
@@ -299,6 +333,9 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
       }
     }
   }
+  // the variables that select a phase kernel keep the lattice on that kernel
+  h->resident = resident_default(g) && !std::getenv("CCMC_NO_TILE") &&
+                !std::getenv("CCMC_TILE_GRID") && !std::getenv("CCMC_NO_RESIDENT") && resident_ready();
   while (((int64_t)1 << (2 * h->h)) < (int64_t)N) ++h->h;
   h->ring_cap = obs_capacity > 0 ? obs_capacity : 4096;
   cudaGetDevice(&h->device);
@@ -511,6 +548,12 @@ int ccmc_sweep(ccmc_lattice *h, int64_t nsweeps, double beta, double Delta, doub
                         h->stream));
     --nsweeps;
   }
+  if (h->resident) {
+    rc = resident_sweeps(h, nsweeps, obs_every);
+    if (rc) return rc;
+    h->phases_done += 8 * nsweeps;
+    return CCMC_OK;
+  }
   rc = drive_sweeps(
       h->phases_done / 8, nsweeps, obs_every,
       [&](int g, int obs) { return run_graph(h, g, obs); },
@@ -717,15 +760,16 @@ struct ccmc_batch {
   int cap = 0;  // largest number of lattices one launch may hold
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  JobDesc *d_jobs = nullptr;
-  int *d_queue = nullptr;
+  ResJob *d_jobs = nullptr;  // resident lattices
   int threads = 256;
-  int64_t resident_max_sites = (int64_t)1 << 18;
+  int64_t resident_max_sites = -1;  // -1: the lattices that ccmc_sweep holds resident
   int ctas_per_sm = 2;
   int max_tpw = 4;
   int sms = 152;
   cudaEvent_t ev = nullptr;
   std::vector<cudaEvent_t> lat_ev;
+  std::vector<cudaStream_t> side;   // resident launches of different shapes run side by side
+  std::vector<cudaEvent_t> side_ev;
   MultiJob *d_multi = nullptr;  // lock-step groups of large lattices
   struct MultiGraph {
     std::vector<ccmc_lattice *> members;
@@ -737,20 +781,96 @@ struct ccmc_batch {
 };
 
 namespace {
-JobDesc job_of(ccmc_lattice *h, int64_t nsweeps, int obs_every) {
-  JobDesc d{};
-  d.g = h->g;
-  d.thrT = h->t.thrT;
-  d.thr32 = h->t.thr32;
-  d.trans = h->t.trans;
-  d.nsweeps = nsweeps;
-  d.ring = h->d_ring;
-  d.ring_cap = h->ring_cap;
-  d.hist = h->d_hist;
-  d.nbins = h->nbins;
-  d.obs_every = obs_every;
-  return d;
+
+// Whether a batch holds a lattice in shared memory: below the configured limit, or
+// what ccmc_sweep would hold.
+bool batch_resident(const ccmc_batch *b, const ccmc_lattice *h) {
+  if (b->resident_max_sites < 0) return h->resident;
+  return 16 * h->g.cstride * 16 <= b->resident_max_sites;
 }
+
+// A resident launch of a batch: lattices of one shape.
+struct ResGroup {
+  ResShape shape;
+  bool aligned;
+  double cost;             // of its longest lattice
+  std::vector<ResJob> jobs;
+};
+
+constexpr int kSideStreams = 8;
+
+int side_streams(ccmc_batch *b, int n) {
+  while ((int)b->side.size() < n) {
+    cudaStream_t s = nullptr;
+    cudaEvent_t e = nullptr;
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return CCMC_E_CUDA;
+    b->side.push_back(s);
+    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return CCMC_E_CUDA;
+    b->side_ev.push_back(e);
+  }
+  return CCMC_OK;
+}
+
+// Queue the resident launches of lats[which] (ordered after the batch stream's
+// work; the batch stream waits for them).
+int run_resident(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats,
+                 const std::vector<int> &which, const int64_t *nsweeps, const int *obs_every) {
+  // every lattice's share of the CTAs the GPU holds, by its words a phase
+  double words = 0;
+  for (int i : which) words += (double)lats[i]->g.cstride;
+  const double ctas = (double)b->sms * b->ctas_per_sm;
+  std::vector<ResGroup> groups;
+  for (int i : which) {
+    ccmc_lattice *h = lats[i];
+    const ResShape sh =
+        resident_shape(h->g, ctas * (double)h->g.cstride / words, words / b->sms,
+                       b->threads, b->max_tpw);
+    const bool al = (h->g.Cx & 15) == 0;
+    ResGroup *hit = nullptr;
+    for (ResGroup &G : groups)
+      if (G.shape.cluster == sh.cluster && G.shape.tpw == sh.tpw &&
+          G.shape.threads == sh.threads && G.aligned == al)
+        hit = &G;
+    if (!hit) {
+      groups.push_back(ResGroup{sh, al, 0.0, {}});
+      hit = &groups.back();
+    }
+    hit->shape.smem = std::max(hit->shape.smem, sh.smem);
+    hit->cost = std::max(hit->cost, (double)sh.rows * h->g.W * (double)nsweeps[i]);
+    hit->jobs.push_back(resident_job(h, nsweeps[i], obs_every[i], sh.rows));
+  }
+  // the longest first, in every launch and over the launches
+  std::sort(groups.begin(), groups.end(),
+            [](const ResGroup &x, const ResGroup &y) { return x.cost > y.cost; });
+  std::vector<ResJob> jobs;
+  for (ResGroup &G : groups) {
+    std::stable_sort(G.jobs.begin(), G.jobs.end(), [](const ResJob &x, const ResJob &y) {
+      return (double)x.rows * x.g.W * x.nsweeps > (double)y.rows * y.g.W * y.nsweeps;
+    });
+    jobs.insert(jobs.end(), G.jobs.begin(), G.jobs.end());
+  }
+  CK(cudaMemcpyAsync(b->d_jobs, jobs.data(), sizeof(ResJob) * jobs.size(), cudaMemcpyHostToDevice,
+                     b->stream));
+  const int n = (int)groups.size(), side = std::min(n - 1, kSideStreams);
+  const int rc = side_streams(b, side);
+  if (rc) return rc;
+  if (side > 0) CK(cudaEventRecord(b->ev, b->stream));
+  for (int k = 0; k < side; ++k) CK(cudaStreamWaitEvent(b->side[k], b->ev, 0));
+  int64_t off = 0;
+  for (int k = 0; k < n; ++k) {
+    const ResGroup &G = groups[k];
+    const int on = k % (side + 1);
+    CK(launch_resident_sweep(nullptr, b->d_jobs + off, (int)G.jobs.size(), G.shape, G.aligned,
+                             on == 0 ? b->stream : b->side[on - 1]));
+    off += (int64_t)G.jobs.size();
+  }
+  for (int k = 0; k < side; ++k) {
+    CK(cudaEventRecord(b->side_ev[k], b->side[k]));
+    CK(cudaStreamWaitEvent(b->stream, b->side_ev[k], 0));
+  }
+  return CCMC_OK;
+}
+
 }  // namespace
 
 namespace {
@@ -885,12 +1005,10 @@ int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int6
     for (int k = 0; k < i; ++k)
       if (lats[k] == h) return CCMC_E_INVAL;  // a lattice may appear once
   }
-  std::vector<JobDesc> jobs;
   std::vector<int> resident;
   for (int i = 0; i < n; ++i) {
     ccmc_lattice *h = lats[i];
-    const int64_t sites = 16 * h->g.cstride * 16;  // padded sites held in words
-    if (nsweeps[i] == 0 || sites > b->resident_max_sites) continue;
+    if (nsweeps[i] == 0 || !batch_resident(b, h)) continue;
     // order the batch stream after work already queued on this lattice's stream
     if (h->stream != b->stream) {
       CK(cudaEventRecord(b->lat_ev[i], h->stream));
@@ -898,46 +1016,18 @@ int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int6
     }
     int rc = upload_params_on(h, beta[i], Delta[i], V[i], J[i], b->stream);
     if (rc) return rc;
-    jobs.push_back(job_of(h, nsweeps[i], obs_every[i]));
-    jobs.back().max_tpw = b->max_tpw;
     resident.push_back(i);
   }
-  if (!jobs.empty()) {
-    // When there are more lattices than CTAs resident at once, those whose
-    // words fit one warp's share of the CTA's shared memory run one a warp
-    // (eight in a CTA of 256 threads): run by a whole CTA they would leave
-    // most of its threads idle through every phase and hold back the lattices
-    // queued behind them.  With CTAs to spare, a whole CTA runs each lattice
-    // (its eight phase schedules drawn in parallel, its tables in shared
-    // memory: 10.3 against 13.6 us a sweep for a 16x16 lattice alone).
-    // One-warp lattices come last; before them, and among them, largest
-    // first, so that the queue hands the longest jobs out before the short
-    // ones.
-    int64_t max_words = 0;
-    for (const JobDesc &j : jobs) max_words = std::max(max_words, 16 * j.g.cstride);
-    const int64_t warp_words = resident_warp_words(b->threads, max_words);
-    const int64_t resident_ctas =
-        (int64_t)b->sms *
-        std::min(b->ctas_per_sm, resident_ctas_per_sm(b->threads, max_words));
-    const bool pack = (int64_t)jobs.size() > resident_ctas;
-    for (JobDesc &j : jobs) j.warp = pack && 16 * j.g.cstride <= warp_words ? 1 : 0;
-    std::vector<int> order(jobs.size());
-    for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
-    std::sort(order.begin(), order.end(), [&](int x, int y) {
-      if (jobs[x].warp != jobs[y].warp) return jobs[x].warp < jobs[y].warp;
-      const int64_t wx = (int64_t)jobs[x].g.Lx * jobs[x].g.Ly * jobs[x].nsweeps;
-      const int64_t wy = (int64_t)jobs[y].g.Lx * jobs[y].g.Ly * jobs[y].nsweeps;
-      return wx > wy;
-    });
-    std::vector<JobDesc> sorted;
-    for (int k : order) sorted.push_back(jobs[k]);
-    CK(cudaMemcpyAsync(b->d_jobs, sorted.data(), sizeof(JobDesc) * sorted.size(),
-                       cudaMemcpyHostToDevice, b->stream));
-    CK(cudaMemsetAsync(b->d_queue, 0, sizeof(int), b->stream));
-    int grid = b->sms * b->ctas_per_sm;
-    if (grid > (int)sorted.size()) grid = (int)sorted.size();
-    CK(launch_resident(b->d_jobs, (int)sorted.size(), b->d_queue, grid, b->threads, max_words,
-                       b->stream));
+  if (!resident.empty()) {
+    // a bounded number of sweeps a launch
+    std::vector<int64_t> left(nsweeps, nsweeps + n), now(n);
+    for (std::vector<int> go = resident; !go.empty();) {
+      for (int i : go) left[i] -= now[i] = std::min<int64_t>(left[i], kResMaxSweeps);
+      const int rc = run_resident(b, lats, go, now.data(), obs_every);
+      if (rc) return rc;
+      go.erase(std::remove_if(go.begin(), go.end(), [&](int i) { return left[i] == 0; }),
+               go.end());
+    }
     CK(cudaEventRecord(b->ev, b->stream));
     for (int i : resident) {
       ccmc_lattice *h = lats[i];
@@ -953,8 +1043,7 @@ int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int6
   int64_t off = 0;
   for (int i = 0; i < n; ++i) {
     ccmc_lattice *h = lats[i];
-    const int64_t sites = 16 * h->g.cstride * 16;
-    if (used[i] || nsweeps[i] == 0 || sites <= b->resident_max_sites) continue;
+    if (used[i] || nsweeps[i] == 0 || batch_resident(b, h)) continue;
     MultiGroup G{{h}, off, 0, (h->g.Cx & 15) == 0, h->cfg.tile_grid > 0};
     used[i] = 1;
     auto small = [](const ccmc_lattice *x) { return (int64_t)x->g.Cy * x->g.W < kLockstepMaxWords; };
@@ -962,8 +1051,7 @@ int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int6
       ccmc_lattice *o = lats[k];
       if (used[k] || nsweeps[k] != nsweeps[i] || obs_every[k] != obs_every[i] ||
           o->phases_done != h->phases_done || ((o->g.Cx & 15) == 0) != G.aligned ||
-          (o->cfg.tile_grid > 0) != G.tiled || !small(o) ||
-          16 * o->g.cstride * 16 <= b->resident_max_sites)
+          (o->cfg.tile_grid > 0) != G.tiled || !small(o) || batch_resident(b, o))
         continue;
       G.m.push_back(o);
       used[k] = 1;
@@ -1037,14 +1125,10 @@ int ccmc::batch_new(int cap, cudaStream_t stream, ccmc_batch **out) {
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
-  int optin = 0;
-  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const int64_t max_words = optin / 4 - kConfigTableWords - 64;
-  if (b->resident_max_sites / 4 > max_words) b->resident_max_sites = max_words * 4;
-  if (cudaMalloc(&b->d_jobs, sizeof(JobDesc) * count) != cudaSuccess ||
-      cudaMalloc(&b->d_multi, sizeof(MultiJob) * count) != cudaSuccess ||
-      cudaMalloc(&b->d_queue, sizeof(int)) != cudaSuccess)
+  if (cudaMalloc(&b->d_jobs, sizeof(ResJob) * count) != cudaSuccess ||
+      cudaMalloc(&b->d_multi, sizeof(MultiJob) * count) != cudaSuccess)
     return fail(CCMC_E_NOMEM);
+  if (!resident_ready()) return fail(CCMC_E_CUDA);
   if (cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess)
     return fail(CCMC_E_CUDA);
   b->lat_ev.assign(count, nullptr);
@@ -1064,7 +1148,9 @@ int ccmc_batch_destroy(ccmc_batch *b) {
     if (e.exec) cudaGraphExecDestroy(e.exec);
   cudaFree(b->d_jobs);
   cudaFree(b->d_multi);
-  cudaFree(b->d_queue);
+  for (cudaStream_t x : b->side) cudaStreamSynchronize(x);
+  for (cudaStream_t x : b->side) cudaStreamDestroy(x);
+  for (cudaEvent_t e : b->side_ev) cudaEventDestroy(e);
   if (b->ev) cudaEventDestroy(b->ev);
   for (auto e : b->lat_ev)
     if (e) cudaEventDestroy(e);

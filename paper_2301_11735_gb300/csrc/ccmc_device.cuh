@@ -173,9 +173,9 @@ __device__ __forceinline__ Sched draw_schedule(const Geo &g, uint64_t P) {
     const U4 w = philox(base + lane, (uint32_t)P, (uint32_t)(P >> 32), TAG_SCHED, g.k0, g.k1);
     const uint64_t x = ((uint64_t)w.z << 32) | (uint64_t)w.y;
     const uint64_t lo = x * N;
-    const uint64_t idx = __umul64hi(x, N);
-    const int rx = (int)(idx % (uint64_t)g.Lx);
-    const int ry = (int)(idx / (uint64_t)g.Lx);
+    const uint32_t idx = (uint32_t)__umul64hi(x, N);  // below N <= 2^30
+    const int ry = (int)(idx / (uint32_t)g.Lx);
+    const int rx = (int)(idx - (uint32_t)ry * (uint32_t)g.Lx);
     const bool ok = (lo >= g.rej) && offset_allowed(g.Lx, g.Ly, rx, ry);
     const unsigned ballot = __ballot_sync(0xFFFFFFFFu, ok);
     if (ballot) {

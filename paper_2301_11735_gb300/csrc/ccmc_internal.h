@@ -92,23 +92,35 @@ struct LaunchCfg {
   int tile_grid_small = 0;       // one wave of the compact tile kernel (16-bit tops)
 };
 
-// One lattice of a resident batch launch (device array, filled on the host).
-struct JobDesc {
-  Geo g;                    // the lattice in global memory
-  const uint16_t *thrT;     // its tables
+// One lattice of a resident launch (ccmc_resident.cu): held in the shared memory
+// of one CTA or of a cluster, each CTA owning `rows` rows of every class.
+struct ResJob {
+  Geo g;                  // the lattice in global memory
+  const uint16_t *thrT;   // its tables (levels, then moves: one block)
   const uint32_t *thr32;
-  const uint32_t *trans;
-  int64_t nsweeps;          // sweeps to run in this launch
-  int64_t *ring;            // observable ring (records every obs_every sweeps)
+  int nsweeps;            // sweeps to run in this launch, at most kResMaxSweeps
+  int64_t *ring;          // observable ring (records every obs_every sweeps)
   int64_t ring_cap;
-  int64_t *hist;            // histograms (nullptr: none)
+  int64_t *hist;          // histograms (nullptr: none)
   int nbins;
   int obs_every;
-  int max_tpw;              // threads a word: the most of 4, 2, 1 (at most max_tpw) that
-                            // take a phase's words in one pass of the CTA, else 1
-  int warp;                 // 1: run by one warp of a CTA, the lattice in that warp's
-                            // share of the shared memory (the launch's warp_words)
+  int rows;
 };
+
+// Launch shape of a resident launch: CTAs a lattice, rows of each class a CTA,
+// threads a word, threads a CTA (the workers and the auxiliary warp), dynamic
+// shared memory.
+struct ResShape {
+  int cluster = 0, rows = 0, tpw = 1, threads = 0;
+  int64_t smem = 0;
+};
+
+constexpr int kResMaxThreads = 1024;
+constexpr int kResMaxCluster = 16;
+constexpr int kResClusterWords = 128;  // lattices of fewer a-words a phase take one CTA
+constexpr int kResMinWords = 16;       // a-words a CTA of a cluster at least
+constexpr int kResMaxSweeps = 1 << 14;
+constexpr int kResMaxSmem = 224 << 10;
 
 // One lattice of a lock-step multi-lattice phase launch: CTAs
 // [cta_begin, cta_begin + cta_count) of the grid work on it.
@@ -120,8 +132,6 @@ struct MultiJob {
   int cta_begin, cta_count;
 };
 
-// Shared memory of the resident kernel besides the lattice words.
-constexpr int kResTableWords = kThrT / 2 + 2 * kMoveN;
 // What ccmc_batch_config's upper limit of resident_max_sites sets aside of a
 // CTA's shared memory (words).
 constexpr int kConfigTableWords = 3292;
@@ -161,17 +171,18 @@ cudaError_t launch_advance(int64_t *ctl, int64_t phases, cudaStream_t s);
 cudaError_t launch_set_ctl(int64_t *ctl, int64_t phase_base, cudaStream_t s);
 cudaError_t launch_unpack(const Geo &g, uint8_t *out, cudaStream_t s);
 cudaError_t launch_pack(const Geo &g, const uint8_t *in, int *bad, cudaStream_t s);
-// Resident batch kernel: grid CTAs of `threads` threads take jobs from *queue
-// (zeroed by the caller) until njobs are done; max_words bounds 16 Cy W of
-// the jobs a whole CTA runs.  Jobs with `warp` set come last in d_jobs and
-// have 16 Cy W <= resident_warp_words(threads, max_words).
-cudaError_t launch_resident(const JobDesc *d_jobs, int njobs, int *d_queue, int grid, int threads,
-                            int64_t max_words, cudaStream_t s);
-// Words of one warp's share of a resident CTA's shared memory, and the
-// resident CTAs of `threads` threads an SM holds at once.
-int64_t resident_warp_words(int threads, int64_t max_words);
-int resident_ctas_per_sm(int threads, int64_t max_words);
-int64_t resident_smem_bytes(int64_t max_words);
+// Resident sweeps (ccmc_resident.cu): whether the current device can run them
+// (raises the kernels' limits once per device; call outside a capture), a CTA's
+// shared memory for `rows` rows of every class, and the launch of `one` lattice or
+// of the njobs lattices of d_jobs (in device memory), all of one shape.
+bool resident_ready();
+int64_t resident_smem(const Geo &g, int rows);
+// The launch shape of a lattice that may take `ctas` CTAs of the GPU (at least
+// one) while `load` a-words a phase run on an average SM, with at most
+// max_threads workers a CTA and max_tpw threads a word.
+ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads, int max_tpw);
+cudaError_t launch_resident_sweep(const ResJob *one, const ResJob *d_jobs, int njobs,
+                                  const ResShape &shape, bool aligned, cudaStream_t s);
 cudaError_t launch_philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,
                           uint32_t k1, int64_t count, uint32_t *out, cudaStream_t s);
 

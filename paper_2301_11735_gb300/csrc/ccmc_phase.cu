@@ -1,7 +1,8 @@
 // ccmc_phase.cu -- the colour-phase kernels of the coupled-pair Metropolis
 // sweep for sm_103a (one lattice per launch: direct and tile-staged; several
-// lattices in lock step; the resident batch kernel) and their launchers
-// (declared in ccmc_internal.h).
+// lattices in lock step) and their launchers (declared in ccmc_internal.h).  The
+// resident kernel, whole sweeps of lattices that fit shared memory, is in
+// ccmc_resident.cu.
 #include <cuda_runtime.h>
 
 #include <cstddef>
@@ -11,6 +12,7 @@
 #include "ccmc_device.cuh"
 #include "ccmc_internal.h"
 #include "ccmc_launch.cuh"
+#include "ccmc_word.cuh"
 
 namespace ccmc {
 
@@ -110,68 +112,6 @@ __device__ __forceinline__ uint32_t window(const uint32_t *cls, const Geo &g, co
   }
 }
 
-// Move entry of choice class r (v mod 12) and r264 = 264 r + 128 near: entry
-// (2 r + near) 16 + (pc XOR r) of the move table, at byte offset
-// 256 r + 128 near + 8 (pc XOR r) = r264 XOR 8 pc.  The XOR spreads a warp's
-// lookups over the banks: with entry (2 r + near) 16 + pc the bank pair of a
-// lookup was its pair state alone, and the few common states (both sites
-// magnetic) piled onto four of sixteen bank pairs.  Word 0: the level
-// offset's base and, at bits 24-27, the move pc XOR npc; word 1: the signed byte
-// coefficients of (2 n1_a, n0_a, 2 n1_b, n0_b).
-__device__ __forceinline__ uint2 move_entry(const uint2 *trans, uint32_t off) {
-  return *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(trans) + off);
-}
-
-// The threshold level at byte offset `off` (the offset is formed in bytes, so
-// that it is the load's address without a shift).
-__device__ __forceinline__ uint32_t level_at(const uint16_t *thrT, uint32_t off) {
-  return *reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(thrT) + off);
-}
-
-// floor(v / 12) for v < 2^16 by a multiply-high: floor(v m / 2^32) with
-// m = ceil(2^32 / 12) is exact there.
-__device__ __forceinline__ uint32_t div12(uint32_t v) { return __umulhi(v, 357913942u); }
-
-// A pair's neighbour counts as dp4a's byte operands.  A word's pairs form four
-// groups k (sites k, k + 4, k + 8, k + 12: one a byte); group k = 2 c + h is
-// half h of MOVE call c.
-constexpr uint32_t kEnvMask = 0x070E070Eu;  // 2 n1 at bits 1-3, n0 at bits 0-2 of a nibble
-
-// The counts of half h's pairs of both calls: byte q of ev[q] .. is lane q's
-// (2 n1_a, n0_a, 2 n1_b, n0_b), call 0 in the low nibbles, call 1 in the high
-// ones (bits outside kEnvMask are whatever the planes hold there).  Two
-// selections put a count's three bits side by side (its unwanted neighbours
-// are masked with the nibble), then eight byte permutes transpose the four
-// counts: 30 instructions for eight pairs, where masked additions, byte
-// extraction per group and a permute per pair took about 70.
-struct Env {
-  uint32_t ev[4];
-};
-
-__device__ __forceinline__ Env half_env(const Planes &a, const Planes &b, int h) {
-  // bits of half h's sites at the low two bits of every nibble
-  const uint32_t m1 = 0x22222222u, m2 = 0x88888888u, m3 = 0x11111111u, m4 = 0x44444444u;
-  const uint32_t aO = h ? a.O >> 2 : a.O, aT = h ? a.T >> 1 : a.T << 1,
-                 aF = h ? a.F : a.F << 2;
-  const uint32_t bO = h ? b.O >> 2 : b.O, bT = h ? b.T >> 1 : b.T << 1,
-                 bF = h ? b.F : b.F << 2;
-  const uint32_t a1 = lop3<kLutMux>(aF, lop3<kLutMux>(aO, aT, m1), m2);
-  const uint32_t a0 = lop3<kLutMux>(aF, lop3<kLutMux>(aO, aT, m3), m4);
-  const uint32_t b1 = lop3<kLutMux>(bF, lop3<kLutMux>(bO, bT, m1), m2);
-  const uint32_t b0 = lop3<kLutMux>(bF, lop3<kLutMux>(bO, bT, m3), m4);
-  const uint32_t x01 = prmt(a1, a0, 0x5140u), x23 = prmt(a1, a0, 0x7362u);
-  const uint32_t y01 = prmt(b1, b0, 0x5140u), y23 = prmt(b1, b0, 0x7362u);
-  return Env{{prmt(x01, y01, 0x5410u), prmt(x01, y01, 0x7632u), prmt(x23, y23, 0x5410u),
-              prmt(x23, y23, 0x7632u)}};
-}
-
-// The inputs of a word's pairs: its a word, its b window and the neighbour
-// counts of both sides.
-struct WordIn {
-  uint32_t A, B;
-  Planes na, nb;
-};
-
 // Row jr + dy of a class (periodic in Cy); staged bands start at the right row.
 template <int kMode>
 __device__ __forceinline__ int band_row(const Geo &g, int r0, int dy) {
@@ -194,83 +134,6 @@ __device__ __forceinline__ WordIn gather(const Geo &g, const PhaseU &u, int jr, 
                          window<kMode>(u.cBU, g, u, band_row<kMode>(g, jb, u.dyBU), w, u.offB, n),
                          window<kMode>(u.cBD, g, u, band_row<kMode>(g, jb, u.dyBD), w, u.offB, n));
   return in;
-}
-
-// The pair states pc (a's code above b's) of half h's pairs: lane q of call c at
-// bits 8 q + 4 c .. + 3.
-__device__ __forceinline__ uint32_t half_pc(const WordIn &in, int h) {
-  return h ? lop3<kLutMux>(in.A, in.B >> 2, 0xCCCCCCCCu)
-           : lop3<kLutMux>(in.A << 2, in.B, 0xCCCCCCCCu);
-}
-
-// 264 r + 128 near XOR 8 pc, the move entry's offset (pcs >> sh: the pair's pc
-// at bits 3-6; sh < 0 shifts left).
-__device__ __forceinline__ uint32_t entry_offset(uint32_t pcs, int sh, uint32_t r264) {
-  return lop3<kLutAndXor>(sh < 0 ? pcs << -sh : pcs >> sh, 0x78u, r264);
-}
-
-// The fast path of the pairs of a word one thread evaluates: kTPW threads
-// share a word (1, 2 or 4), thread `sub` of them takes MOVE call(s) and
-// half(s):
-//   kTPW 1: both calls, both halves (all 16 pairs);
-//   kTPW 2: call sub, both halves (8 pairs);
-//   kTPW 4: call sub / 2, half sub mod 2 (4 pairs: group k = sub).
-// Returns the (dA, dB) of the fast decisions and, in z, bit c for every call
-// c with a rare pair (a tie or a field >= 65532; the fast path rejected it).
-template <int kTPW, class Keys>
-__device__ __forceinline__ uint3 fast_moves(const Geo &g, const uint2 *trans,
-                                            const uint16_t *thrT, int j, int w, int sub,
-                                            const WordIn &in, uint64_t P, uint32_t near128,
-                                            const Keys &keys) {
-  static_assert(kTPW == 1 || kTPW == 2 || kTPW == 4, "one, two or four threads a word");
-  constexpr int kCalls = kTPW == 1 ? 2 : 1;
-  constexpr int kHalves = kTPW == 4 ? 1 : 2;
-  const int c0 = kTPW == 1 ? 0 : (kTPW == 2 ? sub : sub >> 1);
-  const int h0 = kTPW == 4 ? (sub & 1) : 0;
-  const uint32_t gbase = (uint32_t)j * (uint32_t)(2 * g.W) + (uint32_t)(2 * w);
-  Env env[kHalves];
-  uint32_t pcs[kHalves];
-#pragma unroll
-  for (int hi = 0; hi < kHalves; ++hi) {
-    env[hi] = half_env(in.na, in.nb, h0 + hi);
-    pcs[hi] = half_pc(in, h0 + hi);
-  }
-  uint32_t dA = 0u, dB = 0u, slow = 0u;
-#pragma unroll
-  for (int ci = 0; ci < kCalls; ++ci) {
-    const int c = c0 + ci;
-    const U4 r = keys(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE);
-    uint32_t mn = 0xFFFFFFFFu;  // smallest w - T of the call
-#pragma unroll
-    for (int hi = 0; hi < kHalves; ++hi) {
-      const int h = h0 + hi;
-      const int k = 2 * c + h;
-      uint32_t d[4], t[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
-        const uint32_t v = h ? X >> 16 : X & 0xFFFFu;
-        const uint32_t wq = div12(v);
-        const uint2 e = move_entry(
-            trans, entry_offset(pcs[hi], 8 * q + 4 * c - 3, (v - 12u * wq) * 264u + near128));
-        t[q] = (uint32_t)__dp4a((int)e.y, (int)((env[hi].ev[q] >> (4 * c)) & kEnvMask), (int)e.x);
-        d[q] = wq - level_at(thrT, t[q] & 0xFFFFu);  // negative: accept; zero: a tie
-      }
-      mn = __vimin3_u32(mn, d[0], d[1]);
-      mn = __vimin3_u32(mn, d[2], d[3]);
-      // byte q: the accepted move of lane q, i.e. byte 3 of t[q] under the sign
-      // of d[q] (byte permutes: bit 3 of a selector replicates a byte's sign)
-      const uint32_t acc = prmt(prmt(d[0], d[1], 0x00FBu), prmt(d[2], d[3], 0x00FBu), 0x5410u) &
-                           prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
-      // byte q of acc -> site k + 4 q: b bits to 2 (k + 4 q) of dB, a bits of dA
-      dB |= (acc & 0x03030303u) << (2 * k);
-      dA |= ((acc >> 2) & 0x03030303u) << (2 * k);
-    }
-    // a rare pair: a tie, or a field >= 65532 in either half of the call's words
-    const uint32_t mx = __vmaxu2(__vimax3_u16x2(r.x, r.y, r.z), r.w);
-    if (mn == 0u || mx >= 0xFFFC0000u || (mx & 0xFFFFu) >= 0xFFFCu) slow |= 1u << c;
-  }
-  return make_uint3(dA, dB, slow);
 }
 
 // Apply the moves (dA, dB) of word w (row jr of u's arrays, n sites): the a
@@ -319,47 +182,17 @@ __device__ __forceinline__ void apply_moves(const Geo &g, const PhaseU &u, int j
 }
 
 // The exact path of one pair, by one lane of a warp that takes the rare calls
-// of a word together: pair t = k + 4 q (group k = 2 c + h, lane q of the
-// group) of MOVE call c of word w (inputs `in`, n sites in the row), decided
-// with its SLOW words if it is rare (the fast path rejected it), and applied
-// to the word's a and b sites by atomic XOR.
+// of a word together: decided and applied to the word's a and b sites by atomic
+// XOR (see exact_move).
 template <int kMode>
 __device__ __forceinline__ void exact_pair(const Geo &g, const PhaseU &u, const uint2 *trans,
                                            const uint16_t *thrT, const uint32_t *thr32, int j,
                                            int jr, int w, int n, int c, int h, int q,
                                            const WordIn &in, uint64_t P, uint32_t near128) {
-  const int k = 2 * c + h;
-  const int t = k + 4 * q;
+  const int t = 2 * c + h + 4 * q;
   if (t >= n) return;  // past the end of the row: no pair
-  const uint32_t gbase = (uint32_t)j * (uint32_t)(2 * g.W) + (uint32_t)(2 * w);
-  const U4 r = philox(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE, g.k0, g.k1);
-  const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
-  const uint32_t v = h ? X >> 16 : X & 0xFFFFu;
-  const uint32_t wq = div12(v);
-  // the pair's own counts and state, from bits 2 t and 2 t + 1 of the planes
-  auto counts = [&](const Planes &p) {
-    const uint32_t O = p.O >> (2 * t), T = p.T >> (2 * t), F = p.F >> (2 * t);
-    return ((O & 2u) + 2u * (T & 2u) + 4u * (F & 2u)) |
-           (((O & 1u) + 2u * (T & 1u) + 4u * (F & 1u)) << 8);
-  };
-  const uint32_t env = counts(in.na) | (counts(in.nb) << 16);
-  const uint32_t pc8 = ((((in.A >> (2 * t)) & 3u) << 2) | ((in.B >> (2 * t)) & 3u)) << 3;
-  uint2 e = move_entry(trans, ((v - 12u * wq) * 264u + near128) ^ pc8);
-  if (v < 65532u && wq != level_at(thrT, (uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu))
-    return;  // not rare
-  const uint32_t slow0 = (uint32_t)((uint64_t)j * g.Cx + (uint32_t)(w << 4));
-  const U4 sl = philox(slow0 + (uint32_t)t, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, g.k0, g.k1);
-  if (v >= 65532u) {
-    if (sl.y >= 4294967292u) return;  // keep the current configuration
-    e = move_entry(trans, ((sl.y % 12u) * 264u + near128) ^ pc8);
-  }
-  const uint32_t thr = thr32[((uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu) >> 1];
-  const bool accept = thr == 0xFFFFFFFFu ||
-                      (v < 65532u ? ((uint64_t)wq << 32) + sl.x < 5461ull * thr : sl.x < thr);
-  if (accept) {
-    const uint32_t x = e.x >> 24;
-    apply_moves<kMode, false>(g, u, jr, w, n, (x >> 2) << (2 * t), (x & 3u) << (2 * t));
-  }
+  const uint32_t x = exact_move(g, trans, thrT, thr32, j, w, c, h, q, in, P, near128);
+  if (x) apply_moves<kMode, false>(g, u, jr, w, n, (x >> 2) << (2 * t), (x & 3u) << (2 * t));
 }
 
 // One word's pairs by one lane, with all 32 lanes of the warp calling
@@ -384,7 +217,10 @@ __device__ __forceinline__ void warp_word(const Geo &g, const PhaseU &u, const u
   uint32_t rz = 0u;
   if (active) {
     in = gather<kMode>(g, u, jr, w, n);
-    const uint3 d = fast_moves<kTPW>(g, trans, thrT, j, w, sub, in, P, near128, keys);
+    const uint32_t gbase = (uint32_t)j * (uint32_t)(2 * g.W) + (uint32_t)(2 * w);
+    const uint3 d = fast_moves<kTPW>(trans, thrT, sub, in, near128, [&](int c) {
+      return keys(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE);
+    });
     apply_moves<kMode, kTPW == 1>(g, u, jr, w, n, d.x, d.y);
     rz = d.z;
   }
@@ -890,298 +726,6 @@ __global__ void __launch_bounds__(256, 4) phase_multi_kernel(const MultiJob *__r
     warp_word<kAligned ? kRowAligned : kRowGeneral>(g, u, sm.trans, sm.thrT, J.thr32, j, j, w, P,
                                                      near128, SeedKeys{g.k0, g.k1}, 0, act);
   }
-}
-
-// One lattice run by one warp of a resident CTA (JobDesc.warp): its words in
-// the warp's share of the shared memory, its tables read through L1 from
-// global memory, the warp's own barrier between phases.  The same per-word
-// code as the CTA path, so results are identical.
-template <int kMode, int kTPW>
-__device__ __forceinline__ void warp_job_phase(const Geo &gs, const PhaseU &u, const uint2 *trans,
-                                               const uint16_t *thrT, const uint32_t *thr32,
-                                               int nwa, uint64_t P, uint32_t near128) {
-  const int lane = threadIdx.x & 31;
-  const SeedKeys keys{gs.k0, gs.k1};
-  for (int base = 0; base < kTPW * nwa; base += 32) {  // uniform trip count
-    const int i = base + lane;
-    const bool act = i < kTPW * nwa;
-    const int wid = !act ? 0 : (kTPW == 1 ? i : (kTPW == 2 ? i >> 1 : i >> 2));
-    const int sub = act ? i - kTPW * wid : 0;
-    const int j = wid / gs.W, w = wid - j * gs.W;
-    warp_word<kMode, kTPW>(gs, u, trans, thrT, thr32, j, j, w, P, near128, keys, sub, act);
-  }
-}
-
-__device__ __forceinline__ void warp_job(const JobDesc &J, uint32_t *region, PhaseU &su) {
-  const int lane = threadIdx.x & 31;
-  const Geo g = J.g;
-  const int64_t nw = 16 * g.cstride;
-  for (int64_t t = lane; t < nw; t += 32) region[t] = g.words[t];
-  const int64_t P0 = g.ctl[kCtlPhaseBase];
-  const int64_t nsweeps = J.nsweeps;
-  const int obs_every = J.obs_every;
-  Geo gs = g;
-  gs.words = region;
-  const bool aligned = (g.Cx & 15) == 0;
-  const int nwa = g.Cy * g.W;  // a-words per phase
-  const int tpw = J.max_tpw >= 4 && 4 * nwa <= 32 ? 4 : J.max_tpw >= 2 && 2 * nwa <= 32 ? 2 : 1;
-  const uint2 *trans = reinterpret_cast<const uint2 *>(J.trans);
-  int64_t obs_cnt = 0, obs_slot = 0;
-  if (lane == 0 && obs_every > 0) {
-    obs_cnt = g.ctl[kCtlObsCount];
-    obs_slot = obs_cnt % J.ring_cap;
-  }
-  __syncwarp();
-  for (int64_t s = 0; s < nsweeps; ++s) {
-    for (int p = 0; p < 8; ++p) {
-      const uint64_t P = (uint64_t)(P0 + 8 * s + p);
-      const Sched sc = draw_schedule(gs, P);
-      if (lane == 0) su = phase_uniform(gs, sc);
-      __syncwarp();
-      const PhaseU &u = su;  // read from shared memory where used
-      const uint32_t near128 = sc.near ? 128u : 0u;
-      if (aligned) {
-        if (tpw == 1)
-          warp_job_phase<kRowAligned, 1>(gs, u, trans, J.thrT, J.thr32, nwa, P, near128);
-        else if (tpw == 2)
-          warp_job_phase<kRowAligned, 2>(gs, u, trans, J.thrT, J.thr32, nwa, P, near128);
-        else
-          warp_job_phase<kRowAligned, 4>(gs, u, trans, J.thrT, J.thr32, nwa, P, near128);
-      } else {
-        if (tpw == 1)
-          warp_job_phase<kRowGeneral, 1>(gs, u, trans, J.thrT, J.thr32, nwa, P, near128);
-        else if (tpw == 2)
-          warp_job_phase<kRowGeneral, 2>(gs, u, trans, J.thrT, J.thr32, nwa, P, near128);
-        else
-          warp_job_phase<kRowGeneral, 4>(gs, u, trans, J.thrT, J.thr32, nwa, P, near128);
-      }
-      __syncwarp();  // the phase's writes before the next phase's reads
-    }
-    const int64_t done = P0 / 8 + s + 1;
-    if (obs_every > 0 && done % obs_every == 0) {
-      // the 16 classes side by side, two lanes a class
-      int c[7] = {0, 0, 0, 0, 0, 0, 0};
-      count_class(gs, lane >> 1, lane & 1, 2, c);
-      int64_t rec[8];
-      rec[0] = done;
-#pragma unroll
-      for (int k = 0; k < 7; ++k) rec[1 + k] = warp_sum((int64_t)c[k]);
-      if (lane == 0) {
-        for (int k = 0; k < 8; ++k) g.ctl[kCtlLatest + k] = rec[k];
-        int64_t *dst = J.ring + obs_slot * 8;
-        for (int k = 0; k < 8; ++k) dst[k] = rec[k];
-        g.ctl[kCtlObsCount] = ++obs_cnt;
-        if (++obs_slot == J.ring_cap) obs_slot = 0;
-        if (J.hist) {
-          const int64_t N = (int64_t)g.Lx * g.Ly;
-          const int64_t vals[3] = {rec[4], rec[5], rec[7]};
-          for (int h = 0; h < 3; ++h)
-            atomicAdd(reinterpret_cast<unsigned long long *>(
-                          J.hist + h * J.nbins + (vals[h] + N) * J.nbins / (2 * N + 1)),
-                      1ull);
-        }
-      }
-      __syncwarp();
-    }
-  }
-  for (int64_t t = lane; t < nw; t += 32) g.words[t] = region[t];
-  if (lane == 0) g.ctl[kCtlPhaseBase] = P0 + 8 * nsweeps;
-  __syncwarp();
-}
-
-// ============================================================================
-// Resident batch kernel (many lattices of uneven size, one persistent launch).
-// Each CTA takes lattices from a work queue, largest first; it holds the whole
-// packed lattice and its tables in shared memory and runs all of that lattice's
-// sweeps with block barriers between phases, recounting into the lattice's ring
-// when due; then it writes the lattice back and takes the next one.  The same
-// per-word code as phase_kernel runs against shared memory, so results are
-// identical to the per-phase launches.
-__global__ void __launch_bounds__(512, 1) resident_kernel(const JobDesc *__restrict__ jobs, int njobs,
-                                                       int *queue, int warp_words) {
-  extern __shared__ __align__(16) uint32_t dyn[];
-  uint16_t *s_thrT = reinterpret_cast<uint16_t *>(dyn);
-  uint2 *s_trans = reinterpret_cast<uint2 *>(dyn + kThrT / 2);
-  uint32_t *s_words = dyn + kResTableWords;
-  __shared__ Sched s_sched[8];  // the schedules of the current sweep's phases
-  __shared__ PhaseU s_u[8];     // and their class pointers and offsets
-  __shared__ int s_job;
-  __shared__ int64_t s_red[32][7];
-  __shared__ PhaseU s_wu[16];  // one-warp jobs: each warp's current phase
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (;;) {
-    if (threadIdx.x == 0) s_job = atomicAdd(queue, 1);
-    __syncthreads();
-    const int job = s_job;
-    if (job >= njobs) break;
-    if (jobs[job].warp) {
-      // the rest of the queue is one-warp jobs (the planner orders them
-      // last): every warp takes its own from here on, warp 0 this one
-      uint32_t *region = dyn + (int64_t)warp * warp_words;
-      for (int jw = warp == 0 ? job : -1;;) {
-        if (jw < 0) {
-          int x = 0;
-          if (lane == 0) x = atomicAdd(queue, 1);
-          jw = __shfl_sync(0xFFFFFFFFu, x, 0);
-        }
-        if (jw >= njobs) return;
-        if (jobs[jw].warp && 16 * jobs[jw].g.cstride <= warp_words)
-          warp_job(jobs[jw], region, s_wu[warp]);
-        else if (lane == 0)
-          jobs[jw].g.ctl[kCtlStatus] = 1;  // not a one-warp job: the planner's order broke
-        jw = -1;
-      }
-    }
-    const JobDesc &J = jobs[job];
-    const Geo g = J.g;
-    const int64_t nw = 16 * g.cstride;
-    for (int t = threadIdx.x; t < kThrT / 2; t += blockDim.x)
-      dyn[t] = reinterpret_cast<const uint32_t *>(J.thrT)[t];
-    for (int t = threadIdx.x; t < kMoveN; t += blockDim.x)
-      s_trans[t] = make_uint2(J.trans[2 * t], J.trans[2 * t + 1]);
-    for (int64_t t = threadIdx.x; t < nw; t += blockDim.x) s_words[t] = g.words[t];
-    const int64_t P0 = g.ctl[kCtlPhaseBase];
-    const int64_t nsweeps = J.nsweeps;
-    const int obs_every = J.obs_every;
-    Geo gs = g;
-    gs.words = s_words;
-    const bool aligned = (g.Cx & 15) == 0;
-    const int nwa = g.Cy * g.W;  // a-words per phase
-    // threads a word: the most (four, two; at most J.max_tpw) that still take
-    // a phase's words in one pass of the CTA, else one
-    const int tpw = J.max_tpw >= 4 && 4 * nwa <= (int)blockDim.x ? 4
-                  : J.max_tpw >= 2 && 2 * nwa <= (int)blockDim.x ? 2 : 1;
-    // thread 0's copies of the record count and its ring slot: read once per
-    // job, so that a record costs no global load on the sweep's critical path
-    int64_t obs_cnt = 0, obs_slot = 0;
-    if (threadIdx.x == 0 && obs_every > 0) {
-      obs_cnt = g.ctl[kCtlObsCount];
-      obs_slot = obs_cnt % J.ring_cap;
-    }
-    __syncthreads();
-    const int nwarps = blockDim.x >> 5;
-    for (int64_t s = 0; s < nsweeps; ++s) {
-      // the eight schedules of the sweep depend on nothing but the phase
-      // index: the warps draw them (and derive each phase's class pointers)
-      // together, then every phase needs only the barrier that orders it
-      // after the previous one
-      for (int q = warp; q < 8; q += nwarps) {
-        const Sched sc = draw_schedule(gs, (uint64_t)(P0 + 8 * s + q));
-        if (lane == 0) {
-          s_sched[q] = sc;
-          s_u[q] = phase_uniform(gs, sc);
-        }
-      }
-      __syncthreads();
-      for (int p = 0; p < 8; ++p) {
-        const uint64_t P = (uint64_t)(P0 + 8 * s + p);
-        const PhaseU &u = s_u[p];  // read from shared memory where used
-        const uint32_t near128 = s_sched[p].near ? 128u : 0u;
-        for (int base = 0; base < tpw * nwa; base += blockDim.x) {  // uniform trip count
-          const int i = base + threadIdx.x;
-          const bool act = i < tpw * nwa;
-          const int wid = !act ? 0 : tpw == 1 ? i : (tpw == 2 ? i >> 1 : i >> 2);
-          const int sub = act ? i - tpw * wid : 0;
-          const int j = wid / g.W, w = wid - j * g.W;
-          const SeedKeys keys{gs.k0, gs.k1};
-          if (aligned) {
-            if (tpw == 1)
-              warp_word<kRowAligned, 1>(gs, u, s_trans, s_thrT, J.thr32, j, j, w, P, near128, keys,
-                                        sub, act);
-            else if (tpw == 2)
-              warp_word<kRowAligned, 2>(gs, u, s_trans, s_thrT, J.thr32, j, j, w, P, near128, keys,
-                                        sub, act);
-            else
-              warp_word<kRowAligned, 4>(gs, u, s_trans, s_thrT, J.thr32, j, j, w, P, near128, keys,
-                                        sub, act);
-          } else {
-            if (tpw == 1)
-              warp_word<kRowGeneral, 1>(gs, u, s_trans, s_thrT, J.thr32, j, j, w, P, near128, keys,
-                                        sub, act);
-            else if (tpw == 2)
-              warp_word<kRowGeneral, 2>(gs, u, s_trans, s_thrT, J.thr32, j, j, w, P, near128, keys,
-                                        sub, act);
-            else
-              warp_word<kRowGeneral, 4>(gs, u, s_trans, s_thrT, J.thr32, j, j, w, P, near128, keys,
-                                        sub, act);
-          }
-        }
-        __syncthreads();
-      }
-      const int64_t done = P0 / 8 + s + 1;
-      if (obs_every > 0 && done % obs_every == 0) {
-        // the 16 classes side by side: thread t takes words t mod (blockDim / 16),
-        // ... of class 16 t / blockDim (blockDim a multiple of 16)
-        int c[7] = {0, 0, 0, 0, 0, 0, 0};
-        const int per_cls = (int)blockDim.x >> 4;
-        count_class(gs, (int)threadIdx.x / per_cls, (int)threadIdx.x % per_cls, per_cls, c);
-#pragma unroll
-        for (int k = 0; k < 7; ++k) {
-          const int64_t v = warp_sum((int64_t)c[k]);
-          if (lane == 0) s_red[warp][k] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-          int64_t rec[8];
-          rec[0] = done;
-          for (int k = 0; k < 7; ++k) {
-            int64_t v = 0;
-            for (int wv = 0; wv < (int)(blockDim.x >> 5); ++wv) v += s_red[wv][k];
-            rec[1 + k] = v;
-          }
-          for (int k = 0; k < 8; ++k) g.ctl[kCtlLatest + k] = rec[k];
-          int64_t *dst = J.ring + obs_slot * 8;
-          for (int k = 0; k < 8; ++k) dst[k] = rec[k];
-          g.ctl[kCtlObsCount] = ++obs_cnt;
-          if (++obs_slot == J.ring_cap) obs_slot = 0;
-          if (J.hist) {  // reductions: no load to wait for
-            const int64_t N = (int64_t)g.Lx * g.Ly;
-            const int64_t vals[3] = {rec[4], rec[5], rec[7]};
-            for (int h = 0; h < 3; ++h)
-              atomicAdd(reinterpret_cast<unsigned long long *>(
-                            J.hist + h * J.nbins + (vals[h] + N) * J.nbins / (2 * N + 1)),
-                        1ull);
-          }
-        }
-        __syncthreads();
-      }
-    }
-    for (int64_t t = threadIdx.x; t < nw; t += blockDim.x) g.words[t] = s_words[t];
-    if (threadIdx.x == 0) g.ctl[kCtlPhaseBase] = P0 + 8 * nsweeps;
-    __syncthreads();
-  }
-}
-
-int64_t resident_smem_bytes(int64_t max_words) {
-  return (int64_t)sizeof(uint32_t) * (kResTableWords + max_words);
-}
-
-int resident_ctas_per_sm(int threads, int64_t max_words) {
-  const int smem = (int)resident_smem_bytes(max_words);
-  int per_sm = 0;
-  if (cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
-          cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, resident_kernel, threads, smem) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return 1;
-  }
-  return per_sm < 1 ? 1 : per_sm;
-}
-
-int64_t resident_warp_words(int threads, int64_t max_words) {
-  return ((kResTableWords + max_words) / (threads / 32)) & ~(int64_t)3;
-}
-
-cudaError_t launch_resident(const JobDesc *d_jobs, int njobs, int *d_queue, int grid, int threads,
-                            int64_t max_words, cudaStream_t s) {
-  const int64_t smem = resident_smem_bytes(max_words);
-  cudaError_t e = cudaFuncSetAttribute(resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  resident_kernel<<<grid, threads, (size_t)smem, s>>>(
-      d_jobs, njobs, d_queue, (int)resident_warp_words(threads, max_words));
-  return cudaGetLastError();
 }
 
 // ============================================================================

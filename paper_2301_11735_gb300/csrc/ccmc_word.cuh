@@ -1,0 +1,196 @@
+// ccmc_word.cuh -- the per-word core of a colour phase, shared by the phase
+// kernels and the resident kernel: the 16 pairs of one a-class word decided from
+// the word's inputs (its a word, b window and both sides' neighbour counts).
+// How those inputs are read and where the moves go is each kernel's own.
+#pragma once
+
+#include <cstdint>
+
+#include "ccmc_device.cuh"
+#include "ccmc_internal.h"
+
+namespace ccmc {
+
+// Move entry of choice class r (v mod 12) and r264 = 264 r + 128 near: entry
+// (2 r + near) 16 + (pc XOR r) of the move table, at byte offset
+// 256 r + 128 near + 8 (pc XOR r) = r264 XOR 8 pc.  The XOR spreads a warp's
+// lookups over the banks: with entry (2 r + near) 16 + pc the bank pair of a
+// lookup was its pair state alone, and the few common states (both sites
+// magnetic) piled onto four of sixteen bank pairs.  Word 0: the level
+// offset's base and, at bits 24-27, the move pc XOR npc; word 1: the signed byte
+// coefficients of (2 n1_a, n0_a, 2 n1_b, n0_b).
+__device__ __forceinline__ uint2 move_entry(const uint2 *trans, uint32_t off) {
+  return *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(trans) + off);
+}
+
+// The threshold level at byte offset `off` (the offset is formed in bytes, so
+// that it is the load's address without a shift).
+__device__ __forceinline__ uint32_t level_at(const uint16_t *thrT, uint32_t off) {
+  return *reinterpret_cast<const uint16_t *>(reinterpret_cast<const char *>(thrT) + off);
+}
+
+// floor(v / 12) for v < 2^16 by a multiply-high: floor(v m / 2^32) with
+// m = ceil(2^32 / 12) is exact there.
+__device__ __forceinline__ uint32_t div12(uint32_t v) { return __umulhi(v, 357913942u); }
+
+// A pair's neighbour counts as dp4a's byte operands.  A word's pairs form four
+// groups k (sites k, k + 4, k + 8, k + 12: one a byte); group k = 2 c + h is
+// half h of MOVE call c.
+constexpr uint32_t kEnvMask = 0x070E070Eu;  // 2 n1 at bits 1-3, n0 at bits 0-2 of a nibble
+
+// The counts of half h's pairs of both calls: byte q of ev[q] .. is lane q's
+// (2 n1_a, n0_a, 2 n1_b, n0_b), call 0 in the low nibbles, call 1 in the high
+// ones (bits outside kEnvMask are whatever the planes hold there).  Two
+// selections put a count's three bits side by side (its unwanted neighbours
+// are masked with the nibble), then eight byte permutes transpose the four
+// counts: 30 instructions for eight pairs, where masked additions, byte
+// extraction per group and a permute per pair took about 70.
+struct Env {
+  uint32_t ev[4];
+};
+
+__device__ __forceinline__ Env half_env(const Planes &a, const Planes &b, int h) {
+  // bits of half h's sites at the low two bits of every nibble
+  const uint32_t m1 = 0x22222222u, m2 = 0x88888888u, m3 = 0x11111111u, m4 = 0x44444444u;
+  const uint32_t aO = h ? a.O >> 2 : a.O, aT = h ? a.T >> 1 : a.T << 1,
+                 aF = h ? a.F : a.F << 2;
+  const uint32_t bO = h ? b.O >> 2 : b.O, bT = h ? b.T >> 1 : b.T << 1,
+                 bF = h ? b.F : b.F << 2;
+  const uint32_t a1 = lop3<kLutMux>(aF, lop3<kLutMux>(aO, aT, m1), m2);
+  const uint32_t a0 = lop3<kLutMux>(aF, lop3<kLutMux>(aO, aT, m3), m4);
+  const uint32_t b1 = lop3<kLutMux>(bF, lop3<kLutMux>(bO, bT, m1), m2);
+  const uint32_t b0 = lop3<kLutMux>(bF, lop3<kLutMux>(bO, bT, m3), m4);
+  const uint32_t x01 = prmt(a1, a0, 0x5140u), x23 = prmt(a1, a0, 0x7362u);
+  const uint32_t y01 = prmt(b1, b0, 0x5140u), y23 = prmt(b1, b0, 0x7362u);
+  return Env{{prmt(x01, y01, 0x5410u), prmt(x01, y01, 0x7632u), prmt(x23, y23, 0x5410u),
+              prmt(x23, y23, 0x7632u)}};
+}
+
+// The inputs of a word's pairs: its a word, its b window and the neighbour
+// counts of both sides.
+struct WordIn {
+  uint32_t A, B;
+  Planes na, nb;
+};
+
+// The pair states pc (a's code above b's) of half h's pairs: lane q of call c at
+// bits 8 q + 4 c .. + 3.
+__device__ __forceinline__ uint32_t half_pc(uint32_t A, uint32_t B, int h) {
+  return h ? lop3<kLutMux>(A, B >> 2, 0xCCCCCCCCu) : lop3<kLutMux>(A << 2, B, 0xCCCCCCCCu);
+}
+
+// 264 r + 128 near XOR 8 pc, the move entry's offset: the pair's pc at bits 3-6
+// of pcs >> 8 q (of the half's pair states rotated left by 3 - 4 c).
+__device__ __forceinline__ uint32_t entry_offset(uint32_t pcs, int q, uint32_t r264) {
+  return lop3<kLutAndXor>(pcs >> (8 * q), 0x78u, r264);
+}
+
+// The fast path of the pairs of a word one thread evaluates: kTPW threads
+// share a word (1, 2 or 4), thread `sub` of them takes MOVE call(s) and
+// half(s):
+//   kTPW 1: both calls, both halves (all 16 pairs);
+//   kTPW 2: call sub, both halves (8 pairs);
+//   kTPW 4: call sub / 2, half sub mod 2 (4 pairs: group k = sub).
+// Returns the (dA, dB) of the fast decisions and, in z, bit c for every call
+// c with a rare pair (a tie or a field >= 65532; the fast path rejected it).
+// rand(c): the four words of the word's MOVE call c.
+template <int kTPW, class Rand>
+__device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *thrT, int sub,
+                                            const WordIn &in, uint32_t near128,
+                                            const Rand &rand) {
+  static_assert(kTPW == 1 || kTPW == 2 || kTPW == 4, "one, two or four threads a word");
+  constexpr int kCalls = kTPW == 1 ? 2 : 1;
+  constexpr int kHalves = kTPW == 4 ? 1 : 2;
+  const int c0 = kTPW == 1 ? 0 : (kTPW == 2 ? sub : sub >> 1);
+  const int h0 = kTPW == 4 ? (sub & 1) : 0;
+  Env env[kHalves];
+  uint32_t pcs[kHalves];
+#pragma unroll
+  for (int hi = 0; hi < kHalves; ++hi) {
+    if constexpr (kTPW == 4) {  // the thread's half moved to half 0's place
+      auto half = [&](const Planes &p) {
+        return Planes{p.O >> (2 * h0), p.T >> (2 * h0), p.F >> (2 * h0)};
+      };
+      env[hi] = half_env(half(in.na), half(in.nb), 0);
+      pcs[hi] = half_pc(in.A >> (2 * h0), in.B >> (2 * h0), 0);
+    } else {
+      env[hi] = half_env(in.na, in.nb, hi);
+      pcs[hi] = half_pc(in.A, in.B, hi);
+    }
+  }
+  uint32_t dA = 0u, dB = 0u, slow = 0u;
+#pragma unroll
+  for (int ci = 0; ci < kCalls; ++ci) {
+    const int c = c0 + ci;
+    const U4 r = rand(c);
+    uint32_t mn = 0xFFFFFFFFu;  // smallest w - T of the call
+#pragma unroll
+    for (int hi = 0; hi < kHalves; ++hi) {
+      const int h = h0 + hi;
+      const int k = 2 * c + h;
+      uint32_t d[4], t[4];
+      const uint32_t pc = __funnelshift_l(pcs[hi], pcs[hi], 3 - 4 * c);  // counts modulo 32
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
+        const uint32_t v = (X >> (16 * h)) & 0xFFFFu;
+        const uint32_t wq = div12(v);
+        const uint2 e =
+            move_entry(trans, entry_offset(pc, q, (v - 12u * wq) * 264u + near128));
+        t[q] = (uint32_t)__dp4a((int)e.y, (int)((env[hi].ev[q] >> (4 * c)) & kEnvMask), (int)e.x);
+        d[q] = wq - level_at(thrT, t[q] & 0xFFFFu);  // negative: accept; zero: a tie
+      }
+      mn = __vimin3_u32(mn, d[0], d[1]);
+      mn = __vimin3_u32(mn, d[2], d[3]);
+      // byte q: the accepted move of lane q, i.e. byte 3 of t[q] under the sign
+      // of d[q] (byte permutes: bit 3 of a selector replicates a byte's sign)
+      const uint32_t acc = prmt(prmt(d[0], d[1], 0x00FBu), prmt(d[2], d[3], 0x00FBu), 0x5410u) &
+                           prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
+      // byte q of acc -> site k + 4 q: b bits to 2 (k + 4 q) of dB, a bits of dA
+      dB |= (acc & 0x03030303u) << (2 * k);
+      dA |= ((acc >> 2) & 0x03030303u) << (2 * k);
+    }
+    // a rare pair: a tie, or a field >= 65532 in either half of the call's words
+    const uint32_t mx = __vmaxu2(__vimax3_u16x2(r.x, r.y, r.z), r.w);
+    if (mn == 0u || mx >= 0xFFFC0000u || (mx & 0xFFFFu) >= 0xFFFCu) slow |= 1u << c;
+  }
+  return make_uint3(dA, dB, slow);
+}
+
+// The exact decision of pair t = k + 4 q (group k = 2 c + h, lane q of the group)
+// of MOVE call c of word w of class row j: the accepted move if the pair is rare
+// (the fast path rejected it), decided with its SLOW words, else 0.
+__device__ __forceinline__ uint32_t exact_move(const Geo &g, const uint2 *trans,
+                                               const uint16_t *thrT, const uint32_t *thr32, int j,
+                                               int w, int c, int h, int q, const WordIn &in,
+                                               uint64_t P, uint32_t near128) {
+  const int t = 2 * c + h + 4 * q;
+  const uint32_t gbase = (uint32_t)j * (uint32_t)(2 * g.W) + (uint32_t)(2 * w);
+  const U4 r = philox(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE, g.k0, g.k1);
+  const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
+  const uint32_t v = h ? X >> 16 : X & 0xFFFFu;
+  const uint32_t wq = div12(v);
+  // the pair's own counts and state, from bits 2 t and 2 t + 1 of the planes
+  auto counts = [&](const Planes &p) {
+    const uint32_t O = p.O >> (2 * t), T = p.T >> (2 * t), F = p.F >> (2 * t);
+    return ((O & 2u) + 2u * (T & 2u) + 4u * (F & 2u)) |
+           (((O & 1u) + 2u * (T & 1u) + 4u * (F & 1u)) << 8);
+  };
+  const uint32_t env = counts(in.na) | (counts(in.nb) << 16);
+  const uint32_t pc8 = ((((in.A >> (2 * t)) & 3u) << 2) | ((in.B >> (2 * t)) & 3u)) << 3;
+  uint2 e = move_entry(trans, ((v - 12u * wq) * 264u + near128) ^ pc8);
+  if (v < 65532u && wq != level_at(thrT, (uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu))
+    return 0u;  // not rare
+  const uint32_t slow0 = (uint32_t)((uint64_t)j * g.Cx + (uint32_t)(w << 4));
+  const U4 sl = philox(slow0 + (uint32_t)t, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, g.k0, g.k1);
+  if (v >= 65532u) {
+    if (sl.y >= 4294967292u) return 0u;  // keep the current configuration
+    e = move_entry(trans, ((sl.y % 12u) * 264u + near128) ^ pc8);
+  }
+  const uint32_t thr = thr32[((uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu) >> 1];
+  const bool accept = thr == 0xFFFFFFFFu ||
+                      (v < 65532u ? ((uint64_t)wq << 32) + sl.x < 5461ull * thr : sl.x < thr);
+  return accept ? e.x >> 24 : 0u;
+}
+
+}  // namespace ccmc
