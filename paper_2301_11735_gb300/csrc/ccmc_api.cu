@@ -155,7 +155,7 @@ int upload_params_on(ccmc_lattice *h, double beta, double Delta, double V, doubl
   if (h->have_params && h->params[0] == beta && h->params[1] == Delta && h->params[2] == V &&
       h->params[3] == J)
     return CCMC_OK;
-  uint32_t thr32[kDevN];
+  uint32_t thr32[kDevPad] = {};
   uint16_t thrT[kThrT] = {};
   build_device_thresholds(beta, Delta, V, J, thr32);
   for (int i = 0; i < kDevN; ++i) thrT[i] = threshold_level(thr32[i]);
@@ -217,7 +217,6 @@ ResJob resident_job(const ccmc_lattice *h, int64_t nsweeps, int obs_every, int r
   ResJob j{};
   j.g = h->g;
   j.thrT = h->t.thrT;
-  j.thr32 = h->t.thr32;
   j.nsweeps = (int)nsweeps;
   j.ring = h->d_ring;
   j.ring_cap = h->ring_cap;
@@ -225,12 +224,16 @@ ResJob resident_job(const ccmc_lattice *h, int64_t nsweeps, int obs_every, int r
   j.nbins = h->nbins;
   j.obs_every = obs_every;
   j.rows = rows;
+  for (uint32_t r = 0; r < 10; ++r) {
+    j.rk[2 * r] = h->g.k0 + r * 0x9E3779B9u;
+    j.rk[2 * r + 1] = h->g.k1 + r * 0xBB67AE85u;
+  }
   return j;
 }
 
 // Sweep one lattice by the resident kernel, a bounded number of sweeps a launch.
 int resident_sweeps(ccmc_lattice *h, int64_t nsweeps, int obs_every) {
-  const ResShape sh = resident_shape(h->g, kResMaxCluster, 0.0, 512, 4);
+  const ResShape sh = resident_shape(h->g, kResMaxCluster, 0.0, kResMaxWorkers, 4);
   for (int64_t s = 0; s < nsweeps; s += kResMaxSweeps) {
     const ResJob j =
         resident_job(h, std::min<int64_t>(nsweeps - s, kResMaxSweeps), obs_every, sh.rows);
@@ -352,7 +355,7 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
   }
   const int np = recount_grid(g);
   const int dev = h->device;
-  const size_t tb = sizeof(uint32_t) * (kDevN + 2 * kMoveN) + sizeof(uint16_t) * kThrT;
+  const size_t tb = sizeof(uint32_t) * (kDevPad + 2 * kMoveN) + sizeof(uint16_t) * kThrT;
   if (!dalloc((void **)&h->d_words, sizeof(uint32_t) * 16 * g.cstride, dev, h->stream) ||
       !dalloc((void **)&h->d_ctl, sizeof(int64_t) * kCtlWords, dev, h->stream) ||
       !dalloc((void **)&h->d_partials, sizeof(int64_t) * 7 * np, dev, h->stream) ||
@@ -761,9 +764,9 @@ struct ccmc_batch {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   ResJob *d_jobs = nullptr;  // resident lattices
-  int threads = 256;
+  int threads = kResMaxWorkers;
   int64_t resident_max_sites = -1;  // -1: the lattices that ccmc_sweep holds resident
-  int ctas_per_sm = 2;
+  int ctas_per_sm = 1;
   int max_tpw = 4;
   int sms = 152;
   cudaEvent_t ev = nullptr;
@@ -819,25 +822,41 @@ int run_resident(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats,
   double words = 0;
   for (int i : which) words += (double)lats[i]->g.cstride;
   const double ctas = (double)b->sms * b->ctas_per_sm;
-  std::vector<ResGroup> groups;
+  struct Plan {
+    int i;
+    ResShape shape;
+    bool aligned;
+  };
+  std::vector<Plan> plans;
   for (int i : which) {
-    ccmc_lattice *h = lats[i];
-    const ResShape sh =
-        resident_shape(h->g, ctas * (double)h->g.cstride / words, words / b->sms,
-                       b->threads, b->max_tpw);
-    const bool al = (h->g.Cx & 15) == 0;
+    const Geo &g = lats[i]->g;
+    plans.push_back({i,
+                     resident_shape(g, ctas * (double)g.cstride / words, words / b->sms,
+                                    b->threads, b->max_tpw),
+                     (g.Cx & 15) == 0});
+  }
+  auto same = [](const ResShape &x, const ResShape &y) {
+    return x.cluster == y.cluster && x.tpw == y.tpw && x.workers == y.workers;
+  };
+  std::vector<ResGroup> groups;
+  for (const Plan &p : plans) {
+    const ccmc_lattice *h = lats[p.i];
+    ResShape sh = p.shape;
+    if (sh.cluster > 1) {
+      int n = 0;
+      for (const Plan &o : plans) n += same(o.shape, p.shape);
+      sh = resident_fit(h->g, sh, p.aligned, n);
+    }
     ResGroup *hit = nullptr;
     for (ResGroup &G : groups)
-      if (G.shape.cluster == sh.cluster && G.shape.tpw == sh.tpw &&
-          G.shape.threads == sh.threads && G.aligned == al)
-        hit = &G;
+      if (same(G.shape, sh) && G.aligned == p.aligned) hit = &G;
     if (!hit) {
-      groups.push_back(ResGroup{sh, al, 0.0, {}});
+      groups.push_back(ResGroup{sh, p.aligned, 0.0, {}});
       hit = &groups.back();
     }
     hit->shape.smem = std::max(hit->shape.smem, sh.smem);
-    hit->cost = std::max(hit->cost, (double)sh.rows * h->g.W * (double)nsweeps[i]);
-    hit->jobs.push_back(resident_job(h, nsweeps[i], obs_every[i], sh.rows));
+    hit->cost = std::max(hit->cost, (double)sh.rows * h->g.W * (double)nsweeps[p.i]);
+    hit->jobs.push_back(resident_job(h, nsweeps[p.i], obs_every[p.i], sh.rows));
   }
   // the longest first, in every launch and over the launches
   std::sort(groups.begin(), groups.end(),

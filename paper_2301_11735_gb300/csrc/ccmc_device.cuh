@@ -44,8 +44,9 @@ __device__ __forceinline__ U4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint
                                      uint32_t k0, uint32_t k1) {
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
-    const uint32_t lo0 = 0xD2511F53u * c0, hi0 = __umulhi(0xD2511F53u, c0);
-    const uint32_t lo1 = 0xCD9E8D57u * c2, hi1 = __umulhi(0xCD9E8D57u, c2);
+    uint32_t lo0, hi0, lo1, hi1;
+    mul_wide(0xD2511F53u, c0, lo0, hi0);
+    mul_wide(0xCD9E8D57u, c2, lo1, hi1);
     c0 = hi1 ^ c1 ^ k0;
     c2 = hi0 ^ c3 ^ k1;
     c1 = lo1;
@@ -164,6 +165,11 @@ __device__ __forceinline__ bool offset_allowed(int Lx, int Ly, int rx, int ry) {
   return true;
 }
 
+// Whether the offset joins nearest neighbours.
+__device__ __forceinline__ int is_near(const Geo &g, int rx, int ry) {
+  return (ry == 0 && (rx == 1 || rx == g.Lx - 1)) || (rx == 0 && (ry == 1 || ry == g.Ly - 1));
+}
+
 // Executed by one full warp; every lane returns the same schedule.
 __device__ __forceinline__ Sched draw_schedule(const Geo &g, uint64_t P) {
   const unsigned lane = threadIdx.x & 31u;
@@ -187,8 +193,7 @@ __device__ __forceinline__ Sched draw_schedule(const Geo &g, uint64_t P) {
       break;
     }
   }
-  s.near = (s.ry == 0 && (s.rx == 1 || s.rx == g.Lx - 1)) ||
-           (s.rx == 0 && (s.ry == 1 || s.ry == g.Ly - 1));
+  s.near = is_near(g, s.rx, s.ry);
   return s;
 }
 

@@ -63,13 +63,14 @@ constexpr int kSegW = 2 * kSegR + 1;          // 19
 constexpr int kSegSwap = 3 * kSegW * kSegW;   // first entry of the second segment: 1083
 constexpr int kSegFlip = kSegSwap + kNB;      // and of the third: 1124
 constexpr int kDevN = kSegFlip + kNB;         // 1165
+constexpr int kDevPad = (kDevN + 3) / 4 * 4;  // thr32 padded to 16 bytes
 
 // Per-lattice parameter tables in device memory (built on the host).
 struct DevTables {
   uint16_t *thrT;   // kThrT: threshold levels T = floor(5461 thr / 2^32), 5461 for
                     // thr = 0xFFFFFFFF (fast path)
   uint32_t *trans;  // kMoveN x 2 words: move entries (see kMoveN), directly after thrT
-  uint32_t *thr32;  // kDevN: full thresholds (exact path)
+  uint32_t *thr32;  // kDevPad: full thresholds (exact path), directly after trans
 };
 
 // The fast path's threshold level of a 32-bit threshold: a field's w = v / 12
@@ -96,8 +97,7 @@ struct LaunchCfg {
 // of one CTA or of a cluster, each CTA owning `rows` rows of every class.
 struct ResJob {
   Geo g;                  // the lattice in global memory
-  const uint16_t *thrT;   // its tables (levels, then moves: one block)
-  const uint32_t *thr32;
+  const uint16_t *thrT;   // its tables (levels, moves, full thresholds: one block)
   int nsweeps;            // sweeps to run in this launch, at most kResMaxSweeps
   int64_t *ring;          // observable ring (records every obs_every sweeps)
   int64_t ring_cap;
@@ -105,17 +105,19 @@ struct ResJob {
   int nbins;
   int obs_every;
   int rows;
+  alignas(16) uint32_t rk[20];  // Philox round keys: round r's at 2 r, 2 r + 1
 };
 
 // Launch shape of a resident launch: CTAs a lattice, rows of each class a CTA,
-// threads a word, threads a CTA (the workers and the auxiliary warp), dynamic
-// shared memory.
+// threads a word, workers a CTA and all its threads, dynamic shared memory.
 struct ResShape {
-  int cluster = 0, rows = 0, tpw = 1, threads = 0;
+  int cluster = 0, rows = 0, tpw = 1, workers = 0, threads = 0;
   int64_t smem = 0;
 };
 
-constexpr int kResMaxThreads = 1024;
+constexpr int kResMaxWorkers = 512;
+constexpr int kResMaxThreads = kResMaxWorkers + 32;                        // 1, 2 threads a word
+constexpr int kResMaxThreads4 = kResMaxWorkers + kResMaxWorkers / 2 + 32;  // four
 constexpr int kResMaxCluster = 16;
 constexpr int kResClusterWords = 128;  // lattices of fewer a-words a phase take one CTA
 constexpr int kResMinWords = 16;       // a-words a CTA of a cluster at least
@@ -181,6 +183,9 @@ int64_t resident_smem(const Geo &g, int rows);
 // one) while `load` a-words a phase run on an average SM, with at most
 // max_threads workers a CTA and max_tpw threads a word.
 ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads, int max_tpw);
+// The shape for n such lattices in one launch: another one when their clusters
+// would not all fit the GPU at once.
+ResShape resident_fit(const Geo &g, const ResShape &shape, bool aligned, int n);
 cudaError_t launch_resident_sweep(const ResJob *one, const ResJob *d_jobs, int njobs,
                                   const ResShape &shape, bool aligned, cudaStream_t s);
 cudaError_t launch_philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,

@@ -35,10 +35,8 @@ namespace ccmc {
 //   accept = w < T(offset), with T = floor(5461 thr / 2^32) (5461 when thr is
 //            0xFFFFFFFF): w < T implies w 2^32 + s < 5461 thr for every 32-bit
 //            s, w > T the opposite
-// The fast decision is always applied.  A tie (w == T) or a field v >= 65532
-// sends the call's pairs through the exact path, which decides each truly rare
-// pair (the fast path rejected it) with its SLOW random words (about one pair
-// in 4000).
+// A tie (w == T) or a field v >= 65532 (about one pair in 4000, rejected by the
+// fast decision) is decided exactly, with the pair's SLOW random words.
 struct PhaseSmem {
   uint2 trans[kMoveN];
   uint16_t thrT[kThrT];
@@ -191,7 +189,7 @@ __device__ __forceinline__ void exact_pair(const Geo &g, const PhaseU &u, const 
                                            const WordIn &in, uint64_t P, uint32_t near128) {
   const int t = 2 * c + h + 4 * q;
   if (t >= n) return;  // past the end of the row: no pair
-  const uint32_t x = exact_move(g, trans, thrT, thr32, j, w, c, h, q, in, P, near128);
+  const uint32_t x = exact_move(g, trans, thrT, thr32, j, w, t, in, P, near128);
   if (x) apply_moves<kMode, false>(g, u, jr, w, n, (x >> 2) << (2 * t), (x & 3u) << (2 * t));
 }
 
@@ -205,23 +203,22 @@ __device__ __forceinline__ void exact_pair(const Geo &g, const PhaseU &u, const 
 // u's arrays (j itself for a lattice in global memory, the row inside a
 // staged tile otherwise); near128: 128 if the phase's partners are nearest
 // neighbours, else 0; keys: the source of the Philox keys (SeedKeys or
-// TableKeys of the lattice's seed); kTPW threads share the word, this lane is
-// thread `sub` of them (see fast_moves).
-template <int kMode, int kTPW = 1, class Keys = SeedKeys>
+// TableKeys of the lattice's seed).
+template <int kMode, class Keys>
 __device__ __forceinline__ void warp_word(const Geo &g, const PhaseU &u, const uint2 *trans,
                                           const uint16_t *thrT, const uint32_t *thr32, int j,
                                           int jr, int w, uint64_t P, uint32_t near128,
-                                          const Keys &keys, int sub = 0, bool active = true) {
+                                          const Keys &keys, bool active = true) {
   const int n = active ? (kMode == kRowGeneral ? min(16, g.Cx - (w << 4)) : 16) : 0;
   WordIn in{};
   uint32_t rz = 0u;
   if (active) {
     in = gather<kMode>(g, u, jr, w, n);
     const uint32_t gbase = (uint32_t)j * (uint32_t)(2 * g.W) + (uint32_t)(2 * w);
-    const uint3 d = fast_moves<kTPW>(trans, thrT, sub, in, near128, [&](int c) {
+    const uint3 d = fast_moves<1, false>(trans, thrT, 0, in, near128, [&](int c) {
       return keys(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE);
     });
-    apply_moves<kMode, kTPW == 1>(g, u, jr, w, n, d.x, d.y);
+    apply_moves<kMode, true>(g, u, jr, w, n, d.x, d.y);
     rz = d.z;
   }
   unsigned ball = __ballot_sync(0xFFFFFFFFu, rz != 0u);
@@ -244,17 +241,9 @@ __device__ __forceinline__ void warp_word(const Geo &g, const PhaseU &u, const u
       o.nb.F = __shfl_sync(0xFFFFFFFFu, in.nb.F, src);
       const int oj = __shfl_sync(0xFFFFFFFFu, j, src), ojr = __shfl_sync(0xFFFFFFFFu, jr, src),
                 ow = __shfl_sync(0xFFFFFFFFu, w, src), on = __shfl_sync(0xFFFFFFFFu, n, src);
-      // the owner's pairs, one a lane: 16 (both calls), 8 (one call) or 4
-      int c, h;
-      if constexpr (kTPW == 1) {
-        c = (lane >> 3) & 1;
-        h = (lane >> 2) & 1;
-      } else {
-        const int osub = __shfl_sync(0xFFFFFFFFu, sub, src);
-        c = kTPW == 2 ? osub : osub >> 1;
-        h = kTPW == 2 ? (lane >> 2) & 1 : osub & 1;
-      }
-      if (lane < 16 / kTPW && ((orz >> c) & 1u))
+      // the owner's pairs, one a lane
+      const int c = (lane >> 3) & 1, h = (lane >> 2) & 1;
+      if (lane < 16 && ((orz >> c) & 1u))
         exact_pair<kMode>(g, u, trans, thrT, thr32, oj, ojr, ow, on, c, h, lane & 3, o, P,
                           near128);
     }
@@ -290,14 +279,12 @@ __global__ void __launch_bounds__(256, 4) phase_kernel(Geo g, const uint16_t *th
   const uint32_t near128 = sc.near ? 128u : 0u;
   const int nw = g.Cy * g.W;
   const int stride = gridDim.x * blockDim.x;
-  // a trip count uniform across the block, so that every warp's lanes stay
-  // together for the cooperative exact path
   for (int base = blockIdx.x * blockDim.x; base < nw; base += stride) {
     const int wid = base + threadIdx.x;
     const bool act = wid < nw;
     const int j = act ? wid / g.W : 0, w = act ? wid - j * g.W : 0;
     warp_word<kAligned ? kRowAligned : kRowGeneral>(g, u, sm.trans, sm.thrT, thr32, j, j, w, P,
-                                                     near128, SeedKeys{g.k0, g.k1}, 0, act);
+                                                     near128, SeedKeys{g.k0, g.k1}, act);
   }
 }
 
@@ -427,14 +414,13 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // One tile-staged phase of lattice g by CTA `cta` of the `ncta` CTAs that
 // work on it; keys: the source of its Philox keys.
 // kSingle: every CTA takes at most one tile (ncta == tiles): one band buffer.
-// kTPW: threads a word (the CTA has kTileWords kTPW threads; see fast_moves).
-template <bool kSingle, int kTPW, class Keys>
+template <bool kSingle, class Keys>
 __device__ __forceinline__ void tile_phase(const Geo &g, const uint16_t *thrT,
                                            const uint32_t *thr32, int64_t p_off, int cta,
                                            int ncta, const Keys &keys) {
   extern __shared__ __align__(128) unsigned char tile_smem[];
   constexpr int kBufs = kSingle ? 1 : kTileBufs;
-  constexpr int kWarps = kTileWords * kTPW / 32;
+  constexpr int kWarps = kTileWords / 32;
   using Smem = TileSmem<kBufs>;
   Smem &sm = *reinterpret_cast<Smem *>(tile_smem);
   static_assert(offsetof(Smem, trans) == 2 * kThrT, "tables staged as one block");
@@ -565,7 +551,7 @@ __device__ __forceinline__ void tile_phase(const Geo &g, const uint16_t *thrT,
   if (!mbar_wait(smem_u32(&sm.tables), 0u)) sm.err = 1;
 
   const int lw = __ffs(W) - 1;  // W is a power of two
-  const int wi = (int)threadIdx.x / kTPW, sub = (int)threadIdx.x % kTPW;  // word of the tile
+  const int wi = (int)threadIdx.x;  // word of the tile
   const int jr = wi >> lw, w = wi & (W - 1);
   // a tile's bands in buffer b as the windows' sources
   auto local_u = [&](int b) {
@@ -592,8 +578,8 @@ __device__ __forceinline__ void tile_phase(const Geo &g, const uint16_t *thrT,
     }
     const int tile = sm.tile[b];
     if (tile < 0) break;
-    warp_word<kRowTile, kTPW>(g, local_u(b), sm.trans, sm.thrT, thr32, tile * R + jr, jr, w, P,
-                              near128, keys, sub);
+    warp_word<kRowTile>(g, local_u(b), sm.trans, sm.thrT, thr32, tile * R + jr, jr, w, P, near128,
+                        keys);
     // (2) this warp is done with the tile: its shared-memory writes are ordered
     // before the async copies that will refill the buffer, and before the
     // last warp's reads
@@ -664,11 +650,11 @@ __device__ __forceinline__ void tile_phase(const Geo &g, const uint16_t *thrT,
 // large-lattice kernel), or five CTAs per SM, one tile per CTA and one band
 // buffer (the compact kernel for lattices whose phase fits one wave: more CTAs
 // resident for several lattices on their own streams, at 48 registers).
-template <int kMinBlocks, bool kSingle, int kTPW = 1>
-__global__ void __launch_bounds__(256 * kTPW, kMinBlocks) phase_tile_kernel(
+template <int kMinBlocks, bool kSingle>
+__global__ void __launch_bounds__(kTileWords, kMinBlocks) phase_tile_kernel(
     Geo g, const uint16_t *thrT, const uint32_t *thr32, int64_t p_off,
     const __grid_constant__ RoundKeys rk) {
-  tile_phase<kSingle, kTPW>(g, thrT, thr32, p_off, (int)blockIdx.x, (int)gridDim.x,
+  tile_phase<kSingle>(g, thrT, thr32, p_off, (int)blockIdx.x, (int)gridDim.x,
                             TableKeys{&rk});
 }
 
@@ -681,7 +667,7 @@ __global__ void __launch_bounds__(256, 4) phase_tile_multi_kernel(const MultiJob
   while (j + 1 < njobs && (int)blockIdx.x >= jobs[j + 1].cta_begin) ++j;
   const MultiJob &J = jobs[j];
   const Geo g = J.g;
-  tile_phase<false, 1>(g, J.thrT, J.thr32, p_off, (int)blockIdx.x - J.cta_begin, J.cta_count,
+  tile_phase<false>(g, J.thrT, J.thr32, p_off, (int)blockIdx.x - J.cta_begin, J.cta_count,
                        SeedKeys{g.k0, g.k1});
 }
 
@@ -724,7 +710,7 @@ __global__ void __launch_bounds__(256, 4) phase_multi_kernel(const MultiJob *__r
     const bool act = wid < nw;
     const int j = act ? wid / g.W : 0, w = act ? wid - j * g.W : 0;
     warp_word<kAligned ? kRowAligned : kRowGeneral>(g, u, sm.trans, sm.thrT, J.thr32, j, j, w, P,
-                                                     near128, SeedKeys{g.k0, g.k1}, 0, act);
+                                                     near128, SeedKeys{g.k0, g.k1}, act);
   }
 }
 
@@ -769,13 +755,8 @@ int tile_resident_grid() {
   return per_sm * sms;
 }
 
-// The single-tile kernel: one thread a word, five CTAs per SM (48 registers;
-// six at 40 registers spilled more and measured slower).  Two threads a word
-// (512-thread CTAs, two per SM) measured 5.6 us a 4096^2 phase against 5.4,
-// and half the throughput for four such lattices on their own streams: the
-// phase is bound by the issue rate of the SMs that hold two tiles, not by the
-// chain of one thread.
-constexpr int kSmallTPW = 1;
+// The single-tile kernel: five CTAs per SM (48 registers; six at 40 registers
+// spilled more and measured slower).
 constexpr int kSmallMinB = 5;
 
 int tile_resident_grid_small() {
@@ -783,10 +764,10 @@ int tile_resident_grid_small() {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   constexpr int bytes = (int)sizeof(TileSmem<1>);
-  if (cudaFuncSetAttribute(phase_tile_kernel<kSmallMinB, true, kSmallTPW>,
+  if (cudaFuncSetAttribute(phase_tile_kernel<kSmallMinB, true>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &per_sm, phase_tile_kernel<kSmallMinB, true, kSmallTPW>, 256 * kSmallTPW, bytes) !=
+          &per_sm, phase_tile_kernel<kSmallMinB, true>, 256, bytes) !=
           cudaSuccess ||
       per_sm < 1 || sms < 1) {
     cudaGetLastError();
@@ -807,8 +788,8 @@ cudaError_t launch_phase(const Geo &g, const DevTables &t, int64_t p_off, const 
     // A phase that fits one wave of the compact kernel (one tile per CTA)
     // takes it: measured faster for several such lattices on their own streams.
     if (cfg.tile_grid_small > 0 && tiles <= cfg.tile_grid_small)
-      return launch_pdl_smem(phase_tile_kernel<kSmallMinB, true, kSmallTPW>, (int)tiles,
-                             256 * kSmallTPW, sizeof(TileSmem<1>), s, g,
+      return launch_pdl_smem(phase_tile_kernel<kSmallMinB, true>, (int)tiles,
+                             256, sizeof(TileSmem<1>), s, g,
                              (const uint16_t *)t.thrT, t.thr32, p_off, round_keys(g.k0, g.k1));
     const int grid = (int)(tiles < cfg.tile_grid ? tiles : cfg.tile_grid);
     return launch_pdl_smem(phase_tile_kernel<4, false>, grid, 256, sizeof(TileSmem<>),

@@ -4,7 +4,7 @@
 // A CTA (or every CTA of a cluster of C) owns `rows` consecutive rows of each of
 // the 16 residue classes; its worker threads evaluate the a-class words of those
 // rows in every phase, one, two or four threads a word, and one more warp, the
-// auxiliary warp, draws the phase schedules two phases ahead (double Philox
+// auxiliary warp, draws the next sweep's eight phase schedules side by side (Philox
 // and divisions off the workers' chain) and writes the observable records.
 // The a side of a word is the CTA's own; the b side (the partner rows) may
 // belong to another CTA of the cluster and is read and changed through
@@ -19,6 +19,7 @@
 // larger ones are bound by integer issue on their CTAs' SMs.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <mutex>
 
@@ -30,21 +31,27 @@ namespace ccmc {
 
 namespace {
 
-constexpr uint32_t kTableBytes = 2u * kThrT + 8u * kMoveN;
-static_assert(kTableBytes % 16 == 0, "the lattice words start on 16 bytes");
+// Levels, moves and full thresholds (the rare pairs' path must not wait for
+// global memory while the CTA waits at the barrier).
+constexpr uint32_t kFastBytes = 2u * kThrT + 8u * kMoveN;
+constexpr uint32_t kTableBytes = kFastBytes + 4u * kDevPad;
+static_assert(kFastBytes % 16 == 0 && kTableBytes % 16 == 0, "copied 16 bytes at a time");
 
-// One phase's uniforms: classes as byte offsets into a CTA's words, column
-// offsets in sites.  Of a site's two column neighbours at most one lies in
-// another column block, and of its two row neighbours at most one in another
-// row: the neighbour sums do not care which is which, so each side has its own
-// class, one column neighbour read at the side's own column (cAm, cBm) and one
-// at a column xA, xB sites further (cAx, cBx: -1, 0 or 1; for b as the offset
-// offX), one row neighbour in its own row (cAr, cBr) and one yA, yB rows further
-// (cAy, cBy).
+// One phase's uniforms of one side (a or b): classes as byte offsets into a CTA's
+// words, column offsets in sites, row offsets.  Of a site's two column neighbours
+// at most one lies in another column block, and of its two row neighbours at most
+// one in another row: the neighbour sums do not care which is which, so a side
+// has its own class c, one column neighbour read at the side's own column (m) and
+// one xs = -1, 0 or 1 sites further (x), one row neighbour in its own row (r)
+// and one ys rows further (y).  The side's sites lie qx columns and qy rows from
+// the a sites (0, 0 for a itself); offX = qx + xs in [0, Cx).
+struct alignas(16) SideD {
+  uint32_t c, m, x, r, y;
+  int qx, offX, qy, ys, xs;
+  int pad[2];
+};
 struct alignas(16) PhaseD {
-  uint32_t cA, cAm, cAx, cAr, cAy;
-  uint32_t cB, cBm, cBx, cBr, cBy;
-  int xA, yA, yB, qx, qy, offX;
+  SideD side[2];
   uint32_t near128;
 };
 
@@ -116,30 +123,57 @@ __device__ __forceinline__ PhaseD phase_desc(const Geo &g, const Sched &sc, uint
   // -1 when the left (upper) neighbours lie in the block (row) before, +1 when the
   // right (lower) ones lie in the next
   auto shift = [](int c) { return c == 0 ? -1 : c == 3 ? 1 : 0; };
-  auto side = [&](int cx, int cy, uint32_t &c, uint32_t &m, uint32_t &x, uint32_t &r,
-                  uint32_t &y) {
+  auto side = [&](SideD &d, int x, int y) {
+    const int cx = x & 3, cy = y & 3;
     const int dx = cx == 3 ? 1 : -1, dy = cy == 3 ? 1 : -1;  // the further ones
-    c = cls(cx, cy);
-    m = cls(cx - dx, cy);
-    x = cls(cx + dx, cy);
-    r = cls(cx, cy - dy);
-    y = cls(cx, cy + dy);
+    d.c = cls(cx, cy);
+    d.m = cls(cx - dx, cy);
+    d.x = cls(cx + dx, cy);
+    d.r = cls(cx, cy - dy);
+    d.y = cls(cx, cy + dy);
+    int qx = x >> 2, qy = y >> 2;  // an offset is below the size: at most one turn
+    if (qx >= g.Cx) qx -= g.Cx;
+    if (qy >= g.Cy) qy -= g.Cy;
+    d.qx = qx;
+    d.qy = qy;
+    d.xs = shift(cx);
+    d.ys = shift(cy);
+    d.offX = wrap_row(qx + d.xs, g.Cx);
   };
-  const int ax = sc.a0x, ay = sc.a0y;
-  const int bx = ax + sc.rx, by = ay + sc.ry, cbx = bx & 3, cby = by & 3;
-  side(ax, ay, u.cA, u.cAm, u.cAx, u.cAr, u.cAy);
-  side(cbx, cby, u.cB, u.cBm, u.cBx, u.cBr, u.cBy);
-  u.xA = shift(ax);
-  u.yA = shift(ay);
-  u.yB = shift(cby);
-  int qx = bx >> 2, qy = by >> 2;  // rx < Lx: at most one turn
-  if (qx >= g.Cx) qx -= g.Cx;
-  if (qy >= g.Cy) qy -= g.Cy;
-  u.qx = qx;
-  u.qy = qy;
-  u.offX = wrap_row(qx + shift(cbx), g.Cx);
+  side(u.side[0], sc.a0x, sc.a0y);
+  side(u.side[1], sc.a0x + sc.rx, sc.a0y + sc.ry);
   u.near128 = sc.near ? 128u : 0u;
   return u;
+}
+
+// The uniforms of phases P .. P + 7 by one warp: four lanes a phase, each trying
+// attempts lane mod 4, + 4, ... (draw_schedule's: the first allowed one of at most
+// 64 wins, then the fixed offset); one round settles a phase with probability 0.99.
+__device__ __forceinline__ void describe_sweep(const Geo &g, uint64_t P, uint32_t cls_bytes,
+                                               PhaseD *s_d) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t p = P + (lane >> 2), N = (uint64_t)g.Lx * (uint64_t)g.Ly;
+  bool done = false;
+#pragma unroll 1
+  for (uint32_t round = 0; round < 16u; ++round) {
+    const U4 w = philox(4u * round + (lane & 3u), (uint32_t)p, (uint32_t)(p >> 32), TAG_SCHED,
+                        g.k0, g.k1);
+    const uint64_t x = ((uint64_t)w.z << 32) | (uint64_t)w.y;
+    const uint32_t idx = (uint32_t)__umul64hi(x, N);
+    Sched s;
+    s.a0x = (int)(w.x & 3u);
+    s.a0y = (int)((w.x >> 2) & 3u);
+    s.ry = (int)(idx / (uint32_t)g.Lx);
+    s.rx = (int)(idx - (uint32_t)s.ry * (uint32_t)g.Lx);
+    s.near = is_near(g, s.rx, s.ry);
+    const bool ok = !done && x * N >= g.rej && offset_allowed(g.Lx, g.Ly, s.rx, s.ry);
+    const uint32_t m = (__ballot_sync(0xFFFFFFFFu, ok) >> (lane & ~3u)) & 15u;
+    if (m && (lane & 3u) == (uint32_t)__ffs((int)m) - 1u) s_d[p & 15u] = phase_desc(g, s, cls_bytes);
+    done = done || m;
+    if (__all_sync(0xFFFFFFFFu, done)) return;
+  }
+  if (!done && (lane & 3u) == 0)
+    s_d[p & 15u] = phase_desc(g, Sched{0, 0, 2, 2, is_near(g, 2, 2)}, cls_bytes);
 }
 
 // The words and shift of the window of 16 sites at column 16 w + off (mod Cx) of
@@ -243,95 +277,212 @@ __device__ __forceinline__ uint32_t side_window(const Geo &g, const Spot &p, uin
   return __funnelshift_r(lo, hi, 2 * x);  // the shift counts modulo 32
 }
 
+// Row jb of a side's sites for the a sites' row l of this CTA.
+__device__ __forceinline__ int side_row(const Geo &g, const Place &pl, const SideD &d, int l) {
+  const int jb = pl.row0 + l + d.qy;
+  return jb >= g.Cy ? jb - g.Cy : jb;
+}
+
+// One side of a word read the general way (rows anywhere in the cluster): the
+// 16 sites and their neighbours' counts.
+struct SideIn {
+  uint32_t X;
+  Planes n;
+};
+
+template <bool kCl, bool kAl>
+__device__ __forceinline__ SideIn gather_side(const Geo &g, const SideD &d, const Place &pl,
+                                              int l, const Win &win, uint32_t row, int w) {
+  SideIn in;
+  const uint32_t ry = d.ys ? row_addr<kCl>(pl, wrap_row(side_row(g, pl, d, l) + d.ys, g.Cy)) : row;
+  in.X = read_window<kCl, kAl>(row + d.c, win);
+  const uint32_t m = read_window<kCl, kAl>(row + d.m, win);
+  const uint32_t r = read_window<kCl, kAl>(row + d.r, win);
+  const uint32_t x = read_window<kCl, kAl>(row + d.x, window_at<kAl>(g, w, d.offX));
+  const uint32_t y = read_window<kCl, kAl>(ry + d.y, win);
+  in.n = neighbour_planes(m, r, x, y);
+  return in;
+}
+
+// Both sides of a word, the a side (this CTA's rows, whole words) read directly.
 template <bool kCl, bool kAl>
 __device__ __forceinline__ WordIn gather_word(const Geo &g, const PhaseD &u, const Place &pl,
                                               const Spot &p) {
   WordIn in;
+  const SideD &a = u.side[0], &b = u.side[1];
+  {
+    const uint32_t row = row_addr<kCl>(pl, side_row(g, pl, b, p.l));
+    const SideIn s =
+        gather_side<kCl, kAl>(g, b, pl, p.l, window_at<kAl>(g, p.w, b.qx), row, p.w);
+    in.B = s.X;
+    in.nb = s.n;
+  }
   const int j = pl.row0 + p.l;
-  int jb = j + u.qy;
-  jb = jb >= g.Cy ? jb - g.Cy : jb;
-  const uint32_t rb = row_addr<kCl>(pl, jb);
-  const uint32_t ry = u.yB ? row_addr<kCl>(pl, wrap_row(jb + u.yB, g.Cy)) : rb;
-  const Win wb = window_at<kAl>(g, p.w, u.qx);
-  in.B = read_window<kCl, kAl>(rb + u.cB, wb);
-  const uint32_t bm = read_window<kCl, kAl>(rb + u.cBm, wb);
-  const uint32_t br = read_window<kCl, kAl>(rb + u.cBr, wb);
-  const uint32_t bx = read_window<kCl, kAl>(rb + u.cBx, window_at<kAl>(g, p.w, u.offX));
-  const uint32_t by = read_window<kCl, kAl>(ry + u.cBy, wb);
   const uint32_t own = pl.base + p.off;
-  in.A = ld_word<false>(own + u.cA);
-  const uint32_t am = ld_word<false>(own + u.cAm);
-  const uint32_t ar = ld_word<false>(own + u.cAr);
-  const uint32_t ax = side_window<kAl>(g, p, own + u.cAx, u.xA);
+  in.A = ld_word<false>(own + a.c);
+  const uint32_t am = ld_word<false>(own + a.m);
+  const uint32_t ar = ld_word<false>(own + a.r);
+  const uint32_t ax = side_window<kAl>(g, p, own + a.x, a.xs);
   uint32_t ay;
   if constexpr (kCl) {
-    ay = u.yA ? ld_word<true>(row_addr<true>(pl, wrap_row(j + u.yA, g.Cy)) + u.cAy +
+    ay = a.ys ? ld_word<true>(row_addr<true>(pl, wrap_row(j + a.ys, g.Cy)) + a.y +
                               4u * (uint32_t)p.w)
-              : ld_word<false>(own + u.cAy);
+              : ld_word<false>(own + a.y);
   } else {
-    const int jy = wrap_row(j + u.yA, g.Cy);
-    ay = ld_word<false>(own + u.cAy + (uint32_t)(jy - j) * pl.row_bytes);
+    const int jy = wrap_row(j + a.ys, g.Cy);
+    ay = ld_word<false>(own + a.y + (uint32_t)(jy - j) * pl.row_bytes);
   }
   in.na = neighbour_planes(am, ar, ax, ay);
-  in.nb = neighbour_planes(bm, br, bx, by);
   return in;
 }
 
-// Apply the moves (dA, dB) of a word; n: its sites.
+// Apply the moves (dA, dB) of a word's sites.
 template <bool kCl, bool kAl>
 __device__ __forceinline__ void apply_word(const Geo &g, const PhaseD &u, const Place &pl,
-                                           const Spot &p, int n, uint32_t dA, uint32_t dB) {
-  if constexpr (!kAl) {
-    if (n < 16) {  // pairs past the end of the row do not exist
-      const uint32_t valid = (1u << (2 * n)) - 1u;
-      dA &= valid;
-      dB &= valid;
-    }
-  }
-  xor_word<false>(pl.base + p.off + u.cA, dA);
-  int jb = pl.row0 + p.l + u.qy;
-  jb = jb >= g.Cy ? jb - g.Cy : jb;
-  xor_window<kCl, kAl>(row_addr<kCl>(pl, jb) + u.cB, window_at<kAl>(g, p.w, u.qx), dB);
+                                           const Spot &p, uint32_t dA, uint32_t dB) {
+  xor_word<false>(pl.base + p.off + u.side[0].c, dA);
+  const SideD &b = u.side[1];
+  xor_window<kCl, kAl>(row_addr<kCl>(pl, side_row(g, pl, b, p.l)) + b.c,
+                       window_at<kAl>(g, p.w, b.qx), dB);
 }
 
-// The rare pairs of a warp's words, warp-cooperatively: for every lane with
-// flagged calls, 16 / kTPW lanes each decide one of its pairs from its inputs
-// (see the phase kernels' warp_word).
-template <bool kCl, bool kAl, int kTPW>
-__device__ __forceinline__ void rare_pairs(const Geo &g, const PhaseD &u, const Place &pl,
-                                        const uint2 *trans, const uint16_t *thrT,
-                                        const uint32_t *thr32, unsigned ball, uint32_t rz,
-                                        const WordIn &in, const Spot &p, int n, int sub,
-                                        uint64_t P) {
-  const int lane = threadIdx.x & 31;
-  __syncwarp();  // the fast moves of every lane are in memory
+// Bits of a word's sites that exist (the row may end in it), none for a thread
+// without a word.
+template <bool kAl>
+__device__ __forceinline__ uint32_t valid_bits(const Geo &g, const Spot &p, bool act) {
+  uint32_t v = 0xFFFFFFFFu;
+  if constexpr (!kAl) {
+    const int n = g.Cx - (p.w << 4);
+    if (n < 16) v = (1u << (2 * n)) - 1u;
+  }
+  return act ? v : 0u;
+}
+
+// Round keys in shared memory (five 16-byte loads a call instead of twenty
+// additions on the drawing thread's chain).
+__device__ __forceinline__ U4 philox_keys(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
+                                          const uint32_t *rk) {
+  const uint4 *k4 = reinterpret_cast<const uint4 *>(rk);
+#pragma unroll
+  for (int r = 0; r < 5; ++r) {
+    const uint4 k = k4[r];
+    uint32_t lo0, hi0, lo1, hi1;
+    mul_wide(0xD2511F53u, c0, lo0, hi0);
+    mul_wide(0xCD9E8D57u, c2, lo1, hi1);
+    c0 = hi1 ^ c1 ^ k.x;
+    c2 = hi0 ^ c3 ^ k.y;
+    c1 = lo1;
+    c3 = lo0;
+    mul_wide(0xD2511F53u, c0, lo0, hi0);
+    mul_wide(0xCD9E8D57u, c2, lo1, hi1);
+    c0 = hi1 ^ c1 ^ k.z;
+    c2 = hi0 ^ c3 ^ k.w;
+    c1 = lo1;
+    c3 = lo0;
+  }
+  return U4{c0, c1, c2, c3};
+}
+
+// ----------------------------------------------------------------------------
+// Four lanes a word (lattices with few words an SM, bound by one thread's chain).
+// Lane sub decides group k = sub (call sub / 2, half sub mod 2).  Lanes 0 and 1
+// read the a side, lanes 2 and 3 the b side, each for its half; three exchanges
+// with lane sub XOR 2 bring the other side.  The random words come from draw
+// threads (two a word, one a call) one phase ahead, already divided by 12.
+
+// A draw thread's call: for every half the four pairs' fields as wq << 16 |
+// 264 r (a field >= 65532 has wq = 5461; bit 15 of the first: the call has one).
+__device__ __forceinline__ void draw_call(uint32_t gbase, int c, uint64_t P, const uint32_t *rk,
+                                          uint4 *out) {
+  const U4 r = philox_keys(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE, rk);
+  const uint32_t mx = __vmaxu2(__vimax3_u16x2(r.x, r.y, r.z), r.w);
+  const uint32_t flag = mx >= 0xFFFC0000u || (mx & 0xFFFFu) >= 0xFFFCu ? 0x8000u : 0u;
+  const uint32_t X[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t f[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t v = h ? X[q] >> 16 : X[q] & 0xFFFFu;
+      const uint32_t wq = div12(v);
+      f[q] = (wq << 16) + (v - 12u * wq) * 264u;
+    }
+    out[h] = make_uint4(f[0] | flag, f[1], f[2], f[3]);
+  }
+}
+
+// One phase of a word by its four lanes (inactive lanes: valid 0): the word's
+// moves applied.
+template <bool kCl, bool kAl>
+__device__ __forceinline__ void quad_word(const Geo &g, const PhaseD &u, const Place &pl,
+                                          const uint2 *trans, const uint16_t *thrT,
+                                          const uint32_t *thr32, const uint32_t *rk,
+                                          const Spot &p, int sub, uint32_t valid, const uint4 &f,
+                                          uint64_t P) {
+  const SideD &d = u.side[sub >> 1];
+  const int h2 = 2 * (sub & 1), c4 = 4 * (sub >> 1);
+  const uint32_t row = row_addr<kCl>(pl, side_row(g, pl, d, p.l));
+  const Win win = window_at<kAl>(g, p.w, d.qx);
+  const SideIn s = gather_side<kCl, kAl>(g, d, pl, p.l, win, row, p.w);
+  // this side's (2 n1, n0) of the half's pairs, two pairs a word (see half_env)
+  const uint32_t O = s.n.O >> h2, T = (s.n.T >> h2) << 1, F = (s.n.F >> h2) << 2;
+  const uint32_t n1 = lop3<kLutMux>(F, lop3<kLutMux>(O, T, 0x22222222u), 0x88888888u);
+  const uint32_t n0 = lop3<kLutMux>(F, lop3<kLutMux>(O, T, 0x11111111u), 0x44444444u);
+  const uint32_t x01 = prmt(n1, n0, 0x5140u), x23 = prmt(n1, n0, 0x7362u);
+  const uint32_t o01 = __shfl_xor_sync(0xFFFFFFFFu, x01, 2);
+  const uint32_t o23 = __shfl_xor_sync(0xFFFFFFFFu, x23, 2);
+  const uint32_t oX = __shfl_xor_sync(0xFFFFFFFFu, s.X, 2);
+  // operands (a's counts below b's): the lane's own side first or second
+  const uint32_t lo = sub < 2 ? 0x5410u : 0x1054u, hi = sub < 2 ? 0x7632u : 0x3276u;
+  const uint32_t ev[4] = {prmt(x01, o01, lo), prmt(x01, o01, hi), prmt(x23, o23, lo),
+                          prmt(x23, o23, hi)};
+  const uint32_t A = sub < 2 ? s.X : oX, B = sub < 2 ? oX : s.X;
+  const uint32_t pcs = half_pc(A >> h2, B >> h2, 0);
+  const uint32_t pc = __funnelshift_l(pcs, pcs, 3 - c4);
+  const uint2 *moves = trans + (u.near128 >> 3);  // + 128 near bytes
+  const uint32_t fs[4] = {f.x, f.y, f.z, f.w};
+  uint32_t df[4], t[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const uint2 e = move_entry(moves, entry_offset(pc, q, fs[q] & 0x7FFFu));
+    t[q] = (uint32_t)__dp4a((int)e.y, (int)((ev[q] >> c4) & kEnvMask), (int)e.x);
+    df[q] = fs[q] - (level_at(thrT, t[q] & 0xFFFFu) << 16);  // negative: accept; < 2^16: a tie
+  }
+  const uint32_t mn = __vimin3_u32(__vimin3_u32(df[0], df[1], df[2]), df[3], df[3]);
+  uint32_t acc = prmt(prmt(df[0], df[1], 0x00FBu), prmt(df[2], df[3], 0x00FBu), 0x5410u) &
+                 prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
+  if ((mn < 0x10000u || (f.x & 0x8000u)) && valid) {  // rare pairs: decided exactly (see exact_move)
 #pragma unroll 1
-  while (ball) {
-    const int src = __ffs(ball) - 1;
-    ball &= ball - 1u;
-    const uint32_t orz = __shfl_sync(0xFFFFFFFFu, rz, src);
-    WordIn o;
-    o.A = __shfl_sync(0xFFFFFFFFu, in.A, src);
-    o.B = __shfl_sync(0xFFFFFFFFu, in.B, src);
-    o.na.O = __shfl_sync(0xFFFFFFFFu, in.na.O, src);
-    o.na.T = __shfl_sync(0xFFFFFFFFu, in.na.T, src);
-    o.na.F = __shfl_sync(0xFFFFFFFFu, in.na.F, src);
-    o.nb.O = __shfl_sync(0xFFFFFFFFu, in.nb.O, src);
-    o.nb.T = __shfl_sync(0xFFFFFFFFu, in.nb.T, src);
-    o.nb.F = __shfl_sync(0xFFFFFFFFu, in.nb.F, src);
-    const int ol = __shfl_sync(0xFFFFFFFFu, p.l, src), ow = __shfl_sync(0xFFFFFFFFu, p.w, src),
-              on = __shfl_sync(0xFFFFFFFFu, n, src), osub = __shfl_sync(0xFFFFFFFFu, sub, src);
-    const int c = kTPW == 1 ? (lane >> 3) & 1 : kTPW == 2 ? osub : osub >> 1;
-    const int h = kTPW == 4 ? osub & 1 : (lane >> 2) & 1;
-    const int t = 2 * c + h + 4 * (lane & 3);
-    if (lane < 16 / kTPW && ((orz >> c) & 1u) && t < on) {
-      const uint32_t x = exact_move(g, trans, thrT, thr32, pl.row0 + ol, ow, c, h, lane & 3, o, P,
-                                    u.near128);
-      if (x)
-        apply_word<kCl, kAl>(g, u, pl, spot_of(g, pl, ol, ow), on, (x >> 2) << (2 * t),
-                             (x & 3u) << (2 * t));
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t fq = q == 0 ? fs[0] : q == 1 ? fs[1] : q == 2 ? fs[2] : fs[3];
+      const uint32_t dq = q == 0 ? df[0] : q == 1 ? df[1] : q == 2 ? df[2] : df[3];
+      uint32_t tq = q == 0 ? t[0] : q == 1 ? t[1] : q == 2 ? t[2] : t[3];
+      const uint32_t wq = fq >> 16;
+      const bool big = wq == 5461u;
+      if (dq >= 0x10000u && !big) continue;
+      const uint32_t slow0 =
+          (uint32_t)((uint64_t)(pl.row0 + p.l) * g.Cx + (uint32_t)(p.w << 4)) + (uint32_t)sub + 4u * q;
+      const U4 sl = philox_keys(slow0, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, rk);
+      if (big) {
+        if (sl.y >= 4294967292u) continue;  // keep the current configuration
+        const uint32_t eq = q == 0 ? ev[0] : q == 1 ? ev[1] : q == 2 ? ev[2] : ev[3];
+        const uint2 e = move_entry(moves, entry_offset(pc, q, (sl.y % 12u) * 264u));
+        tq = (uint32_t)__dp4a((int)e.y, (int)((eq >> c4) & kEnvMask), (int)e.x);
+      }
+      const uint32_t thr = thr32[(tq & 0xFFFFu) >> 1];
+      if (thr == 0xFFFFFFFFu ||
+          (big ? sl.x < thr : ((uint64_t)wq << 32) + sl.x < 5461ull * thr))
+        acc |= (tq >> 24) << (8 * q);  // the fast path left this lane's byte zero
     }
   }
+  uint32_t dB = (acc & 0x03030303u) << (2 * sub);
+  uint32_t dA = ((acc >> 2) & 0x03030303u) << (2 * sub);
+  // the word's moves together; one lane a side writes its sites
+  uint32_t mine = sub < 2 ? dA : dB, other = sub < 2 ? dB : dA;
+  mine |= __shfl_xor_sync(0xFFFFFFFFu, other, 2);
+  mine |= __shfl_xor_sync(0xFFFFFFFFu, mine, 1);
+  if (sub & 1) mine = 0u;
+  xor_window<kCl, kAl>(row + d.c, win, mine & valid);
 }
 
 // Observables of this CTA's words by definition, as sums over bit products of
@@ -378,19 +529,25 @@ __device__ __forceinline__ void count_words(const Geo &g, const Place &pl, int n
 
 }  // namespace
 
+// Threads: `workers` (a multiple of 32), with four lanes a word then workers / 2
+// draw threads, then the auxiliary warp.  The register limits (96 and 72 a thread,
+// by the largest CTA) leave no spills: a spilled value read after a cluster
+// barrier comes from L2, as the barrier's acquire empties L1 (1024^2 on sixteen
+// CTAs: 19.4 us a sweep, 23.6 at 72 registers).
 template <bool kCl, bool kAl, int kTPW>
-__global__ void __launch_bounds__(kResMaxThreads, 1)
+__global__ void __launch_bounds__(kTPW == 4 ? kResMaxThreads4 : kResMaxThreads, 1)
     resident_sweep_kernel(const __grid_constant__ ResJob one, const ResJob *__restrict__ jobs,
-                    int cluster) {
+                          int cluster, int workers) {
   extern __shared__ __align__(16) unsigned char res_smem[];
-  __shared__ PhaseD s_d[4];   // phase P's uniforms in slot P mod 4
+  __shared__ PhaseD s_d[16];  // phase P's uniforms in slot P mod 16
   __shared__ int s_obs[2][8]; // the counts of even and odd records
+  __shared__ ResJob s_job;    // read where used: its fields would fill the registers
   uint16_t *thrT = reinterpret_cast<uint16_t *>(res_smem);
   uint2 *trans = reinterpret_cast<uint2 *>(res_smem + 2 * kThrT);
-  __shared__ ResJob s_job;  // read where used: its fields would fill the registers
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int nworkers = (int)blockDim.x - 32;
-  const bool aux = tid >= nworkers;
+  const uint32_t *thr32 = reinterpret_cast<const uint32_t *>(res_smem + kFastBytes);
+  int tid;  // opaque: the compiler would read the special register again every phase
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+  const int lane = tid & 31;
   {
     const uint32_t *src = reinterpret_cast<const uint32_t *>(
         jobs ? jobs + (kCl ? blockIdx.x / cluster : blockIdx.x) : &one);
@@ -400,6 +557,8 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
   }
   const ResJob &J = s_job;
   const Geo &g = s_job.g;
+  const bool aux = tid >= (int)blockDim.x - 32;
+  const bool worker = tid < workers;
   Place pl;
   uint32_t rank = 0;
   if constexpr (kCl) asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
@@ -413,7 +572,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
   const uint32_t mw = g.W > 1 ? 0xFFFFFFFFu / (uint32_t)g.W + 1u : 0u;
   // tables and words in
   {
-    const uint4 *src = reinterpret_cast<const uint4 *>(J.thrT);  // levels, then moves
+    const uint4 *src = reinterpret_cast<const uint4 *>(J.thrT);  // one block in this order
     uint4 *dst = reinterpret_cast<uint4 *>(res_smem);
     for (int t = tid; t < (int)(kTableBytes / 16); t += blockDim.x) dst[t] = src[t];
     uint32_t *words = reinterpret_cast<uint32_t *>(res_smem + kTableBytes);
@@ -427,82 +586,118 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
   }
   const int64_t P0 = g.ctl[kCtlPhaseBase];
   const int obs_every = J.obs_every;
-  auto describe = [&](uint64_t P) {  // the auxiliary warp
-    const Sched sc = draw_schedule(g, P);
-    if (lane == 0) s_d[P & 3u] = phase_desc(g, sc, cls_bytes);
-  };
   // sweeps until the next record, and the record writer's ring position
   int until = obs_every > 0 ? obs_every - (int)((P0 / 8) % obs_every) : 0;
   int64_t obs_cnt = 0, obs_slot = 0;
   if (aux) {
-    describe((uint64_t)P0);
-    describe((uint64_t)P0 + 1u);
+    describe_sweep(g, (uint64_t)P0, cls_bytes, s_d);
     if (obs_every > 0 && rank == 0 && lane == 0) {
       obs_cnt = g.ctl[kCtlObsCount];
       obs_slot = obs_cnt % J.ring_cap;
     }
   }
-  // this thread's place in every phase's first pass, and that pass's random words
+  // a worker's place in every phase's first pass
   const int items = kTPW * nr * g.W;
-  constexpr int kCalls = kTPW == 1 ? 2 : 1;
-  auto place = [&](int i) {
-    const int wid = i / kTPW;
+  auto place = [&](int wid) {
     const int l = g.W > 1 ? (int)__umulhi((uint32_t)wid, mw) : wid;
     return spot_of(g, pl, l, wid - l * g.W);
   };
-  auto call_of = [&](const Spot &p, int c, uint64_t P) {
-    const uint32_t gbase = (uint32_t)(pl.row0 + p.l) * (uint32_t)(2 * g.W) + (uint32_t)(2 * p.w);
-    return philox(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE, g.k0, g.k1);
+  auto base_of = [&](const Spot &p) {
+    return (uint32_t)(pl.row0 + p.l) * (uint32_t)(2 * g.W) + (uint32_t)(2 * p.w);
   };
-  const Spot p0 = place(aux ? 0 : tid);
+  // four lanes a word: the fields of phase P in buffer P mod 2, 16 bytes a worker
+  uint4 *fields =
+      reinterpret_cast<uint4 *>(res_smem + kTableBytes + 16u * cls_bytes);
+  const int call = tid - workers;  // a draw thread's call
+  const bool drawer = kTPW == 4 && !worker && !aux && 2 * call < items;
+  const Spot p0 = place(worker ? (tid < items ? tid / kTPW : 0) : drawer ? call >> 1 : 0);
   const int sub = tid % kTPW;
-  U4 rn[kCalls];
+  constexpr int kCalls = kTPW == 1 ? 2 : 1;
+  U4 rn[kCalls];  // one or two threads a word: the first word's random words
   auto draw_first = [&](uint64_t P) {
+    if constexpr (kTPW == 4) {
+      if (drawer)
+        draw_call(base_of(p0), call & 1, P, J.rk, fields + (P & 1u) * workers + 2 * call);
+    } else {
 #pragma unroll
-    for (int ci = 0; ci < kCalls; ++ci)
-      rn[ci] = call_of(p0, kTPW == 1 ? ci : kTPW == 2 ? sub : sub >> 1, P);
+      for (int ci = 0; ci < kCalls; ++ci)
+        rn[ci] = philox_keys(base_of(p0) + (uint32_t)(kTPW == 1 ? ci : sub), (uint32_t)P,
+                             (uint32_t)(P >> 32), TAG_MOVE, J.rk);
+    }
   };
-  draw_first((uint64_t)P0);
+  if (!aux) draw_first((uint64_t)P0);
+  const uint32_t valid0 = valid_bits<kAl>(g, p0, tid < items);
+  const bool warp_has = tid - lane < items;
   bar_arrive<kCl>();
   bar_wait<kCl>();
   int obs_buf = 0;
   const int nphases = 8 * J.nsweeps;
   for (int q = 0; q < nphases; ++q) {
     const uint64_t P = (uint64_t)(P0 + q);
-    if (!aux) {
-      const PhaseD &u = s_d[P & 3u];
-      for (int base = tid - lane; base < items; base += nworkers) {  // uniform over the warp
-        const bool act = base + lane < items;
-        const bool first = base < nworkers;
-        Spot p = p0;
-        if (!first) p = place(base + lane);
-        const int n = !act ? 0 : kAl ? 16 : min(16, g.Cx - (p.w << 4));
-        WordIn in{};
-        uint32_t rz = 0u;
-        if (act) {
-          in = gather_word<kCl, kAl>(g, u, pl, p);
-          const uint3 d = fast_moves<kTPW>(trans, thrT, sub, in, u.near128, [&](int c) {
-            return first ? rn[kTPW == 1 ? c : 0] : call_of(p, c, P);
-          });
-          apply_word<kCl, kAl>(g, u, pl, p, n, d.x, d.y);
-          rz = d.z;
+    const PhaseD &u = s_d[P & 15u];
+    if constexpr (kTPW == 4) {
+      if (worker) {
+        if (warp_has) {
+          // lanes without a word decide word 0 on zero fields (nobody draws theirs, and
+          // what the buffer holds there is no table offset); valid0 drops their moves
+          const uint4 f = tid < items ? fields[(P & 1u) * workers + tid] : uint4{0u, 0u, 0u, 0u};
+          quad_word<kCl, kAl>(g, u, pl, trans, thrT, thr32, J.rk, p0, sub, valid0, f, P);
         }
-        const unsigned ball = __ballot_sync(0xFFFFFFFFu, rz != 0u);
-        if (ball)
-          rare_pairs<kCl, kAl, kTPW>(g, u, pl, trans, thrT, J.thr32, ball, rz, in, p, n, sub, P);
+      } else if (!aux) {
+        draw_first(P + 1u);
       }
+      bar_arrive<kCl>();
+    } else {
+      if (worker) {
+        for (int base = tid - lane; base < items; base += workers) {  // uniform over the warp
+          const bool first = base < workers;
+          Spot p = p0;
+          uint32_t valid = valid0;
+          if (!first) {
+            const bool act = base + lane < items;
+            p = place(act ? (base + lane) / kTPW : 0);
+            valid = valid_bits<kAl>(g, p, act);
+          }
+          const WordIn in = gather_word<kCl, kAl>(g, u, pl, p);
+          uint3 d = fast_moves<kTPW, true>(trans, thrT, sub, in, u.near128, [&](int c) {
+            return first ? rn[kTPW == 1 ? c : 0]
+                         : philox_keys(base_of(p) + (uint32_t)c, (uint32_t)P,
+                                       (uint32_t)(P >> 32), TAG_MOVE, J.rk);
+          });
+          // rare pairs, decided by their own thread from the inputs it holds (all
+          // lanes together after exchanging them took longer, and the whole cluster
+          // waits at its barrier for the last warp of a phase)
+          if (!valid) d.z = 0u;
+#pragma unroll 1
+          while (d.z) {
+            const int t = __ffs((int)d.z) - 1;
+            d.z &= d.z - 1u;
+            const uint32_t x =
+                exact_move(g, trans, thrT, thr32, pl.row0 + p.l, p.w, t, in, P, u.near128);
+            d.x |= (x >> 2) << (2 * t);
+            d.y |= (x & 3u) << (2 * t);
+          }
+          apply_word<kCl, kAl>(g, u, pl, p, d.x & valid, d.y & valid);
+        }
+      }
+      bar_arrive<kCl>();
+      if (!aux) draw_first(P + 1u);
     }
-    bar_arrive<kCl>();
-    if (aux)
-      describe(P + 2u);
-    else
-      draw_first(P + 1u);
-    bar_wait<kCl>();
+    // the next sweep's schedules, in the first phase of this one (the other eight
+    // slots): on one CTA the auxiliary warp has the whole sweep for them
+    if (aux && (q & 7) == 0) describe_sweep(g, P + 8u, cls_bytes, s_d);
+    if constexpr (kCl) {
+      bar_wait<kCl>();
+    } else if ((q & 7) == 7) {
+      __syncthreads();
+    } else if (!aux) {
+      asm volatile("bar.sync 1, %0;" ::"r"((int)blockDim.x - 32) : "memory");
+    }
     if (obs_every > 0 && (q & 7) == 7 && --until == 0) {
       until = obs_every;
       int n[7] = {0, 0, 0, 0, 0, 0, 0};
-      if (!aux) count_words<kCl, kAl>(g, pl, nr, cls_bytes, tid, nworkers, n);
       if (!aux) {
+        count_words<kCl, kAl>(g, pl, nr, cls_bytes, tid, (int)blockDim.x - 32, n);
         uint32_t dst = smem_addr(s_obs[obs_buf]);
         if constexpr (kCl) dst = map_rank(dst, 0u);
 #pragma unroll
@@ -564,7 +759,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
 
 namespace {
 
-using Kernel = void (*)(const ResJob, const ResJob *, int);
+using Kernel = void (*)(const ResJob, const ResJob *, int, int);
 
 Kernel kernel_of(bool cluster, bool aligned, int tpw) {
   static const Kernel k[2][2][3] = {
@@ -582,6 +777,20 @@ Kernel kernel_of(bool cluster, bool aligned, int tpw) {
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 bool g_ready[kMaxDevices] = {};
+
+void launch_config(const ResShape &shape, int njobs, cudaStream_t s, cudaLaunchConfig_t &cfg,
+                   cudaLaunchAttribute *attr) {
+  cfg.gridDim = dim3((unsigned)(njobs * shape.cluster));
+  cfg.blockDim = dim3((unsigned)shape.threads);
+  cfg.dynamicSmemBytes = (size_t)shape.smem;
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)shape.cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = shape.cluster > 1 ? 1 : 0;
+}
 
 // Raises every instance's shared-memory limit and allows clusters of 16, once
 // per device (outside any capture: called when a lattice or a batch is created).
@@ -616,49 +825,83 @@ int64_t resident_smem(const Geo &g, int rows) {
   return (int64_t)kTableBytes + 64ll * rows * g.W;
 }
 
-// Shapes, measured on GB300 (us a sweep, records off).  A cluster's barrier and
-// remote windows cost 0.7 us a phase, which only pays for lattices of enough
-// words: 256^2 (256 words a phase) 15.0 on one CTA, 12.4 on four, 11.5 on sixteen;
-// 1024^2 51.8 on four, 33.1 on eight, 26.1 on sixteen; 128 lattices of 128^2 12.6
-// on one CTA each, 16.6 on two.  Four threads a word shorten the chain while few
-// words share an SM (64^2: 5.7, 6.3 with two, 10.1 with one), two up to 256; with
-// more, the work repeated for threads that share a word costs more than it hides
-// (512 replicas: 22.9 with one, 25.8 with two, 30.8 with four).
-ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads, int max_tpw) {
+// The shape of `rows` rows a CTA of a cluster of C.
+static ResShape shape_of(const Geo &g, int C, int tpw, int max_workers) {
   ResShape sh;
+  sh.cluster = C;
+  sh.rows = (g.Cy + C - 1) / C;
+  sh.tpw = tpw;
+  const int words = sh.rows * g.W;
+  int workers = 32;
+  while (workers < tpw * words && workers < max_workers) workers *= 2;
+  sh.workers = workers;
+  sh.threads = workers + (tpw == 4 ? workers / 2 + (workers & 32 ? 16 : 0) : 0) + 32;
+  sh.smem = resident_smem(g, sh.rows) + (tpw == 4 ? 32 * workers : 0);
+  return sh;
+}
+
+// Shapes, measured on GB300 (us a sweep, records off).  A cluster's barrier and
+// remote windows cost 0.5 us a phase, which pays from 128 words a phase: 128^2
+// (64 words) 6.5 on one CTA, 6.9 on four; 256^2 13.5 on one, 9.8 on four, 8.1 on
+// sixteen; 1024^2 43.5 on four, 26.4 on eight, 19.4 on sixteen.  Four lanes a
+// word up to 64 words a CTA (64^2: 4.3, 6.3 with two, 9.4 with one; 512^2 on
+// sixteen CTAs: 12.2, 12.9 with two), also when many lattices share the SMs:
+// their four kinds of warps fall on the four schedulers, while lone worker warps
+// all land on the same one (128 lattices of 256^2 and 128 of 64^2: 23 against
+// 34).  Above that the work repeated for threads that share a word costs more
+// than the shorter chain hides (1024^2 on sixteen: 19.4 with one thread, 21.8
+// with two); two for up to 128 words on SMs of their own.
+ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads, int max_tpw) {
   int C = 1;
   if (g.cstride >= kResClusterWords)
     while (C < kResMaxCluster && 2 * C <= ctas && g.cstride >= 2 * C * kResMinWords) C *= 2;
   while (C < kResMaxCluster && resident_smem(g, (g.Cy + C - 1) / C) > kResMaxSmem) C *= 2;
-  sh.rows = (g.Cy + C - 1) / C;
-  sh.cluster = C;
-  const int words = sh.rows * g.W;
-  const double busy = words > load ? words : load;
-  sh.tpw = max_tpw >= 4 && busy <= 24 ? 4 : max_tpw >= 2 && busy <= 256 ? 2 : 1;
-  while (sh.tpw > 1 && sh.tpw * words > max_threads) sh.tpw /= 2;
-  int workers = 32;
-  while (workers < sh.tpw * words && workers < max_threads) workers *= 2;
-  sh.threads = workers + 32;
-  sh.smem = resident_smem(g, sh.rows);
-  return sh;
+  const int words = (g.Cy + C - 1) / C * g.W;
+  int tpw = max_tpw >= 4 && words <= 64 ? 4 : max_tpw >= 2 && words <= 128 && load <= 128.0 ? 2 : 1;
+  while (tpw > 1 && tpw * words > max_threads) tpw /= 2;
+  return shape_of(g, C, tpw, max_threads);
+}
+
+// Clusters of eight full CTAs do not all find eight free SMs of one processing
+// cluster: for 16 lattices of 1024^2 two waited for the others (54 us a sweep).
+// CTAs of 128 workers that take their words in several passes fit four to an SM:
+// 37 us (eight CTAs of 256 workers, two to an SM: 43).
+ResShape resident_fit(const Geo &g, const ResShape &shape, bool aligned, int n) {
+  auto fits = [&](const ResShape &sh) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    launch_config(sh, n, nullptr, cfg, attr);
+    int most = 0;
+    if (cudaOccupancyMaxActiveClusters(
+            &most, reinterpret_cast<const void *>(kernel_of(true, aligned, sh.tpw)), &cfg) !=
+        cudaSuccess) {
+      cudaGetLastError();
+      return true;
+    }
+    return n <= most;
+  };
+  if (shape.cluster == 1 || fits(shape)) return shape;
+  if (g.cstride >= kResMaxCluster * 128) {
+    const ResShape wide = shape_of(g, kResMaxCluster, 1, std::min(128, shape.workers));
+    if (fits(wide)) return wide;
+  }
+  if (shape.cluster > 2) {
+    const ResShape half = shape_of(g, shape.cluster / 2, shape.tpw, shape.workers);
+    if (half.smem <= kResMaxSmem &&
+        (half.tpw == 1 || half.tpw * half.rows * g.W <= half.workers) && fits(half))
+      return half;
+  }
+  return shape;
 }
 
 cudaError_t launch_resident_sweep(const ResJob *one, const ResJob *d_jobs, int njobs,
                             const ResShape &shape, bool aligned, cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(njobs * shape.cluster));
-  cfg.blockDim = dim3((unsigned)shape.threads);
-  cfg.dynamicSmemBytes = (size_t)shape.smem;
-  cfg.stream = s;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)shape.cluster;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = shape.cluster > 1 ? 1 : 0;
+  launch_config(shape, njobs, s, cfg, attr);
   return cudaLaunchKernelEx(&cfg, kernel_of(shape.cluster > 1, aligned, shape.tpw),
-                            one ? *one : ResJob{}, one ? nullptr : d_jobs, shape.cluster);
+                            one ? *one : ResJob{}, one ? nullptr : d_jobs, shape.cluster,
+                            shape.workers);
 }
 
 }  // namespace ccmc

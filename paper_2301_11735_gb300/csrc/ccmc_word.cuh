@@ -85,16 +85,53 @@ __device__ __forceinline__ uint32_t entry_offset(uint32_t pcs, int q, uint32_t r
   return lop3<kLutAndXor>(pcs >> (8 * q), 0x78u, r264);
 }
 
+// The exact decision of pair t of word w of class row j, with its SLOW words, if it
+// is rare (a tie or a field >= 65532, which the fast path rejected): the accepted
+// move, else 0.
+__device__ __forceinline__ uint32_t exact_move(const Geo &g, const uint2 *trans,
+                                               const uint16_t *thrT, const uint32_t *thr32, int j,
+                                               int w, int t, const WordIn &in, uint64_t P,
+                                               uint32_t near128) {
+  const int c = (t >> 1) & 1, h = t & 1, q = t >> 2;  // its MOVE call, half and word
+  const uint32_t gbase = (uint32_t)j * (uint32_t)(2 * g.W) + (uint32_t)(2 * w);
+  const U4 r = philox(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE, g.k0, g.k1);
+  const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
+  const uint32_t v = h ? X >> 16 : X & 0xFFFFu;
+  const uint32_t wq = div12(v);
+  // the pair's own counts and state, from bits 2 t and 2 t + 1 of the planes
+  auto counts = [&](const Planes &p) {
+    const uint32_t O = p.O >> (2 * t), T = p.T >> (2 * t), F = p.F >> (2 * t);
+    return ((O & 2u) + 2u * (T & 2u) + 4u * (F & 2u)) |
+           (((O & 1u) + 2u * (T & 1u) + 4u * (F & 1u)) << 8);
+  };
+  const uint32_t env = counts(in.na) | (counts(in.nb) << 16);
+  const uint32_t pc8 = ((((in.A >> (2 * t)) & 3u) << 2) | ((in.B >> (2 * t)) & 3u)) << 3;
+  uint2 e = move_entry(trans, ((v - 12u * wq) * 264u + near128) ^ pc8);
+  if (v < 65532u && wq != level_at(thrT, (uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu))
+    return 0u;  // not rare
+  const uint32_t slow0 = (uint32_t)((uint64_t)j * g.Cx + (uint32_t)(w << 4));
+  const U4 sl = philox(slow0 + (uint32_t)t, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, g.k0, g.k1);
+  if (v >= 65532u) {
+    if (sl.y >= 4294967292u) return 0u;  // keep the current configuration
+    e = move_entry(trans, ((sl.y % 12u) * 264u + near128) ^ pc8);
+  }
+  const uint32_t thr = thr32[((uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu) >> 1];
+  const bool accept = thr == 0xFFFFFFFFu ||
+                      (v < 65532u ? ((uint64_t)wq << 32) + sl.x < 5461ull * thr : sl.x < thr);
+  return accept ? e.x >> 24 : 0u;
+}
+
 // The fast path of the pairs of a word one thread evaluates: kTPW threads
 // share a word (1, 2 or 4), thread `sub` of them takes MOVE call(s) and
 // half(s):
 //   kTPW 1: both calls, both halves (all 16 pairs);
 //   kTPW 2: call sub, both halves (8 pairs);
 //   kTPW 4: call sub / 2, half sub mod 2 (4 pairs: group k = sub).
-// Returns the (dA, dB) of the fast decisions and, in z, bit c for every call
-// c with a rare pair (a tie or a field >= 65532; the fast path rejected it).
-// rand(c): the four words of the word's MOVE call c.
-template <int kTPW, class Rand>
+// rand(c): the four words of the word's MOVE call c.  Returns the (dA, dB) of the
+// fast decisions and, in z, what needs the exact path (a tie or a field >= 65532,
+// rejected here): bit t for every such pair t (kPairs), or bit c for every call c
+// with one (fewer instructions, for a path that looks at the call's pairs anyway).
+template <int kTPW, bool kPairs, class Rand>
 __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *thrT, int sub,
                                             const WordIn &in, uint32_t near128,
                                             const Rand &rand) {
@@ -123,6 +160,8 @@ __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *
   for (int ci = 0; ci < kCalls; ++ci) {
     const int c = c0 + ci;
     const U4 r = rand(c);
+    const uint32_t mx = __vmaxu2(__vimax3_u16x2(r.x, r.y, r.z), r.w);
+    const bool big = mx >= 0xFFFC0000u || (mx & 0xFFFFu) >= 0xFFFCu;  // a field >= 65532
     uint32_t mn = 0xFFFFFFFFu;  // smallest w - T of the call
 #pragma unroll
     for (int hi = 0; hi < kHalves; ++hi) {
@@ -140,8 +179,18 @@ __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *
         t[q] = (uint32_t)__dp4a((int)e.y, (int)((env[hi].ev[q] >> (4 * c)) & kEnvMask), (int)e.x);
         d[q] = wq - level_at(thrT, t[q] & 0xFFFFu);  // negative: accept; zero: a tie
       }
-      mn = __vimin3_u32(mn, d[0], d[1]);
-      mn = __vimin3_u32(mn, d[2], d[3]);
+      if constexpr (kPairs) {
+        if (__vimin3_u32(__vimin3_u32(d[0], d[1], d[2]), d[3], d[3]) == 0u || big) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
+            if (d[q] == 0u || ((X >> (16 * h)) & 0xFFFFu) >= 65532u) slow |= 1u << (k + 4 * q);
+          }
+        }
+      } else {
+        mn = __vimin3_u32(mn, d[0], d[1]);
+        mn = __vimin3_u32(mn, d[2], d[3]);
+      }
       // byte q: the accepted move of lane q, i.e. byte 3 of t[q] under the sign
       // of d[q] (byte permutes: bit 3 of a selector replicates a byte's sign)
       const uint32_t acc = prmt(prmt(d[0], d[1], 0x00FBu), prmt(d[2], d[3], 0x00FBu), 0x5410u) &
@@ -150,47 +199,9 @@ __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *
       dB |= (acc & 0x03030303u) << (2 * k);
       dA |= ((acc >> 2) & 0x03030303u) << (2 * k);
     }
-    // a rare pair: a tie, or a field >= 65532 in either half of the call's words
-    const uint32_t mx = __vmaxu2(__vimax3_u16x2(r.x, r.y, r.z), r.w);
-    if (mn == 0u || mx >= 0xFFFC0000u || (mx & 0xFFFFu) >= 0xFFFCu) slow |= 1u << c;
+    if (!kPairs && (mn == 0u || big)) slow |= 1u << c;
   }
   return make_uint3(dA, dB, slow);
-}
-
-// The exact decision of pair t = k + 4 q (group k = 2 c + h, lane q of the group)
-// of MOVE call c of word w of class row j: the accepted move if the pair is rare
-// (the fast path rejected it), decided with its SLOW words, else 0.
-__device__ __forceinline__ uint32_t exact_move(const Geo &g, const uint2 *trans,
-                                               const uint16_t *thrT, const uint32_t *thr32, int j,
-                                               int w, int c, int h, int q, const WordIn &in,
-                                               uint64_t P, uint32_t near128) {
-  const int t = 2 * c + h + 4 * q;
-  const uint32_t gbase = (uint32_t)j * (uint32_t)(2 * g.W) + (uint32_t)(2 * w);
-  const U4 r = philox(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE, g.k0, g.k1);
-  const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
-  const uint32_t v = h ? X >> 16 : X & 0xFFFFu;
-  const uint32_t wq = div12(v);
-  // the pair's own counts and state, from bits 2 t and 2 t + 1 of the planes
-  auto counts = [&](const Planes &p) {
-    const uint32_t O = p.O >> (2 * t), T = p.T >> (2 * t), F = p.F >> (2 * t);
-    return ((O & 2u) + 2u * (T & 2u) + 4u * (F & 2u)) |
-           (((O & 1u) + 2u * (T & 1u) + 4u * (F & 1u)) << 8);
-  };
-  const uint32_t env = counts(in.na) | (counts(in.nb) << 16);
-  const uint32_t pc8 = ((((in.A >> (2 * t)) & 3u) << 2) | ((in.B >> (2 * t)) & 3u)) << 3;
-  uint2 e = move_entry(trans, ((v - 12u * wq) * 264u + near128) ^ pc8);
-  if (v < 65532u && wq != level_at(thrT, (uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu))
-    return 0u;  // not rare
-  const uint32_t slow0 = (uint32_t)((uint64_t)j * g.Cx + (uint32_t)(w << 4));
-  const U4 sl = philox(slow0 + (uint32_t)t, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, g.k0, g.k1);
-  if (v >= 65532u) {
-    if (sl.y >= 4294967292u) return 0u;  // keep the current configuration
-    e = move_entry(trans, ((sl.y % 12u) * 264u + near128) ^ pc8);
-  }
-  const uint32_t thr = thr32[((uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu) >> 1];
-  const bool accept = thr == 0xFFFFFFFFu ||
-                      (v < 65532u ? ((uint64_t)wq << 32) + sl.x < 5461ull * thr : sl.x < thr);
-  return accept ? e.x >> 24 : 0u;
 }
 
 }  // namespace ccmc
