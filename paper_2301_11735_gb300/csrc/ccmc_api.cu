@@ -47,19 +47,34 @@ constexpr int kChunk = 16;
 constexpr int kLockstepMin = 8;
 constexpr int64_t kLockstepMaxWords = 16384;
 
-// Lattice memory comes from a library-owned stream-ordered pool per device
-// (allocations and frees queued on the lattice's stream, memory kept cached
-// in the pool): creating and destroying lattices then never synchronises the
-// device, which a server admitting and retiring simulations while others run
-// depends on.
+// Lattice memory comes from a library-owned pool per device, kept cached:
+// creating and destroying lattices never synchronises the device, which a server
+// admitting and retiring simulations while others run depends on.  Everything is
+// allocated and freed on one stream of the library's own, which carries nothing
+// else: an allocation is complete when the call returns (any stream may use it),
+// and a free follows the owner's last work, for which the caller has waited.
+// (Allocating on every lattice's own stream made the pool grow by a chunk a
+// stream: 0.2 to 0.8 ms a lattice when 512 were created, or read back for the
+// first time; now 0.02.)
 constexpr int kMaxDevices = 64;
+struct DevicePool {
+  cudaMemPool_t pool = nullptr;
+  cudaStream_t stream = nullptr;
+};
 std::mutex g_pool_mu;
-cudaMemPool_t g_pool[kMaxDevices] = {};
+DevicePool g_pool[kMaxDevices] = {};
 
-cudaMemPool_t lattice_pool(int dev) {
+// The device's pool (made on first use), nullptr when that fails.
+const DevicePool *device_pool(int dev) {
   if (dev < 0 || dev >= kMaxDevices) return nullptr;
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (!g_pool[dev]) {
+  DevicePool &d = g_pool[dev];
+  if (!d.stream && cudaStreamCreateWithFlags(&d.stream, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    d.stream = nullptr;
+    return nullptr;
+  }
+  if (!d.pool) {
     cudaMemPoolProps props{};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -71,25 +86,78 @@ cudaMemPool_t lattice_pool(int dev) {
     }
     uint64_t keep = UINT64_MAX;
     cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
-    g_pool[dev] = p;
+    d.pool = p;
   }
-  return g_pool[dev];
+  return &d;
 }
 
-// bytes of device memory for a lattice of device dev, ordered on stream s
-bool dalloc(void **p, size_t bytes, int dev, cudaStream_t s) {
-  cudaMemPool_t pool = lattice_pool(dev);
-  if (!pool || cudaMallocFromPoolAsync(p, bytes, pool, s) != cudaSuccess) {
+// bytes of device memory of device dev, usable at once on any stream
+bool dalloc(void **p, size_t bytes, int dev) {
+  const DevicePool *d = device_pool(dev);
+  *p = nullptr;
+  if (!d || cudaMallocFromPoolAsync(p, bytes, d->pool, d->stream) != cudaSuccess) {
     cudaGetLastError();
+    *p = nullptr;
+    return false;
+  }
+  if (cudaStreamSynchronize(d->stream) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFreeAsync(*p, d->stream);
     *p = nullptr;
     return false;
   }
   return true;
 }
 
-void dfree(void *p, cudaStream_t s) {
-  if (p) cudaFreeAsync(p, s);
+// the caller has waited for the last work that uses p
+void dfree(void *p, int dev) {
+  const DevicePool *d = p ? device_pool(dev) : nullptr;
+  if (d) cudaFreeAsync(p, d->stream);
 }
+
+// Pinned host buffers through which short results reach the caller: a copy or a
+// kernel writes the buffer, one synchronisation, then a host copy (a copy to
+// pageable memory stages and waits inside the driver: 24 us for a 16 KB state
+// instead of 10).  At most kStages of kStageBytes for the process, lent for the
+// length of one call; a caller that finds none takes the pageable path.
+constexpr size_t kStageBytes = (size_t)1 << 20;
+constexpr int kStages = 8;
+std::mutex g_stage_mu;
+std::vector<void *> g_stage_free;
+int g_stage_made = 0;
+
+class Stage {
+ public:
+  explicit Stage(size_t bytes) {
+    if (bytes > kStageBytes) return;
+    std::lock_guard<std::mutex> lock(g_stage_mu);
+    if (!g_stage_free.empty()) {
+      p_ = g_stage_free.back();
+      g_stage_free.pop_back();
+    } else if (g_stage_made < kStages &&
+               cudaHostAlloc(&p_, kStageBytes, cudaHostAllocPortable) == cudaSuccess) {
+      ++g_stage_made;
+    } else {
+      p_ = nullptr;
+      cudaGetLastError();
+    }
+  }
+  ~Stage() {
+    if (!p_) return;
+    std::lock_guard<std::mutex> lock(g_stage_mu);
+    g_stage_free.push_back(p_);
+  }
+  Stage(const Stage &) = delete;
+  Stage &operator=(const Stage &) = delete;
+  explicit operator bool() const { return p_ != nullptr; }
+  template <class T>
+  T *as(size_t offset = 0) const {
+    return reinterpret_cast<T *>(static_cast<char *>(p_) + offset);
+  }
+
+ private:
+  void *p_ = nullptr;
+};
 
 }  // namespace
 
@@ -99,17 +167,18 @@ struct ccmc_lattice {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int device = 0;
+  void *d_slab = nullptr;  // one allocation: the members down to the flag
   uint32_t *d_words = nullptr;
   int64_t *d_ctl = nullptr;
   int64_t *d_partials = nullptr;
   int64_t *d_ring = nullptr;
   int64_t ring_cap = 0;
+  DevTables t{};
+  int *d_flag = nullptr;
   int64_t *d_hist = nullptr;
   int nbins = 0;
-  void *d_tables = nullptr;
-  DevTables t{};
   uint8_t *d_bytes = nullptr;
-  int *d_flag = nullptr;
+  bool queued = true;  // work may be queued on `stream` that no call has waited for
   bool initialised = false;
   uint64_t seed = 0;
   int64_t phases_done = 0;  // global phase index of the next phase
@@ -294,12 +363,24 @@ void fill_obs(const ccmc_lattice *h, const int64_t *rec, ccmc_obs *o) {
   o->E = Delta * (double)rec[1] + V * (double)rec[2] + (0.25 * J) * (double)rec[3];
 }
 
-int check_status(ccmc_lattice *h) {
-  int64_t st = 0;
-  CK(cudaMemcpyAsync(&st, h->d_ctl + kCtlStatus, sizeof(int64_t), cudaMemcpyDeviceToHost,
-                     h->stream));
+// The control block's words as they are behind the work queued on the lattice's
+// stream (synchronises it).
+int read_ctl(ccmc_lattice *h, int64_t ctl[kCtlWords]) {
+  const size_t n = sizeof(int64_t) * kCtlWords;
+  Stage st(n);
+  int64_t *to = st ? st.as<int64_t>() : ctl;
+  CK(cudaMemcpyAsync(to, h->d_ctl, n, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  return st == 0 ? CCMC_OK : CCMC_E_TIMEOUT;
+  h->queued = false;
+  if (st) std::memcpy(ctl, to, n);
+  return CCMC_OK;
+}
+
+int check_status(ccmc_lattice *h) {
+  int64_t ctl[kCtlWords];
+  const int rc = read_ctl(h, ctl);
+  if (rc) return rc;
+  return ctl[kCtlStatus] == 0 ? CCMC_OK : CCMC_E_TIMEOUT;
 }
 
 }  // namespace
@@ -355,18 +436,30 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
   }
   const int np = recount_grid(g);
   const int dev = h->device;
-  const size_t tb = sizeof(uint32_t) * (kDevPad + 2 * kMoveN) + sizeof(uint16_t) * kThrT;
-  if (!dalloc((void **)&h->d_words, sizeof(uint32_t) * 16 * g.cstride, dev, h->stream) ||
-      !dalloc((void **)&h->d_ctl, sizeof(int64_t) * kCtlWords, dev, h->stream) ||
-      !dalloc((void **)&h->d_partials, sizeof(int64_t) * 7 * np, dev, h->stream) ||
-      !dalloc((void **)&h->d_ring, sizeof(int64_t) * 8 * h->ring_cap, dev, h->stream) ||
-      !dalloc((void **)&h->d_flag, sizeof(int), dev, h->stream) ||
-      !dalloc(&h->d_tables, tb, dev, h->stream))
-    return fail(CCMC_E_NOMEM);
   // the threshold levels and the move table one after another (a multiple of
   // 16 bytes from a 256-byte aligned base): the tile kernels copy them into
   // shared memory with one bulk copy; thr32 after them
-  char *p = (char *)h->d_tables;
+  size_t at = 0;
+  auto part = [&](size_t bytes) {
+    const size_t o = at;
+    at += (bytes + 255) & ~(size_t)255;
+    return o;
+  };
+  const size_t o_words = part(sizeof(uint32_t) * 16 * g.cstride);
+  const size_t o_tables =
+      part(sizeof(uint16_t) * kThrT + sizeof(uint32_t) * (2 * kMoveN + kDevPad));
+  const size_t o_ctl = part(sizeof(int64_t) * kCtlWords);
+  const size_t o_partials = part(sizeof(int64_t) * 7 * np);
+  const size_t o_flag = part(sizeof(int));
+  const size_t o_ring = part(sizeof(int64_t) * 8 * h->ring_cap);
+  if (!dalloc(&h->d_slab, at, dev)) return fail(CCMC_E_NOMEM);
+  char *p = (char *)h->d_slab;
+  h->d_words = (uint32_t *)(p + o_words);
+  h->d_ctl = (int64_t *)(p + o_ctl);
+  h->d_partials = (int64_t *)(p + o_partials);
+  h->d_flag = (int *)(p + o_flag);
+  h->d_ring = (int64_t *)(p + o_ring);
+  p += o_tables;
   h->t.thrT = (uint16_t *)p;
   p += sizeof(uint16_t) * kThrT;
   h->t.trans = (uint32_t *)p;
@@ -390,7 +483,7 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
 static int ensure_bytes(ccmc_lattice *h) {
   if (h->d_bytes) return CCMC_OK;
   const size_t N = (size_t)h->g.Lx * h->g.Ly;
-  if (!dalloc((void **)&h->d_bytes, N, h->device, h->stream)) return CCMC_E_NOMEM;
+  if (!dalloc((void **)&h->d_bytes, N, h->device)) return CCMC_E_NOMEM;
   return CCMC_OK;
 }
 
@@ -398,6 +491,7 @@ int ccmc::init_counts_async(ccmc_lattice *h, uint64_t seed, int64_t n_plus, int6
   if (!h) return CCMC_E_INVAL;
   const int64_t N = (int64_t)h->g.Lx * h->g.Ly;
   if (n_plus < 0 || n_minus < 0 || n_plus + n_minus > N) return CCMC_E_INVAL;
+  h->queued = true;
   set_seed(h, seed);
   CK(launch_set_ctl(h->d_ctl, 0, h->stream));
   CK(launch_init(h->g, h->h, n_plus, n_minus, h->stream));
@@ -425,6 +519,7 @@ int ccmc::init_constrained_async(ccmc_lattice *h, uint64_t seed, double n, doubl
 int ccmc::export_async(ccmc_lattice *h, int64_t *rec, int64_t *status, int64_t *count,
                        int64_t *ring, uint8_t *state, cudaEvent_t ready) {
   if (!h || !rec || !status || !h->initialised) return CCMC_E_INVAL;
+  h->queued = true;
   int rc = write_recount_latest(h);
   if (rc) return rc;
   CK(cudaMemcpyAsync(rec, h->d_ctl + kCtlLatest, sizeof(int64_t) * 8, cudaMemcpyDeviceToHost,
@@ -438,7 +533,9 @@ int ccmc::export_async(ccmc_lattice *h, int64_t *rec, int64_t *status, int64_t *
     CK(cudaMemcpyAsync(ring, h->d_ring, sizeof(int64_t) * 8 * h->ring_cap,
                        cudaMemcpyDeviceToHost, h->stream));
   }
-  if (state) {
+  if (state && (size_t)h->g.Lx * h->g.Ly <= kStageBytes) {
+    CK(launch_unpack(h->g, state, h->stream));  // straight into the pinned buffer
+  } else if (state) {
     rc = ensure_bytes(h);
     if (rc) return rc;
     CK(launch_unpack(h->g, h->d_bytes, h->stream));
@@ -502,15 +599,10 @@ int ccmc_lattice_destroy(ccmc_lattice *h) {
   if (!h) return CCMC_E_INVAL;
   if (h->stream) cudaStreamSynchronize(h->stream);  // this lattice's work only
   drop_graphs(h);
-  dfree(h->d_words, h->stream);
-  dfree(h->d_ctl, h->stream);
-  dfree(h->d_partials, h->stream);
-  dfree(h->d_ring, h->stream);
-  dfree(h->d_hist, h->stream);
-  dfree(h->d_tables, h->stream);
-  dfree(h->d_bytes, h->stream);
-  dfree(h->d_flag, h->stream);
-  dfree(h->d_maps, h->stream);
+  dfree(h->d_slab, h->device);
+  dfree(h->d_hist, h->device);
+  dfree(h->d_bytes, h->device);
+  dfree(h->d_maps, h->device);
   if (h->map_ev) cudaEventDestroy(h->map_ev);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
@@ -521,6 +613,7 @@ int ccmc_init_counts(ccmc_lattice *h, uint64_t seed, int64_t n_plus, int64_t n_m
   const int rc = init_counts_async(h, seed, n_plus, n_minus);
   if (rc) return rc;
   CK(cudaStreamSynchronize(h->stream));
+  h->queued = false;
   return CCMC_OK;
 }
 
@@ -528,6 +621,7 @@ int ccmc_init_constrained(ccmc_lattice *h, uint64_t seed, double n, double charg
   const int rc = init_constrained_async(h, seed, n, charged_frac);
   if (rc) return rc;
   CK(cudaStreamSynchronize(h->stream));
+  h->queued = false;
   return CCMC_OK;
 }
 
@@ -539,6 +633,7 @@ int ccmc_sweep(ccmc_lattice *h, int64_t nsweeps, double beta, double Delta, doub
   if (!h->initialised) return CCMC_E_STATE;
   if (fault_injected("launch")) return CCMC_E_CUDA;
   TraceRange trace("ccmc_sweep");
+  h->queued = true;
   int rc = upload_params(h, beta, Delta, V, J);
   if (rc) return rc;
   if (nsweeps > 0 && h->phases_done % 8) {
@@ -580,6 +675,7 @@ int ccmc_phases(ccmc_lattice *h, int64_t nphases, double beta, double Delta, dou
     return CCMC_E_INVAL;
   if (!h->initialised) return CCMC_E_STATE;
   if (fault_injected("launch")) return CCMC_E_CUDA;
+  h->queued = true;
   int rc = upload_params(h, beta, Delta, V, J);
   if (rc) return rc;
   for (int64_t p = 0; p < nphases; ++p) {
@@ -606,16 +702,18 @@ int ccmc_map_apply(ccmc_lattice *h, const int32_t *pairs, int64_t map0, int64_t 
   const int64_t N = (int64_t)h->g.Lx * h->g.Ly;
   if (nmaps > ((int64_t)1 << 40) / (2 * P)) return CCMC_E_INVAL;
   const int64_t n = 2 * P * nmaps;
+  h->queued = true;
   // the kernel addresses the lattice with these indices: reject any outside it
   for (int64_t i = 0; i < n; ++i)
     if (pairs[i] < 0 || pairs[i] >= N) return CCMC_E_INVAL;
   if (!h->map_ev && cudaEventCreateWithFlags(&h->map_ev, cudaEventDisableTiming) != cudaSuccess)
     return CCMC_E_CUDA;
   if (n > h->map_cap) {
-    dfree(h->d_maps, h->stream);  // after the earlier maps' work on the stream
+    if (h->d_maps) CK(cudaStreamSynchronize(h->stream));  // the earlier maps' work
+    dfree(h->d_maps, h->device);
     h->d_maps = nullptr;
     h->map_cap = 0;
-    if (!dalloc((void **)&h->d_maps, sizeof(int32_t) * n, h->device, h->stream))
+    if (!dalloc((void **)&h->d_maps, sizeof(int32_t) * n, h->device))
       return CCMC_E_NOMEM;
     h->map_cap = n;
   }
@@ -633,33 +731,41 @@ int ccmc_map_apply(ccmc_lattice *h, const int32_t *pairs, int64_t map0, int64_t 
 int ccmc_observables(ccmc_lattice *h, ccmc_obs *out) {
   if (!h || !out) return CCMC_E_INVAL;
   if (!h->initialised) return CCMC_E_STATE;
+  h->queued = true;
   int rc = write_recount_latest(h);
   if (rc) return rc;
-  int64_t rec[8];
-  CK(cudaMemcpyAsync(rec, h->d_ctl + kCtlLatest, sizeof(rec), cudaMemcpyDeviceToHost,
-                     h->stream));
-  CK(cudaStreamSynchronize(h->stream));
+  int64_t ctl[kCtlWords];
+  rc = read_ctl(h, ctl);
+  if (rc) return rc;
+  int64_t *rec = ctl + kCtlLatest;
   rec[0] = h->phases_done / 8;
   fill_obs(h, rec, out);
-  return check_status(h);
+  return ctl[kCtlStatus] == 0 ? CCMC_OK : CCMC_E_TIMEOUT;
 }
 
 int ccmc_obs_series(ccmc_lattice *h, ccmc_obs *out, int64_t cap, int64_t *n_written) {
   if (!h || !n_written || cap < 0 || (cap > 0 && !out)) return CCMC_E_INVAL;
-  int64_t cnt = 0;
-  CK(cudaMemcpyAsync(&cnt, h->d_ctl + kCtlObsCount, sizeof(int64_t), cudaMemcpyDeviceToHost,
-                     h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  const int64_t held = cnt < h->ring_cap ? cnt : h->ring_cap;
-  const int64_t first = cnt - held;
-  std::vector<int64_t> ring((size_t)(8 * h->ring_cap));
-  CK(cudaMemcpyAsync(ring.data(), h->d_ring, sizeof(int64_t) * 8 * h->ring_cap,
-                     cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  int64_t n = 0;
-  for (int64_t r = first; r < cnt && n < cap; ++r, ++n)
-    fill_obs(h, ring.data() + 8 * (r % h->ring_cap), out + n);
-  *n_written = n;
+  const size_t head = sizeof(int64_t) * kCtlWords, bytes = sizeof(int64_t) * 8 * h->ring_cap;
+  Stage st(head + bytes);
+  int64_t ctl[kCtlWords];
+  std::vector<int64_t> own;
+  const int64_t *ring = nullptr;
+  if (st) {  // control block and ring behind one synchronisation
+    CK(cudaMemcpyAsync(st.as<char>(), h->d_ctl, head, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(st.as<char>(head), h->d_ring, bytes, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    h->queued = false;
+    std::memcpy(ctl, st.as<char>(), head);
+    ring = st.as<int64_t>(head);
+  } else {
+    const int rc = read_ctl(h, ctl);
+    if (rc) return rc;
+    own.resize((size_t)(8 * h->ring_cap));
+    CK(cudaMemcpyAsync(own.data(), h->d_ring, bytes, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    ring = own.data();
+  }
+  *n_written = series_of_ring(h, ring, ctl[kCtlObsCount], out, cap);
   return CCMC_OK;
 }
 
@@ -667,12 +773,13 @@ int ccmc_hist_enable(ccmc_lattice *h, int nbins) {
   if (!h || nbins < 1 || nbins > (1 << 20)) return CCMC_E_INVAL;
   CK(cudaStreamSynchronize(h->stream));
   drop_graphs(h);  // captured recounts hold the old histogram pointer
-  dfree(h->d_hist, h->stream);
+  dfree(h->d_hist, h->device);
   h->d_hist = nullptr;
   h->nbins = 0;
-  if (!dalloc((void **)&h->d_hist, sizeof(int64_t) * 3 * nbins, h->device, h->stream))
+  if (!dalloc((void **)&h->d_hist, sizeof(int64_t) * 3 * nbins, h->device))
     return CCMC_E_NOMEM;
   h->nbins = nbins;
+  h->queued = true;
   CK(cudaMemsetAsync(h->d_hist, 0, sizeof(int64_t) * 3 * nbins, h->stream));
   return CCMC_OK;
 }
@@ -687,33 +794,46 @@ int ccmc_hist_get(ccmc_lattice *h, int64_t *out) {
 }
 
 
-int ccmc_get_state(ccmc_lattice *h, uint8_t *host_out) {
+}  // extern "C"
+
+// Hands `n` bytes of state made by `make(device pointer)` to the caller: short ones
+// written into a pinned buffer by the kernel itself.
+template <typename Make>
+static int read_state(ccmc_lattice *h, uint8_t *host_out, size_t n, Make make) {
   if (!h || !host_out) return CCMC_E_INVAL;
   if (!h->initialised) return CCMC_E_STATE;
-  int rc = ensure_bytes(h);
-  if (rc) return rc;
-  const size_t N = (size_t)h->g.Lx * h->g.Ly;
-  CK(launch_unpack(h->g, h->d_bytes, h->stream));
-  CK(cudaMemcpyAsync(host_out, h->d_bytes, N, cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
+  Stage st(n);
+  if (st) {
+    CK(make(st.as<uint8_t>()));
+    CK(cudaStreamSynchronize(h->stream));
+    std::memcpy(host_out, st.as<uint8_t>(), n);
+  } else {
+    const int rc = ensure_bytes(h);
+    if (rc) return rc;
+    CK(make(h->d_bytes));
+    CK(cudaMemcpyAsync(host_out, h->d_bytes, n, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+  }
+  h->queued = false;
   return CCMC_OK;
 }
 
+extern "C" {
+
+int ccmc_get_state(ccmc_lattice *h, uint8_t *host_out) {
+  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly : 0,
+                    [&](uint8_t *to) { return launch_unpack(h->g, to, h->stream); });
+}
+
 int ccmc_get_state_packed(ccmc_lattice *h, uint8_t *host_out) {
-  if (!h || !host_out) return CCMC_E_INVAL;
-  if (!h->initialised) return CCMC_E_STATE;
-  int rc = ensure_bytes(h);
-  if (rc) return rc;
-  const size_t nb = (size_t)h->g.Lx * h->g.Ly / 4;
-  CK(launch_unpack2(h->g, h->d_bytes, h->stream));
-  CK(cudaMemcpyAsync(host_out, h->d_bytes, nb, cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  return CCMC_OK;
+  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly / 4 : 0,
+                    [&](uint8_t *to) { return launch_unpack2(h->g, to, h->stream); });
 }
 
 int ccmc_set_state_packed(ccmc_lattice *h, const uint8_t *host_in, uint64_t seed,
                           int64_t sweeps_done) {
   if (!h || !host_in || sweeps_done < 0 || sweeps_done > ((int64_t)1 << 59)) return CCMC_E_INVAL;
+  h->queued = true;
   int rc = ensure_bytes(h);
   if (rc) return rc;
   const size_t nb = (size_t)h->g.Lx * h->g.Ly / 4;
@@ -730,6 +850,7 @@ int ccmc_set_state_packed(ccmc_lattice *h, const uint8_t *host_in, uint64_t seed
 
 int ccmc_set_state(ccmc_lattice *h, const uint8_t *host_in, uint64_t seed, int64_t sweeps_done) {
   if (!h || !host_in || sweeps_done < 0) return CCMC_E_INVAL;
+  h->queued = true;
   int rc = ensure_bytes(h);
   if (rc) return rc;
   const size_t N = (size_t)h->g.Lx * h->g.Ly;
@@ -764,6 +885,7 @@ struct ccmc_batch {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   ResJob *d_jobs = nullptr;  // resident lattices
+  int64_t **d_ctls = nullptr;  // the members' control blocks (a batch with fixed members)
   int threads = kResMaxWorkers;
   int64_t resident_max_sites = -1;  // -1: the lattices that ccmc_sweep holds resident
   int ctas_per_sm = 1;
@@ -1028,8 +1150,9 @@ int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int6
   for (int i = 0; i < n; ++i) {
     ccmc_lattice *h = lats[i];
     if (nsweeps[i] == 0 || !batch_resident(b, h)) continue;
-    // order the batch stream after work already queued on this lattice's stream
-    if (h->stream != b->stream) {
+    // order the batch stream after work already queued on this lattice's stream (a
+    // stream of the library's own that a call has waited for carries none)
+    if (h->stream != b->stream && (h->queued || !h->own_stream)) {
       CK(cudaEventRecord(b->lat_ev[i], h->stream));
       CK(cudaStreamWaitEvent(b->stream, b->lat_ev[i], 0));
     }
@@ -1051,6 +1174,7 @@ int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int6
     for (int i : resident) {
       ccmc_lattice *h = lats[i];
       h->phases_done += 8 * nsweeps[i];
+      h->queued = true;
       if (h->stream != b->stream) CK(cudaStreamWaitEvent(h->stream, b->ev, 0));
     }
   }
@@ -1097,8 +1221,10 @@ int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int6
     if (rc) return rc;
     off += (int64_t)G.m.size();
     CK(cudaEventRecord(b->ev, b->stream));
-    for (ccmc_lattice *o : G.m)
+    for (ccmc_lattice *o : G.m) {
+      o->queued = true;
       if (o->stream != b->stream) CK(cudaStreamWaitEvent(o->stream, b->ev, 0));
+    }
   }
   return CCMC_OK;
 }
@@ -1117,6 +1243,19 @@ int ccmc_batch_create(int count, ccmc_lattice *const *lattices, void *cuda_strea
   const int rc = ccmc::batch_new(count, (cudaStream_t)cuda_stream, out);
   if (rc != CCMC_OK) return rc;
   (*out)->lats.assign(lattices, lattices + count);
+  std::vector<int64_t *> ctls;
+  for (int i = 0; i < count; ++i) ctls.push_back(lattices[i]->d_ctl);
+  if (cudaMalloc(&(*out)->d_ctls, sizeof(int64_t *) * count) != cudaSuccess) {
+    ccmc_batch_destroy(*out);
+    *out = nullptr;
+    return CCMC_E_NOMEM;
+  }
+  if (cudaMemcpyAsync((*out)->d_ctls, ctls.data(), sizeof(int64_t *) * count,
+                      cudaMemcpyHostToDevice, (*out)->stream) != cudaSuccess) {
+    ccmc_batch_destroy(*out);
+    *out = nullptr;
+    return CCMC_E_CUDA;
+  }
   return CCMC_OK;
 }
 
@@ -1167,6 +1306,7 @@ int ccmc_batch_destroy(ccmc_batch *b) {
     if (e.exec) cudaGraphExecDestroy(e.exec);
   cudaFree(b->d_jobs);
   cudaFree(b->d_multi);
+  cudaFree(b->d_ctls);
   for (cudaStream_t x : b->side) cudaStreamSynchronize(x);
   for (cudaStream_t x : b->side) cudaStreamDestroy(x);
   for (cudaEvent_t e : b->side_ev) cudaEventDestroy(e);
@@ -1210,10 +1350,25 @@ int ccmc_batch_sweep(ccmc_batch *b, const int64_t *nsweeps, const double *beta,
 int ccmc_batch_sync(ccmc_batch *b) {
   if (!b) return CCMC_E_INVAL;
   CK(cudaStreamSynchronize(b->stream));
-  for (ccmc_lattice *h : b->lats) {
-    const int rc = check_status(h);
-    if (rc) return rc;
+  const int n = (int)b->lats.size();
+  const size_t bytes = sizeof(int64_t) * n;
+  Stage st(bytes);
+  if (!st || !b->d_ctls) {
+    for (ccmc_lattice *h : b->lats) {
+      const int rc = check_status(h);
+      if (rc) return rc;
+    }
+    return CCMC_OK;
   }
+  // every member's stream, then all their status words at once
+  for (ccmc_lattice *h : b->lats) {
+    CK(cudaStreamSynchronize(h->stream));
+    h->queued = false;
+  }
+  CK(launch_gather_status(b->d_ctls, n, st.as<int64_t>(), b->stream));
+  CK(cudaStreamSynchronize(b->stream));
+  for (int i = 0; i < n; ++i)
+    if (st.as<int64_t>()[i]) return CCMC_E_TIMEOUT;
   return CCMC_OK;
 }
 

@@ -171,6 +171,7 @@ cudaError_t launch_recount(const Geo &g, int64_t *partials, int64_t *ring, int64
                            int64_t *hist, int nbins, int64_t sweep_off, cudaStream_t s);
 cudaError_t launch_advance(int64_t *ctl, int64_t phases, cudaStream_t s);
 cudaError_t launch_set_ctl(int64_t *ctl, int64_t phase_base, cudaStream_t s);
+cudaError_t launch_gather_status(int64_t *const *ctls, int n, int64_t *out, cudaStream_t s);
 cudaError_t launch_unpack(const Geo &g, uint8_t *out, cudaStream_t s);
 cudaError_t launch_pack(const Geo &g, const uint8_t *in, int *bad, cudaStream_t s);
 // Resident sweeps (ccmc_resident.cu): whether the current device can run them

@@ -166,6 +166,17 @@ __global__ void advance_kernel(int64_t *ctl, int64_t phases) {
   ctl[kCtlPhaseBase] += phases;
 }
 
+// The status words of n lattices side by side (for one copy to the host).
+__global__ void gather_status_kernel(int64_t *const *ctls, int n, int64_t *out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    out[i] = ctls[i][kCtlStatus];
+}
+
+cudaError_t launch_gather_status(int64_t *const *ctls, int n, int64_t *out, cudaStream_t s) {
+  gather_status_kernel<<<grid_for(n, 256, 152), 256, 0, s>>>(ctls, n, out);
+  return cudaGetLastError();
+}
+
 // Self-test of the bounded device waits: one CTA waits on an mbarrier that
 // nothing completes, polling at most `polls` times, then records the timeout in
 // *status and returns -- as the phase kernels' waits do on a bulk copy or an
@@ -204,39 +215,84 @@ __global__ void set_ctl_kernel(int64_t *ctl, int64_t phase_base) {
   if (threadIdx.x == 0) ctl[kCtlPhaseBase] = phase_base;
 }
 
-// Logical bytes (site y Lx + x) <-> packed class words.
+// Logical bytes (site y Lx + x) <-> packed class words.  The four classes of a
+// row of sites hold its sites in turn, so byte q of their four words of column
+// block w is 16 consecutive bytes of the row: one thread per such group, the four
+// words' bytes side by side in B (class cx at byte cx), site 4 i + cx of the group
+// at bits 2 i of byte cx.  Memory-bound: 16-byte accesses on the byte side (4-byte
+// ones on rows that are no multiple of 16), consecutive threads consecutive
+// groups.  A thread a class word, with 16 byte accesses 4 bytes apart, moved
+// every sector of the byte side four times (4096^2: see the launch list).
+struct ByteGroup {
+  int64_t word;  // of class cx = 0
+  int64_t byte;  // of the group's first site
+  int q, sites;  // byte of the words; sites of each class in the row (0 to 4)
+};
+
+__device__ __forceinline__ ByteGroup byte_group(const Geo &g, int64_t id) {
+  const int64_t wid = id >> 2;
+  const int w = (int)(wid % g.W);
+  const int64_t r = wid / g.W;  // r = cy Cy + j
+  const int cy = (int)(r / g.Cy), j = (int)(r - (int64_t)cy * g.Cy);
+  ByteGroup b;
+  b.q = (int)(id & 3);
+  b.word = (int64_t)(cy * 4) * g.cstride + (int64_t)j * g.W + w;
+  b.byte = (int64_t)(4 * j + cy) * g.Lx + 64 * w + 16 * b.q;
+  b.sites = max(0, min(4, g.Cx - 16 * w - 4 * b.q));
+  return b;
+}
+
 __global__ void unpack_kernel(Geo g, uint8_t *out) {
-  const int64_t nwords = 16 * g.cstride;
-  for (int64_t wid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; wid < nwords;
-       wid += (int64_t)gridDim.x * blockDim.x) {
-    const int cls = (int)(wid / g.cstride);
-    const int64_t rem = wid - (int64_t)cls * g.cstride;
-    const int j = (int)(rem / g.W), w = (int)(rem - (int64_t)j * g.W);
-    const int s0 = w << 4, n = min(16, g.Cx - s0);
-    const uint32_t X = linear_code(g.words[wid]);
-    for (int t = 0; t < n; ++t) {
-      const int64_t x = 4 * (s0 + t) + (cls & 3), y = 4 * j + (cls >> 2);
-      out[y * g.Lx + x] = (uint8_t)((X >> (2 * t)) & 3u);
+  const int64_t n = 16 * (int64_t)g.Cy * g.W;  // 4 rows a class row, 4 groups a word
+  const bool vec = (g.Lx & 15) == 0;
+  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < n;
+       id += (int64_t)gridDim.x * blockDim.x) {
+    const ByteGroup b = byte_group(g, id);
+    uint32_t B = 0u;
+#pragma unroll
+    for (int cx = 0; cx < 4; ++cx)
+      B |= ((g.words[b.word + cx * g.cstride] >> (8 * b.q)) & 0xFFu) << (8 * cx);
+    B = linear_code(B);
+    uint32_t v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = (B >> (2 * i)) & 0x03030303u;
+    if (vec && b.sites == 4) {
+      *reinterpret_cast<uint4 *>(out + b.byte) = make_uint4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i < b.sites) *reinterpret_cast<uint32_t *>(out + b.byte + 4 * i) = v[i];
     }
   }
 }
 
 __global__ void pack_kernel(Geo g, const uint8_t *in, int *bad) {
-  const int64_t nwords = 16 * g.cstride;
-  for (int64_t wid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; wid < nwords;
-       wid += (int64_t)gridDim.x * blockDim.x) {
-    const int cls = (int)(wid / g.cstride);
-    const int64_t rem = wid - (int64_t)cls * g.cstride;
-    const int j = (int)(rem / g.W), w = (int)(rem - (int64_t)j * g.W);
-    const int s0 = w << 4, n = min(16, g.Cx - s0);
-    uint32_t X = 0u;
-    for (int t = 0; t < n; ++t) {
-      const int64_t x = 4 * (s0 + t) + (cls & 3), y = 4 * j + (cls >> 2);
-      const uint32_t c = in[y * g.Lx + x];
-      if (c > 3u) *bad = 1;
-      X |= (c & 3u) << (2 * t);
+  const int64_t n = 16 * (int64_t)g.Cy * g.W;
+  const bool vec = (g.Lx & 15) == 0;
+  for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < n;
+       id += (int64_t)gridDim.x * blockDim.x) {
+    const ByteGroup b = byte_group(g, id);
+    uint32_t v[4] = {0u, 0u, 0u, 0u};
+    if (vec && b.sites == 4) {
+      const uint4 x = *reinterpret_cast<const uint4 *>(in + b.byte);
+      v[0] = x.x;
+      v[1] = x.y;
+      v[2] = x.z;
+      v[3] = x.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i < b.sites) v[i] = *reinterpret_cast<const uint32_t *>(in + b.byte + 4 * i);
     }
-    g.words[wid] = linear_code(X);
+    if ((v[0] | v[1] | v[2] | v[3]) & 0xFCFCFCFCu) *bad = 1;
+    uint32_t B = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) B |= (v[i] & 0x03030303u) << (2 * i);
+    B = linear_code(B);
+    uint8_t *words = reinterpret_cast<uint8_t *>(g.words);
+#pragma unroll
+    for (int cx = 0; cx < 4; ++cx)
+      words[4 * (b.word + cx * g.cstride) + b.q] = (uint8_t)(B >> (8 * cx));
   }
 }
 
@@ -361,12 +417,12 @@ cudaError_t launch_set_ctl(int64_t *ctl, int64_t phase_base, cudaStream_t s) {
 }
 
 cudaError_t launch_unpack(const Geo &g, uint8_t *out, cudaStream_t s) {
-  unpack_kernel<<<grid_for(16 * g.cstride, 256, 152 * 16), 256, 0, s>>>(g, out);
+  unpack_kernel<<<grid_for(16 * (int64_t)g.Cy * g.W, 256, 152 * 16), 256, 0, s>>>(g, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_pack(const Geo &g, const uint8_t *in, int *bad, cudaStream_t s) {
-  pack_kernel<<<grid_for(16 * g.cstride, 256, 152 * 16), 256, 0, s>>>(g, in, bad);
+  pack_kernel<<<grid_for(16 * (int64_t)g.Cy * g.W, 256, 152 * 16), 256, 0, s>>>(g, in, bad);
   return cudaGetLastError();
 }
 

@@ -86,10 +86,12 @@ int64_t ring_records(const ccmc_request &r) {
   return r.obs_every > 0 ? std::min<int64_t>(r.nsweeps / r.obs_every + 1, 1 << 16) : 1;
 }
 
-// Estimated wall time of one sweep, for sizing slices: a latency floor for
-// lattices held by one CTA, plus a throughput term.
+// Estimated wall time of one sweep, for sizing slices (measured: 4.3 us at 64^2,
+// 12 at 512^2, 20 at 1024^2, held in shared memory; 43 at 4096^2, 280 at 16384^2,
+// a launch a phase).
 double sweep_us(const ccmc_request &r) {
-  return 12.0 + 5e-6 * (double)r.Lx * (double)r.Ly;
+  const double N = (double)r.Lx * (double)r.Ly;
+  return N <= 1.2e6 ? 5.0 + 1.5e-5 * N : 30.0 + 1e-6 * N;
 }
 
 // Pinned host buffers, cached by power-of-two size (allocating pinned memory
