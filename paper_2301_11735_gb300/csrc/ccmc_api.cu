@@ -199,7 +199,7 @@ namespace {
 // a launch of a phase's own begins to be as fast (1024^2: 3.2 us a phase
 // resident, 3.7 us a launch; 1000^2, ragged: 3.4 against 4.6; 256^2: 1.4 against
 // 3.3; 64^2: 0.7 against 3.3).
-bool resident_default(const Geo &g) { return g.cstride <= 4608; }
+bool resident_default(const Geo &g) { return g.cstride <= 4608 && resident_possible(g); }
 
 int validate_shape(int Lx, int Ly) {
   if (Lx < 4 || Ly < 4 || (Lx & 3) || (Ly & 3)) return CCMC_E_INVAL;

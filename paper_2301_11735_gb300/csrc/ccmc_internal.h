@@ -116,8 +116,10 @@ struct ResShape {
 };
 
 constexpr int kResMaxWorkers = 512;
-constexpr int kResMaxThreads = kResMaxWorkers + 32;                        // 1, 2 threads a word
-constexpr int kResMaxThreads4 = kResMaxWorkers + kResMaxWorkers / 2 + 32;  // four
+constexpr int kResQuadWords = 96;     // words a CTA that may have four threads each
+constexpr int kResMaxThreads = 608;  // 96 registers a thread
+static_assert(kResMaxWorkers + 32 <= kResMaxThreads && 6 * kResQuadWords + 32 <= kResMaxThreads,
+              "workers, draw threads and the auxiliary warp");
 constexpr int kResMaxCluster = 16;
 constexpr int kResClusterWords = 128;  // lattices of fewer a-words a phase take one CTA
 constexpr int kResMinWords = 16;       // a-words a CTA of a cluster at least
@@ -184,6 +186,8 @@ int64_t resident_smem(const Geo &g, int rows);
 // one) while `load` a-words a phase run on an average SM, with at most
 // max_threads workers a CTA and max_tpw threads a word.
 ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads, int max_tpw);
+// Whether the lattice fits shared memory in some shape.
+bool resident_possible(const Geo &g);
 // The shape for n such lattices in one launch: another one when their clusters
 // would not all fit the GPU at once.
 ResShape resident_fit(const Geo &g, const ResShape &shape, bool aligned, int n);

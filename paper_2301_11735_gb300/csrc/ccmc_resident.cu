@@ -43,8 +43,8 @@ static_assert(kFastBytes % 16 == 0 && kTableBytes % 16 == 0, "copied 16 bytes at
 // one in another row: the neighbour sums do not care which is which, so a side
 // has its own class c, one column neighbour read at the side's own column (m) and
 // one xs = -1, 0 or 1 sites further (x), one row neighbour in its own row (r)
-// and one ys rows further (y).  The side's sites lie qx columns and qy rows from
-// the a sites (0, 0 for a itself); offX = qx + xs in [0, Cx).
+// and one 0, 1 or Cy - 1 rows further (y, ys).  The side's sites lie qx columns and
+// qy rows from the a sites (0, 0 for a itself); offX = qx + xs in [0, Cx).
 struct alignas(16) SideD {
   uint32_t c, m, x, r, y;
   int qx, offX, qy, ys, xs;
@@ -112,8 +112,9 @@ __device__ __forceinline__ void bar_wait() {
   }
 }
 
-__device__ __forceinline__ int wrap_row(int v, int n) {
-  return v >= n ? v - n : (v < 0 ? v + n : v);
+// v in [0, 2 n) modulo n: an unsigned minimum instead of a comparison and a choice.
+__device__ __forceinline__ int turn(int v, int n) {
+  return (int)min((uint32_t)v, (uint32_t)(v - n));
 }
 
 // The phase's uniforms from its schedule, for classes of cls_bytes bytes.
@@ -131,14 +132,12 @@ __device__ __forceinline__ PhaseD phase_desc(const Geo &g, const Sched &sc, uint
     d.x = cls(cx + dx, cy);
     d.r = cls(cx, cy - dy);
     d.y = cls(cx, cy + dy);
-    int qx = x >> 2, qy = y >> 2;  // an offset is below the size: at most one turn
-    if (qx >= g.Cx) qx -= g.Cx;
-    if (qy >= g.Cy) qy -= g.Cy;
-    d.qx = qx;
-    d.qy = qy;
+    d.qx = turn(x >> 2, g.Cx);  // an offset is below the size: at most one turn
+    d.qy = turn(y >> 2, g.Cy);
     d.xs = shift(cx);
-    d.ys = shift(cy);
-    d.offX = wrap_row(qx + d.xs, g.Cx);
+    const int ys = shift(cy);
+    d.ys = ys < 0 ? g.Cy - 1 : ys < g.Cy ? ys : 0;
+    d.offX = turn(d.qx + (d.xs < 0 ? g.Cx - 1 : d.xs), g.Cx);
   };
   side(u.side[0], sc.a0x, sc.a0y);
   side(u.side[1], sc.a0x + sc.rx, sc.a0y + sc.ry);
@@ -186,22 +185,19 @@ struct Win {
 template <bool kAl>
 __device__ __forceinline__ Win window_at(const Geo &g, int w, int off) {
   Win x;
+  int wl;
   if constexpr (kAl) {
-    int wl = w + (off >> 4);
-    wl = wl >= g.W ? wl - g.W : wl;
-    x.lo = 4u * (uint32_t)wl;
-    x.hi = wl + 1 == g.W ? 0u : x.lo + 4u;
+    wl = turn(w + (off >> 4), g.W);
     x.sh = 2 * (off & 15);
     x.n1 = 16;
   } else {
-    int s = 16 * w + off;
-    s = s >= g.Cx ? s - g.Cx : s;
-    const int wl = s >> 4;
-    x.lo = 4u * (uint32_t)wl;
-    x.hi = wl + 1 == g.W ? 0u : x.lo + 4u;
+    const int s = turn(16 * w + off, g.Cx);
+    wl = s >> 4;
     x.sh = 2 * (s & 15);
     x.n1 = g.Cx - s;
   }
+  x.lo = 4u * (uint32_t)wl;
+  x.hi = 4u * (uint32_t)turn(wl + 1, g.W);
   return x;
 }
 
@@ -242,7 +238,7 @@ struct Place {
 template <bool kCl>
 __device__ __forceinline__ uint32_t row_addr(const Place &pl, int j) {
   if constexpr (kCl) {
-    const uint32_t rank = pl.rows == 1 ? (uint32_t)j : __umulhi((uint32_t)j, pl.mrows);
+    const uint32_t rank = __umulhi((uint32_t)j, pl.mrows);  // clusters have rows >= 2
     return map_rank(pl.base, rank) + (uint32_t)(j - (int)rank * pl.rows) * pl.row_bytes;
   } else {
     return pl.base + (uint32_t)j * pl.row_bytes;
@@ -279,8 +275,7 @@ __device__ __forceinline__ uint32_t side_window(const Geo &g, const Spot &p, uin
 
 // Row jb of a side's sites for the a sites' row l of this CTA.
 __device__ __forceinline__ int side_row(const Geo &g, const Place &pl, const SideD &d, int l) {
-  const int jb = pl.row0 + l + d.qy;
-  return jb >= g.Cy ? jb - g.Cy : jb;
+  return turn(pl.row0 + l + d.qy, g.Cy);
 }
 
 // One side of a word read the general way (rows anywhere in the cluster): the
@@ -294,7 +289,7 @@ template <bool kCl, bool kAl>
 __device__ __forceinline__ SideIn gather_side(const Geo &g, const SideD &d, const Place &pl,
                                               int l, const Win &win, uint32_t row, int w) {
   SideIn in;
-  const uint32_t ry = d.ys ? row_addr<kCl>(pl, wrap_row(side_row(g, pl, d, l) + d.ys, g.Cy)) : row;
+  const uint32_t ry = row_addr<kCl>(pl, turn(side_row(g, pl, d, l) + d.ys, g.Cy));
   in.X = read_window<kCl, kAl>(row + d.c, win);
   const uint32_t m = read_window<kCl, kAl>(row + d.m, win);
   const uint32_t r = read_window<kCl, kAl>(row + d.r, win);
@@ -323,15 +318,12 @@ __device__ __forceinline__ WordIn gather_word(const Geo &g, const PhaseD &u, con
   const uint32_t am = ld_word<false>(own + a.m);
   const uint32_t ar = ld_word<false>(own + a.r);
   const uint32_t ax = side_window<kAl>(g, p, own + a.x, a.xs);
+  const int jy = turn(j + a.ys, g.Cy);
   uint32_t ay;
-  if constexpr (kCl) {
-    ay = a.ys ? ld_word<true>(row_addr<true>(pl, wrap_row(j + a.ys, g.Cy)) + a.y +
-                              4u * (uint32_t)p.w)
-              : ld_word<false>(own + a.y);
-  } else {
-    const int jy = wrap_row(j + a.ys, g.Cy);
+  if constexpr (kCl)
+    ay = ld_word<true>(row_addr<true>(pl, jy) + a.y + 4u * (uint32_t)p.w);
+  else
     ay = ld_word<false>(own + a.y + (uint32_t)(jy - j) * pl.row_bytes);
-  }
   in.na = neighbour_planes(am, ar, ax, ay);
   return in;
 }
@@ -511,7 +503,7 @@ __device__ __forceinline__ void count_words(const Geo &g, const Place &pl, int n
         window_at<kAl>(g, w, cx == 3 && g.Cx > 1 ? 1 : 0));
     const uint32_t dcls = (uint32_t)(((cy + 1) & 3) * 4 + cx) * cls_bytes + 4u * (uint32_t)w;
     const uint32_t Yd =
-        cy == 3 ? ld_word<kCl>(row_addr<kCl>(pl, wrap_row(pl.row0 + l + 1, g.Cy)) + dcls)
+        cy == 3 ? ld_word<kCl>(row_addr<kCl>(pl, turn(pl.row0 + l + 1, g.Cy)) + dcls)
                 : ld_word<false>(row + dcls);
     const uint32_t odd = X & 0xAAAAAAAAu, even = X & 0x55555555u;
     const uint32_t Xs = (odd >> 1) | (even << 1);
@@ -530,12 +522,12 @@ __device__ __forceinline__ void count_words(const Geo &g, const Place &pl, int n
 }  // namespace
 
 // Threads: `workers` (a multiple of 32), with four lanes a word then workers / 2
-// draw threads, then the auxiliary warp.  The register limits (96 and 72 a thread,
-// by the largest CTA) leave no spills: a spilled value read after a cluster
-// barrier comes from L2, as the barrier's acquire empties L1 (1024^2 on sixteen
-// CTAs: 19.4 us a sweep, 23.6 at 72 registers).
+// draw threads (rounded up to warps), then the auxiliary warp.  The register limit
+// (96 a thread, by the largest CTA) leaves hardly a spill: a spilled value read
+// after a cluster barrier comes from L2, as the barrier's acquire empties L1
+// (1024^2 on sixteen CTAs: 19.4 us a sweep, 23.6 at 72 registers).
 template <bool kCl, bool kAl, int kTPW>
-__global__ void __launch_bounds__(kTPW == 4 ? kResMaxThreads4 : kResMaxThreads, 1)
+__global__ void __launch_bounds__(kResMaxThreads, 1)
     resident_sweep_kernel(const __grid_constant__ ResJob one, const ResJob *__restrict__ jobs,
                           int cluster, int workers) {
   extern __shared__ __align__(16) unsigned char res_smem[];
@@ -630,70 +622,90 @@ __global__ void __launch_bounds__(kTPW == 4 ? kResMaxThreads4 : kResMaxThreads, 
   const bool warp_has = tid - lane < items;
   bar_arrive<kCl>();
   bar_wait<kCl>();
-  int obs_buf = 0;
-  const int nphases = 8 * J.nsweeps;
-  for (int q = 0; q < nphases; ++q) {
-    const uint64_t P = (uint64_t)(P0 + q);
-    const PhaseD &u = s_d[P & 15u];
-    if constexpr (kTPW == 4) {
-      if (worker) {
-        if (warp_has) {
-          // lanes without a word decide word 0 on zero fields (nobody draws theirs, and
-          // what the buffer holds there is no table offset); valid0 drops their moves
-          const uint4 f = tid < items ? fields[(P & 1u) * workers + tid] : uint4{0u, 0u, 0u, 0u};
-          quad_word<kCl, kAl>(g, u, pl, trans, thrT, thr32, J.rk, p0, sub, valid0, f, P);
-        }
-      } else if (!aux) {
-        draw_first(P + 1u);
-      }
-      bar_arrive<kCl>();
-    } else {
-      if (worker) {
-        for (int base = tid - lane; base < items; base += workers) {  // uniform over the warp
-          const bool first = base < workers;
-          Spot p = p0;
-          uint32_t valid = valid0;
-          if (!first) {
-            const bool act = base + lane < items;
-            p = place(act ? (base + lane) / kTPW : 0);
-            valid = valid_bits<kAl>(g, p, act);
-          }
-          const WordIn in = gather_word<kCl, kAl>(g, u, pl, p);
-          uint3 d = fast_moves<kTPW, true>(trans, thrT, sub, in, u.near128, [&](int c) {
-            return first ? rn[kTPW == 1 ? c : 0]
-                         : philox_keys(base_of(p) + (uint32_t)c, (uint32_t)P,
-                                       (uint32_t)(P >> 32), TAG_MOVE, J.rk);
-          });
-          // rare pairs, decided by their own thread from the inputs it holds (all
-          // lanes together after exchanging them took longer, and the whole cluster
-          // waits at its barrier for the last warp of a phase)
-          if (!valid) d.z = 0u;
-#pragma unroll 1
-          while (d.z) {
-            const int t = __ffs((int)d.z) - 1;
-            d.z &= d.z - 1u;
-            const uint32_t x =
-                exact_move(g, trans, thrT, thr32, pl.row0 + p.l, p.w, t, in, P, u.near128);
-            d.x |= (x >> 2) << (2 * t);
-            d.y |= (x & 3u) << (2 * t);
-          }
-          apply_word<kCl, kAl>(g, u, pl, p, d.x & valid, d.y & valid);
-        }
-      }
-      bar_arrive<kCl>();
-      if (!aux) draw_first(P + 1u);
-    }
-    // the next sweep's schedules, in the first phase of this one (the other eight
-    // slots): on one CTA the auxiliary warp has the whole sweep for them
-    if (aux && (q & 7) == 0) describe_sweep(g, P + 8u, cls_bytes, s_d);
-    if constexpr (kCl) {
+  // The barrier of a phase.  On one CTA the auxiliary warp only joins a sweep's last.
+  auto phase_wait = [&](int p) {
+    if (kCl || p == 7)
       bar_wait<kCl>();
-    } else if ((q & 7) == 7) {
-      __syncthreads();
-    } else if (!aux) {
+    else
       asm volatile("bar.sync 1, %0;" ::"r"((int)blockDim.x - 32) : "memory");
+  };
+  int obs_buf = 0;
+  const int nsweeps = J.nsweeps;
+  for (int sweep = 0; sweep < nsweeps; ++sweep) {
+    const uint64_t S = (uint64_t)P0 + 8u * (uint32_t)sweep;
+    if (aux) {
+      // the next sweep's schedules, into the other eight slots
+      if constexpr (kCl) {
+        bar_arrive<true>();
+        describe_sweep(g, S + 8u, cls_bytes, s_d);
+        bar_wait<true>();
+        for (int p = 1; p < 8; ++p) {
+          bar_arrive<true>();
+          bar_wait<true>();
+        }
+      } else {
+        describe_sweep(g, S + 8u, cls_bytes, s_d);
+        __syncthreads();
+      }
+    } else if (kTPW == 4 && !worker) {
+#pragma unroll 1
+      for (int p = 0; p < 8; ++p) {
+        draw_first(S + (uint32_t)p + 1u);
+        bar_arrive<kCl>();
+        phase_wait(p);
+      }
+    } else {
+#pragma unroll 1
+      for (int p = 0; p < 8; ++p) {
+        const uint64_t P = S + (uint32_t)p;
+        const PhaseD &u = s_d[P & 15u];
+        if constexpr (kTPW == 4) {
+          if (warp_has) {
+            // lanes without a word decide word 0 on zero fields (nobody draws theirs, and
+            // what the buffer holds there is no table offset); valid0 drops their moves
+            const uint4 f =
+                tid < items ? fields[(P & 1u) * workers + tid] : uint4{0u, 0u, 0u, 0u};
+            quad_word<kCl, kAl>(g, u, pl, trans, thrT, thr32, J.rk, p0, sub, valid0, f, P);
+          }
+          bar_arrive<kCl>();
+        } else {
+          for (int base = tid - lane; base < items; base += workers) {  // uniform in the warp
+            const bool first = base < workers;
+            Spot pt = p0;
+            uint32_t valid = valid0;
+            if (!first) {
+              const bool act = base + lane < items;
+              pt = place(act ? (base + lane) / kTPW : 0);
+              valid = valid_bits<kAl>(g, pt, act);
+            }
+            const WordIn in = gather_word<kCl, kAl>(g, u, pl, pt);
+            uint3 d = fast_moves<kTPW, true>(trans, thrT, sub, in, u.near128, [&](int c) {
+              return first ? rn[kTPW == 1 ? c : 0]
+                           : philox_keys(base_of(pt) + (uint32_t)c, (uint32_t)P,
+                                         (uint32_t)(P >> 32), TAG_MOVE, J.rk);
+            });
+            // rare pairs, decided by their own thread from the inputs it holds (all
+            // lanes together after exchanging them took longer, and the whole cluster
+            // waits at its barrier for the last warp of a phase)
+            if (!valid) d.z = 0u;
+#pragma unroll 1
+            while (d.z) {
+              const int t = __ffs((int)d.z) - 1;
+              d.z &= d.z - 1u;
+              const uint32_t x =
+                  exact_move(g, trans, thrT, thr32, pl.row0 + pt.l, pt.w, t, in, P, u.near128);
+              d.x |= (x >> 2) << (2 * t);
+              d.y |= (x & 3u) << (2 * t);
+            }
+            apply_word<kCl, kAl>(g, u, pl, pt, d.x & valid, d.y & valid);
+          }
+          bar_arrive<kCl>();
+          draw_first(P + 1u);
+        }
+        phase_wait(p);
+      }
     }
-    if (obs_every > 0 && (q & 7) == 7 && --until == 0) {
+    if (obs_every > 0 && --until == 0) {
       until = obs_every;
       int n[7] = {0, 0, 0, 0, 0, 0, 0};
       if (!aux) {
@@ -723,7 +735,7 @@ __global__ void __launch_bounds__(kTPW == 4 ? kResMaxThreads4 : kResMaxThreads, 
                       s0 = c[6];
         for (int k = 0; k < 7; ++k) c[k] = 0;  // for the record after the next
         const int64_t N = (int64_t)g.Lx * g.Ly;
-        const int64_t rec[8] = {(int64_t)(P + 1u) / 8, b1 + b0 - 2 * both, like - unlike,
+        const int64_t rec[8] = {(int64_t)(S / 8u) + 1, b1 + b0 - 2 * both, like - unlike,
                                 2 * N - 4 * (b1 + b0) + like + unlike, N - b1 - b0,
                                 -s1 - s0, b1 - b0, s1 - s0};
         int64_t *dst = J.ring + obs_slot * 8;
@@ -753,7 +765,7 @@ __global__ void __launch_bounds__(kTPW == 4 ? kResMaxThreads4 : kResMaxThreads, 
       for (int t = tid; t < nw; t += blockDim.x)
         g.words[(int64_t)cls * g.cstride + (int64_t)pl.row0 * g.W + t] =
             words[cls * J.rows * g.W + t];
-    if (rank == 0 && tid == 0) g.ctl[kCtlPhaseBase] = P0 + nphases;
+    if (rank == 0 && tid == 0) g.ctl[kCtlPhaseBase] = P0 + 8 * (int64_t)nsweeps;
   }
 }
 
@@ -832,34 +844,47 @@ static ResShape shape_of(const Geo &g, int C, int tpw, int max_workers) {
   sh.rows = (g.Cy + C - 1) / C;
   sh.tpw = tpw;
   const int words = sh.rows * g.W;
-  int workers = 32;
-  while (workers < tpw * words && workers < max_workers) workers *= 2;
+  // whole warps, beyond 128 in steps of 64 (fewer different shapes in a batch)
+  const int step = tpw * words <= 128 ? 32 : 64;
+  const int workers = std::min((tpw * words + step - 1) / step * step, max_workers);
   sh.workers = workers;
-  sh.threads = workers + (tpw == 4 ? workers / 2 + (workers & 32 ? 16 : 0) : 0) + 32;
+  sh.threads = workers + (tpw == 4 ? (workers / 2 + 31) / 32 * 32 : 0) + 32;
   sh.smem = resident_smem(g, sh.rows) + (tpw == 4 ? 32 * workers : 0);
   return sh;
 }
 
 // Shapes, measured on GB300 (us a sweep, records off).  A cluster's barrier and
-// remote windows cost 0.5 us a phase, which pays from 128 words a phase: 128^2
-// (64 words) 6.5 on one CTA, 6.9 on four; 256^2 13.5 on one, 9.8 on four, 8.1 on
-// sixteen; 1024^2 43.5 on four, 26.4 on eight, 19.4 on sixteen.  Four lanes a
-// word up to 64 words a CTA (64^2: 4.3, 6.3 with two, 9.4 with one; 512^2 on
-// sixteen CTAs: 12.2, 12.9 with two), also when many lattices share the SMs:
-// their four kinds of warps fall on the four schedulers, while lone worker warps
-// all land on the same one (128 lattices of 256^2 and 128 of 64^2: 23 against
-// 34).  Above that the work repeated for threads that share a word costs more
-// than the shorter chain hides (1024^2 on sixteen: 19.4 with one thread, 21.8
-// with two); two for up to 128 words on SMs of their own.
+// remote windows cost 0.4 us a phase, which pays from 128 words a phase: 128^2
+// (64 words) 5.3 on one CTA, 6.5 on four; 256^2 13.5 on one, 9.8 on four, 7.7 on
+// sixteen; 1024^2 43 on four, 26 on eight, 18.7 on sixteen.  Four lanes a word up
+// to 96 words a CTA (64^2: 3.4, with one 9.4; 516^2, 81 words a CTA: 13.7, with two
+// 15.7); above that the work repeated for threads that share a word costs more
+// than the shorter chain hides (1024^2 on sixteen: 18.7 with one thread, 21.8 with
+// two), two threads paying up to 128 words.  When lattices crowd the SMs only the
+// smallest keep four lanes: their four kinds of warps fall on the four schedulers
+// (a lone worker warp a CTA lands on the same one every time: 128 lattices of 256^2
+// and 128 of 64^2 34 against 23), while a 416-thread CTA finds no room beside
+// another (512 replicas: 19.7 with four lanes for their 128^2 lattices, 15.8 with
+// one thread).
 ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads, int max_tpw) {
   int C = 1;
   if (g.cstride >= kResClusterWords)
-    while (C < kResMaxCluster && 2 * C <= ctas && g.cstride >= 2 * C * kResMinWords) C *= 2;
-  while (C < kResMaxCluster && resident_smem(g, (g.Cy + C - 1) / C) > kResMaxSmem) C *= 2;
+    while (C < kResMaxCluster && 2 * C <= ctas && g.cstride >= 2 * C * kResMinWords &&
+           g.Cy >= 4 * C)  // two rows a CTA at least
+      C *= 2;
+  while (C < kResMaxCluster && g.Cy >= 4 * C && resident_smem(g, (g.Cy + C - 1) / C) > kResMaxSmem)
+    C *= 2;
   const int words = (g.Cy + C - 1) / C * g.W;
-  int tpw = max_tpw >= 4 && words <= 64 ? 4 : max_tpw >= 2 && words <= 128 && load <= 128.0 ? 2 : 1;
+  const bool crowded = load > 128.0;
+  int tpw = max_tpw >= 4 && words <= (crowded ? 32 : kResQuadWords) ? 4
+            : max_tpw >= 2 && words <= 128 && !crowded              ? 2
+                                                                     : 1;
   while (tpw > 1 && tpw * words > max_threads) tpw /= 2;
   return shape_of(g, C, tpw, max_threads);
+}
+
+bool resident_possible(const Geo &g) {
+  return resident_shape(g, kResMaxCluster, 0.0, kResMaxWorkers, 1).smem <= kResMaxSmem;
 }
 
 // Clusters of eight full CTAs do not all find eight free SMs of one processing
@@ -881,7 +906,7 @@ ResShape resident_fit(const Geo &g, const ResShape &shape, bool aligned, int n) 
     return n <= most;
   };
   if (shape.cluster == 1 || fits(shape)) return shape;
-  if (g.cstride >= kResMaxCluster * 128) {
+  if (g.cstride >= kResMaxCluster * 128 && g.Cy >= 2 * kResMaxCluster) {
     const ResShape wide = shape_of(g, kResMaxCluster, 1, std::min(128, shape.workers));
     if (fits(wide)) return wide;
   }

@@ -41,6 +41,8 @@ def _lattice(cc, Lx, Ly, **env):
 SMALL = [(4, 4), (4, 64), (64, 4), (12, 8), (60, 36), (64, 64), (68, 124), (128, 128), (132, 140),
          (192, 256), (256, 260), (2052, 16), (16, 2052)]
 LARGE = [(516, 516), (768, 400), (1000, 1000), (1024, 1024), (64, 4096), (4096, 64), (1088, 1084)]
+# few rows of classes, so that no shape or only one CTA holds them
+WIDE = [(131072, 4), (262144, 4), (131072, 8), (32768, 32)]
 
 
 @pytest.mark.parametrize("shape", SMALL)
@@ -60,7 +62,7 @@ def test_resident_sweeps_match_oracle(cc, shape):
             assert np.array_equal(lat.obs_series()[-len(rec):], rec), (shape, done)
 
 
-@pytest.mark.parametrize("shape", LARGE)
+@pytest.mark.parametrize("shape", LARGE + WIDE)
 def test_resident_sweeps_match_the_phase_kernels(cc, shape):
     out = []
     for env in ({}, {"CCMC_NO_RESIDENT": "1"}):
