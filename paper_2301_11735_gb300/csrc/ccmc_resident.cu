@@ -72,6 +72,16 @@ __device__ __forceinline__ uint32_t ld_word(uint32_t addr) {
   return v;
 }
 
+// v, or the word at addr if p: a predicated load, no branch.
+__device__ __forceinline__ uint32_t ld_remote_if(bool p, uint32_t addr, uint32_t v) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t"
+      "@q ld.shared::cluster.u32 %0, [%1];\n\t}"
+      : "+r"(v)
+      : "r"(addr), "r"((uint32_t)p));
+  return v;
+}
+
 // (nothing to do for 0: predicated, no branch)
 template <bool kCl>
 __device__ __forceinline__ void xor_word(uint32_t addr, uint32_t v) {
@@ -299,13 +309,55 @@ __device__ __forceinline__ SideIn gather_side(const Geo &g, const SideD &d, cons
   return in;
 }
 
+// The b side of the words of a whole warp in a cluster (kTPW lanes a word), as
+// gather_side: a window's second word is the first word of the lane that holds the
+// next word of the row, so it comes from that lane; only lanes without such a
+// neighbour (the warp's last, a ragged row's turn) load it.  Remote shared memory
+// delivers 10 to 13 bytes a cycle to an SM: this halves its share of a phase.
+template <bool kAl, int kTPW>
+__device__ __forceinline__ SideIn gather_remote(const Geo &g, const SideD &d, const Place &pl,
+                                                int l, int w) {
+  const int lane = threadIdx.x & 31;
+  const int next = w + 1 < g.W ? lane + kTPW : lane + kTPW * (1 - g.W);
+  const int src = next >= 0 && next < 32 ? next : lane;
+  const int jb = side_row(g, pl, d, l);
+  const uint32_t row = row_addr<true>(pl, jb), ry = row_addr<true>(pl, turn(jb + d.ys, g.Cy));
+  const Win win = window_at<kAl>(g, w, d.qx), wx = window_at<kAl>(g, w, d.offX);
+  const bool near = __shfl_sync(0xFFFFFFFFu, row + win.lo, src) == row + win.hi;
+  const bool nearx = __shfl_sync(0xFFFFFFFFu, row + wx.lo, src) == row + wx.hi;
+  const uint32_t at[5] = {row + d.c, row + d.m, row + d.r, ry + d.y, row + d.x};
+  uint32_t lo[5], v[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) lo[k] = ld_word<true>(at[k] + (k < 4 ? win.lo : wx.lo));
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const Win &x = k < 4 ? win : wx;
+    const uint32_t hi = ld_remote_if(!(k < 4 ? near : nearx), at[k] + x.hi,
+                                     __shfl_sync(0xFFFFFFFFu, lo[k], src));
+    v[k] = __funnelshift_r(lo[k], hi, x.sh);
+    if constexpr (!kAl) {
+      if (x.n1 < 16)
+        v[k] = (v[k] & ((1u << (2 * x.n1)) - 1u)) | (ld_word<true>(at[k]) << (2 * x.n1));
+    }
+  }
+  SideIn in;
+  in.X = v[0];
+  in.n = neighbour_planes(v[1], v[2], v[3], v[4]);
+  return in;
+}
+
 // Both sides of a word, the a side (this CTA's rows, whole words) read directly.
-template <bool kCl, bool kAl>
+// kTPW: all lanes of the warp call, with so many lanes a word.
+template <bool kCl, bool kAl, int kTPW>
 __device__ __forceinline__ WordIn gather_word(const Geo &g, const PhaseD &u, const Place &pl,
                                               const Spot &p) {
   WordIn in;
   const SideD &a = u.side[0], &b = u.side[1];
-  {
+  if constexpr (kCl) {
+    const SideIn s = gather_remote<kAl, kTPW>(g, b, pl, p.l, p.w);
+    in.B = s.X;
+    in.nb = s.n;
+  } else {
     const uint32_t row = row_addr<kCl>(pl, side_row(g, pl, b, p.l));
     const SideIn s =
         gather_side<kCl, kAl>(g, b, pl, p.l, window_at<kAl>(g, p.w, b.qx), row, p.w);
@@ -588,7 +640,6 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
       obs_slot = obs_cnt % J.ring_cap;
     }
   }
-  // a worker's place in every phase's first pass
   const int items = kTPW * nr * g.W;
   auto place = [&](int wid) {
     const int l = g.W > 1 ? (int)__umulhi((uint32_t)wid, mw) : wid;
@@ -602,23 +653,23 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
       reinterpret_cast<uint4 *>(res_smem + kTableBytes + 16u * cls_bytes);
   const int call = tid - workers;  // a draw thread's call
   const bool drawer = kTPW == 4 && !worker && !aux && 2 * call < items;
-  const Spot p0 = place(worker ? (tid < items ? tid / kTPW : 0) : drawer ? call >> 1 : 0);
+  Spot pt = place(worker ? (tid < items ? tid / kTPW : 0) : drawer ? call >> 1 : 0);
   const int sub = tid % kTPW;
   constexpr int kCalls = kTPW == 1 ? 2 : 1;
-  U4 rn[kCalls];  // one or two threads a word: the first word's random words
-  auto draw_first = [&](uint64_t P) {
+  U4 rn[kCalls];  // one or two threads a word: the random words of the word at pt
+  auto draw_next = [&](uint64_t P) {
     if constexpr (kTPW == 4) {
       if (drawer)
-        draw_call(base_of(p0), call & 1, P, J.rk, fields + (P & 1u) * workers + 2 * call);
+        draw_call(base_of(pt), call & 1, P, J.rk, fields + (P & 1u) * workers + 2 * call);
     } else {
 #pragma unroll
       for (int ci = 0; ci < kCalls; ++ci)
-        rn[ci] = philox_keys(base_of(p0) + (uint32_t)(kTPW == 1 ? ci : sub), (uint32_t)P,
+        rn[ci] = philox_keys(base_of(pt) + (uint32_t)(kTPW == 1 ? ci : sub), (uint32_t)P,
                              (uint32_t)(P >> 32), TAG_MOVE, J.rk);
     }
   };
-  if (!aux) draw_first((uint64_t)P0);
-  const uint32_t valid0 = valid_bits<kAl>(g, p0, tid < items);
+  if (!aux) draw_next((uint64_t)P0);
+  uint32_t valid = valid_bits<kAl>(g, pt, tid < items);
   const bool warp_has = tid - lane < items;
   bar_arrive<kCl>();
   bar_wait<kCl>();
@@ -650,7 +701,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
     } else if (kTPW == 4 && !worker) {
 #pragma unroll 1
       for (int p = 0; p < 8; ++p) {
-        draw_first(S + (uint32_t)p + 1u);
+        draw_next(S + (uint32_t)p + 1u);
         bar_arrive<kCl>();
         phase_wait(p);
       }
@@ -662,28 +713,22 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
         if constexpr (kTPW == 4) {
           if (warp_has) {
             // lanes without a word decide word 0 on zero fields (nobody draws theirs, and
-            // what the buffer holds there is no table offset); valid0 drops their moves
+            // what the buffer holds there is no table offset); valid drops their moves
             const uint4 f =
                 tid < items ? fields[(P & 1u) * workers + tid] : uint4{0u, 0u, 0u, 0u};
-            quad_word<kCl, kAl>(g, u, pl, trans, thrT, thr32, J.rk, p0, sub, valid0, f, P);
+            quad_word<kCl, kAl>(g, u, pl, trans, thrT, thr32, J.rk, pt, sub, valid, f, P);
           }
           bar_arrive<kCl>();
         } else {
-          for (int base = tid - lane; base < items; base += workers) {  // uniform in the warp
-            const bool first = base < workers;
-            Spot pt = p0;
-            uint32_t valid = valid0;
-            if (!first) {
-              const bool act = base + lane < items;
-              pt = place(act ? (base + lane) / kTPW : 0);
-              valid = valid_bits<kAl>(g, pt, act);
-            }
-            const WordIn in = gather_word<kCl, kAl>(g, u, pl, pt);
-            uint3 d = fast_moves<kTPW, true>(trans, thrT, sub, in, u.near128, [&](int c) {
-              return first ? rn[kTPW == 1 ? c : 0]
-                           : philox_keys(base_of(pt) + (uint32_t)c, (uint32_t)P,
-                                         (uint32_t)(P >> 32), TAG_MOVE, J.rk);
-            });
+          if (!warp_has) {
+            bar_arrive<kCl>();
+            phase_wait(p);
+            continue;
+          }
+          for (int base = tid - lane;;) {  // uniform in the warp
+            const WordIn in = gather_word<kCl, kAl, kTPW>(g, u, pl, pt);
+            uint3 d = fast_moves<kTPW, true>(trans, thrT, sub, in, u.near128,
+                                             [&](int c) { return rn[kTPW == 1 ? c : 0]; });
             // rare pairs, decided by their own thread from the inputs it holds (all
             // lanes together after exchanging them took longer, and the whole cluster
             // waits at its barrier for the last warp of a phase)
@@ -698,9 +743,19 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
               d.y |= (x & 3u) << (2 * t);
             }
             apply_word<kCl, kAl>(g, u, pl, pt, d.x & valid, d.y & valid);
+            // on to the next pass, or with the phase's last to the next phase: the next
+            // word's random words are drawn here, behind the arrival at the barrier
+            base += workers;
+            const bool last = base >= items;
+            if (last) bar_arrive<kCl>();
+            const int i = last ? tid : base + lane;
+            if (items > workers) {
+              pt = place(i < items ? i / kTPW : 0);
+              valid = valid_bits<kAl>(g, pt, i < items);
+            }
+            draw_next(P + (last ? 1u : 0u));
+            if (last) break;
           }
-          bar_arrive<kCl>();
-          draw_first(P + 1u);
         }
         phase_wait(p);
       }
