@@ -530,44 +530,86 @@ __device__ __forceinline__ void quad_word(const Geo &g, const PhaseD &u, const P
 }
 
 // Observables of this CTA's words by definition, as sums over bit products of
-// the linear code (S = b1 - b0, sigma = 1 - b1 - b0): a site's bits against its
-// right and down neighbours', like bits (n[0]) and unlike ones (n[1]); the
-// sites' b1, b0 and both (n[2..4]); b1 and b0 with the staggered sign (n[5], n[6]).
+// the linear code (S = b1 - b0, sigma = 1 - b1 - b0), added to out[0..6] (of the
+// cluster's first CTA): a site's bits against its right and down neighbours', like
+// bits and unlike ones; the sites' b1 and b0; both; b1 and b0 on the sites of even
+// x + y.  A thread takes the four classes of a row of sites at one word place: they
+// are each other's right neighbours, so nine loads serve four words and only the
+// last one's window crosses into the next word.  Bits above a ragged row's end are
+// zero in the words, so they count nowhere.  Two 16-bit counts share a register
+// through the warp's sums (a thread takes at most seven places between them: 7 x
+// 256 x 32 < 2^16).
 template <bool kCl, bool kAl>
-__device__ __forceinline__ void count_words(const Geo &g, const Place &pl, int nr,
-                                            uint32_t cls_bytes, int tid, int nthreads, int n[7]) {
-  const int nw = nr * g.W;
-  if (nw == 0) return;
-  const uint32_t mw = 0xFFFFFFFFu / (uint32_t)g.W + 1u, mn = 0xFFFFFFFFu / (uint32_t)nw + 1u;
-  for (int i = tid; i < 16 * nw; i += nthreads) {
-    const int cls = nw == 1 ? i : (int)__umulhi((uint32_t)i, mn);
-    const int wid = i - cls * nw;
-    const int l = g.W == 1 ? wid : (int)__umulhi((uint32_t)wid, mw), w = wid - l * g.W;
-    const int cx = cls & 3, cy = cls >> 2;
-    const uint32_t row = pl.base + (uint32_t)l * pl.row_bytes;
-    uint32_t X = ld_word<false>(row + (uint32_t)cls * cls_bytes + 4u * (uint32_t)w);
-    if constexpr (!kAl) {
-      const int ns = min(16, g.Cx - 16 * w);
-      if (ns < 16) X &= (1u << (2 * ns)) - 1u;
+__device__ __forceinline__ void count_words(const Geo &g, const Place &pl, int nw, uint32_t mw,
+                                            uint32_t mn, uint32_t cls_bytes, int tid, int nthreads,
+                                            int *out) {
+  constexpr uint32_t kOdd = 0xAAAAAAAAu;
+  uint32_t dst = smem_addr(out);
+  if constexpr (kCl) dst = map_rank(dst, 0u);
+  const int lane = threadIdx.x & 31;
+  for (int i = tid; i - lane < 4 * nw;) {  // uniform in the warp
+    uint32_t bonds = 0u, bits = 0u, both = 0u, even = 0u;
+    for (int k = 0; k < 7 && i - lane < 4 * nw; ++k, i += nthreads) {
+      if (i >= 4 * nw) continue;
+      const int cy = nw == 1 ? i : (int)__umulhi((uint32_t)i, mn);
+      const int wid = i - cy * nw;
+      const int l = g.W == 1 ? wid : (int)__umulhi((uint32_t)wid, mw);
+      const Spot p = spot_of(g, pl, l, wid - l * g.W);
+      const uint32_t own = pl.base + p.off + (uint32_t)(4 * cy) * cls_bytes;
+      uint32_t X[4], Yr[4], Yd[4];
+#pragma unroll
+      for (int cx = 0; cx < 4; ++cx) X[cx] = ld_word<false>(own + (uint32_t)cx * cls_bytes);
+      if (kCl && cy == 3) {
+        const uint32_t down =
+            row_addr<true>(pl, turn(pl.row0 + l + 1, g.Cy)) + 4u * (uint32_t)p.w;
+#pragma unroll
+        for (int cx = 0; cx < 4; ++cx) Yd[cx] = ld_word<true>(down + (uint32_t)cx * cls_bytes);
+      } else {
+        const uint32_t down = cy < 3 ? own + 4u * cls_bytes
+                                     : pl.base + p.off + (uint32_t)(turn(l + 1, g.Cy) - l) * pl.row_bytes;
+#pragma unroll
+        for (int cx = 0; cx < 4; ++cx) Yd[cx] = ld_word<false>(down + (uint32_t)cx * cls_bytes);
+      }
+      Yr[0] = X[1];
+      Yr[1] = X[2];
+      Yr[2] = X[3];
+      Yr[3] = side_window<kAl>(g, p, own, g.Cx > 1 ? 1 : 0);
+      uint32_t like = 0u, unlike = 0u, B[4];
+#pragma unroll
+      for (int cx = 0; cx < 4; ++cx) {
+        const uint32_t Xs = lop3<kLutMux>(X[cx] << 1, X[cx] >> 1, kOdd);  // b0, b1 swapped
+        like += (uint32_t)(__popc(X[cx] & Yr[cx]) + __popc(X[cx] & Yd[cx]));
+        unlike += (uint32_t)(__popc(Xs & Yr[cx]) + __popc(Xs & Yd[cx]));
+        B[cx] = X[cx] & Xs;
+      }
+      bonds += like + (unlike << 16);
+      // two classes of one parity share a count
+      uint32_t b[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        b[h] = (uint32_t)__popc(lop3<kLutMux>(X[h], X[h + 2] >> 1, kOdd)) +
+               ((uint32_t)__popc(lop3<kLutMux>(X[h] << 1, X[h + 2], kOdd)) << 16);
+        both += (uint32_t)__popc(lop3<kLutMux>(B[h], B[h + 2], kOdd));
+      }
+      bits += b[0] + b[1];
+      even += cy & 1 ? b[1] : b[0];
     }
-    const uint32_t Yr = read_window<false, kAl>(
-        row + (uint32_t)(cy * 4 + ((cx + 1) & 3)) * cls_bytes,
-        window_at<kAl>(g, w, cx == 3 && g.Cx > 1 ? 1 : 0));
-    const uint32_t dcls = (uint32_t)(((cy + 1) & 3) * 4 + cx) * cls_bytes + 4u * (uint32_t)w;
-    const uint32_t Yd =
-        cy == 3 ? ld_word<kCl>(row_addr<kCl>(pl, turn(pl.row0 + l + 1, g.Cy)) + dcls)
-                : ld_word<false>(row + dcls);
-    const uint32_t odd = X & 0xAAAAAAAAu, even = X & 0x55555555u;
-    const uint32_t Xs = (odd >> 1) | (even << 1);
-    n[0] += __popc(X & Yr) + __popc(X & Yd);
-    n[1] += __popc(Xs & Yr) + __popc(Xs & Yd);
-    const int k1 = __popc(odd), k0 = __popc(even);
-    n[2] += k1;
-    n[3] += k0;
-    n[4] += __popc(odd & Xs);
-    const bool minus = (cx + cy) & 1;
-    n[5] += minus ? -k1 : k1;
-    n[6] += minus ? -k0 : k0;
+    bonds = __reduce_add_sync(0xFFFFFFFFu, bonds);
+    bits = __reduce_add_sync(0xFFFFFFFFu, bits);
+    both = __reduce_add_sync(0xFFFFFFFFu, both);
+    even = __reduce_add_sync(0xFFFFFFFFu, even);
+    const uint32_t v = lane < 2 ? bonds : lane < 4 ? bits : lane == 4 ? both : even;
+    const uint32_t add = lane == 4 ? v
+                         : (lane == 1 || lane == 3 || lane == 6) ? v >> 16 : v & 0xFFFFu;
+    if (lane < 7) {
+      if constexpr (kCl)
+        asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(
+                         dst + 4u * (uint32_t)lane),
+                     "r"(add)
+                     : "memory");
+      else
+        atomicAdd(out + lane, (int)add);
+    }
   }
 }
 
@@ -614,6 +656,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
   const int nr = max(0, min(J.rows, g.Cy - pl.row0));  // rows of this CTA
   const uint32_t cls_bytes = (uint32_t)J.rows * pl.row_bytes;
   const uint32_t mw = g.W > 1 ? 0xFFFFFFFFu / (uint32_t)g.W + 1u : 0u;
+  const uint32_t mn = nr * g.W > 1 ? 0xFFFFFFFFu / (uint32_t)(nr * g.W) + 1u : 0u;
   // tables and words in
   {
     const uint4 *src = reinterpret_cast<const uint4 *>(J.thrT);  // one block in this order
@@ -762,32 +805,16 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
     }
     if (obs_every > 0 && --until == 0) {
       until = obs_every;
-      int n[7] = {0, 0, 0, 0, 0, 0, 0};
-      if (!aux) {
-        count_words<kCl, kAl>(g, pl, nr, cls_bytes, tid, (int)blockDim.x - 32, n);
-        uint32_t dst = smem_addr(s_obs[obs_buf]);
-        if constexpr (kCl) dst = map_rank(dst, 0u);
-#pragma unroll
-        for (int k = 0; k < 7; ++k) {
-          const int v = __reduce_add_sync(0xFFFFFFFFu, n[k]);
-          if (lane == 0) {
-            if constexpr (kCl)
-              asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(
-                               dst + 4u * k),
-                           "r"(v)
-                           : "memory");
-            else
-              atomicAdd(&s_obs[obs_buf][k], v);
-          }
-        }
-      }
+      if (!aux)
+        count_words<kCl, kAl>(g, pl, nr * g.W, mw, mn, cls_bytes, tid, (int)blockDim.x - 32,
+                              s_obs[obs_buf]);
       // the counts are complete, and no word changes before all are counted
       bar_arrive<kCl>();
       bar_wait<kCl>();
       if (aux && rank == 0 && lane == 0) {
         volatile int *c = s_obs[obs_buf];
-        const int64_t like = c[0], unlike = c[1], b1 = c[2], b0 = c[3], both = c[4], s1 = c[5],
-                      s0 = c[6];
+        const int64_t like = c[0], unlike = c[1], b1 = c[2], b0 = c[3], both = c[4],
+                      s1 = 2 * (int64_t)c[5] - b1, s0 = 2 * (int64_t)c[6] - b0;
         for (int k = 0; k < 7; ++k) c[k] = 0;  // for the record after the next
         const int64_t N = (int64_t)g.Lx * g.Ly;
         const int64_t rec[8] = {(int64_t)(S / 8u) + 1, b1 + b0 - 2 * both, like - unlike,
