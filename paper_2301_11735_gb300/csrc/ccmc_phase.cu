@@ -49,14 +49,11 @@ struct PhaseU {
   const uint32_t *cA, *cAL, *cAR, *cAU, *cAD, *cB, *cBL, *cBR, *cBU, *cBD;
   int offAL, offAR, offB, offBL, offBR;
   int dyAU, dyAD, qy, dyBU, dyBD;
-  int wmask;  // W - 1 (rows of power-of-two width only)
 };
 
-// How the word code reads its windows: rows of any width (kRowGeneral), rows
-// of whole words (kRowAligned), or rows of whole words and power-of-two width
-// W, staged as bands whose first row is the tile's first row (kRowTile: column
-// wraps are masks and every row offset dy is 0).
-enum RowMode { kRowGeneral = 0, kRowAligned = 1, kRowTile = 2 };
+// How the direct path reads its windows: rows of any width (kRowGeneral) or rows
+// of whole words (kRowAligned).
+enum RowMode { kRowGeneral = 0, kRowAligned = 1 };
 
 __device__ __forceinline__ int wrap(int v, int n) { return v >= n ? v - n : (v < 0 ? v + n : v); }
 
@@ -87,7 +84,6 @@ __device__ __forceinline__ PhaseU phase_uniform(const Geo &g, const Sched &sc) {
   u.qy = (byy >> 2) % g.Cy;
   u.dyBU = cby == 0 ? -1 : 0;
   u.dyBD = cby == 3 ? 1 : 0;
-  u.wmask = g.W - 1;
   return u;
 }
 
@@ -96,10 +92,7 @@ template <int kMode>
 __device__ __forceinline__ uint32_t window(const uint32_t *cls, const Geo &g, const PhaseU &u,
                                            int row, int w, int off, int n) {
   const uint32_t *r = cls + row * g.W;
-  if constexpr (kMode == kRowTile) {
-    const int wl = (w + (off >> 4)) & u.wmask;
-    return __funnelshift_r(r[wl], r[(wl + 1) & u.wmask], 2 * (off & 15));
-  } else if constexpr (kMode == kRowAligned) {  // the window straddles at most two words
+  if constexpr (kMode == kRowAligned) {  // the window straddles at most two words
     const int wl = wrap(w + (off >> 4), g.W);
     const int sh = 2 * (off & 15);
     if (sh == 0) return r[wl];
@@ -110,27 +103,21 @@ __device__ __forceinline__ uint32_t window(const uint32_t *cls, const Geo &g, co
   }
 }
 
-// Row jr + dy of a class (periodic in Cy); staged bands start at the right row.
-template <int kMode>
-__device__ __forceinline__ int band_row(const Geo &g, int r0, int dy) {
-  return kMode == kRowTile ? r0 : wrap(r0 + dy, g.Cy);
-}
-
 // n: the word's sites inside its row (16 unless the row ends in it).
 template <int kMode>
 __device__ __forceinline__ WordIn gather(const Geo &g, const PhaseU &u, int jr, int w, int n) {
   WordIn in;
   in.A = u.cA[jr * g.W + w];
-  const int jb = band_row<kMode>(g, jr, u.qy);
+  const int jb = wrap(jr + u.qy, g.Cy);
   in.B = window<kMode>(u.cB, g, u, jb, w, u.offB, n);
   in.na = neighbour_planes(window<kMode>(u.cAL, g, u, jr, w, u.offAL, n),
                          window<kMode>(u.cAR, g, u, jr, w, u.offAR, n),
-                         u.cAU[band_row<kMode>(g, jr, u.dyAU) * g.W + w],
-                         u.cAD[band_row<kMode>(g, jr, u.dyAD) * g.W + w]);
+                         u.cAU[wrap(jr + u.dyAU, g.Cy) * g.W + w],
+                         u.cAD[wrap(jr + u.dyAD, g.Cy) * g.W + w]);
   in.nb = neighbour_planes(window<kMode>(u.cBL, g, u, jb, w, u.offBL, n),
                          window<kMode>(u.cBR, g, u, jb, w, u.offBR, n),
-                         window<kMode>(u.cBU, g, u, band_row<kMode>(g, jb, u.dyBU), w, u.offB, n),
-                         window<kMode>(u.cBD, g, u, band_row<kMode>(g, jb, u.dyBD), w, u.offB, n));
+                         window<kMode>(u.cBU, g, u, wrap(jb + u.dyBU, g.Cy), w, u.offB, n),
+                         window<kMode>(u.cBD, g, u, wrap(jb + u.dyBD, g.Cy), w, u.offB, n));
   return in;
 }
 
@@ -156,16 +143,8 @@ __device__ __forceinline__ void apply_moves(const Geo &g, const PhaseU &u, int j
       atomicXor(pa, dA);
   }
   if (dB) {
-    uint32_t *rb = const_cast<uint32_t *>(u.cB) + band_row<kMode>(g, jr, u.qy) * g.W;
-    if constexpr (kMode == kRowTile) {
-      const int wl = (w + (u.offB >> 4)) & u.wmask;
-      const int sh = 2 * (u.offB & 15);
-      atomicXor(rb + wl, dB << sh);
-      if (sh) {
-        const uint32_t hi = dB >> (32 - sh);
-        if (hi) atomicXor(rb + ((wl + 1) & u.wmask), hi);
-      }
-    } else if constexpr (kMode == kRowAligned) {
+    uint32_t *rb = const_cast<uint32_t *>(u.cB) + wrap(jr + u.qy, g.Cy) * g.W;
+    if constexpr (kMode == kRowAligned) {
       const int wl = wrap(w + (u.offB >> 4), g.W);
       const int sh = 2 * (u.offB & 15);
       atomicXor(rb + wl, dB << sh);
@@ -179,19 +158,24 @@ __device__ __forceinline__ void apply_moves(const Geo &g, const PhaseU &u, int j
   }
 }
 
-// The exact path of one pair, by one lane of a warp that takes the rare calls
-// of a word together: decided and applied to the word's a and b sites by atomic
-// XOR (see exact_move).
+// The direct path's view of a word: row j, word w of the classes in global memory.
 template <int kMode>
-__device__ __forceinline__ void exact_pair(const Geo &g, const PhaseU &u, const uint2 *trans,
-                                           const uint16_t *thrT, const uint32_t *thr32, int j,
-                                           int jr, int w, int n, int c, int h, int q,
-                                           const WordIn &in, uint64_t P, uint32_t near128) {
-  const int t = 2 * c + h + 4 * q;
-  if (t >= n) return;  // past the end of the row: no pair
-  const uint32_t x = exact_move(g, trans, thrT, thr32, j, w, t, in, P, near128);
-  if (x) apply_moves<kMode, false>(g, u, jr, w, n, (x >> 2) << (2 * t), (x & 3u) << (2 * t));
-}
+struct DirectView {
+  const Geo &g;
+  const PhaseU &u;
+  int j, w;
+
+  __device__ __forceinline__ int sites(int ww) const {
+    return kMode == kRowGeneral ? min(16, g.Cx - (ww << 4)) : 16;
+  }
+  __device__ __forceinline__ WordIn gather() const { return ccmc::gather<kMode>(g, u, j, w, sites(w)); }
+  __device__ __forceinline__ void apply(uint32_t dA, uint32_t dB) const {
+    apply_moves<kMode, true>(g, u, j, w, sites(w), dA, dB);
+  }
+  __device__ __forceinline__ void apply_other(int oj, int ow, uint32_t dA, uint32_t dB) const {
+    apply_moves<kMode, false>(g, u, oj, ow, sites(ow), dA, dB);
+  }
+};
 
 // One word's pairs by one lane, with all 32 lanes of the warp calling
 // together (inactive lanes: active false): the fast decisions are applied;
@@ -199,26 +183,24 @@ __device__ __forceinline__ void exact_pair(const Geo &g, const PhaseU &u, const 
 // decides that word's rare pairs together, one pair a lane, from the owner's
 // inputs.  The rare pairs were rejected by the fast path, and no other pair of
 // the phase touches their sites or neighbours, so the order does not matter.
-// j: the a word's row in the class (keys the random streams); jr: its row in
-// u's arrays (j itself for a lattice in global memory, the row inside a
-// staged tile otherwise); near128: 128 if the phase's partners are nearest
-// neighbours, else 0; keys: the source of the Philox keys (SeedKeys or
+// view: how the word is read and changed; j: its row in the class (keys the random
+// streams), w its place in the row; near128: 128 if the phase's partners are
+// nearest neighbours, else 0; keys: the source of the Philox keys (SeedKeys or
 // TableKeys of the lattice's seed).
-template <int kMode, class Keys>
-__device__ __forceinline__ void warp_word(const Geo &g, const PhaseU &u, const uint2 *trans,
+template <class View, class Keys>
+__device__ __forceinline__ void warp_word(const Geo &g, const View &view, const uint2 *trans,
                                           const uint16_t *thrT, const uint32_t *thr32, int j,
-                                          int jr, int w, uint64_t P, uint32_t near128,
-                                          const Keys &keys, bool active = true) {
-  const int n = active ? (kMode == kRowGeneral ? min(16, g.Cx - (w << 4)) : 16) : 0;
+                                          int w, uint64_t P, uint32_t near128, const Keys &keys,
+                                          bool active = true) {
   WordIn in{};
   uint32_t rz = 0u;
   if (active) {
-    in = gather<kMode>(g, u, jr, w, n);
+    in = view.gather();
     const uint32_t gbase = (uint32_t)j * (uint32_t)(2 * g.W) + (uint32_t)(2 * w);
     const uint3 d = fast_moves<1, false>(trans, thrT, 0, in, near128, [&](int c) {
       return keys(gbase + (uint32_t)c, (uint32_t)P, (uint32_t)(P >> 32), TAG_MOVE);
     });
-    apply_moves<kMode, true>(g, u, jr, w, n, d.x, d.y);
+    view.apply(d.x, d.y);
     rz = d.z;
   }
   unsigned ball = __ballot_sync(0xFFFFFFFFu, rz != 0u);
@@ -239,13 +221,14 @@ __device__ __forceinline__ void warp_word(const Geo &g, const PhaseU &u, const u
       o.nb.O = __shfl_sync(0xFFFFFFFFu, in.nb.O, src);
       o.nb.T = __shfl_sync(0xFFFFFFFFu, in.nb.T, src);
       o.nb.F = __shfl_sync(0xFFFFFFFFu, in.nb.F, src);
-      const int oj = __shfl_sync(0xFFFFFFFFu, j, src), ojr = __shfl_sync(0xFFFFFFFFu, jr, src),
-                ow = __shfl_sync(0xFFFFFFFFu, w, src), on = __shfl_sync(0xFFFFFFFFu, n, src);
-      // the owner's pairs, one a lane
+      const int oj = __shfl_sync(0xFFFFFFFFu, j, src), ow = __shfl_sync(0xFFFFFFFFu, w, src);
+      // the owner's pairs, one a lane: half h of call c, word lane & 3 of it
       const int c = (lane >> 3) & 1, h = (lane >> 2) & 1;
-      if (lane < 16 && ((orz >> c) & 1u))
-        exact_pair<kMode>(g, u, trans, thrT, thr32, oj, ojr, ow, on, c, h, lane & 3, o, P,
-                          near128);
+      const int t = 2 * c + h + 4 * (lane & 3);
+      if (lane < 16 && ((orz >> c) & 1u) && 16 * ow + t < g.Cx) {
+        const uint32_t x = exact_move(g, trans, thrT, thr32, oj, ow, t, o, P, near128);
+        if (x) view.apply_other(oj, ow, (x >> 2) << (2 * t), (x & 3u) << (2 * t));
+      }
     }
   }
 }
@@ -283,8 +266,8 @@ __global__ void __launch_bounds__(256, 4) phase_kernel(Geo g, const uint16_t *th
     const int wid = base + threadIdx.x;
     const bool act = wid < nw;
     const int j = act ? wid / g.W : 0, w = act ? wid - j * g.W : 0;
-    warp_word<kAligned ? kRowAligned : kRowGeneral>(g, u, sm.trans, sm.thrT, thr32, j, j, w, P,
-                                                     near128, SeedKeys{g.k0, g.k1}, act);
+    warp_word(g, DirectView<kAligned ? kRowAligned : kRowGeneral>{g, u, j, w}, sm.trans, sm.thrT,
+              thr32, j, w, P, near128, SeedKeys{g.k0, g.k1}, act);
   }
 }
 
@@ -339,6 +322,86 @@ struct Band {
   int dy;
 };
 
+// The tile phase's column uniforms.  Each side is staged as five bands: the class
+// itself, the column neighbour in the same columns, the one xs = -1, 0 or 1 sites
+// further, and the two row neighbours, whose band starts at the right row (a side's
+// neighbours differ in no other way: see the resident kernel's SideD).
+enum BandOf { kA = 0, kAm, kAx, kAr, kAy, kB, kBm, kBx, kBr, kBy };
+struct TileCols {
+  int xA;          // a's further column neighbour
+  int qx, offX;    // b's columns and its further column neighbour's
+};
+
+// The tile path's view of a word: its byte offsets in a band, the same in every
+// tile of a phase, so that all sixteen loads are a base, one of seven offsets and
+// the band's constant.  (Taking every window's words from its own column offset,
+// with class pointers, cost 60 more instructions a word.)
+struct TileView {
+  char *band;  // the tile's bands in shared memory
+  uint32_t own, alo, ahi, blo, bhi, xlo, xhi;
+  int ash, bsh, xsh;
+
+  __device__ __forceinline__ TileView(const TileCols &c, int W, int jr, int w) {
+    const int m = W - 1;  // W is a power of two
+    const uint32_t row = 4u * (uint32_t)(jr * W);
+    auto at = [&](int i) { return row + 4u * (uint32_t)(i & m); };
+    band = nullptr;
+    own = at(w);
+    alo = c.xA < 0 ? at(w - 1) : own;
+    ahi = c.xA > 0 ? at(w + 1) : own;
+    ash = 2 * c.xA & 31;
+    blo = at(w + (c.qx >> 4));
+    bhi = at(w + (c.qx >> 4) + 1);
+    bsh = 2 * (c.qx & 15);
+    xlo = at(w + (c.offX >> 4));
+    xhi = at(w + (c.offX >> 4) + 1);
+    xsh = 2 * (c.offX & 15);
+  }
+  __device__ __forceinline__ uint32_t &word(int k, uint32_t off) const {
+    return *reinterpret_cast<uint32_t *>(band + off + (uint32_t)(k * kTileWords * 4));
+  }
+  __device__ __forceinline__ uint32_t window(int k) const {
+    return __funnelshift_r(word(k, blo), word(k, bhi), bsh);
+  }
+  __device__ __forceinline__ WordIn gather() const {
+    WordIn in;
+    in.A = word(kA, own);
+    in.B = window(kB);
+    in.na = neighbour_planes(word(kAm, own), word(kAr, own), word(kAy, own),
+                             __funnelshift_r(word(kAx, alo), word(kAx, ahi), ash));
+    in.nb = neighbour_planes(window(kBm), window(kBr), window(kBy),
+                             __funnelshift_r(word(kBx, xlo), word(kBx, xhi), xsh));
+    return in;
+  }
+  __device__ __forceinline__ void apply_b(uint32_t dB) const {
+    if (dB) {
+      atomicXor(&word(kB, blo), dB << bsh);
+      const uint32_t hi = __funnelshift_l(dB, 0u, bsh);  // dB >> (32 - bsh), 0 for 0
+      if (hi) atomicXor(&word(kB, bhi), hi);
+    }
+  }
+  __device__ __forceinline__ void apply(uint32_t dA, uint32_t dB) const {
+    if (dA) word(kA, own) ^= dA;
+    apply_b(dB);
+  }
+};
+
+// A tile's words seen by the warp's exact path: another lane's word from its place.
+struct TileWord {
+  const TileView &v;
+  const TileCols &c;
+  int W, j0;
+
+  __device__ __forceinline__ WordIn gather() const { return v.gather(); }
+  __device__ __forceinline__ void apply(uint32_t dA, uint32_t dB) const { v.apply(dA, dB); }
+  __device__ __forceinline__ void apply_other(int oj, int ow, uint32_t dA, uint32_t dB) const {
+    TileView o(c, W, oj - j0, ow);
+    o.band = v.band;
+    if (dA) atomicXor(&o.word(kA, o.own), dA);
+    o.apply_b(dB);
+  }
+};
+
 // kBufs: band buffers (three for the pipelined tile loop, one for a CTA that
 // takes a single tile).
 template <int kBufs = kTileBufs>
@@ -352,7 +415,8 @@ struct TileSmem {
   int armed[kBufs];    // times the buffer's `full` barrier was armed
   int tile[kBufs];     // the tile staged in the buffer, -1: no more tiles
   Band bands[kBands];
-  Sched sched;
+  TileCols cols;
+  uint32_t near128;
   int err;
   int busy0, busy1;  // classes the previous phase writes (early staging waits for them)
 };
@@ -468,19 +532,31 @@ __device__ __forceinline__ void tile_phase(const Geo &g, const uint16_t *thrT,
       }
     }
     if (lane == 0) {
-      sm.sched = sc;
-      const PhaseU u0 = phase_uniform(g, sc);
-      const Band bs[kBands] = {{u0.cA, 0},       {u0.cAL, 0},       {u0.cAR, 0},
-                               {u0.cAU, u0.dyAU}, {u0.cAD, u0.dyAD}, {u0.cB, u0.qy},
-                               {u0.cBL, u0.qy},   {u0.cBR, u0.qy},   {u0.cBU, u0.qy + u0.dyBU},
-                               {u0.cBD, u0.qy + u0.dyBD}};
-      for (int k = 0; k < kBands; ++k) sm.bands[k] = bs[k];
+      sm.near128 = sc.near ? 128u : 0u;
+      const int bx = sc.a0x + sc.rx, by = sc.a0y + sc.ry;
+      const int qx = (bx >> 2) % g.Cx, qy = (by >> 2) % g.Cy;
+      auto cls = [&](int x, int y) {
+        return g.words + (int64_t)((y & 3) * 4 + (x & 3)) * g.cstride;
+      };
+      // bands k .. k + 4 of the side at class (cx, cy), dy rows below the a rows;
+      // returns where its further column neighbour lies
+      auto side = [&](int k, int cx, int cy, int dy) {
+        const int dx = cx == 3 ? 1 : -1, dr = cy == 3 ? 1 : -1;
+        sm.bands[k + kA] = {cls(cx, cy), dy};
+        sm.bands[k + kAm] = {cls(cx - dx, cy), dy};
+        sm.bands[k + kAx] = {cls(cx + dx, cy), dy};
+        sm.bands[k + kAr] = {cls(cx, cy - dr), dy};
+        sm.bands[k + kAy] = {cls(cx, cy + dr), dy + (cy == 0 ? -1 : cy == 3 ? 1 : 0)};
+        return cx == 0 ? -1 : cx == 3 ? 1 : 0;
+      };
+      sm.cols.xA = side(kA, sc.a0x, sc.a0y, 0);
+      const int xB = side(kB, bx & 3, by & 3, qy);
+      sm.cols.qx = qx;
+      sm.cols.offX = wrap(qx + xB, g.Cx);
     }
   }
   __syncthreads();
-  const Sched sc = sm.sched;
-  const uint32_t near128 = sc.near ? 128u : 0u;
-  const PhaseU u = phase_uniform(g, sc);
+  const uint32_t near128 = sm.near128;
   const int W = g.W, R = kTileWords / W, Cy = g.Cy;
   const int ntiles = Cy / R;
   const uint32_t row_bytes = (uint32_t)W * 4u;
@@ -551,24 +627,8 @@ __device__ __forceinline__ void tile_phase(const Geo &g, const uint16_t *thrT,
   if (!mbar_wait(smem_u32(&sm.tables), 0u)) sm.err = 1;
 
   const int lw = __ffs(W) - 1;  // W is a power of two
-  const int wi = (int)threadIdx.x;  // word of the tile
-  const int jr = wi >> lw, w = wi & (W - 1);
-  // a tile's bands in buffer b as the windows' sources
-  auto local_u = [&](int b) {
-    const uint32_t *base = sm.band[b][0];
-    PhaseU lu = u;
-    lu.cA = base;
-    lu.cAL = base + 1 * kTileWords;
-    lu.cAR = base + 2 * kTileWords;
-    lu.cAU = base + 3 * kTileWords;
-    lu.cAD = base + 4 * kTileWords;
-    lu.cB = base + 5 * kTileWords;
-    lu.cBL = base + 6 * kTileWords;
-    lu.cBR = base + 7 * kTileWords;
-    lu.cBU = base + 8 * kTileWords;
-    lu.cBD = base + 9 * kTileWords;
-    return lu;
-  };
+  const int jr = (int)threadIdx.x >> lw, w = (int)threadIdx.x & (W - 1);  // word of the tile
+  TileView view(sm.cols, W, jr, w);
   int b = 0;
   for (int t = 0;; ++t) {
     // (1) evaluate this thread's word of the tile in buffer b, if any
@@ -578,8 +638,9 @@ __device__ __forceinline__ void tile_phase(const Geo &g, const uint16_t *thrT,
     }
     const int tile = sm.tile[b];
     if (tile < 0) break;
-    warp_word<kRowTile>(g, local_u(b), sm.trans, sm.thrT, thr32, tile * R + jr, jr, w, P, near128,
-                        keys);
+    view.band = reinterpret_cast<char *>(sm.band[b][0]);
+    warp_word(g, TileWord{view, sm.cols, W, tile * R}, sm.trans, sm.thrT, thr32, tile * R + jr, w,
+              P, near128, keys);
     // (2) this warp is done with the tile: its shared-memory writes are ordered
     // before the async copies that will refill the buffer, and before the
     // last warp's reads
@@ -598,12 +659,13 @@ __device__ __forceinline__ void tile_phase(const Geo &g, const uint16_t *thrT,
       if (*(volatile int *)&sm.err == 0) {
         const int j0 = tile * R;
         const uint4 *sa = reinterpret_cast<const uint4 *>(sm.band[b][0]);
-        const uint4 *sb = reinterpret_cast<const uint4 *>(sm.band[b][5]);
-        uint4 *ga = reinterpret_cast<uint4 *>(const_cast<uint32_t *>(u.cA) + (int64_t)j0 * W);
-        int rb = j0 + u.qy;
+        const uint4 *sb = reinterpret_cast<const uint4 *>(sm.band[b][kB]);
+        uint4 *ga = reinterpret_cast<uint4 *>(const_cast<uint32_t *>(sm.bands[kA].cls) +
+                                              (int64_t)j0 * W);
+        int rb = j0 + sm.bands[kB].dy;
         rb = rb >= Cy ? rb - Cy : rb;
         const int split = min(R, Cy - rb) * W / 4;  // uint4 before the band wraps
-        uint4 *gb = reinterpret_cast<uint4 *>(const_cast<uint32_t *>(u.cB));
+        uint4 *gb = reinterpret_cast<uint4 *>(const_cast<uint32_t *>(sm.bands[kB].cls));
         const int64_t gb1 = (int64_t)rb * W / 4;  // in uint4
 #pragma unroll
         for (int q = lane; q < kTileWords / 4; q += 32) {
@@ -709,8 +771,8 @@ __global__ void __launch_bounds__(256, 4) phase_multi_kernel(const MultiJob *__r
     const int wid = base + threadIdx.x;
     const bool act = wid < nw;
     const int j = act ? wid / g.W : 0, w = act ? wid - j * g.W : 0;
-    warp_word<kAligned ? kRowAligned : kRowGeneral>(g, u, sm.trans, sm.thrT, J.thr32, j, j, w, P,
-                                                     near128, SeedKeys{g.k0, g.k1}, act);
+    warp_word(g, DirectView<kAligned ? kRowAligned : kRowGeneral>{g, u, j, w}, sm.trans, sm.thrT,
+              J.thr32, j, w, P, near128, SeedKeys{g.k0, g.k1}, act);
   }
 }
 
