@@ -1,7 +1,12 @@
 // ccmc_count.cuh -- observables of a packed lattice by definition (Eq. 3 and
-// Eq. 2): popcounts of the charge and sign bit planes of each class word
-// against its right and down neighbour windows.  Used by the recount kernel
-// and by the resident batch kernel.
+// Eq. 2) as sums over bit products.  In the linear code S = b1 - b0 and sigma = 1 -
+// b1 - b0, so with `like` the bonds' products b1 b1' + b0 b0' and `unlike` b1 b0' +
+// b0 b1', summed over all 2N right and down bonds,
+//   BV = like - unlike,
+//   BJ = 2N - 4 (b1 + b0) + like + unlike   (every site has four bond ends),
+// and Nc = b1 + b0 - 2 both, M = N - b1 - b0, S = b1 - b0 from the sites' sums; the
+// staggered ones from the sums over the sites of even x + y (half of all).
+// Used by the recount kernel; the resident kernel counts the same sums.
 #pragma once
 
 #include <cstdint>
@@ -17,86 +22,55 @@ __device__ __forceinline__ int64_t warp_sum(int64_t v) {
   return v;
 }
 
-// Bit planes of a class word X (linear code) against its right and down
-// neighbour windows Yr, Yd, a site's type (1 = charged, b1 XOR b0) at its odd
-// bit and its sign (b0, 1 = minus) at the even bit below it.  `vo` holds the
-// odd bits of the valid sites.  Bonds are laid out two to a site: the right
-// bond at the odd bit, the down bond at the even bit (the down masks shifted
-// down one place, which adds to the right ones without carries).
-struct WordPlanes {
-  uint32_t k, kg, ug;  // charged, charged with S = -1, magnetic with sigma = -1
-  uint32_t kk, uu;     // charged-charged and magnetic-magnetic bonds
-  uint32_t f;          // bonds whose two signs differ
-};
+// like, unlike, b1, b0, both, and b1, b0 over the sites of even x + y.
+constexpr int kSums = 7;
 
-__device__ __forceinline__ WordPlanes word_planes(uint32_t X, uint32_t Yr, uint32_t Yd,
-                                                  uint32_t vo) {
-  constexpr uint32_t kEven = 0x55555555u, kOdd = 0xAAAAAAAAu;
-  WordPlanes p;
-  const uint32_t Xs = X << 1;  // sign bits moved up to the odd bits
-  const uint32_t K = X ^ Xs, Kr = Yr ^ (Yr << 1), Kd = Yd ^ (Yd << 1);
-  p.k = K & vo;
-  p.kg = ~X & Xs & vo;
-  p.ug = X & Xs & vo;
-  p.kk = (K & Kr & vo) + ((K & Kd & vo) >> 1);
-  p.uu = (~(K | Kr) & vo) + ((~(K | Kd) & vo) >> 1);
-  p.f = (((X ^ Yr) << 1) & kOdd) | ((X ^ Yd) & kEven);
-  return p;
+// The observables Nc, BV, BJ, M, M_stag, S_sum, S_stag of the lattice's sums.
+__device__ __forceinline__ void observables_of(const Geo &g, const int64_t s[kSums],
+                                               int64_t obs[7]) {
+  const int64_t N = (int64_t)g.Lx * g.Ly;
+  const int64_t like = s[0], unlike = s[1], b1 = s[2], b0 = s[3], both = s[4];
+  const int64_t d1 = 2 * s[5] - b1, d0 = 2 * s[6] - b0;  // even minus odd sites
+  obs[0] = b1 + b0 - 2 * both;
+  obs[1] = like - unlike;
+  obs[2] = 2 * N - 4 * (b1 + b0) + like + unlike;
+  obs[3] = N - b1 - b0;
+  obs[4] = -d1 - d0;
+  obs[5] = b1 - b0;
+  obs[6] = d1 - d0;
 }
 
-// Popcount sums of one class: the sites' planes and the bonds' planes, and
-// the number of sites counted.  fold() turns them into c[7] (Nc, BV, BJ, M,
-// M_stag, S_sum, S_stag); the staggered sign is uniform over a class.
-struct ClassCounts {
-  int sites = 0, nK = 0, nKG = 0, nUG = 0, nKK = 0, nKKd = 0, nUU = 0, nUUd = 0;
+// Bits b1 and b0 of every site exchanged.
+__device__ __forceinline__ uint32_t swapped(uint32_t X) {
+  return lop3<kLutMux>(X << 1, X >> 1, 0xAAAAAAAAu);
+}
 
-  __device__ __forceinline__ void bonds(const WordPlanes &p) {
-    nKK += __popc(p.kk);
-    nKKd += __popc(p.kk & p.f);
-    nUU += __popc(p.uu);
-    nUUd += __popc(p.uu & p.f);
-  }
-  __device__ __forceinline__ void fold(int cls, int c[7]) const {
-    const int sgn = (((cls & 3) + (cls >> 2)) & 1) ? -1 : 1;
-    const int M = sites - nK - 2 * nUG, S = nK - 2 * nKG;
-    c[0] += nK;
-    c[1] += nKK - 2 * nKKd;
-    c[2] += nUU - 2 * nUUd;
-    c[3] += M;
-    c[4] += sgn * M;
-    c[5] += S;
-    c[6] += sgn * S;
-  }
-};
-
-// Adds the observables of words tid, tid + nthreads, ... of class `cls` to
-// c[7] (Nc, BV, BJ, M, M_stag, S_sum, S_stag), any row width.
+// Adds the sums of words tid, tid + nthreads, ... of class `cls`, any row width
+// (bits above a row's end are zero in the words).
 __device__ __forceinline__ void count_class(const Geo &g, int cls, int tid, int nthreads,
-                                            int c[7]) {
+                                            int s[kSums]) {
   const int W = g.W, nw = g.Cy * W;
   const int cx = cls & 3, cy = cls >> 2;
   const uint32_t *X0 = g.words + (int64_t)cls * g.cstride;
   const uint32_t *R0 = g.words + (int64_t)(cy * 4 + ((cx + 1) & 3)) * g.cstride;
   const uint32_t *D0 = g.words + (int64_t)(((cy + 1) & 3) * 4 + cx) * g.cstride;
-  ClassCounts n;
   int wid = tid;
   int j = wid / W, w = wid - j * W;
   const int sj = nthreads / W, sw = nthreads - sj * W;
+  int k1 = 0, k0 = 0;
   for (; wid < nw; wid += nthreads) {
     const int s0 = w << 4;
-    const int ns = min(16, g.Cx - s0);
-    const uint32_t vo = ns == 16 ? 0xAAAAAAAAu : (((1u << (2 * ns)) - 1u) & 0xAAAAAAAAu);
-    const uint32_t X = X0[wid];
-    const uint32_t Xr = fetch_window(R0 + j * W, W, g.Cx,
-                                     cx == 3 ? (s0 + 1 == g.Cx ? 0 : s0 + 1) : s0, ns);
+    const uint32_t X = X0[wid], Xs = swapped(X);
+    const uint32_t Yr = fetch_window(R0 + j * W, W, g.Cx,
+                                     cx == 3 ? (s0 + 1 == g.Cx ? 0 : s0 + 1) : s0,
+                                     min(16, g.Cx - s0));
     const int jd = cy == 3 ? (j + 1 == g.Cy ? 0 : j + 1) : j;
-    const uint32_t Xd = D0[jd * W + w];
-    const WordPlanes p = word_planes(X, Xr, Xd, vo);
-    n.sites += ns;
-    n.nK += __popc(p.k);
-    n.nKG += __popc(p.kg);
-    n.nUG += __popc(p.ug);
-    n.bonds(p);
+    const uint32_t Yd = D0[jd * W + w];
+    s[0] += __popc(X & Yr) + __popc(X & Yd);
+    s[1] += __popc(Xs & Yr) + __popc(Xs & Yd);
+    k1 += __popc(X & 0xAAAAAAAAu);
+    k0 += __popc(X & 0x55555555u);
+    s[4] += __popc(X & Xs & 0xAAAAAAAAu);
     w += sw;
     j += sj;
     if (w >= W) {
@@ -104,118 +78,101 @@ __device__ __forceinline__ void count_class(const Geo &g, int cls, int tid, int 
       ++j;
     }
   }
-  n.fold(cls, c);
+  s[2] += k1;
+  s[3] += k0;
+  if (!((cx + cy) & 1)) {
+    s[5] += k1;
+    s[6] += k0;
+  }
 }
 
-// The quad path: rows of whole words (Cx a multiple of 16) with W a multiple
-// of 4, four consecutive words of a class row per step with 16-byte loads.
-// Every site's type bit (odd) and sign bit (even) are first copied into both
-// bits of its pair, one plane per word for the word and one for its two
-// neighbour windows (right window at the odd bits, down window at the even
-// bits); then one AND is the charged-charged bonds of both directions, and an
-// XOR of the sign planes marks the bonds whose signs differ.  The count of
-// magnetic-magnetic bonds is not formed: over the whole lattice it follows
-// from the others (below).  Sites of two words share one popcount (types of
-// the first at the odd bits, of the second at the even bits).
-struct QuadCounts {
-  int nK = 0, nKG = 0, nUG = 0, nKK = 0, nKKd = 0, nUUd = 0, quads = 0;
-};
+// The quad path: rows of whole words (Cx a multiple of 16) with W a multiple of 4.
+// A thread takes four consecutive words of the four classes of a row of sites at
+// once with 16-byte loads: the classes are each other's right neighbours, so eight
+// loads (and one word across the quad's end) serve sixteen words, 8.25 bytes a word
+// where a class at a time took 12.  The logic pipe and the population counts (a
+// quarter of its rate) share the work: a half adder joins a word's two bonds, a full
+// adder three words, and two classes share the site counts: 4 counts and 15 logic
+// instructions a word.
 
-constexpr uint32_t kLutNorAnd = 0x02;   // ~(a | b) & c
-constexpr uint32_t kLutAndNot = 0x0C;   // ~a & b
+// The bond products of four words against their right and down windows.
+__device__ __forceinline__ int bond_count(const uint32_t X[4], const uint32_t R[4],
+                                          const uint32_t D[4]) {
+  constexpr uint32_t kLutAndXor2 = 0x60;  // a & (b ^ c)
+  uint32_t s[4], c[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    s[k] = lop3<kLutAndXor2>(X[k], R[k], D[k]);
+    c[k] = lop3<kLutAnd3>(X[k], R[k], D[k]);
+  }
+  const uint32_t s1 = lop3<kLutXor3>(s[0], s[1], s[2]), t0 = lop3<kLutMaj>(s[0], s[1], s[2]);
+  const uint32_t t1 = lop3<kLutXor3>(t0, c[0], c[1]), f0 = lop3<kLutMaj>(t0, c[0], c[1]);
+  const uint32_t t2 = lop3<kLutXor3>(t1, c[2], c[3]), f1 = lop3<kLutMaj>(t1, c[2], c[3]);
+  return __popc(s1) + __popc(s[3]) + 2 * __popc(t2) + 4 * (__popc(f0) + __popc(f1));
+}
 
-template <bool kColR, bool kRowD>
-__device__ __forceinline__ void count_quads(const uint32_t *__restrict__ X0,
-                                            const uint32_t *__restrict__ R0,
-                                            const uint32_t *__restrict__ D0, int W, int Cy,
-                                            int q, int nthreads, QuadCounts &n) {
+__device__ __forceinline__ void count_quads(const Geo &g, int cy, int q, int nthreads,
+                                            int s[kSums]) {
   constexpr uint32_t kOdd = 0xAAAAAAAAu;
-  const int Wq = W >> 2, nq = Cy * Wq, last_row = (Cy - 1) * Wq;
+  const int W = g.W, Wq = W >> 2, nq = g.Cy * Wq, last_row = (g.Cy - 1) * Wq;
+  const uint32_t *own = g.words + (int64_t)(4 * cy) * g.cstride;
+  const uint32_t *below = g.words + (int64_t)(4 * ((cy + 1) & 3)) * g.cstride;
   int wq = q % Wq;
   const int sw = nthreads % Wq;
-#pragma unroll 2
   for (; q < nq; q += nthreads) {
     const int o = 4 * q;  // word offset of the quad: row j, column 4 wq
-    // the down neighbours of class row Cy-1 of the last class row wrap to row 0
-    const int od = kRowD ? (q < last_row ? o + W : o - last_row * 4) : o;
-    const uint4 x = *reinterpret_cast<const uint4 *>(X0 + o);
-    const uint4 r = *reinterpret_cast<const uint4 *>(R0 + o);
-    const uint4 d = *reinterpret_cast<const uint4 *>(D0 + od);
-    // right neighbours of class column 3 are one column further on: the
-    // windows start one site later (the last one wraps to the row's start)
-    uint32_t rn = 0u;
-    if (kColR) {
-      rn = R0[wq == Wq - 1 ? o + 4 - W : o + 4];
-      wq += sw;
-      if (wq >= Wq) wq -= Wq;
-    }
-    const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
-    const uint32_t ds[4] = {d.x, d.y, d.z, d.w};
-    const uint32_t rs[5] = {r.x, r.y, r.z, r.w, rn};
+    // the down neighbours of class row 3 lie one class row further down
+    const int od = cy < 3 ? o : q < last_row ? o + W : o - last_row * 4;
+    uint4 x[4], d[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint32_t X = xs[k], Yd = ds[k];
-      const uint32_t Yr = kColR ? __funnelshift_r(rs[k], rs[k + 1], 2) : rs[k];
-      const uint32_t gX = lop3<kLutMux>(X << 1, X, kOdd);        // sign in both bits
-      const uint32_t tX = lop3<kLutMux>(X, X >> 1, kOdd) ^ gX;   // type in both bits
-      const uint32_t gY = lop3<kLutMux>(Yr << 1, Yd, kOdd);
-      const uint32_t tY = lop3<kLutMux>(Yr, Yd >> 1, kOdd) ^ gY;
-      const uint32_t f = gX ^ gY;
-      n.nKK += __popc(tX & tY);
-      n.nKKd += __popc(lop3<kLutAnd3>(tX, tY, f));
-      n.nUUd += __popc(lop3<kLutNorAnd>(tX, tY, f));
+    for (int cx = 0; cx < 4; ++cx) {
+      x[cx] = *reinterpret_cast<const uint4 *>(own + cx * g.cstride + o);
+      d[cx] = *reinterpret_cast<const uint4 *>(below + cx * g.cstride + od);
+    }
+    const uint32_t next = own[wq == Wq - 1 ? o + 4 - W : o + 4];
+    wq += sw;
+    if (wq >= Wq) wq -= Wq;
+    uint32_t X[4][4], B[4][4];
+#pragma unroll
+    for (int cx = 0; cx < 4; ++cx) {
+      X[cx][0] = x[cx].x;
+      X[cx][1] = x[cx].y;
+      X[cx][2] = x[cx].z;
+      X[cx][3] = x[cx].w;
     }
 #pragma unroll
-    for (int k = 0; k < 4; k += 2) {
-      const uint32_t S = lop3<kLutMux>(xs[k] << 1, xs[k + 1], kOdd);
-      const uint32_t T = lop3<kLutMux>(xs[k], xs[k + 1] >> 1, kOdd) ^ S;
-      n.nK += __popc(T);
-      n.nKG += __popc(T & S);
-      n.nUG += __popc(lop3<kLutAndNot>(T, S, 0u));
+    for (int cx = 0; cx < 4; ++cx) {
+      const uint32_t D[4] = {d[cx].x, d[cx].y, d[cx].z, d[cx].w};
+      uint32_t R[4], Xs[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        // the last class's right neighbours: the first class one site further
+        R[k] = cx < 3 ? X[(cx + 1) & 3][k]
+                      : __funnelshift_r(X[0][k], k < 3 ? X[0][(k + 1) & 3] : next, 2);
+        Xs[k] = swapped(X[cx][k]);
+        B[cx][k] = X[cx][k] & Xs[k];
+      }
+      s[0] += bond_count(X[cx], R, D);
+      s[1] += bond_count(Xs, R, D);
     }
-    ++n.quads;
+    int b1[2] = {0, 0}, b0[2] = {0, 0};
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        b1[h] += __popc(lop3<kLutMux>(X[h][k], X[h + 2][k] >> 1, kOdd));
+        b0[h] += __popc(lop3<kLutMux>(X[h][k] << 1, X[h + 2][k], kOdd));
+        s[4] += __popc(lop3<kLutMux>(B[h][k], B[h + 2][k], kOdd));
+      }
+    s[2] += b1[0] + b1[1];
+    s[3] += b0[0] + b0[1];
+    s[5] += cy & 1 ? b1[1] : b1[0];
+    s[6] += cy & 1 ? b0[1] : b0[0];
   }
 }
 
-// Adds the quad path's counts of class `cls` to c[7].  c[2] receives
-// nKK - 2 nUUd only: with nUU the magnetic-magnetic bonds, every site having
-// two bonds (2N in all) and every charged site four bond ends
-// (4 Nc = 2 nKK + n_mixed), the lattice total is nUU = 2N - 4 Nc + nKK, so
-// BJ = nUU - 2 nUUd lacks the term 2N - 4 Nc, which bj_completion() gives
-// once for the whole lattice.
-__device__ __forceinline__ void count_class_quads(const Geo &g, int cls, int tid, int nthreads,
-                                                  int c[7]) {
-  const int cx = cls & 3, cy = cls >> 2;
-  const uint32_t *X0 = g.words + (int64_t)cls * g.cstride;
-  const uint32_t *R0 = g.words + (int64_t)(cy * 4 + ((cx + 1) & 3)) * g.cstride;
-  const uint32_t *D0 = g.words + (int64_t)(((cy + 1) & 3) * 4 + cx) * g.cstride;
-  QuadCounts n;
-  if (cx == 3) {
-    if (cy == 3) count_quads<true, true>(X0, R0, D0, g.W, g.Cy, tid, nthreads, n);
-    else count_quads<true, false>(X0, R0, D0, g.W, g.Cy, tid, nthreads, n);
-  } else {
-    if (cy == 3) count_quads<false, true>(X0, R0, D0, g.W, g.Cy, tid, nthreads, n);
-    else count_quads<false, false>(X0, R0, D0, g.W, g.Cy, tid, nthreads, n);
-  }
-  const int sgn = ((cx + cy) & 1) ? -1 : 1;
-  const int M = 64 * n.quads - n.nK - 2 * n.nUG, S = n.nK - 2 * n.nKG;
-  c[0] += n.nK;
-  c[1] += n.nKK - 2 * n.nKKd;
-  c[2] += n.nKK - 2 * n.nUUd;
-  c[3] += M;
-  c[4] += sgn * M;
-  c[5] += S;
-  c[6] += sgn * S;
-}
-
-__device__ __forceinline__ bool quads_ok(const Geo &g) {
+__host__ __device__ inline bool quads_ok(const Geo &g) {
   return (g.Cx & 15) == 0 && (g.W & 3) == 0;
-}
-
-// The part of BJ that count_class_quads leaves to the lattice total, given the
-// lattice's number of charged sites Nc.
-__device__ __forceinline__ int64_t bj_completion(const Geo &g, int64_t Nc) {
-  return quads_ok(g) ? 2 * (int64_t)g.Lx * g.Ly - 4 * Nc : 0;
 }
 
 }  // namespace ccmc

@@ -69,8 +69,8 @@ __global__ void init_kernel(Geo g, int h, int64_t n_plus, int64_t n_minus) {
 }
 
 // ============================================================================
-// Recount (Eq. 3 and Eq. 2 by definition): per class word, popcounts of the
-// charge/sign bit planes against the right and down neighbour windows.  Block
+// Recount (Eq. 3 and Eq. 2 by definition): sums of bit products of the class words
+// against their right and down neighbour windows (ccmc_count.cuh).  Block
 // partials go to scratch; the last block to arrive sums them into a record,
 // appends it to the ring and the histograms, and re-arms the ticket.
 struct RecountArgs {
@@ -82,14 +82,14 @@ struct RecountArgs {
   int64_t sweep_off;    // sweeps_done = phase_base / 8 + sweep_off
 };
 
-// Grid (gx, 16): grid row y counts class y.
-__global__ void __launch_bounds__(256, 5) recount_kernel(Geo g, RecountArgs a) {
+// Grid (gx, 4): grid row y counts the classes of site rows y mod 4; or (gx, 16),
+// class y, for rows that are not whole quads of words.
+__global__ void __launch_bounds__(256, 4) recount_kernel(Geo g, RecountArgs a) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
-  int c[7] = {0, 0, 0, 0, 0, 0, 0};  // Nc, BV, BJ, M, Ms, S, Ss
+  int c[kSums] = {0, 0, 0, 0, 0, 0, 0};
   if (quads_ok(g))
-    count_class_quads(g, blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x,
-                      gridDim.x * blockDim.x, c);
+    count_quads(g, blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, c);
   else
     count_class(g, blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, c);
   const unsigned nblocks = gridDim.x * gridDim.y;
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256, 5) recount_kernel(Geo g, RecountArgs a) {
   __threadfence();
   // the last block sums the partials with all its threads (L2 loads: the
   // partials were written by other blocks)
-  __shared__ int64_t rec[8];
+  __shared__ int64_t sums[kSums];
   int64_t v[7] = {0, 0, 0, 0, 0, 0, 0};
   for (unsigned b = threadIdx.x; b < nblocks; b += blockDim.x) {
 #pragma unroll
@@ -135,12 +135,13 @@ __global__ void __launch_bounds__(256, 5) recount_kernel(Geo g, RecountArgs a) {
   if (threadIdx.x < 7) {
     int64_t x = 0;
     for (int wv = 0; wv < (int)(blockDim.x >> 5); ++wv) x += red[wv][threadIdx.x];
-    rec[1 + threadIdx.x] = x;
+    sums[threadIdx.x] = x;
   }
-  if (threadIdx.x == 0) rec[0] = g.ctl[kCtlPhaseBase] / 8 + a.sweep_off;
   __syncthreads();
   if (threadIdx.x == 0) {
-    rec[3] += bj_completion(g, rec[1]);
+    int64_t rec[8];
+    rec[0] = g.ctl[kCtlPhaseBase] / 8 + a.sweep_off;
+    observables_of(g, sums, rec + 1);
     for (int k = 0; k < 8; ++k) g.ctl[kCtlLatest + k] = rec[k];
     if (a.ring) {
       const int64_t cnt = g.ctl[kCtlObsCount];
@@ -391,20 +392,23 @@ cudaError_t launch_init(const Geo &g, int h, int64_t n_plus, int64_t n_minus, cu
   return cudaGetLastError();
 }
 
-// Grid x-extent of recount_kernel (its y-extent is the 16 classes): at most
-// 16 x 47 = 752 blocks, one wave at five blocks per SM (48 registers).  A
-// thread's unit is a word, or four words on rows that allow 16-byte loads.
-static int recount_gx(const Geo &g) {
-  const int64_t units = (int64_t)g.Cy * g.W / (((g.Cx & 15) == 0 && (g.W & 3) == 0) ? 4 : 1);
-  return grid_for(units, 256, 47);
+// Grid of recount_kernel: one wave at four blocks per SM (64 registers).  A
+// thread's unit is a word, or a quad of words of four classes.
+static dim3 recount_dim(const Geo &g) {
+  const int64_t words = (int64_t)g.Cy * g.W;
+  if (quads_ok(g)) return dim3((unsigned)grid_for(words / 4, 256, 152), 4u);
+  return dim3((unsigned)grid_for(words, 256, 38), 16u);
 }
 
-int recount_grid(const Geo &g) { return 16 * recount_gx(g); }
+int recount_grid(const Geo &g) {
+  const dim3 d = recount_dim(g);
+  return (int)(d.x * d.y);
+}
 
 cudaError_t launch_recount(const Geo &g, int64_t *partials, int64_t *ring, int64_t ring_cap,
                            int64_t *hist, int nbins, int64_t sweep_off, cudaStream_t s) {
   RecountArgs a{partials, ring, ring_cap, hist, nbins, sweep_off};
-  return launch_pdl(recount_kernel, dim3((unsigned)recount_gx(g), 16u), 256, s, g, a);
+  return launch_pdl(recount_kernel, recount_dim(g), 256, s, g, a);
 }
 
 cudaError_t launch_advance(int64_t *ctl, int64_t phases, cudaStream_t s) {

@@ -8,7 +8,6 @@
 #include <cstddef>
 #include <cstdint>
 
-#include "ccmc_count.cuh"
 #include "ccmc_device.cuh"
 #include "ccmc_internal.h"
 #include "ccmc_launch.cuh"
