@@ -121,6 +121,7 @@ void dfree(void *p, int dev) {
 // instead of 10).  At most kStages of kStageBytes for the process, lent for the
 // length of one call; a caller that finds none takes the pageable path.
 constexpr size_t kStageBytes = (size_t)1 << 20;
+constexpr size_t kStateBytes = (size_t)256 << 10;  // lattice states at most this long
 constexpr int kStages = 8;
 std::mutex g_stage_mu;
 std::vector<void *> g_stage_free;
@@ -200,6 +201,21 @@ namespace {
 // resident, 3.7 us a launch; 1000^2, ragged: 3.4 against 4.6; 256^2: 1.4 against
 // 3.3; 64^2: 0.7 against 3.3).
 bool resident_default(const Geo &g) { return g.cstride <= 4608 && resident_possible(g); }
+
+// The move table, the same for every lattice (built and checked once: 25 us).
+struct MoveTable {
+  uint32_t words[2 * kMoveN];
+  bool ok;
+};
+
+const MoveTable &move_table() {
+  static const MoveTable t = [] {
+    MoveTable m;
+    m.ok = build_transitions(m.words);
+    return m;
+  }();
+  return t;
+}
 
 int validate_shape(int Lx, int Ly) {
   if (Lx < 4 || Ly < 4 || (Lx & 3) || (Ly & 3)) return CCMC_E_INVAL;
@@ -467,10 +483,10 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
   h->t.thr32 = (uint32_t *)p;
   g.words = h->d_words;
   g.ctl = h->d_ctl;
-  uint32_t tr[2 * kMoveN];
-  if (!build_transitions(tr)) return fail(CCMC_E_INVAL);
-  if (cudaMemcpyAsync(h->t.trans, tr, sizeof(tr), cudaMemcpyHostToDevice, h->stream) !=
-          cudaSuccess ||
+  const MoveTable &moves = move_table();
+  if (!moves.ok) return fail(CCMC_E_INVAL);
+  if (cudaMemcpyAsync(h->t.trans, moves.words, sizeof(moves.words), cudaMemcpyHostToDevice,
+                      h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->d_words, 0, sizeof(uint32_t) * 16 * g.cstride, h->stream) !=
           cudaSuccess ||
       launch_set_ctl(h->d_ctl, 0, h->stream) != cudaSuccess ||
@@ -533,7 +549,7 @@ int ccmc::export_async(ccmc_lattice *h, int64_t *rec, int64_t *status, int64_t *
     CK(cudaMemcpyAsync(ring, h->d_ring, sizeof(int64_t) * 8 * h->ring_cap,
                        cudaMemcpyDeviceToHost, h->stream));
   }
-  if (state && (size_t)h->g.Lx * h->g.Ly <= kStageBytes) {
+  if (state && (size_t)h->g.Lx * h->g.Ly <= (h->g.Lx % 16 ? 4096 : kStateBytes)) {
     CK(launch_unpack(h->g, state, h->stream));  // straight into the pinned buffer
   } else if (state) {
     rc = ensure_bytes(h);
@@ -797,13 +813,15 @@ int ccmc_hist_get(ccmc_lattice *h, int64_t *out) {
 }  // extern "C"
 
 // Hands `n` bytes of state made by `make(device pointer)` to the caller: short ones
-// written into a pinned buffer by the kernel itself.
+// through a pinned buffer, which the kernel writes itself when its rows are whole
+// 16-byte groups (wide) or there are few of them (1648 x 2048 in single bytes: 80 us
+// more than a copy).
 template <typename Make>
-static int read_state(ccmc_lattice *h, uint8_t *host_out, size_t n, Make make) {
+static int read_state(ccmc_lattice *h, uint8_t *host_out, size_t n, bool wide, Make make) {
   if (!h || !host_out) return CCMC_E_INVAL;
   if (!h->initialised) return CCMC_E_STATE;
-  Stage st(n);
-  if (st) {
+  Stage st(n <= kStateBytes ? n : kStageBytes + 1);  // longer ones: the driver's own staging
+  if (st && (wide || n <= 4096)) {
     CK(make(st.as<uint8_t>()));
     CK(cudaStreamSynchronize(h->stream));
     std::memcpy(host_out, st.as<uint8_t>(), n);
@@ -811,8 +829,10 @@ static int read_state(ccmc_lattice *h, uint8_t *host_out, size_t n, Make make) {
     const int rc = ensure_bytes(h);
     if (rc) return rc;
     CK(make(h->d_bytes));
-    CK(cudaMemcpyAsync(host_out, h->d_bytes, n, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaMemcpyAsync(st ? st.as<uint8_t>() : host_out, h->d_bytes, n, cudaMemcpyDeviceToHost,
+                       h->stream));
     CK(cudaStreamSynchronize(h->stream));
+    if (st) std::memcpy(host_out, st.as<uint8_t>(), n);
   }
   h->queued = false;
   return CCMC_OK;
@@ -821,12 +841,12 @@ static int read_state(ccmc_lattice *h, uint8_t *host_out, size_t n, Make make) {
 extern "C" {
 
 int ccmc_get_state(ccmc_lattice *h, uint8_t *host_out) {
-  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly : 0,
+  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly : 0, h && h->g.Lx % 16 == 0,
                     [&](uint8_t *to) { return launch_unpack(h->g, to, h->stream); });
 }
 
 int ccmc_get_state_packed(ccmc_lattice *h, uint8_t *host_out) {
-  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly / 4 : 0,
+  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly / 4 : 0, h && h->g.Lx % 64 == 0,
                     [&](uint8_t *to) { return launch_unpack2(h->g, to, h->stream); });
 }
 
@@ -884,6 +904,8 @@ struct ccmc_batch {
   int cap = 0;  // largest number of lattices one launch may hold
   cudaStream_t stream = nullptr;
   bool own_stream = false;
+  int device = 0;
+  void *d_slab = nullptr;    // one allocation: the next two and d_multi
   ResJob *d_jobs = nullptr;  // resident lattices
   int64_t **d_ctls = nullptr;  // the members' control blocks (a batch with fixed members)
   int threads = kResMaxWorkers;
@@ -940,9 +962,13 @@ int side_streams(ccmc_batch *b, int n) {
 // work; the batch stream waits for them).
 int run_resident(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats,
                  const std::vector<int> &which, const int64_t *nsweeps, const int *obs_every) {
-  // every lattice's share of the CTAs the GPU holds, by its words a phase
-  double words = 0;
-  for (int i : which) words += (double)lats[i]->g.cstride;
+  // every lattice's share of the CTAs the GPU holds, by its work in this launch (a
+  // lattice with many sweeps left gets more, so that it does not end alone)
+  double words = 0, work = 0;
+  for (int i : which) {
+    words += (double)lats[i]->g.cstride;
+    work += (double)lats[i]->g.cstride * (double)nsweeps[i];
+  }
   const double ctas = (double)b->sms * b->ctas_per_sm;
   struct Plan {
     int i;
@@ -953,8 +979,8 @@ int run_resident(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats,
   for (int i : which) {
     const Geo &g = lats[i]->g;
     plans.push_back({i,
-                     resident_shape(g, ctas * (double)g.cstride / words, words / b->sms,
-                                    b->threads, b->max_tpw),
+                     resident_shape(g, ctas * (double)g.cstride * (double)nsweeps[i] / work,
+                                    words / b->sms, b->threads, b->max_tpw),
                      (g.Cx & 15) == 0});
   }
   auto same = [](const ResShape &x, const ResShape &y) {
@@ -1245,11 +1271,6 @@ int ccmc_batch_create(int count, ccmc_lattice *const *lattices, void *cuda_strea
   (*out)->lats.assign(lattices, lattices + count);
   std::vector<int64_t *> ctls;
   for (int i = 0; i < count; ++i) ctls.push_back(lattices[i]->d_ctl);
-  if (cudaMalloc(&(*out)->d_ctls, sizeof(int64_t *) * count) != cudaSuccess) {
-    ccmc_batch_destroy(*out);
-    *out = nullptr;
-    return CCMC_E_NOMEM;
-  }
   if (cudaMemcpyAsync((*out)->d_ctls, ctls.data(), sizeof(int64_t *) * count,
                       cudaMemcpyHostToDevice, (*out)->stream) != cudaSuccess) {
     ccmc_batch_destroy(*out);
@@ -1283,9 +1304,13 @@ int ccmc::batch_new(int cap, cudaStream_t stream, ccmc_batch **out) {
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaMalloc(&b->d_jobs, sizeof(ResJob) * count) != cudaSuccess ||
-      cudaMalloc(&b->d_multi, sizeof(MultiJob) * count) != cudaSuccess)
-    return fail(CCMC_E_NOMEM);
+  b->device = dev;
+  const size_t o_multi = (sizeof(ResJob) * count + 255) & ~(size_t)255;
+  const size_t o_ctls = o_multi + ((sizeof(MultiJob) * count + 255) & ~(size_t)255);
+  if (!dalloc(&b->d_slab, o_ctls + sizeof(int64_t *) * count, dev)) return fail(CCMC_E_NOMEM);
+  b->d_jobs = (ResJob *)b->d_slab;
+  b->d_multi = (MultiJob *)((char *)b->d_slab + o_multi);
+  b->d_ctls = (int64_t **)((char *)b->d_slab + o_ctls);
   if (!resident_ready()) return fail(CCMC_E_CUDA);
   if (cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess)
     return fail(CCMC_E_CUDA);
@@ -1304,10 +1329,8 @@ int ccmc_batch_destroy(ccmc_batch *b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   for (auto &e : b->graphs)
     if (e.exec) cudaGraphExecDestroy(e.exec);
-  cudaFree(b->d_jobs);
-  cudaFree(b->d_multi);
-  cudaFree(b->d_ctls);
   for (cudaStream_t x : b->side) cudaStreamSynchronize(x);
+  dfree(b->d_slab, b->device);
   for (cudaStream_t x : b->side) cudaStreamDestroy(x);
   for (cudaEvent_t e : b->side_ev) cudaEventDestroy(e);
   if (b->ev) cudaEventDestroy(b->ev);
@@ -1353,7 +1376,7 @@ int ccmc_batch_sync(ccmc_batch *b) {
   const int n = (int)b->lats.size();
   const size_t bytes = sizeof(int64_t) * n;
   Stage st(bytes);
-  if (!st || !b->d_ctls) {
+  if (!st) {
     for (ccmc_lattice *h : b->lats) {
       const int rc = check_status(h);
       if (rc) return rc;

@@ -42,6 +42,11 @@ namespace {
 using Clock = std::chrono::steady_clock;
 
 constexpr int kSlicesInFlight = 2;
+// The first slice after the GPU ran dry holds the one or two requests that woke the
+// scheduler, while the rest of a burst arrives: it is kept short, so that they join
+// soon (48 requests at once: 56 ms to the last result, the first 14 of them spent
+// on the first request alone).
+constexpr double kFirstSliceMs = 1.0;
 
 struct Pending {
   uint64_t ticket;
@@ -353,9 +358,10 @@ void ccmc_server::run() {
     std::vector<int64_t> sw(n);
     std::vector<double> beta(n), Delta(n), V(n), J(n);
     std::vector<int> every(n);
+    const double ms = slices.empty() ? std::min(slice_ms, kFirstSliceMs) : slice_ms;
     for (int i = 0; i < n; ++i) {
       Running &r = active[i];
-      int64_t q = (int64_t)(slice_ms * 1e3 / sweep_us(r.req));
+      int64_t q = (int64_t)(ms * 1e3 / sweep_us(r.req));
       if (q < 1) q = 1;
       if (r.req.obs_every > 1) q = std::max<int64_t>(r.req.obs_every, q / r.req.obs_every * r.req.obs_every);
       lats[i] = r.lat;
