@@ -123,27 +123,6 @@ __device__ __forceinline__ uint32_t fetch_window(const uint32_t *row, int W, int
   return v;
 }
 
-// XOR the first n sites of D into the class row at column `start` (periodic).
-// Only bits of the caller's own sites are nonzero, so concurrent XORs from other
-// threads into the same words commute.
-__device__ __forceinline__ void scatter_xor(uint32_t *row, int Cx, int start, int n, uint32_t D) {
-  if (D == 0u) return;
-  const int n1 = min(n, Cx - start);
-  const uint32_t d1 = (n1 < 16) ? (D & ((1u << (2 * n1)) - 1u)) : D;
-  const int wi = start >> 4, o = start & 15;
-  if (d1) {
-    atomicXor(row + wi, d1 << (2 * o));
-    if (o) {
-      const uint32_t h = d1 >> (32 - 2 * o);
-      if (h) atomicXor(row + wi + 1, h);
-    }
-  }
-  if (n1 < n) {
-    const uint32_t d2 = D >> (2 * n1);
-    if (d2) atomicXor(row, d2);
-  }
-}
-
 // ----------------------------------------------------------------------------
 // Colour schedule of global phase P (Sec. 3.2, a "map" of non-interacting
 // pairs): attempt t draws Philox(seed, (t, P_lo, P_hi, SCHED)); class a0 from

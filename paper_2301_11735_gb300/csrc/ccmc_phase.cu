@@ -37,142 +37,90 @@ namespace ccmc {
 // A tie (w == T) or a field v >= 65532 (about one pair in 4000, rejected by the
 // fast decision) is decided exactly, with the pair's SLOW random words.
 struct PhaseSmem {
-  uint2 trans[kMoveN];
-  uint16_t thrT[kThrT];
-  Sched sched;
+  alignas(16) uint16_t thrT[kThrT];
+  uint2 trans[kMoveN];  // directly after thrT, as in device memory
+  PhaseD u;
+  uint64_t P;
 };
-
-// Uniform per phase: where the ten windows of a word come from.  Column offsets
-// are in sites, normalised to [0, Cx).
-struct PhaseU {
-  const uint32_t *cA, *cAL, *cAR, *cAU, *cAD, *cB, *cBL, *cBR, *cBU, *cBD;
-  int offAL, offAR, offB, offBL, offBR;
-  int dyAU, dyAD, qy, dyBU, dyBD;
-};
-
-// How the direct path reads its windows: rows of any width (kRowGeneral) or rows
-// of whole words (kRowAligned).
-enum RowMode { kRowGeneral = 0, kRowAligned = 1 };
 
 __device__ __forceinline__ int wrap(int v, int n) { return v >= n ? v - n : (v < 0 ? v + n : v); }
 
-__device__ __forceinline__ PhaseU phase_uniform(const Geo &g, const Sched &sc) {
-  PhaseU u;
-  const int ax = sc.a0x, ay = sc.a0y;
-  const int bxx = ax + sc.rx, byy = ay + sc.ry;
-  const int cbx = bxx & 3, cby = byy & 3;
-  auto cls = [&](int cx, int cy) { return g.words + (int64_t)(cy * 4 + cx) * g.cstride; };
-  u.cA = cls(ax, ay);
-  u.cAL = cls((ax + 3) & 3, ay);
-  u.cAR = cls((ax + 1) & 3, ay);
-  u.cAU = cls(ax, (ay + 3) & 3);
-  u.cAD = cls(ax, (ay + 1) & 3);
-  u.cB = cls(cbx, cby);
-  u.cBL = cls((cbx + 3) & 3, cby);
-  u.cBR = cls((cbx + 1) & 3, cby);
-  u.cBU = cls(cbx, (cby + 3) & 3);
-  u.cBD = cls(cbx, (cby + 1) & 3);
-  const int qx = (bxx >> 2) % g.Cx;
-  u.offAL = ax == 0 ? g.Cx - 1 : 0;
-  u.offAR = ax == 3 ? (g.Cx == 1 ? 0 : 1) : 0;
-  u.offB = qx;
-  u.offBL = cbx == 0 ? wrap(qx - 1, g.Cx) : qx;
-  u.offBR = cbx == 3 ? wrap(qx + 1, g.Cx) : qx;
-  u.dyAU = ay == 0 ? -1 : 0;
-  u.dyAD = ay == 3 ? 1 : 0;
-  u.qy = (byy >> 2) % g.Cy;
-  u.dyBU = cby == 0 ? -1 : 0;
-  u.dyBD = cby == 3 ? 1 : 0;
-  return u;
-}
-
-// Window of n sites at column 16 w + off (mod Cx) of one class row.
-template <int kMode>
-__device__ __forceinline__ uint32_t window(const uint32_t *cls, const Geo &g, const PhaseU &u,
-                                           int row, int w, int off, int n) {
-  const uint32_t *r = cls + row * g.W;
-  if constexpr (kMode == kRowAligned) {  // the window straddles at most two words
-    const int wl = wrap(w + (off >> 4), g.W);
-    const int sh = 2 * (off & 15);
-    if (sh == 0) return r[wl];
-    const int wh = wl + 1 == g.W ? 0 : wl + 1;
-    return __funnelshift_r(r[wl], r[wh], sh);
-  } else {
-    return fetch_window(r, g.W, g.Cx, wrap(16 * w + off, g.Cx), n);
-  }
-}
-
-// n: the word's sites inside its row (16 unless the row ends in it).
-template <int kMode>
-__device__ __forceinline__ WordIn gather(const Geo &g, const PhaseU &u, int jr, int w, int n) {
-  WordIn in;
-  in.A = u.cA[jr * g.W + w];
-  const int jb = wrap(jr + u.qy, g.Cy);
-  in.B = window<kMode>(u.cB, g, u, jb, w, u.offB, n);
-  in.na = neighbour_planes(window<kMode>(u.cAL, g, u, jr, w, u.offAL, n),
-                         window<kMode>(u.cAR, g, u, jr, w, u.offAR, n),
-                         u.cAU[wrap(jr + u.dyAU, g.Cy) * g.W + w],
-                         u.cAD[wrap(jr + u.dyAD, g.Cy) * g.W + w]);
-  in.nb = neighbour_planes(window<kMode>(u.cBL, g, u, jb, w, u.offBL, n),
-                         window<kMode>(u.cBR, g, u, jb, w, u.offBR, n),
-                         window<kMode>(u.cBU, g, u, wrap(jb + u.dyBU, g.Cy), w, u.offB, n),
-                         window<kMode>(u.cBD, g, u, wrap(jb + u.dyBD, g.Cy), w, u.offB, n));
-  return in;
-}
-
-// Apply the moves (dA, dB) of word w (row jr of u's arrays, n sites): the a
-// word by a plain read-modify-write when this thread owns it (kOwnA), else by
-// atomic XOR; the b sites by atomic XOR (their words are shared with the
-// partners of neighbouring words).
-template <int kMode, bool kOwnA>
-__device__ __forceinline__ void apply_moves(const Geo &g, const PhaseU &u, int jr, int w, int n,
-                                            uint32_t dA, uint32_t dB) {
-  if constexpr (kMode == kRowGeneral) {
-    if (n < 16) {  // pairs past the end of the row do not exist
-      const uint32_t valid = (1u << (2 * n)) - 1u;
-      dA &= valid;
-      dB &= valid;
-    }
-  }
-  if (dA) {
-    uint32_t *pa = const_cast<uint32_t *>(u.cA) + jr * g.W + w;
-    if constexpr (kOwnA)
-      *pa ^= dA;
-    else
-      atomicXor(pa, dA);
-  }
-  if (dB) {
-    uint32_t *rb = const_cast<uint32_t *>(u.cB) + wrap(jr + u.qy, g.Cy) * g.W;
-    if constexpr (kMode == kRowAligned) {
-      const int wl = wrap(w + (u.offB >> 4), g.W);
-      const int sh = 2 * (u.offB & 15);
-      atomicXor(rb + wl, dB << sh);
-      if (sh) {
-        const uint32_t hi = dB >> (32 - sh);
-        if (hi) atomicXor(rb + (wl + 1 == g.W ? 0 : wl + 1), hi);
-      }
-    } else {
-      scatter_xor(rb, g.Cx, wrap((w << 4) + u.offB, g.Cx), n, dB);
-    }
-  }
-}
-
-// The direct path's view of a word: row j, word w of the classes in global memory.
-template <int kMode>
+// The direct path's view of a word: row j, word w of the classes in global memory
+// (class offsets in words), rows of whole words (kAl) or of any width.
+template <bool kAl>
 struct DirectView {
   const Geo &g;
-  const PhaseU &u;
+  const PhaseD &u;
   int j, w;
 
-  __device__ __forceinline__ int sites(int ww) const {
-    return kMode == kRowGeneral ? min(16, g.Cx - (ww << 4)) : 16;
+  // sites of the window from one class row
+  __device__ __forceinline__ uint32_t window(const uint32_t *row, const Win &x) const {
+    uint32_t v = __funnelshift_r(row[x.lo], row[x.hi], x.sh);
+    if constexpr (!kAl) {
+      if (x.n1 < 16)  // the row ends inside the window: go on at its start
+        v = (v & ((1u << (2 * x.n1)) - 1u)) | (row[0] << (2 * x.n1));
+    }
+    return v;
   }
-  __device__ __forceinline__ WordIn gather() const { return ccmc::gather<kMode>(g, u, j, w, sites(w)); }
+  __device__ __forceinline__ WordIn gather() const {
+    WordIn in;
+    const SideD &a = u.side[0], &b = u.side[1];
+    const int jb = turn(j + b.qy, g.Cy);
+    const uint32_t *rb = g.words + (int64_t)jb * g.W,
+                   *ry = g.words + (int64_t)turn(jb + b.ys, g.Cy) * g.W;
+    const Win win = window_at<kAl>(g, w, b.qx);
+    in.B = window(rb + b.c, win);
+    in.nb = neighbour_planes(window(rb + b.m, win), window(rb + b.r, win), window(ry + b.y, win),
+                             window(rb + b.x, window_at<kAl>(g, w, b.offX)));
+    const uint32_t *ra = g.words + (int64_t)j * g.W;
+    in.A = ra[a.c + w];
+    in.na = neighbour_planes(ra[a.m + w], ra[a.r + w],
+                             g.words[a.y + (int64_t)turn(j + a.ys, g.Cy) * g.W + w],
+                             window(ra + a.x, window_at<kAl>(g, w, a.offX)));
+    return in;
+  }
+  // a's word by a plain read-modify-write (kOwn: its thread's own) or by atomic XOR;
+  // the b sites by atomic XOR (their words are shared with the partners of
+  // neighbouring words)
+  template <bool kOwn>
+  __device__ __forceinline__ void change(int jj, int ww, uint32_t dA, uint32_t dB) const {
+    const SideD &a = u.side[0], &b = u.side[1];
+    if constexpr (!kAl) {
+      const int n = g.Cx - (ww << 4);
+      if (n < 16) {  // pairs past the end of the row do not exist
+        const uint32_t valid = (1u << (2 * n)) - 1u;
+        dA &= valid;
+        dB &= valid;
+      }
+    }
+    if (dA) {
+      uint32_t *pa = g.words + a.c + (int64_t)jj * g.W + ww;
+      if constexpr (kOwn)
+        *pa ^= dA;
+      else
+        atomicXor(pa, dA);
+    }
+    if (dB) {
+      uint32_t *row = g.words + b.c + (int64_t)turn(jj + b.qy, g.Cy) * g.W;
+      const Win x = window_at<kAl>(g, ww, b.qx);
+      uint32_t d1 = dB;
+      if constexpr (!kAl) {
+        if (x.n1 < 16) {
+          d1 = dB & ((1u << (2 * x.n1)) - 1u);
+          const uint32_t d2 = dB >> (2 * x.n1);
+          if (d2) atomicXor(row, d2);
+        }
+      }
+      const uint32_t lo = d1 << x.sh, hi = __funnelshift_l(d1, 0u, x.sh);
+      if (lo) atomicXor(row + x.lo, lo);
+      if (hi) atomicXor(row + x.hi, hi);
+    }
+  }
   __device__ __forceinline__ void apply(uint32_t dA, uint32_t dB) const {
-    apply_moves<kMode, true>(g, u, j, w, sites(w), dA, dB);
+    change<true>(j, w, dA, dB);
   }
   __device__ __forceinline__ void apply_other(int oj, int ow, uint32_t dA, uint32_t dB) const {
-    apply_moves<kMode, false>(g, u, oj, ow, sites(ow), dA, dB);
+    change<false>(oj, ow, dA, dB);
   }
 };
 
@@ -232,41 +180,48 @@ __device__ __forceinline__ void warp_word(const Geo &g, const View &view, const 
   }
 }
 
+// One phase on the direct path.  The prologue (tables, and for a launch after the
+// first of a chain the phase index and its schedule) runs before the kernel waits
+// for its predecessor, as in the tile kernels.  Small lattices take small CTAs: a
+// thread's chain is what they wait for, and it is shorter on an SM of its own.
 template <bool kAligned>
 __global__ void __launch_bounds__(256, 4) phase_kernel(Geo g, const uint16_t *thrT,
-                                                    const uint32_t *thr32, const uint32_t *trans,
-                                                    int64_t p_off) {
+                                                       const uint32_t *thr32, int64_t p_off,
+                                                       const __grid_constant__ RoundKeys rk) {
   __shared__ PhaseSmem sm;
-  // The tables come from host uploads that precede the whole launch chain, so
-  // they are loaded before waiting for the previous kernel of the stream (which
-  // lets this prologue overlap its tail under programmatic dependent launch).
-  for (int t = threadIdx.x; t < kThrT / 2; t += blockDim.x)
-    reinterpret_cast<uint32_t *>(sm.thrT)[t] = reinterpret_cast<const uint32_t *>(thrT)[t];
+  // The tables come from host uploads that precede the whole launch chain.
+  for (int t = threadIdx.x; t < (int)((2u * kThrT + 8u * kMoveN) / 16u); t += blockDim.x)
+    reinterpret_cast<uint4 *>(sm.thrT)[t] = reinterpret_cast<const uint4 *>(thrT)[t];
+  auto prologue = [&] {
+    if (threadIdx.x < 32) {
+      const uint64_t P = (uint64_t)(g.ctl[kCtlPhaseBase] + p_off);
+      const Sched s = draw_schedule(g, P);
+      if (threadIdx.x == 0) {
+        sm.u = phase_desc(g, s, (uint32_t)g.cstride);
+        sm.P = P;
+      }
+    }
+  };
+  const bool pre = p_off > 0;  // the counter's base is two launches old (see tile_phase)
+  if (pre) prologue();
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // The next kernel may launch now: with one resident wave its blocks only take
   // the slots of blocks that finish, and it waits for this whole grid before
   // touching the lattice.
   asm volatile("griddepcontrol.launch_dependents;");
-  const uint64_t P = (uint64_t)(g.ctl[kCtlPhaseBase] + p_off);
-  if (threadIdx.x < 32) {
-    const Sched s = draw_schedule(g, P);
-    if (threadIdx.x == 0) sm.sched = s;
-  }
+  if (!pre) prologue();
   __syncthreads();
-  const Sched sc = sm.sched;
-  for (int t = threadIdx.x; t < kMoveN; t += blockDim.x)
-    sm.trans[t] = make_uint2(trans[2 * t], trans[2 * t + 1]);
-  __syncthreads();
-  const PhaseU u = phase_uniform(g, sc);
-  const uint32_t near128 = sc.near ? 128u : 0u;
+  const PhaseD &u = sm.u;
+  const uint64_t P = sm.P;
+  const uint32_t near128 = u.near128;
   const int nw = g.Cy * g.W;
   const int stride = gridDim.x * blockDim.x;
   for (int base = blockIdx.x * blockDim.x; base < nw; base += stride) {
     const int wid = base + threadIdx.x;
     const bool act = wid < nw;
     const int j = act ? wid / g.W : 0, w = act ? wid - j * g.W : 0;
-    warp_word(g, DirectView<kAligned ? kRowAligned : kRowGeneral>{g, u, j, w}, sm.trans, sm.thrT,
-              thr32, j, w, P, near128, SeedKeys{g.k0, g.k1}, act);
+    warp_word(g, DirectView<kAligned>{g, u, j, w}, sm.trans, sm.thrT, thr32, j, w, P, near128,
+              TableKeys{&rk}, act);
   }
 }
 
@@ -748,30 +703,26 @@ __global__ void __launch_bounds__(256, 4) phase_multi_kernel(const MultiJob *__r
   __syncthreads();
   const MultiJob &J = jobs[s_job];
   const Geo g = J.g;
-  for (int t = threadIdx.x; t < kThrT / 2; t += blockDim.x)
-    reinterpret_cast<uint32_t *>(sm.thrT)[t] = reinterpret_cast<const uint32_t *>(J.thrT)[t];
+  for (int t = threadIdx.x; t < (int)((2u * kThrT + 8u * kMoveN) / 16u); t += blockDim.x)
+    reinterpret_cast<uint4 *>(sm.thrT)[t] = reinterpret_cast<const uint4 *>(J.thrT)[t];
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
   const uint64_t P = (uint64_t)(g.ctl[kCtlPhaseBase] + p_off);
   if (threadIdx.x < 32) {
     const Sched sc = draw_schedule(g, P);
-    if (threadIdx.x == 0) sm.sched = sc;
+    if (threadIdx.x == 0) sm.u = phase_desc(g, sc, (uint32_t)g.cstride);
   }
   __syncthreads();
-  const Sched sc = sm.sched;
-  for (int t = threadIdx.x; t < kMoveN; t += blockDim.x)
-    sm.trans[t] = make_uint2(J.trans[2 * t], J.trans[2 * t + 1]);
-  __syncthreads();
-  const PhaseU u = phase_uniform(g, sc);
-  const uint32_t near128 = sc.near ? 128u : 0u;
+  const PhaseD &u = sm.u;
+  const uint32_t near128 = u.near128;
   const int nw = g.Cy * g.W;
   const int stride = J.cta_count * blockDim.x;
   for (int base = ((int)blockIdx.x - J.cta_begin) * blockDim.x; base < nw; base += stride) {
     const int wid = base + threadIdx.x;
     const bool act = wid < nw;
     const int j = act ? wid / g.W : 0, w = act ? wid - j * g.W : 0;
-    warp_word(g, DirectView<kAligned ? kRowAligned : kRowGeneral>{g, u, j, w}, sm.trans, sm.thrT,
-              J.thr32, j, w, P, near128, SeedKeys{g.k0, g.k1}, act);
+    warp_word(g, DirectView<kAligned>{g, u, j, w}, sm.trans, sm.thrT, J.thr32, j, w, P, near128,
+              SeedKeys{g.k0, g.k1}, act);
   }
 }
 
@@ -837,6 +788,10 @@ int tile_resident_grid_small() {
   return per_sm * sms;
 }
 
+// a-words up to which the direct path takes CTAs of 64 and 128 threads: two and
+// four warps on each of the 152 SMs.
+constexpr int64_t kDirectSmall64 = 152 * 64, kDirectSmall128 = 152 * 128;
+
 cudaError_t launch_phase(const Geo &g, const DevTables &t, int64_t p_off, const LaunchCfg &cfg,
                          cudaStream_t s) {
   const int64_t nw = (int64_t)g.Cy * g.W;
@@ -857,12 +812,10 @@ cudaError_t launch_phase(const Geo &g, const DevTables &t, int64_t p_off, const 
                            s, g, (const uint16_t *)t.thrT, t.thr32, p_off,
                            round_keys(g.k0, g.k1));
   }
-  const int grid = grid_for(nw, 256, cfg.phase_grid_cap);
-  const uint16_t *thrT = t.thrT;
-  const uint32_t *thr32 = t.thr32, *tr = t.trans;
-  if ((g.Cx & 15) == 0)
-    return launch_pdl(phase_kernel<true>, grid, 256, s, g, thrT, thr32, tr, p_off);
-  return launch_pdl(phase_kernel<false>, grid, 256, s, g, thrT, thr32, tr, p_off);
+  const int block = nw <= kDirectSmall64 ? 64 : nw <= kDirectSmall128 ? 128 : 256;
+  const int grid = grid_for(nw, block, cfg.phase_grid_cap);
+  return launch_pdl((g.Cx & 15) == 0 ? phase_kernel<true> : phase_kernel<false>, grid, block, s, g,
+                    (const uint16_t *)t.thrT, t.thr32, p_off, round_keys(g.k0, g.k1));
 }
 
 cudaError_t launch_phase_tile_multi(const MultiJob *d_jobs, int njobs, int grid, int64_t p_off,

@@ -37,24 +37,6 @@ constexpr uint32_t kFastBytes = 2u * kThrT + 8u * kMoveN;
 constexpr uint32_t kTableBytes = kFastBytes + 4u * kDevPad;
 static_assert(kFastBytes % 16 == 0 && kTableBytes % 16 == 0, "copied 16 bytes at a time");
 
-// One phase's uniforms of one side (a or b): classes as byte offsets into a CTA's
-// words, column offsets in sites, row offsets.  Of a site's two column neighbours
-// at most one lies in another column block, and of its two row neighbours at most
-// one in another row: the neighbour sums do not care which is which, so a side
-// has its own class c, one column neighbour read at the side's own column (m) and
-// one xs = -1, 0 or 1 sites further (x), one row neighbour in its own row (r)
-// and one 0, 1 or Cy - 1 rows further (y, ys).  The side's sites lie qx columns and
-// qy rows from the a sites (0, 0 for a itself); offX = qx + xs in [0, Cx).
-struct alignas(16) SideD {
-  uint32_t c, m, x, r, y;
-  int qx, offX, qy, ys, xs;
-  int pad[2];
-};
-struct alignas(16) PhaseD {
-  SideD side[2];
-  uint32_t near128;
-};
-
 __device__ __forceinline__ uint32_t smem_addr(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -122,39 +104,6 @@ __device__ __forceinline__ void bar_wait() {
   }
 }
 
-// v in [0, 2 n) modulo n: an unsigned minimum instead of a comparison and a choice.
-__device__ __forceinline__ int turn(int v, int n) {
-  return (int)min((uint32_t)v, (uint32_t)(v - n));
-}
-
-// The phase's uniforms from its schedule, for classes of cls_bytes bytes.
-__device__ __forceinline__ PhaseD phase_desc(const Geo &g, const Sched &sc, uint32_t cls_bytes) {
-  PhaseD u;
-  auto cls = [&](int cx, int cy) { return (uint32_t)((cy & 3) * 4 + (cx & 3)) * cls_bytes; };
-  // -1 when the left (upper) neighbours lie in the block (row) before, +1 when the
-  // right (lower) ones lie in the next
-  auto shift = [](int c) { return c == 0 ? -1 : c == 3 ? 1 : 0; };
-  auto side = [&](SideD &d, int x, int y) {
-    const int cx = x & 3, cy = y & 3;
-    const int dx = cx == 3 ? 1 : -1, dy = cy == 3 ? 1 : -1;  // the further ones
-    d.c = cls(cx, cy);
-    d.m = cls(cx - dx, cy);
-    d.x = cls(cx + dx, cy);
-    d.r = cls(cx, cy - dy);
-    d.y = cls(cx, cy + dy);
-    d.qx = turn(x >> 2, g.Cx);  // an offset is below the size: at most one turn
-    d.qy = turn(y >> 2, g.Cy);
-    d.xs = shift(cx);
-    const int ys = shift(cy);
-    d.ys = ys < 0 ? g.Cy - 1 : ys < g.Cy ? ys : 0;
-    d.offX = turn(d.qx + (d.xs < 0 ? g.Cx - 1 : d.xs), g.Cx);
-  };
-  side(u.side[0], sc.a0x, sc.a0y);
-  side(u.side[1], sc.a0x + sc.rx, sc.a0y + sc.ry);
-  u.near128 = sc.near ? 128u : 0u;
-  return u;
-}
-
 // The uniforms of phases P .. P + 7 by one warp: four lanes a phase, each trying
 // attempts lane mod 4, + 4, ... (draw_schedule's: the first allowed one of at most
 // 64 wins, then the fixed offset); one round settles a phase with probability 0.99.
@@ -185,35 +134,10 @@ __device__ __forceinline__ void describe_sweep(const Geo &g, uint64_t P, uint32_
     s_d[p & 15u] = phase_desc(g, Sched{0, 0, 2, 2, is_near(g, 2, 2)}, cls_bytes);
 }
 
-// The words and shift of the window of 16 sites at column 16 w + off (mod Cx) of
-// a row; n1: sites before the row's end (rows of whole words: never cut).
-struct Win {
-  uint32_t lo, hi;  // byte offsets of its two words
-  int sh, n1;
-};
-
-template <bool kAl>
-__device__ __forceinline__ Win window_at(const Geo &g, int w, int off) {
-  Win x;
-  int wl;
-  if constexpr (kAl) {
-    wl = turn(w + (off >> 4), g.W);
-    x.sh = 2 * (off & 15);
-    x.n1 = 16;
-  } else {
-    const int s = turn(16 * w + off, g.Cx);
-    wl = s >> 4;
-    x.sh = 2 * (s & 15);
-    x.n1 = g.Cx - s;
-  }
-  x.lo = 4u * (uint32_t)wl;
-  x.hi = 4u * (uint32_t)turn(wl + 1, g.W);
-  return x;
-}
-
 template <bool kCl, bool kAl>
 __device__ __forceinline__ uint32_t read_window(uint32_t row, const Win &x) {
-  uint32_t v = __funnelshift_r(ld_word<kCl>(row + x.lo), ld_word<kCl>(row + x.hi), x.sh);
+  uint32_t v = __funnelshift_r(ld_word<kCl>(row + 4u * (uint32_t)x.lo),
+                               ld_word<kCl>(row + 4u * (uint32_t)x.hi), x.sh);
   if constexpr (!kAl) {
     if (x.n1 < 16)  // the row ends inside the window: go on at its start
       v = (v & ((1u << (2 * x.n1)) - 1u)) | (ld_word<kCl>(row) << (2 * x.n1));
@@ -231,8 +155,8 @@ __device__ __forceinline__ void xor_window(uint32_t row, const Win &x, uint32_t 
       xor_word<kCl>(row, D >> (2 * x.n1));
     }
   }
-  xor_word<kCl>(row + x.lo, d1 << x.sh);
-  xor_word<kCl>(row + x.hi, __funnelshift_l(d1, 0u, x.sh));  // d1 >> (32 - sh), 0 for sh = 0
+  xor_word<kCl>(row + 4u * (uint32_t)x.lo, d1 << x.sh);
+  xor_word<kCl>(row + 4u * (uint32_t)x.hi, __funnelshift_l(d1, 0u, x.sh));  // d1 >> (32 - sh), 0 for sh = 0
 }
 
 // Where a CTA's rows lie.
@@ -323,16 +247,16 @@ __device__ __forceinline__ SideIn gather_remote(const Geo &g, const SideD &d, co
   const int jb = side_row(g, pl, d, l);
   const uint32_t row = row_addr<true>(pl, jb), ry = row_addr<true>(pl, turn(jb + d.ys, g.Cy));
   const Win win = window_at<kAl>(g, w, d.qx), wx = window_at<kAl>(g, w, d.offX);
-  const bool near = __shfl_sync(0xFFFFFFFFu, row + win.lo, src) == row + win.hi;
-  const bool nearx = __shfl_sync(0xFFFFFFFFu, row + wx.lo, src) == row + wx.hi;
+  const bool near = __shfl_sync(0xFFFFFFFFu, row + 4u * (uint32_t)win.lo, src) == row + 4u * (uint32_t)win.hi;
+  const bool nearx = __shfl_sync(0xFFFFFFFFu, row + 4u * (uint32_t)wx.lo, src) == row + 4u * (uint32_t)wx.hi;
   const uint32_t at[5] = {row + d.c, row + d.m, row + d.r, ry + d.y, row + d.x};
   uint32_t lo[5], v[5];
 #pragma unroll
-  for (int k = 0; k < 5; ++k) lo[k] = ld_word<true>(at[k] + (k < 4 ? win.lo : wx.lo));
+  for (int k = 0; k < 5; ++k) lo[k] = ld_word<true>(at[k] + 4u * (uint32_t)(k < 4 ? win.lo : wx.lo));
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const Win &x = k < 4 ? win : wx;
-    const uint32_t hi = ld_remote_if(!(k < 4 ? near : nearx), at[k] + x.hi,
+    const uint32_t hi = ld_remote_if(!(k < 4 ? near : nearx), at[k] + 4u * (uint32_t)x.hi,
                                      __shfl_sync(0xFFFFFFFFu, lo[k], src));
     v[k] = __funnelshift_r(lo[k], hi, x.sh);
     if constexpr (!kAl) {

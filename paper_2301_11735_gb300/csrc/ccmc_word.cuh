@@ -1,7 +1,8 @@
 // ccmc_word.cuh -- the per-word core of a colour phase, shared by the phase
 // kernels and the resident kernel: the 16 pairs of one a-class word decided from
-// the word's inputs (its a word, b window and both sides' neighbour counts).
-// How those inputs are read and where the moves go is each kernel's own.
+// the word's inputs (its a word, b window and both sides' neighbour counts), and the
+// phase's uniforms from which a kernel reads those inputs.  How it reads them and
+// where the moves go is each kernel's own.
 #pragma once
 
 #include <cstdint>
@@ -10,6 +11,81 @@
 #include "ccmc_internal.h"
 
 namespace ccmc {
+
+// One phase's uniforms of one side (a or b): classes as offsets of a unit of the
+// kernel's, column offsets in sites, row offsets.  Of a site's two column neighbours
+// at most one lies in another column block, and of its two row neighbours at most
+// one in another row: the neighbour sums do not care which is which, so a side
+// has its own class c, one column neighbour read at the side's own column (m) and
+// one xs = -1, 0 or 1 sites further (x), one row neighbour in its own row (r)
+// and one 0, 1 or Cy - 1 rows further (y, ys).  The side's sites lie qx columns and
+// qy rows from the a sites (0, 0 for a itself); offX = qx + xs in [0, Cx).
+struct alignas(16) SideD {
+  uint32_t c, m, x, r, y;
+  int qx, offX, qy, ys, xs;
+  int pad[2];
+};
+struct alignas(16) PhaseD {
+  SideD side[2];
+  uint32_t near128;
+};
+
+// v in [0, 2 n) modulo n: an unsigned minimum instead of a comparison and a choice.
+__device__ __forceinline__ int turn(int v, int n) {
+  return (int)min((uint32_t)v, (uint32_t)(v - n));
+}
+
+// The phase's uniforms from its schedule, class c at offset c * unit.
+__device__ __forceinline__ PhaseD phase_desc(const Geo &g, const Sched &sc, uint32_t unit) {
+  PhaseD u;
+  auto cls = [&](int cx, int cy) { return (uint32_t)((cy & 3) * 4 + (cx & 3)) * unit; };
+  // -1 when the left (upper) neighbours lie in the block (row) before, +1 when the
+  // right (lower) ones lie in the next
+  auto shift = [](int c) { return c == 0 ? -1 : c == 3 ? 1 : 0; };
+  auto side = [&](SideD &d, int x, int y) {
+    const int cx = x & 3, cy = y & 3;
+    const int dx = cx == 3 ? 1 : -1, dy = cy == 3 ? 1 : -1;  // the further ones
+    d.c = cls(cx, cy);
+    d.m = cls(cx - dx, cy);
+    d.x = cls(cx + dx, cy);
+    d.r = cls(cx, cy - dy);
+    d.y = cls(cx, cy + dy);
+    d.qx = turn(x >> 2, g.Cx);  // an offset is below the size: at most one turn
+    d.qy = turn(y >> 2, g.Cy);
+    d.xs = shift(cx);
+    const int ys = shift(cy);
+    d.ys = ys < 0 ? g.Cy - 1 : ys < g.Cy ? ys : 0;
+    d.offX = turn(d.qx + (d.xs < 0 ? g.Cx - 1 : d.xs), g.Cx);
+  };
+  side(u.side[0], sc.a0x, sc.a0y);
+  side(u.side[1], sc.a0x + sc.rx, sc.a0y + sc.ry);
+  u.near128 = sc.near ? 128u : 0u;
+  return u;
+}
+
+// The words and shift of the window of 16 sites at column 16 w + off (mod Cx) of
+// a row; n1: sites before the row's end (rows of whole words: never cut).
+struct Win {
+  int lo, hi;  // its two words
+  int sh, n1;
+};
+
+template <bool kAl>
+__device__ __forceinline__ Win window_at(const Geo &g, int w, int off) {
+  Win x;
+  if constexpr (kAl) {
+    x.lo = turn(w + (off >> 4), g.W);
+    x.sh = 2 * (off & 15);
+    x.n1 = 16;
+  } else {
+    const int s = turn(16 * w + off, g.Cx);
+    x.lo = s >> 4;
+    x.sh = 2 * (s & 15);
+    x.n1 = g.Cx - s;
+  }
+  x.hi = turn(x.lo + 1, g.W);
+  return x;
+}
 
 // Move entry of choice class r (v mod 12) and r264 = 264 r + 128 near: entry
 // (2 r + near) 16 + (pc XOR r) of the move table, at byte offset
