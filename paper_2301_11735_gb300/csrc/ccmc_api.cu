@@ -40,12 +40,13 @@ struct GraphEntry {
 
 constexpr int kChunk = 16;
 // Lock-step groups: at least kLockstepMin lattices, each with fewer than
-// kLockstepMaxWords a-words per phase.  Measured on GB300: 16 lattices of
-// 1024^2 run faster in lock step than on their own streams; 8 of 2048^2 or
-// 4 of 4096^2 run faster on their own streams, whose phases fill each other's
-// tails.
-constexpr int kLockstepMin = 8;
-constexpr int64_t kLockstepMaxWords = 16384;
+// kLockstepMaxWords a-words per phase.  Measured on GB300, us a phase of all, lock
+// step against their own streams, whose phases fill each other's tails: 8 of 1536^2
+// (9216 words) 4.7 against 4.0, 16 6.8 against 7.4, 32 11.4 against 13.5; 16 of 1200^2
+// 6.5 against 6.9, 40 11.7 against 16.5; 16 of 1980^2 (15345 words) 10.9 against 9.5,
+// 64 33.1 against 32.0.
+constexpr int kLockstepMin = 12;
+constexpr int64_t kLockstepMaxWords = 12288;
 
 // Lattice memory comes from a library-owned pool per device, kept cached:
 // creating and destroying lattices never synchronises the device, which a server
@@ -420,20 +421,7 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
   const uint64_t N = (uint64_t)Lx * (uint64_t)Ly;
   g.rej = (0 - N) % N;
   h->cfg.phase_grid_cap = phase_resident_grid((g.Cx & 15) == 0);
-  if (tile_path_ok(g) && !std::getenv("CCMC_NO_TILE")) {
-    h->cfg.tile_grid = tile_resident_grid();
-    h->cfg.tile_grid_small = tile_resident_grid_small();
-    // CCMC_TILE_GRID=n (tests): the pipelined tile kernel with at most n CTAs,
-    // so that small lattices take several tiles per CTA
-    if (const char *e = std::getenv("CCMC_TILE_GRID")) {
-      const int n = std::atoi(e);
-      if (n > 0 && h->cfg.tile_grid > 0) {
-        h->cfg.tile_grid = n < h->cfg.tile_grid ? n : h->cfg.tile_grid;
-        h->cfg.tile_grid_small = 0;
-      }
-    }
-  }
-  // the variables that select a phase kernel keep the lattice on that kernel
+  // any of these variables (tests) keeps the lattice on the phase kernels
   h->resident = resident_default(g) && !std::getenv("CCMC_NO_TILE") &&
                 !std::getenv("CCMC_TILE_GRID") && !std::getenv("CCMC_NO_RESIDENT") && resident_ready();
   while (((int64_t)1 << (2 * h->h)) < (int64_t)N) ++h->h;
@@ -452,9 +440,9 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
   }
   const int np = recount_grid(g);
   const int dev = h->device;
-  // the threshold levels and the move table one after another (a multiple of
-  // 16 bytes from a 256-byte aligned base): the tile kernels copy them into
-  // shared memory with one bulk copy; thr32 after them
+  // the threshold levels, the move table and the full thresholds one after another
+  // (multiples of 16 bytes from a 256-byte aligned base): the kernels copy the first
+  // two, or all three, into shared memory as one block
   size_t at = 0;
   auto part = [&](size_t bytes) {
     const size_t o = at;
@@ -1047,15 +1035,12 @@ struct MultiGroup {
   int64_t off;  // first slot in d_multi
   int grid;
   bool aligned;
-  bool tiled;  // every member takes the tile-staged phase
 };
 
 int enqueue_multi_chunk(ccmc_batch *b, const MultiGroup &G, int sweeps, int obs_every) {
   for (int s = 0; s < sweeps; ++s) {
     for (int p = 0; p < 8; ++p)
-      CK(G.tiled ? launch_phase_tile_multi(b->d_multi + G.off, (int)G.m.size(), G.grid,
-                                           8LL * s + p, b->stream)
-                 : launch_phase_multi(b->d_multi + G.off, (int)G.m.size(), G.grid, G.aligned,
+      CK(launch_phase_multi(b->d_multi + G.off, (int)G.m.size(), G.grid, G.aligned,
                                       8LL * s + p, b->stream));
     if (obs_every > 0 && (s + 1) % obs_every == 0)
       for (ccmc_lattice *h : G.m)
@@ -1092,38 +1077,22 @@ int run_multi_graph(ccmc_batch *b, const MultiGroup &G, int sweeps, int obs_ever
 // Sweep a lock-step group (same position, sweeps, observable interval and
 // alignment) with one phase launch per phase for all of them.
 int run_multi(ccmc_batch *b, MultiGroup &G, int64_t nsweeps, int obs_every) {
-  int64_t words = 0, tiles = 0;
+  int64_t words = 0;
   for (ccmc_lattice *h : G.m) words += (int64_t)h->g.Cy * h->g.W;
-  for (ccmc_lattice *h : G.m) tiles += G.tiled ? tile_count(h->g) : 0;
-  const int wave = G.tiled ? G.m[0]->cfg.tile_grid : phase_resident_grid(G.aligned);
-  // tile path: the same number of tiles per CTA for every member, as few as
-  // one wave of CTAs allows
-  int64_t per_cta = G.tiled ? (tiles + wave - 1) / wave : 1;
-  if (G.tiled)
-    for (;;) {
-      int64_t ctas = 0;
-      for (ccmc_lattice *h : G.m) ctas += (tile_count(h->g) + per_cta - 1) / per_cta;
-      if (ctas <= wave) break;
-      ++per_cta;
-    }
+  const int wave = phase_resident_grid(G.aligned);
   std::vector<MultiJob> jobs;
   int begin = 0;
   for (ccmc_lattice *h : G.m) {
     const int64_t w = (int64_t)h->g.Cy * h->g.W;
-    int share;
-    if (G.tiled) {
-      share = (int)((tile_count(h->g) + per_cta - 1) / per_cta);
-    } else {
-      share = (int)((double)wave * (double)w / (double)words);
-      const int64_t need = (w + 255) / 256;  // more CTAs than a word each would idle
-      if (share > need) share = (int)need;
-      if (share < 1) share = 1;
-    }
+    int share = (int)((double)wave * (double)w / (double)words);
+    const int64_t need = (w + 255) / 256;  // more CTAs than a word each would idle
+    if (share > need) share = (int)need;
+    if (share < 1) share = 1;
     MultiJob j{};
     j.g = h->g;
     j.thrT = h->t.thrT;
     j.thr32 = h->t.thr32;
-    j.trans = h->t.trans;
+    j.mw = row_magic(h->g);
     j.cta_begin = begin;
     j.cta_count = share;
     begin += share;
@@ -1137,9 +1106,7 @@ int run_multi(ccmc_batch *b, MultiGroup &G, int64_t nsweeps, int obs_every) {
       [&](int g, int obs) { return run_multi_graph(b, G, g, obs); },
       [&](bool obs_due) {
         for (int p = 0; p < 8; ++p)
-          CK(G.tiled ? launch_phase_tile_multi(b->d_multi + G.off, (int)G.m.size(), G.grid, p,
-                                               b->stream)
-                     : launch_phase_multi(b->d_multi + G.off, (int)G.m.size(), G.grid, G.aligned,
+          CK(launch_phase_multi(b->d_multi + G.off, (int)G.m.size(), G.grid, G.aligned,
                                           p, b->stream));
         if (obs_due)
           for (ccmc_lattice *h : G.m)
@@ -1213,14 +1180,14 @@ int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int6
   for (int i = 0; i < n; ++i) {
     ccmc_lattice *h = lats[i];
     if (used[i] || nsweeps[i] == 0 || batch_resident(b, h)) continue;
-    MultiGroup G{{h}, off, 0, (h->g.Cx & 15) == 0, h->cfg.tile_grid > 0};
+    MultiGroup G{{h}, off, 0, (h->g.Cx & 15) == 0};
     used[i] = 1;
     auto small = [](const ccmc_lattice *x) { return (int64_t)x->g.Cy * x->g.W < kLockstepMaxWords; };
     for (int k = i + 1; k < n && lockstep && small(h); ++k) {
       ccmc_lattice *o = lats[k];
       if (used[k] || nsweeps[k] != nsweeps[i] || obs_every[k] != obs_every[i] ||
           o->phases_done != h->phases_done || ((o->g.Cx & 15) == 0) != G.aligned ||
-          (o->cfg.tile_grid > 0) != G.tiled || !small(o) || batch_resident(b, o))
+          !small(o) || batch_resident(b, o))
         continue;
       G.m.push_back(o);
       used[k] = 1;

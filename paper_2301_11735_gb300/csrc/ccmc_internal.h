@@ -31,8 +31,6 @@ enum CtlSlot : int {
   kCtlTicket = 2,     // arrival counter of the recount's last-block reduction
   kCtlStatus = 3,     // device-side error flag
   kCtlLatest = 4,     // 8 words: the last recount record
-  kCtlTileClaim = 12,  // 2 words: tile claims of the tile-staged phases of even
-                       // and odd P (phase P's low 32 bits above the claim count)
   kCtlWords = 16
 };
 
@@ -89,8 +87,6 @@ constexpr int kThrT = (kDevN + 7) / 8 * 8;  // 16-bit levels, padded to 16 bytes
 
 struct LaunchCfg {
   int phase_grid_cap = 152 * 3;  // one resident wave of phase_kernel (set at create)
-  int tile_grid = 0;             // > 0: tile-staged phases, this many CTAs at most
-  int tile_grid_small = 0;       // one wave of the compact tile kernel (16-bit tops)
 };
 
 // One lattice of a resident launch (ccmc_resident.cu): held in the shared memory
@@ -132,7 +128,7 @@ struct MultiJob {
   Geo g;
   const uint16_t *thrT;
   const uint32_t *thr32;
-  const uint32_t *trans;
+  uint32_t mw;  // row_magic
   int cta_begin, cta_count;
 };
 
@@ -155,20 +151,11 @@ cudaError_t launch_phase(const Geo &g, const DevTables &t, int64_t p_off, const 
 int recount_grid(const Geo &g);
 // CTAs of phase_kernel that fit the device at once (one wave).
 int phase_resident_grid(bool aligned);
-// Whether a lattice can take the tile-staged phase kernel, and its one wave.
-bool tile_path_ok(const Geo &g);
-int tile_resident_grid();
-// One wave of the compact tile kernel (more CTAs per SM), 0 if unavailable.
-int tile_resident_grid_small();
 // One colour phase of every lattice in d_jobs (all aligned or all not).
 cudaError_t launch_phase_multi(const MultiJob *d_jobs, int njobs, int grid, bool aligned,
                                int64_t p_off, cudaStream_t s);
-// One tile-staged phase of every lattice in d_jobs (all take the tile path;
-// their tables one staged block each, as launch_phase requires).
-cudaError_t launch_phase_tile_multi(const MultiJob *d_jobs, int njobs, int grid, int64_t p_off,
-                                    cudaStream_t s);
-// Tiles of one tile-staged phase of lattice g.
-int tile_count(const Geo &g);
+// What the lock-step kernel's MultiJob::mw is for a lattice.
+uint32_t row_magic(const Geo &g);
 cudaError_t launch_recount(const Geo &g, int64_t *partials, int64_t *ring, int64_t ring_cap,
                            int64_t *hist, int nbins, int64_t sweep_off, cudaStream_t s);
 cudaError_t launch_advance(int64_t *ctl, int64_t phases, cudaStream_t s);

@@ -110,3 +110,26 @@ def test_batches_of_every_shape_match_single_sweeps(cc, cfg):
         assert np.array_equal(lat.obs_series(), one.obs_series()), (cfg, shapes[i])
         lat.close()
         one.close()
+
+
+@pytest.mark.parametrize("shapes", [[(516, 260)] * 7 + [(260, 1024)] * 6, [(512, 256)] * 13])
+def test_lock_step_groups_match_single_sweeps(cc, shapes):
+    """Enough lattices beyond the resident limit to advance with one launch a phase."""
+    lats, ref = [], []
+    for i, (Lx, Ly) in enumerate(shapes):
+        for group in (lats, ref):
+            lat = cc.Lattice(Lx, Ly, obs_capacity=16)
+            lat.init_constrained(80 + i, 0.1, 0.3)
+            group.append(lat)
+    T = [0.3 + 0.2 * i for i in range(len(shapes))]
+    with cc.Batch(lats) as b:
+        b.config(256, 1024, 2)
+        for _ in range(2):  # the second call replays the captured group graph
+            b.sweep(18, [1 / t for t in T], 0.1, 0.5, 1.0, obs_every=2)
+        b.sync()
+    for lat, one, t in zip(lats, ref, T):
+        one.sweep(36, 1 / t, 0.1, 0.5, 1.0, obs_every=2)
+        assert np.array_equal(lat.get_state(), one.get_state())
+        assert np.array_equal(lat.obs_series(), one.obs_series())
+        lat.close()
+        one.close()
