@@ -417,32 +417,8 @@ __device__ __forceinline__ void quad_word(const Geo &g, const PhaseD &u, const P
     df[q] = fs[q] - (level_at(thrT, t[q] & 0xFFFFu) << 16);  // negative: accept; < 2^16: a tie
   }
   const uint32_t mn = __vimin3_u32(__vimin3_u32(df[0], df[1], df[2]), df[3], df[3]);
-  uint32_t acc = prmt(prmt(df[0], df[1], 0x00FBu), prmt(df[2], df[3], 0x00FBu), 0x5410u) &
-                 prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
-  if ((mn < 0x10000u || (f.x & 0x8000u)) && valid) {  // rare pairs: decided exactly (see exact_move)
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t fq = q == 0 ? fs[0] : q == 1 ? fs[1] : q == 2 ? fs[2] : fs[3];
-      const uint32_t dq = q == 0 ? df[0] : q == 1 ? df[1] : q == 2 ? df[2] : df[3];
-      uint32_t tq = q == 0 ? t[0] : q == 1 ? t[1] : q == 2 ? t[2] : t[3];
-      const uint32_t wq = fq >> 16;
-      const bool big = wq == 5461u;
-      if (dq >= 0x10000u && !big) continue;
-      const uint32_t slow0 =
-          (uint32_t)((uint64_t)(pl.row0 + p.l) * g.Cx + (uint32_t)(p.w << 4)) + (uint32_t)sub + 4u * q;
-      const U4 sl = philox_keys(slow0, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, rk);
-      if (big) {
-        if (sl.y >= 4294967292u) continue;  // keep the current configuration
-        const uint32_t eq = q == 0 ? ev[0] : q == 1 ? ev[1] : q == 2 ? ev[2] : ev[3];
-        const uint2 e = move_entry(moves, entry_offset(pc, q, (sl.y % 12u) * 264u));
-        tq = (uint32_t)__dp4a((int)e.y, (int)((eq >> c4) & kEnvMask), (int)e.x);
-      }
-      const uint32_t thr = thr32[(tq & 0xFFFFu) >> 1];
-      if (thr == 0xFFFFFFFFu ||
-          (big ? sl.x < thr : ((uint64_t)wq << 32) + sl.x < 5461ull * thr))
-        acc |= (tq >> 24) << (8 * q);  // the fast path left this lane's byte zero
-    }
-  }
+  const uint32_t acc = prmt(prmt(df[0], df[1], 0x00FBu), prmt(df[2], df[3], 0x00FBu), 0x5410u) &
+                       prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
   uint32_t dB = (acc & 0x03030303u) << (2 * sub);
   uint32_t dA = ((acc >> 2) & 0x03030303u) << (2 * sub);
   // the word's moves together; one lane a side writes its sites
@@ -451,6 +427,25 @@ __device__ __forceinline__ void quad_word(const Geo &g, const PhaseD &u, const P
   mine |= __shfl_xor_sync(0xFFFFFFFFu, mine, 1);
   if (sub & 1) mine = 0u;
   xor_window<kCl, kAl>(row + d.c, win, mine & valid);
+  // The rare pairs, which the fast path left as they were, decided exactly behind the
+  // word's other moves: no lane waits at this branch before the exchange (256^2: 7.8 us
+  // a sweep with it there, 7.2 here; 16^2: 4.06, 3.93).
+  if ((mn < 0x10000u || (f.x & 0x8000u)) && valid) {
+    uint32_t m = 0u, wq[4], e4[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      wq[q] = fs[q] >> 16;
+      e4[q] = (ev[q] >> c4) & kEnvMask;
+      if (df[q] < 0x10000u || wq[q] == 5461u) m |= 1u << q;
+    }
+    const uint32_t slow0 = (uint32_t)(pl.row0 + p.l) * (uint32_t)g.Cx + (uint32_t)(p.w << 4);
+    const uint32_t x = exact_group(
+        trans, thr32, m, wq, t, e4, pc, u.near128, slow0 + (uint32_t)sub, [&](uint32_t i) {
+          return philox_keys(i, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, rk);
+        });
+    apply_word<kCl, kAl>(g, u, pl, p, (((x >> 2) & 0x03030303u) << (2 * sub)) & valid,
+                         ((x & 0x03030303u) << (2 * sub)) & valid);
+  }
 }
 
 // Observables of this CTA's words by definition, as sums over bit products of
@@ -702,10 +697,19 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
             if (!valid) d.z = 0u;
 #pragma unroll 1
             while (d.z) {
-              const int t = __ffs((int)d.z) - 1;
+              const int t = __ffs((int)d.z) - 1, q = t >> 2;
               d.z &= d.z - 1u;
-              const uint32_t x =
-                  exact_move(g, trans, thrT, thr32, pl.row0 + pt.l, pt.w, t, in, P, u.near128);
+              uint32_t X = q == 0 ? rn[0].x : q == 1 ? rn[0].y : q == 2 ? rn[0].z : rn[0].w;
+              if constexpr (kTPW == 1) {  // no indexing: rn stays in registers
+                const U4 &r = rn[kCalls - 1];
+                if (t & 2) X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
+              }
+              const uint32_t x = rare_move(
+                  trans, thr32, t, in, X,
+                  (uint32_t)(pl.row0 + pt.l) * (uint32_t)g.Cx + (uint32_t)(pt.w << 4), u.near128,
+                  [&](uint32_t i) {
+                    return philox_keys(i, (uint32_t)P, (uint32_t)(P >> 32), TAG_SLOW, J.rk);
+                  });
               d.x |= (x >> 2) << (2 * t);
               d.y |= (x & 3u) << (2 * t);
             }

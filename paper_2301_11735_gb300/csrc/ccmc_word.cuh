@@ -161,6 +161,27 @@ __device__ __forceinline__ uint32_t entry_offset(uint32_t pcs, int q, uint32_t r
   return lop3<kLutAndXor>(pcs >> (8 * q), 0x78u, r264);
 }
 
+// Pair t's own counts (dp4a's operand) and state (times 8), from bits 2 t and 2 t + 1
+// of the word's planes and words.
+__device__ __forceinline__ uint32_t pair_env(const WordIn &in, int t) {
+  auto counts = [&](const Planes &p) {
+    const uint32_t O = p.O >> (2 * t), T = p.T >> (2 * t), F = p.F >> (2 * t);
+    return ((O & 2u) + 2u * (T & 2u) + 4u * (F & 2u)) |
+           (((O & 1u) + 2u * (T & 1u) + 4u * (F & 1u)) << 8);
+  };
+  return counts(in.na) | (counts(in.nb) << 16);
+}
+__device__ __forceinline__ uint32_t pair_pc8(const WordIn &in, int t) {
+  return ((((in.A >> (2 * t)) & 3u) << 2) | ((in.B >> (2 * t)) & 3u)) << 3;
+}
+
+// The exact decision against the full threshold of a pair with w = wq (5461: its choice
+// class was drawn again) and SLOW word s.
+__device__ __forceinline__ bool exact_accept(uint32_t thr, uint32_t wq, uint32_t s) {
+  return thr == 0xFFFFFFFFu ||
+         (wq != 5461u ? ((uint64_t)wq << 32) + s < 5461ull * thr : s < thr);
+}
+
 // The exact decision of pair t of word w of class row j, with its SLOW words, if it
 // is rare (a tie or a field >= 65532, which the fast path rejected): the accepted
 // move, else 0.
@@ -174,14 +195,7 @@ __device__ __forceinline__ uint32_t exact_move(const Geo &g, const uint2 *trans,
   const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
   const uint32_t v = h ? X >> 16 : X & 0xFFFFu;
   const uint32_t wq = div12(v);
-  // the pair's own counts and state, from bits 2 t and 2 t + 1 of the planes
-  auto counts = [&](const Planes &p) {
-    const uint32_t O = p.O >> (2 * t), T = p.T >> (2 * t), F = p.F >> (2 * t);
-    return ((O & 2u) + 2u * (T & 2u) + 4u * (F & 2u)) |
-           (((O & 1u) + 2u * (T & 1u) + 4u * (F & 1u)) << 8);
-  };
-  const uint32_t env = counts(in.na) | (counts(in.nb) << 16);
-  const uint32_t pc8 = ((((in.A >> (2 * t)) & 3u) << 2) | ((in.B >> (2 * t)) & 3u)) << 3;
+  const uint32_t env = pair_env(in, t), pc8 = pair_pc8(in, t);
   uint2 e = move_entry(trans, ((v - 12u * wq) * 264u + near128) ^ pc8);
   if (v < 65532u && wq != level_at(thrT, (uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu))
     return 0u;  // not rare
@@ -192,9 +206,69 @@ __device__ __forceinline__ uint32_t exact_move(const Geo &g, const uint2 *trans,
     e = move_entry(trans, ((sl.y % 12u) * 264u + near128) ^ pc8);
   }
   const uint32_t thr = thr32[((uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu) >> 1];
-  const bool accept = thr == 0xFFFFFFFFu ||
-                      (v < 65532u ? ((uint64_t)wq << 32) + sl.x < 5461ull * thr : sl.x < thr);
-  return accept ? e.x >> 24 : 0u;
+  return exact_accept(thr, wq, sl.x) ? e.x >> 24 : 0u;
+}
+
+// The same of a pair known to be rare, with the random word X of its MOVE call at hand;
+// slow0: the SLOW index of the word's pair 0, slow(i): the SLOW words of index i, which
+// do not wait for the level and the exact threshold.  A resident phase waits for its
+// slowest warp, and of a lattice of 256 words one has a rare pair in most phases: with
+// exact_move there, 800 cycles, 1000^2 took 18.7 us a sweep, now 17.1.
+template <class Slow>
+__device__ __forceinline__ uint32_t rare_move(const uint2 *trans, const uint32_t *thr32, int t,
+                                              const WordIn &in, uint32_t X, uint32_t slow0,
+                                              uint32_t near128, const Slow &slow) {
+  const uint32_t v = t & 1 ? X >> 16 : X & 0xFFFFu;
+  const uint32_t wq = div12(v);
+  const uint32_t env = pair_env(in, t), pc8 = pair_pc8(in, t);
+  // (a field >= 65532 has v - 12 wq = 0 .. 3: an entry of the table, not the pair's)
+  uint2 e = move_entry(trans, ((v - 12u * wq) * 264u + near128) ^ pc8);
+  auto threshold = [&]() {
+    return thr32[((uint32_t)__dp4a((int)e.y, (int)env, (int)e.x) & 0xFFFFu) >> 1];
+  };
+  uint32_t thr = threshold();
+  const U4 sl = slow(slow0 + (uint32_t)t);
+  if (v >= 65532u) {
+    if (sl.y >= 4294967292u) return 0u;  // keep the current configuration
+    e = move_entry(trans, ((sl.y % 12u) * 264u + near128) ^ pc8);
+    thr = threshold();
+  }
+  return exact_accept(thr, wq, sl.x) ? e.x >> 24 : 0u;
+}
+
+// The exact decisions of a group's rare pairs (mask m of its lanes q, not empty), by
+// the thread that holds the group: the accepted moves, byte q for lane q.  wq, t, ev:
+// the lanes' w, level offset with the move in byte 3, and dp4a operand; pc: the pair
+// states as entry_offset takes them; slow0: the SLOW index of lane 0, slow(i): the
+// SLOW words of index i.  The threshold is on its way while the words are drawn.
+template <class Slow>
+__device__ __forceinline__ uint32_t exact_group(const uint2 *trans, const uint32_t *thr32,
+                                                uint32_t m, const uint32_t (&wq)[4],
+                                                const uint32_t (&t)[4], const uint32_t (&ev)[4],
+                                                uint32_t pc, uint32_t near128, uint32_t slow0,
+                                                const Slow &slow) {
+  auto lane = [](const uint32_t (&x)[4], int q) {  // no indexing: the array stays in registers
+    return q == 0 ? x[0] : q == 1 ? x[1] : q == 2 ? x[2] : x[3];
+  };
+  uint32_t acc = 0u;
+#pragma unroll 1
+  do {
+    const int q = __ffs((int)m) - 1;
+    m &= m - 1u;
+    const uint32_t w = lane(wq, q);
+    uint32_t tq = lane(t, q);
+    uint32_t thr = thr32[(tq & 0xFFFFu) >> 1];
+    const U4 sl = slow(slow0 + 4u * (uint32_t)q);
+    const bool big = w == 5461u;  // a field >= 65532: the choice class drawn again
+    if (big) {
+      if (sl.y >= 4294967292u) continue;  // keep the current configuration
+      const uint2 e = move_entry(trans, entry_offset(pc, q, (sl.y % 12u) * 264u + near128));
+      tq = (uint32_t)__dp4a((int)e.y, (int)lane(ev, q), (int)e.x);
+      thr = thr32[(tq & 0xFFFFu) >> 1];
+    }
+    if (exact_accept(thr, w, sl.x)) acc |= (tq >> 24) << (8 * q);
+  } while (m);
+  return acc;
 }
 
 // The fast path of the pairs of a word one thread evaluates: kTPW threads
@@ -206,7 +280,9 @@ __device__ __forceinline__ uint32_t exact_move(const Geo &g, const uint2 *trans,
 // rand(c): the four words of the word's MOVE call c.  Returns the (dA, dB) of the
 // fast decisions and, in z, what needs the exact path (a tie or a field >= 65532,
 // rejected here): bit t for every such pair t (kPairs), or bit c for every call c
-// with one (fewer instructions, for a path that looks at the call's pairs anyway).
+// with one (fewer instructions, for a path that looks at the call's pairs anyway).  A
+// call asks once for all its pairs: a branch for every four kept the groups of a call
+// from being worked on together (1000^2: 0.1 us a phase).
 template <int kTPW, bool kPairs, class Rand>
 __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *thrT, int sub,
                                             const WordIn &in, uint32_t near128,
@@ -239,11 +315,12 @@ __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *
     const uint32_t mx = __vmaxu2(__vimax3_u16x2(r.x, r.y, r.z), r.w);
     const bool big = mx >= 0xFFFC0000u || (mx & 0xFFFFu) >= 0xFFFCu;  // a field >= 65532
     uint32_t mn = 0xFFFFFFFFu;  // smallest w - T of the call
+    uint32_t d[kHalves][4];
 #pragma unroll
     for (int hi = 0; hi < kHalves; ++hi) {
       const int h = h0 + hi;
       const int k = 2 * c + h;
-      uint32_t d[4], t[4];
+      uint32_t t[4];
       const uint32_t pc = __funnelshift_l(pcs[hi], pcs[hi], 3 - 4 * c);  // counts modulo 32
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -253,29 +330,33 @@ __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *
         const uint2 e =
             move_entry(trans, entry_offset(pc, q, (v - 12u * wq) * 264u + near128));
         t[q] = (uint32_t)__dp4a((int)e.y, (int)((env[hi].ev[q] >> (4 * c)) & kEnvMask), (int)e.x);
-        d[q] = wq - level_at(thrT, t[q] & 0xFFFFu);  // negative: accept; zero: a tie
+        d[hi][q] = wq - level_at(thrT, t[q] & 0xFFFFu);  // negative: accept; zero: a tie
       }
-      if constexpr (kPairs) {
-        if (__vimin3_u32(__vimin3_u32(d[0], d[1], d[2]), d[3], d[3]) == 0u || big) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
-            if (d[q] == 0u || ((X >> (16 * h)) & 0xFFFFu) >= 65532u) slow |= 1u << (k + 4 * q);
-          }
-        }
-      } else {
-        mn = __vimin3_u32(mn, d[0], d[1]);
-        mn = __vimin3_u32(mn, d[2], d[3]);
-      }
+      mn = __vimin3_u32(mn, d[hi][0], d[hi][1]);
+      mn = __vimin3_u32(mn, d[hi][2], d[hi][3]);
       // byte q: the accepted move of lane q, i.e. byte 3 of t[q] under the sign
       // of d[q] (byte permutes: bit 3 of a selector replicates a byte's sign)
-      const uint32_t acc = prmt(prmt(d[0], d[1], 0x00FBu), prmt(d[2], d[3], 0x00FBu), 0x5410u) &
-                           prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
+      const uint32_t acc =
+          prmt(prmt(d[hi][0], d[hi][1], 0x00FBu), prmt(d[hi][2], d[hi][3], 0x00FBu), 0x5410u) &
+          prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
       // byte q of acc -> site k + 4 q: b bits to 2 (k + 4 q) of dB, a bits of dA
       dB |= (acc & 0x03030303u) << (2 * k);
       dA |= ((acc >> 2) & 0x03030303u) << (2 * k);
     }
-    if (!kPairs && (mn == 0u || big)) slow |= 1u << c;
+    if (mn == 0u || big) {
+      if constexpr (kPairs) {
+#pragma unroll
+        for (int hi = 0; hi < kHalves; ++hi)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
+            if (d[hi][q] == 0u || ((X >> (16 * (h0 + hi))) & 0xFFFFu) >= 65532u)
+              slow |= 1u << (2 * c + h0 + hi + 4 * q);
+          }
+      } else {
+        slow |= 1u << c;
+      }
+    }
   }
   return make_uint3(dA, dB, slow);
 }
