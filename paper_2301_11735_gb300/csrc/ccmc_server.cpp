@@ -43,10 +43,14 @@ using Clock = std::chrono::steady_clock;
 
 constexpr int kSlicesInFlight = 2;
 // The first slice after the GPU ran dry holds the one or two requests that woke the
-// scheduler, while the rest of a burst arrives: it is kept short, so that they join
-// soon (48 requests at once: 56 ms to the last result, the first 14 of them spent
-// on the first request alone).
+// scheduler, and the second, queued at once behind it, what arrived meanwhile: both are
+// kept short, so that a burst's requests are soon together (48 requests at once: 56 ms
+// to the last result with full slices, the first 14 of them spent on the first request
+// alone; with the first kept short 43 or 68, as the second held all of them or 34; with
+// both 44 to 45; a third of 4 ms costs 6 more, as it advances every lattice by as much
+// time and not by its share of the work left).
 constexpr double kFirstSliceMs = 1.0;
+constexpr int kFirstSlices = 2;
 
 struct Pending {
   uint64_t ticket;
@@ -91,12 +95,12 @@ int64_t ring_records(const ccmc_request &r) {
   return r.obs_every > 0 ? std::min<int64_t>(r.nsweeps / r.obs_every + 1, 1 << 16) : 1;
 }
 
-// Estimated wall time of one sweep, for sizing slices (measured: 4.3 us at 64^2,
-// 12 at 512^2, 20 at 1024^2, held in shared memory; 43 at 4096^2, 280 at 16384^2,
-// a launch a phase).
+// Estimated wall time of one sweep, for sizing slices (measured: 3.5 us at 64^2, 11 at
+// 512^2, 19 at 1024^2, held in shared memory; 24 at 2048^2, 33 at 4096^2, 213 at
+// 16384^2, a launch a phase).
 double sweep_us(const ccmc_request &r) {
   const double N = (double)r.Lx * (double)r.Ly;
-  return N <= 1.2e6 ? 5.0 + 1.5e-5 * N : 30.0 + 1e-6 * N;
+  return N <= 1.2e6 ? 5.0 + 1.5e-5 * N : 22.0 + 0.7e-6 * N;
 }
 
 // Pinned host buffers, cached by power-of-two size (allocating pinned memory
@@ -275,6 +279,7 @@ bool ccmc_server::collect(Retiring &x) {
 
 void ccmc_server::run() {
   cudaSetDevice(device);
+  int first_slices = 0;  // short slices left since the GPU ran dry
   for (;;) {
     // (1) admission: first come, first served, while slots and budget allow
     std::vector<Pending> admit;
@@ -358,7 +363,9 @@ void ccmc_server::run() {
     std::vector<int64_t> sw(n);
     std::vector<double> beta(n), Delta(n), V(n), J(n);
     std::vector<int> every(n);
-    const double ms = slices.empty() ? std::min(slice_ms, kFirstSliceMs) : slice_ms;
+    if (slices.empty()) first_slices = kFirstSlices;
+    const double ms = first_slices > 0 ? std::min(slice_ms, kFirstSliceMs) : slice_ms;
+    if (first_slices > 0) --first_slices;
     for (int i = 0; i < n; ++i) {
       Running &r = active[i];
       int64_t q = (int64_t)(ms * 1e3 / sweep_us(r.req));
