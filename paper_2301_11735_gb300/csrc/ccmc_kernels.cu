@@ -84,7 +84,7 @@ struct RecountArgs {
 
 // Grid (gx, 4): grid row y counts the classes of site rows y mod 4; or (gx, 16),
 // class y, for rows that are not whole quads of words.
-__global__ void __launch_bounds__(256, 4) recount_kernel(Geo g, RecountArgs a) {
+__global__ void __launch_bounds__(1024, 1) recount_kernel(Geo g, RecountArgs a) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;");
   int c[kSums] = {0, 0, 0, 0, 0, 0, 0};
@@ -94,19 +94,20 @@ __global__ void __launch_bounds__(256, 4) recount_kernel(Geo g, RecountArgs a) {
     count_class(g, blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, c);
   const unsigned nblocks = gridDim.x * gridDim.y;
   const unsigned bid = blockIdx.y * gridDim.x + blockIdx.x;
-  __shared__ int64_t red[8][7];
+  constexpr int kRuns = 256 / kSums;  // threads that share a sum in the last block
+  __shared__ int64_t red[kRuns][kSums];
   __shared__ bool last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < 7; ++k) {
-    const int64_t v = warp_sum((int64_t)c[k]);
+  for (int k = 0; k < kSums; ++k) {  // a warp counts below 2^31
+    const int v = __reduce_add_sync(0xFFFFFFFFu, c[k]);
     if (lane == 0) red[warp][k] = v;
   }
   __syncthreads();
-  if (threadIdx.x < 7) {
+  if (threadIdx.x < kSums) {
     int64_t v = 0;
     for (int wv = 0; wv < (int)(blockDim.x >> 5); ++wv) v += red[wv][threadIdx.x];
-    a.partials[bid * 7 + threadIdx.x] = v;
+    a.partials[bid * kSums + threadIdx.x] = v;
   }
   __threadfence();
   __syncthreads();
@@ -118,47 +119,43 @@ __global__ void __launch_bounds__(256, 4) recount_kernel(Geo g, RecountArgs a) {
   __syncthreads();
   if (!last) return;
   __threadfence();
-  // the last block sums the partials with all its threads (L2 loads: the
-  // partials were written by other blocks)
-  __shared__ int64_t sums[kSums];
-  int64_t v[7] = {0, 0, 0, 0, 0, 0, 0};
-  for (unsigned b = threadIdx.x; b < nblocks; b += blockDim.x) {
-#pragma unroll
-    for (int k = 0; k < 7; ++k) v[k] += __ldcg(a.partials + (int64_t)b * 7 + k);
-  }
-#pragma unroll
-  for (int k = 0; k < 7; ++k) {
-    const int64_t x = warp_sum(v[k]);
-    if (lane == 0) red[warp][k] = x;
+  // The last block's end is what the next phase waits for: consecutive threads read
+  // consecutive partials (L2 loads: other blocks wrote them), then one warp writes the
+  // record, a lane a word, and the three bins side by side.
+  const int64_t base = g.ctl[kCtlPhaseBase], cnt = g.ctl[kCtlObsCount];
+  if (threadIdx.x < kRuns * kSums) {
+    int64_t v = 0;
+#pragma unroll 8
+    for (unsigned b = threadIdx.x; b < nblocks * kSums; b += kRuns * kSums)
+      v += __ldcg(a.partials + b);
+    red[threadIdx.x / kSums][threadIdx.x % kSums] = v;
   }
   __syncthreads();
-  if (threadIdx.x < 7) {
-    int64_t x = 0;
-    for (int wv = 0; wv < (int)(blockDim.x >> 5); ++wv) x += red[wv][threadIdx.x];
-    sums[threadIdx.x] = x;
+  if (warp != 0) return;
+  int64_t x = 0;
+  if (lane < kSums) {
+#pragma unroll
+    for (int r = 0; r < kRuns; ++r) x += red[r][lane];
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int64_t rec[8];
-    rec[0] = g.ctl[kCtlPhaseBase] / 8 + a.sweep_off;
-    observables_of(g, sums, rec + 1);
-    for (int k = 0; k < 8; ++k) g.ctl[kCtlLatest + k] = rec[k];
-    if (a.ring) {
-      const int64_t cnt = g.ctl[kCtlObsCount];
-      int64_t *dst = a.ring + (cnt % a.ring_cap) * 8;
-      for (int k = 0; k < 8; ++k) dst[k] = rec[k];
-      g.ctl[kCtlObsCount] = cnt + 1;
-      if (a.hist) {
-        const int64_t N = (int64_t)g.Lx * g.Ly;
-        const int64_t vals[3] = {rec[4], rec[5], rec[7]};
-        for (int h = 0; h < 3; ++h) {
-          const int64_t bin = (vals[h] + N) * a.nbins / (2 * N + 1);
-          a.hist[h * a.nbins + bin] += 1;
-        }
-      }
+  int64_t sums[kSums], rec[8];
+#pragma unroll
+  for (int k = 0; k < kSums; ++k) sums[k] = __shfl_sync(0xFFFFFFFFu, x, k);
+  rec[0] = base / 8 + a.sweep_off;
+  observables_of(g, sums, rec + 1);
+  int64_t mine = rec[0];  // lane k: word k
+#pragma unroll
+  for (int k = 1; k < 8; ++k) mine = lane == k ? rec[k] : mine;
+  if (lane < 8) g.ctl[kCtlLatest + lane] = mine;
+  if (a.ring) {
+    if (lane < 8) a.ring[(cnt % a.ring_cap) * 8 + lane] = mine;
+    if (lane == 0) g.ctl[kCtlObsCount] = cnt + 1;
+    if (a.hist && (lane == 4 || lane == 5 || lane == 7)) {  // M, M_stag, S_stag
+      const int64_t N = (int64_t)g.Lx * g.Ly;
+      const int64_t bin = (mine + N) * a.nbins / (2 * N + 1);
+      a.hist[(lane == 7 ? 2 : lane - 4) * a.nbins + bin] += 1;
     }
-    g.ctl[kCtlTicket] = 0;
   }
+  if (lane == 0) g.ctl[kCtlTicket] = 0;
 }
 
 // ============================================================================
@@ -392,23 +389,33 @@ cudaError_t launch_init(const Geo &g, int h, int64_t n_plus, int64_t n_minus, cu
   return cudaGetLastError();
 }
 
-// Grid of recount_kernel: one wave at four blocks per SM (64 registers).  A
-// thread's unit is a word, or a quad of words of four classes.
-static dim3 recount_dim(const Geo &g) {
+// Launch of recount_kernel: one wave of 1024 threads an SM (64 registers).  A thread's
+// unit is a word, or a quad of words of four classes.  A block's end (its sums, its
+// fence and ticket) costs what a block of 256 counts in 4 us, so a wave that is full of
+// work takes one block an SM (16384^2: 26.6 us a recount with four, 24.7; 8192^2 13.8,
+// 11.1) and one that is not takes small blocks, for more SMs (4096^2: 7.5 us, 14.2 with
+// blocks of 1024).  Rows that are not whole quads: four blocks an SM.
+struct RecountShape {
+  dim3 grid;
+  int block;
+};
+static RecountShape recount_shape(const Geo &g) {
   const int64_t words = (int64_t)g.Cy * g.W;
-  if (quads_ok(g)) return dim3((unsigned)grid_for(words / 4, 256, 152), 4u);
-  return dim3((unsigned)grid_for(words, 256, 38), 16u);
+  if (!quads_ok(g)) return {dim3((unsigned)grid_for(words, 256, 38), 16u), 256};
+  const int block = words / 4 >= 38 * 1024 ? 1024 : 256;
+  return {dim3((unsigned)grid_for(words / 4, block, 152 * 256 / block), 4u), block};
 }
 
 int recount_grid(const Geo &g) {
-  const dim3 d = recount_dim(g);
+  const dim3 d = recount_shape(g).grid;
   return (int)(d.x * d.y);
 }
 
 cudaError_t launch_recount(const Geo &g, int64_t *partials, int64_t *ring, int64_t ring_cap,
                            int64_t *hist, int nbins, int64_t sweep_off, cudaStream_t s) {
   RecountArgs a{partials, ring, ring_cap, hist, nbins, sweep_off};
-  return launch_pdl(recount_kernel, recount_dim(g), 256, s, g, a);
+  const RecountShape sh = recount_shape(g);
+  return launch_pdl(recount_kernel, sh.grid, sh.block, s, g, a);
 }
 
 cudaError_t launch_advance(int64_t *ctl, int64_t phases, cudaStream_t s) {
