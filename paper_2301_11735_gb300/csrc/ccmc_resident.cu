@@ -865,17 +865,18 @@ static ResShape shape_of(const Geo &g, int C, int tpw, int max_workers) {
 
 // Shapes, measured on GB300 (us a sweep, records off).  A cluster's barrier and
 // remote windows cost 0.4 us a phase, which pays from 128 words a phase: 128^2
-// (64 words) 5.3 on one CTA, 6.5 on four; 256^2 13.5 on one, 9.8 on four, 7.7 on
-// sixteen; 1024^2 43 on four, 26 on eight, 18.7 on sixteen.  Four lanes a word up
-// to 96 words a CTA (64^2: 3.4, with one 9.4; 516^2, 81 words a CTA: 13.7, with two
-// 15.7); above that the work repeated for threads that share a word costs more
-// than the shorter chain hides (1024^2 on sixteen: 18.7 with one thread, 21.8 with
-// two), two threads paying up to 128 words.  When lattices crowd the SMs only the
-// smallest keep four lanes: their four kinds of warps fall on the four schedulers
-// (a lone worker warp a CTA lands on the same one every time: 128 lattices of 256^2
-// and 128 of 64^2 34 against 23), while a 416-thread CTA finds no room beside
-// another (512 replicas: 19.7 with four lanes for their 128^2 lattices, 15.8 with
-// one thread).
+// (64 words) 5.2 on one CTA, 6.1 on four; 256^2 10.6 on one, 8.7 on four, 7.2 on
+// sixteen; 1024^2 37.7 on four, 21.8 on eight, 15.0 on sixteen.  Four lanes a word up
+// to 96 words a CTA (64^2: 3.3, with one 6.5; 516^2, 81 words a CTA: 12.9, with two
+// 13.3), of rows of whole words up to 48 (448^2, 49 words: 10.6 both; 512^2, 64: 10.9,
+// with two 10.2; 576^2, 81: 12.5, 12.1); above that the work repeated for threads that
+// share a word costs more than the shorter chain hides (1024^2 on sixteen: 15.0 with
+// one thread, 16.8 with two), two threads paying up to 128 words.  When lattices crowd
+// the SMs only the smallest keep four lanes: their four kinds of warps fall on the four
+// schedulers (a lone worker warp a CTA lands on the same one every time: 128 lattices of
+// 256^2 and 128 of 64^2 34 against 23; 512 replicas: 28 against 14.7), while a
+// 416-thread CTA finds no room beside another (512 replicas: 18.5 with four lanes for
+// their 128^2 lattices, 14.7 with one thread).
 ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads, int max_tpw) {
   int C = 1;
   if (g.cstride >= kResClusterWords)
@@ -886,9 +887,12 @@ ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads,
     C *= 2;
   const int words = (g.Cy + C - 1) / C * g.W;
   const bool crowded = load > 128.0;
-  int tpw = max_tpw >= 4 && words <= (crowded ? 32 : kResQuadWords) ? 4
-            : max_tpw >= 2 && words <= 128 && !crowded              ? 2
-                                                                     : 1;
+  const int quad = crowded ? 32 : (g.Cx & 15) == 0 ? 48 : kResQuadWords;
+  int tpw = 1;
+  if (max_tpw >= 4 && words <= quad)
+    tpw = 4;
+  else if (max_tpw >= 2 && words <= 128 && !crowded)
+    tpw = 2;
   while (tpw > 1 && tpw * words > max_threads) tpw /= 2;
   return shape_of(g, C, tpw, max_threads);
 }
@@ -931,6 +935,9 @@ ResShape resident_fit(const Geo &g, const ResShape &shape, bool aligned, int n) 
 
 cudaError_t launch_resident_sweep(const ResJob *one, const ResJob *d_jobs, int njobs,
                             const ResShape &shape, bool aligned, cudaStream_t s) {
+  // (a block barrier of a part of a warp would never complete)
+  if (shape.workers % 32 || shape.threads % 32 || shape.threads > kResMaxThreads)
+    return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[1];
   launch_config(shape, njobs, s, cfg, attr);

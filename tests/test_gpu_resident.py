@@ -40,7 +40,7 @@ def _lattice(cc, Lx, Ly, **env):
 # not divide by the CTAs, words that do not divide by the warps)
 SMALL = [(4, 4), (4, 64), (64, 4), (12, 8), (60, 36), (64, 64), (68, 124), (128, 128), (132, 140),
          (192, 256), (256, 260), (2052, 16), (16, 2052)]
-LARGE = [(516, 516), (768, 400), (1000, 1000), (1024, 1024), (64, 4096), (4096, 64), (1088, 1084)]
+LARGE = [(448, 384), (448, 448), (516, 516), (768, 400), (1000, 1000), (1024, 1024), (64, 4096), (4096, 64), (1088, 1084)]
 # few rows of classes, so that no shape or only one CTA holds them
 WIDE = [(131072, 4), (262144, 4), (131072, 8), (32768, 32)]
 
