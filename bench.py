@@ -25,8 +25,8 @@ stream-ordered), and reads the observable records back (ccmc_obs_series).
 Beside the headline the same JSON line carries side measurements:
 `temperature4096` (the four 4096^2 lattices above, with their own roofline),
 `paper_maps` (the paper's own host-built maps against the colour schedule),
-`batched` (512 replicas of uneven L in one persistent launch, against the same
-lattices swept one at a time), `served` (a Poisson request stream through the
+`batched` (512 replicas of uneven L, one resident launch a shape, against the
+same lattices swept one at a time), `served` (a Poisson request stream through the
 continuous-batching server: p50/p99 latency, achieved vs offered
 site-updates/s, against the same requests run one at a time) and `small16`
 (the 16x16 lattice's microseconds a sweep, plain and as a batch of one).
@@ -62,26 +62,27 @@ OBS_EVERY = {"temperature4096": 10, "large16384": 1}
 # They hold only for the kernel sources they were taken with (kernel_digest);
 # after any change to those sources the bench reports them as null.
 PHASE_COUNTERS = {
-    "large16384": {"digest": "e6ddb005f8d5ceedad68da55ac243d2d058a839479b6933f3ebea067275a9715",
-                   "traffic": 33_638_144 + 118_528, "warp_inst": 26_336_685},
-    "temperature4096": {"digest": "e6ddb005f8d5ceedad68da55ac243d2d058a839479b6933f3ebea067275a9715",
-                        "traffic": 2_152_960, "warp_inst": 1_906_504},
+    "large16384": {"digest": "f881680a544843509018256b10e951cdfabaa09ccebc2f342c5615618fae22f9",
+                   "traffic": 33_596_928 + 17_152, "warp_inst": 21_016_353},
+    "temperature4096": {"digest": "f881680a544843509018256b10e951cdfabaa09ccebc2f342c5615618fae22f9",
+                        "traffic": 2_137_344, "warp_inst": 1_549_387},
 }
 # What bounds the dominant kernel, from the same captures: the HBM roofline is
 # the algorithm's bound, these are the kernel's.
 PHASE_LIMITER = {
-    "large16384": "integer instruction issue, then the shared-memory pipe (issue active 61 %, "
-                  "ALU pipe 59 %, shared-memory wavefronts 44 % of peak, half of them bank "
-                  "conflicts of the table lookups; DRAM 11 %)",
+    "large16384": "integer instruction issue and the shared-memory pipe together (issue active "
+                  "64 %, ALU pipe 60 %, l1tex 63 %, half of the shared wavefronts bank conflicts "
+                  "of the table lookups; DRAM 13 %)",
     "temperature4096": "latency: one lattice's phase fills a fifth of the warp slots (warps "
-                       "active 21 %, issue 27 %); the four lattices overlap on their streams",
+                       "active 19 %, issue 28 %); the four lattices overlap on their streams",
 }
-# (file, first line, end line): the sources that define the tile phase kernel
-# and its launch -- ccmc_phase.cu from the per-word code through the tile
-# kernel, and its launchers; the headers whole.
+# (file, first line, end line): the sources that define the phase kernel and its
+# launch -- ccmc_phase.cu from the per-word code through the kernel, and its
+# launchers; the word's code and the headers whole.
 KERNEL_SOURCES = (
     ("ccmc_phase.cu", "// One colour phase", "// Lock-step phase of several lattices"),
     ("ccmc_phase.cu", "// Launchers.", None),
+    ("ccmc_word.cuh", None, None),
     ("ccmc_device.cuh", None, None),
     ("ccmc_launch.cuh", None, None),
     ("ccmc_internal.h", None, None),
@@ -89,7 +90,7 @@ KERNEL_SOURCES = (
 
 
 def kernel_digest() -> str:
-    """sha256 over the tile phase kernel's sources (KERNEL_SOURCES, in order)."""
+    """sha256 over the phase kernel's sources (KERNEL_SOURCES, in order)."""
     h = hashlib.sha256()
     for name, first, end in KERNEL_SOURCES:
         with open(os.path.join(ROOT, "paper_2301_11735_gb300", "csrc", name)) as f:
@@ -177,10 +178,11 @@ class ClockSampler:
 
 
 def launches_per_call(nsweeps: int, obs_every: int, done: int) -> int:
-    """Kernel launches of one ccmc_sweep call, following the library's rule:
-    16-sweep (or obs_every-aligned) captured chunks when they fit, single
-    sweeps otherwise; a sweep is 8 phase kernels, each recount one kernel, each
-    chunk or single sweep ends with one counter-advance kernel."""
+    """Kernel launches of one ccmc_sweep call of a lattice too large for shared
+    memory, following the library's rule: 16-sweep (or obs_every-aligned)
+    captured chunks when they fit, single sweeps otherwise; a sweep is 8 phase
+    kernels, each recount one kernel, each chunk or single sweep ends with one
+    counter-advance kernel."""
     n, s = 0, 0
     while s < nsweeps:
         a = done + s
@@ -200,23 +202,6 @@ def launches_per_call(nsweeps: int, obs_every: int, done: int) -> int:
         n += 8 + (1 if obs_every > 0 and (a + 1) % obs_every == 0 else 0) + 1
         s += 1
     return n
-
-
-def tile_ok(s) -> bool:
-    """Whether the lattice takes the tile-staged phase kernel (rows of W words
-    with W a multiple of 4 dividing 256, and Ly/4 a multiple of 256/W)."""
-    W = (s.Lx // 4 + 15) // 16
-    return (s.Lx // 4) % 16 == 0 and W % 4 == 0 and 256 % W == 0 and (s.Ly // 4) % (256 // W) == 0
-
-
-def tile_kernel_name(s) -> str:
-    """The tile-staged phase kernel a lattice takes: the single-tile compact
-    instantiation when its phase fits one wave of it (five CTAs per SM on the
-    152 SMs of a GB300), the pipelined one otherwise."""
-    W = (s.Lx // 4 + 15) // 16
-    tiles = (s.Ly // 4) // (256 // W)
-    return ("phase_tile_kernel<5, true, 1> (one tile per CTA)" if tiles <= 5 * 152
-            else "phase_tile_kernel<4, false, 1> (pipelined tiles)")
 
 
 def _dist():
@@ -389,11 +374,10 @@ def measure_batched(cc, nsweeps=5000, plain_per_size=4):
 
 def measure_small(cc, reps=3):
     """The 16x16 lattice of 48 + 16 charges (Delta = 0.5, V = J = 1, T = 1):
-    2000 sweeps with observables after every sweep, as microseconds a sweep on
-    the plain single-lattice path (eight phase launches and a recount a sweep,
-    replayed as graphs) and as a batch of one (one resident launch with the
-    lattice in shared memory, autotuned launch shape); best of reps, host clock
-    around a synchronised call."""
+    2000 sweeps with observables after every sweep, as microseconds a sweep of
+    ccmc_sweep (one launch with the lattice in shared memory) and of a batch of
+    one with the autotuned launch shape; best of reps, host clock around a
+    synchronised call."""
     from workloads import SMALL_16 as c
 
     beta, nsw = 1.0 / c["T"], c["nsweeps"]
@@ -673,7 +657,7 @@ def roofline(name, s0, m, value, peak, peak_kind, clocks, local):
             "issue": issue,
             "limiter": PHASE_LIMITER.get(name) if counters else None,
             "kernel": f"colour phase of one {s0.Lx}^2 lattice "
-                      f"({tile_kernel_name(s0) if tile_ok(s0) else 'phase_kernel'})",
+                      "(phase_kernel)",
             "peak_source": peak_kind, "launch_ms": m["phase_ms"],
             # the same algorithmic bytes over the whole timed run (every lattice's
             # phases, recounts and histograms included)

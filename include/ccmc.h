@@ -63,10 +63,10 @@ typedef struct ccmc_lattice ccmc_lattice;
 /* Allocate an Lx x Ly lattice on the current CUDA device (Lx, Ly multiples of
  * 4, at least 4, Lx Ly <= 2^30).  cuda_stream is a cudaStream_t (NULL: the
  * library creates one).  The observable ring holds the last obs_capacity
- * records (<= 0: 4096).  Device memory comes from a stream-ordered pool the
- * library keeps per device (allocated and freed in order on the lattice's
- * stream, cached for reuse until the process exits), so creating and
- * destroying lattices never synchronises the device.  Returns once the
+ * records (<= 0: 4096).  Device memory comes from a pool the library keeps per
+ * device (allocated and freed on a stream of its own, cached for reuse until
+ * the process exits), so creating and destroying lattices never synchronises
+ * the device.  Returns once the
  * lattice is ready.  Errors: E_INVAL, E_NOMEM, E_CUDA. */
 int ccmc_lattice_create(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity,
                         ccmc_lattice **out);
@@ -106,14 +106,16 @@ int ccmc_phases(ccmc_lattice *h, int64_t nphases, double beta, double Delta, dou
  * A batch groups existing, initialised lattices (each with its own size,
  * seed and parameters; Sec. 3.2 runs "several copies of the lattice").
  * ccmc_batch_sweep advances lattice i by nsweeps[i] sweeps at (beta[i],
- * Delta[i], V[i], J[i]).  Lattices of at most resident_max_sites sites run
- * together in one persistent launch on the batch stream: each CTA keeps a
- * whole lattice and its tables in shared memory and runs all its sweeps,
- * taking lattices from a work queue largest first.  Larger lattices run the
- * per-phase path at the same time: eight or more of them at the same sweep
- * count with fewer than 16384 class-row words a phase (below 2048^2) advance
- * in lock step, one launch per phase for all of them on the batch stream; the
- * others each on their own stream.  Every lattice ends in
+ * Delta[i], V[i], J[i]).  Lattices that ccmc_sweep holds in shared memory (up
+ * to about 1070^2; after ccmc_batch_config those of at most resident_max_sites
+ * sites) run together, side by side, ordered on the batch stream: a CTA or a
+ * cluster of CTAs keeps a whole lattice and its tables in shared memory and
+ * runs all its sweeps, one launch for all lattices of one shape, each with its
+ * share of the CTAs by its work.  Larger lattices run the per-phase path at
+ * the same time: twelve or more of them at the same sweep count with fewer
+ * than 12288 class-row words a phase (below about 1770^2) advance in lock step,
+ * one launch per phase for all of them on the batch stream; the others each on
+ * their own stream.  Every lattice ends in
  * exactly the state ccmc_sweep would give it (same random streams), and its
  * observable ring gets the same records.  Ordering: the batch waits for work
  * already queued on each lattice's stream, and each lattice's stream waits for
@@ -123,12 +125,12 @@ typedef struct ccmc_batch ccmc_batch;
 int ccmc_batch_create(int count, ccmc_lattice *const *lattices, void *cuda_stream,
                       ccmc_batch **out);
 int ccmc_batch_destroy(ccmc_batch *b);
-/* Launch shape of the resident launch (autotuner knobs; results do not depend
- * on them): threads per CTA (64, 128, 256 or 512), the largest lattice (in
- * sites) kept in shared memory, CTAs per SM of the persistent grid, and the
- * most threads that share one packed word (16 pairs) of a lattice: 1, 2 or 4
- * (each lattice takes the most, up to this, that still covers a phase's words
- * in one pass of its CTA).  Errors: E_INVAL (a value out of range, or a
+/* Launch shape of the resident launches (autotuner knobs; results do not depend
+ * on them): the most worker threads per CTA (64, 128, 256 or 512), the largest
+ * lattice (in sites) kept in shared memory, the CTAs per SM that the lattices
+ * share out, and the most threads that share one packed word (16 pairs) of a
+ * lattice: 1, 2 or 4 (a lattice takes more than one where they shorten its
+ * phases).  Errors: E_INVAL (a value out of range, or a
  * resident limit beyond the device's shared memory). */
 int ccmc_batch_config(ccmc_batch *b, int resident_threads, int64_t resident_max_sites,
                       int ctas_per_sm, int max_threads_per_word);
@@ -271,10 +273,9 @@ int ccmc_threshold_table(double beta, double Delta, double V, double J, uint32_t
 
 /* Diagnostic (the paper has no counterpart): the bounded-wait self-test.  One
  * CTA waits on a device barrier that nothing completes, giving up after
- * `polls` polls (1 .. 2^24), records the timeout and returns, as every wait of
- * the phase kernels does; the call then returns CCMC_E_TIMEOUT and the CUDA
- * context stays usable.  Errors: E_INVAL (polls out of range), E_NOMEM,
- * E_CUDA.  Host-side failures can be injected with the environment variable
+ * `polls` polls (1 .. 2^24), records the timeout and returns; the call then
+ * returns CCMC_E_TIMEOUT and the CUDA context stays usable.  Errors: E_INVAL
+ * (polls out of range), E_NOMEM, E_CUDA.  Host-side failures can be injected with the environment variable
  * CCMC_FAULT (comma-separated): "alloc" makes ccmc_lattice_create and
  * ccmc_batch_create return E_NOMEM before allocating anything, "launch" makes
  * ccmc_sweep, ccmc_phases and ccmc_batch_sweep return E_CUDA before queuing

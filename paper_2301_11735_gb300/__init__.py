@@ -325,8 +325,8 @@ class Lattice:
 
 
 class Batch:
-    """Several lattices swept together (ccmc_batch_*): small ones share one
-    persistent shared-memory-resident launch, large ones run alongside."""
+    """Several lattices swept together (ccmc_batch_*): small ones held in shared
+    memory, one launch a shape, large ones run alongside."""
 
     def __init__(self, lattices, stream=None):
         self.lattices = list(lattices)

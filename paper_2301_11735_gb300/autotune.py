@@ -1,10 +1,11 @@
 """Autotuner for batched sweeps: picks the launch shape of a batch by timing.
 
-The knobs (ccmc_batch_config) are the threads per CTA of the resident launch
-(64 to 512), its CTAs per SM, the largest lattice kept in shared memory (the
-shared-memory path; the rest take the per-phase L2/HBM path), and the most
-threads that share one packed word of a lattice (1, 2 or 4: the pairs each
-thread evaluates, 16, 8 or 4).  None of them changes results -- the random
+The knobs (ccmc_batch_config) are the most threads per CTA of the resident
+launches (64 to 512), the CTAs per SM the lattices share out among them, the
+largest lattice kept in shared memory (the shared-memory path; the rest take the
+per-phase L2/HBM path; a batch that was never configured keeps what ccmc_sweep
+would), and the most threads that share one packed word of a lattice (1, 2 or 4:
+the pairs each thread evaluates, 16, 8 or 4).  None of them changes results -- the random
 streams are keyed by (seed, phase, site) -- so the tuner may pick freely.
 
 A probe batch of synthetic lattices with the same shapes is swept for a few

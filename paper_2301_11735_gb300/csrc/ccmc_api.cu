@@ -197,10 +197,10 @@ struct ccmc_lattice {
 namespace {
 
 // Lattices that the resident kernel sweeps unless the caller says otherwise: up
-// to 4608 a-words a phase (1024^2 has 4096), 288 a CTA of a cluster of 16, where
-// a launch of a phase's own begins to be as fast (1024^2: 3.2 us a phase
-// resident, 3.7 us a launch; 1000^2, ragged: 3.4 against 4.6; 256^2: 1.4 against
-// 3.3; 64^2: 0.7 against 3.3).
+// to 4608 a-words a phase (1024^2 has 4096), 288 a CTA of a cluster of 16; a little
+// further on a launch of a phase's own is as fast (us a sweep resident and with a
+// launch a phase: 64^2 3.5, 16.9; 256^2 7.5, 18.3; 1000^2, ragged, 17.9, 23.6; 1024^2
+// 15.0, 21.4; 1200^2 22.6, 23.4; 1280^2 22.5, 22.1; 1536^2 33.3, 22.9).
 bool resident_default(const Geo &g) { return g.cstride <= 4608 && resident_possible(g); }
 
 // The move table, the same for every lattice (built and checked once: 25 us).
@@ -883,10 +883,10 @@ int ccmc_set_state(ccmc_lattice *h, const uint8_t *host_in, uint64_t seed, int64
 }  // extern "C"
 
 // ----------------------------------------------------------------------------
-// Batches: many lattices swept together.  Lattices whose packed words fit the
-// resident limit run in one persistent resident_kernel launch on the batch
-// stream (each CTA holds a whole lattice in shared memory); larger ones run the
-// per-phase path on their own streams at the same time.
+// Batches: many lattices swept together.  Lattices up to the resident limit run in
+// shared memory, one resident_sweep_kernel launch a shape, side by side on streams
+// that fork from the batch stream and join it; larger ones run the per-phase path
+// on their own streams, or in lock step, at the same time.
 struct ccmc_batch {
   std::vector<ccmc_lattice *> lats;
   int cap = 0;  // largest number of lattices one launch may hold

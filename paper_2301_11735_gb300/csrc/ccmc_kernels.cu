@@ -177,8 +177,8 @@ cudaError_t launch_gather_status(int64_t *const *ctls, int n, int64_t *out, cuda
 
 // Self-test of the bounded device waits: one CTA waits on an mbarrier that
 // nothing completes, polling at most `polls` times, then records the timeout in
-// *status and returns -- as the phase kernels' waits do on a bulk copy or an
-// arrival that never comes, so that the context stays usable.
+// *status and returns, so that the context stays usable.  (The sweep kernels wait
+// only at hardware barriers of their own block or cluster, and on their predecessor.)
 __global__ void wait_selftest_kernel(uint32_t polls, int *status) {
   __shared__ __align__(8) unsigned long long bar;
   const uint32_t a = (uint32_t)__cvta_generic_to_shared(&bar);

@@ -226,8 +226,10 @@ __device__ __forceinline__ void phase_word(const Geo &g, const PhaseSmem &sm,
 // are in flight together, and 32 warps an SM hide them behind the integer work that
 // bounds the phase.  (Staging tiles of class rows into shared memory by bulk copies,
 // with the last warp of a tile writing it back, held that rate too, but a phase then
-// began and ended with a tile's latency on every SM: 16384^2 28.5 us against 26.8
-// here, 4096^2 5.1 against 4.1, 2048^2 4.1 against 3.1.)  The prologue (tables, and
+// began and ended with a tile's latency on every SM: 16384^2 28.5 us against 26.6
+// here, 4096^2 5.1 against 4.1, 2048^2 4.1 against 3.0.)  Four CTAs of 64 registers an
+// SM: with 48 registers and five 16384^2 takes 28.0 us, with 56 and nine of 128 threads
+// 28.1, with 384-thread CTAs 27.0.  The prologue (tables, and
 // for a launch after the first of a chain the phase index and its schedule) runs
 // before the kernel waits for its predecessor.  Small lattices take small CTAs: a
 // thread's chain is what they wait for, and it is shorter on an SM of its own

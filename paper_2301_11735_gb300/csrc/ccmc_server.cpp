@@ -4,14 +4,14 @@
 // admitted as memory and slots free up, under a device-memory budget.  Every
 // admitted simulation keeps its lattice and random-stream position resident on
 // the GPU.  A scheduler thread advances all admitted simulations in slices: one
-// slice is one batched sweep launch (small lattices share one persistent
-// shared-memory launch, large ones run beside it on their own streams), each
+// slice is one batched sweep (small lattices held in shared memory, one launch a
+// shape, large ones beside them on their own streams), each
 // simulation advancing by as many sweeps as fit a slice's time budget.
 //
 // The GPU never waits for the host: the scheduler keeps two slices queued, so
 // slice k + 1 is on the device before slice k ends; a request is created and
 // initialised by work queued on its own stream (lattice memory comes from a
-// stream-ordered pool, so no call synchronises the device); a request that
+// pool that is kept, so no call synchronises the device); a request that
 // finishes in a slice has its results (latest exact recount, status, the
 // observable ring and the final state when asked) copied into pinned host
 // buffers by work queued behind its last sweep, and the scheduler collects
