@@ -22,6 +22,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <cmath>
 #include <condition_variable>
 #include <cstring>
 #include <deque>
@@ -95,12 +96,12 @@ int64_t ring_records(const ccmc_request &r) {
   return r.obs_every > 0 ? std::min<int64_t>(r.nsweeps / r.obs_every + 1, 1 << 16) : 1;
 }
 
-// Estimated wall time of one sweep, for sizing slices (measured: 3.5 us at 64^2, 11 at
-// 512^2, 19 at 1024^2, held in shared memory; 24 at 2048^2, 33 at 4096^2, 213 at
-// 16384^2, a launch a phase).
+// Estimated wall time of one sweep, for sizing slices (measured: 3.5 us at 64^2, 7.5 at
+// 256^2, 10.5 at 512^2, 15 to 18 at 1000^2, held in shared memory; 24 at 2048^2, 33 at
+// 4096^2, 213 at 16384^2, a launch a phase).
 double sweep_us(const ccmc_request &r) {
   const double N = (double)r.Lx * (double)r.Ly;
-  return N <= 1.2e6 ? 5.0 + 1.5e-5 * N : 22.0 + 0.7e-6 * N;
+  return N <= 1.2e6 ? 3.2 + 0.0145 * std::sqrt(N) : 22.0 + 0.7e-6 * N;
 }
 
 // Pinned host buffers, cached by power-of-two size (allocating pinned memory
@@ -281,7 +282,18 @@ void ccmc_server::run() {
   cudaSetDevice(device);
   int first_slices = 0;  // short slices left since the GPU ran dry
   for (;;) {
-    // (1) admission: first come, first served, while slots and budget allow
+    // (1) at most kSlicesInFlight slices queued: wait for the oldest; with nothing left to
+    // queue, for one at a time, so that what it finished is handed out before the next
+    // ends.  (Waiting after the admission instead, what arrived during the wait missed a
+    // slice.)
+    while ((int)slices.size() >= kSlicesInFlight || (!slices.empty() && active.empty())) {
+      cudaEventSynchronize(slices.front());
+      events.push_back(slices.front());
+      slices.pop_front();
+      if (active.empty()) break;
+    }
+
+    // (2) admission: first come, first served, while slots and budget allow
     std::vector<Pending> admit;
     {
       std::unique_lock<std::mutex> lock(mu);
@@ -333,25 +345,18 @@ void ccmc_server::run() {
         active.push_back(r);
     }
 
-    // (2) results that have landed
-    for (size_t i = 0; i < retiring.size();) {
-      if (collect(retiring[i])) {
-        retiring[i] = retiring.back();
-        retiring.pop_back();
-      } else {
-        ++i;
-      }
-    }
+    // (3) results that have landed, of those that landed together the smallest first
+    std::stable_sort(retiring.begin(), retiring.end(), [](const Retiring &a, const Retiring &b) {
+      return a.r.bytes < b.r.bytes;
+    });
+    size_t kept = 0;
+    for (size_t i = 0; i < retiring.size(); ++i)
+      if (!collect(retiring[i])) retiring[kept++] = retiring[i];
+    retiring.erase(retiring.begin() + (ptrdiff_t)kept, retiring.end());
 
-    // (3) at most kSlicesInFlight slices queued: wait for the oldest
-    while ((int)slices.size() >= kSlicesInFlight ||
-           (!slices.empty() && active.empty())) {
-      cudaEventSynchronize(slices.front());
-      events.push_back(slices.front());
-      slices.pop_front();
-    }
     if (active.empty()) {
-      if (!retiring.empty()) std::this_thread::sleep_for(std::chrono::microseconds(100));
+      if (slices.empty() && !retiring.empty())
+        std::this_thread::sleep_for(std::chrono::microseconds(100));
       continue;
     }
 
