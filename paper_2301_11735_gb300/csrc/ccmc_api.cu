@@ -224,16 +224,18 @@ int validate_shape(int Lx, int Ly) {
   return CCMC_OK;
 }
 
-void set_seed(ccmc_lattice *h, uint64_t seed) {
-  h->seed = seed;
-  h->g.k0 = (uint32_t)(seed & 0xFFFFFFFFu);
-  h->g.k1 = (uint32_t)(seed >> 32);
-}
-
+// (a graph that is still running is freed when it has ended)
 void drop_graphs(ccmc_lattice *h) {
   for (auto &e : h->graphs)
     if (e.exec) cudaGraphExecDestroy(e.exec);
   h->graphs.clear();
+}
+
+void set_seed(ccmc_lattice *h, uint64_t seed) {
+  if (seed != h->seed) drop_graphs(h);  // captured phases hold the seed's Philox keys
+  h->seed = seed;
+  h->g.k0 = (uint32_t)(seed & 0xFFFFFFFFu);
+  h->g.k1 = (uint32_t)(seed >> 32);
 }
 
 int upload_params_on(ccmc_lattice *h, double beta, double Delta, double V, double J,
