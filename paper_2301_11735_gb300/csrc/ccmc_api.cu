@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "../../include/ccmc.h"
@@ -913,6 +914,7 @@ struct ccmc_batch {
     int sweeps, obs_every;
     int64_t off;
     cudaGraphExec_t exec;
+    std::vector<std::pair<int64_t *, int>> hists;  // the members', held by its recounts
   };
   std::vector<MultiGraph> graphs;
 };
@@ -1054,11 +1056,21 @@ int enqueue_multi_chunk(ccmc_batch *b, const MultiGroup &G, int sweeps, int obs_
 }
 
 int run_multi_graph(ccmc_batch *b, const MultiGroup &G, int sweeps, int obs_every) {
-  for (auto &e : b->graphs)
-    if (e.members == G.m && e.sweeps == sweeps && e.obs_every == obs_every && e.off == G.off) {
+  std::vector<std::pair<int64_t *, int>> hists;
+  for (const ccmc_lattice *h : G.m) hists.emplace_back(h->d_hist, h->nbins);
+  for (size_t i = 0; i < b->graphs.size(); ++i) {
+    ccmc_batch::MultiGraph &e = b->graphs[i];
+    if (e.members != G.m || e.sweeps != sweeps || e.obs_every != obs_every || e.off != G.off)
+      continue;
+    if (e.hists == hists) {
       CK(cudaGraphLaunch(e.exec, b->stream));
       return CCMC_OK;
     }
+    // a member's histograms were enabled since: its captured recounts hold the old ones
+    cudaGraphExecDestroy(e.exec);
+    b->graphs.erase(b->graphs.begin() + (ptrdiff_t)i);
+    break;
+  }
   cudaGraph_t graph = nullptr;
   CK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
   const int rc = enqueue_multi_chunk(b, G, sweeps, obs_every);
@@ -1067,7 +1079,7 @@ int run_multi_graph(ccmc_batch *b, const MultiGroup &G, int sweeps, int obs_ever
     if (graph) cudaGraphDestroy(graph);
     return CCMC_E_CUDA;
   }
-  ccmc_batch::MultiGraph e{G.m, sweeps, obs_every, G.off, nullptr};
+  ccmc_batch::MultiGraph e{G.m, sweeps, obs_every, G.off, nullptr, hists};
   const cudaError_t ie = cudaGraphInstantiate(&e.exec, graph, 0);
   cudaGraphDestroy(graph);
   if (ie != cudaSuccess) return CCMC_E_CUDA;
