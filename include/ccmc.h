@@ -279,9 +279,19 @@ int ccmc_threshold_table(double beta, double Delta, double V, double J, uint32_t
  * CCMC_FAULT (comma-separated): "alloc" makes ccmc_lattice_create and
  * ccmc_batch_create return E_NOMEM before allocating anything, "launch" makes
  * ccmc_sweep, ccmc_phases and ccmc_batch_sweep return E_CUDA before queuing
- * anything (the handle stays usable), "admit" makes the server refuse every
- * request at admission (result status E_BUDGET). */
+ * anything (the handle stays usable), "cluster" makes ccmc_lattice_create take
+ * the device for one that places no thread-block cluster (the lattice is held by
+ * one CTA or swept a launch a phase, with the same results), "admit" makes the
+ * server refuse every request at admission (result status E_BUDGET). */
 int ccmc_selftest_wait(uint32_t polls);
+
+/* Diagnostic, host-only (no GPU needed): how ccmc_sweep holds an Lx x Ly lattice
+ * in shared memory on a device that places clusters of max_cluster CTAs (16, 8,
+ * 4, 2, 1; 0: a device that runs no such kernel).  plan receives the number of
+ * CTAs (0: the lattice is swept a launch a phase), the rows of each residue class
+ * a CTA owns, the threads that share a packed word, and a CTA's shared memory in
+ * bytes.  Errors: E_INVAL. */
+int ccmc_resident_plan(int Lx, int Ly, int max_cluster, int64_t plan[4]);
 
 /* Diagnostic: Philox4x32-10 on the device for counters (c0 + i mod 2^32, c1,
  * c2, c3), i < count, key (k0, k1); out receives 4 * count words (host buffer

@@ -90,6 +90,7 @@ def _load():
         "ccmc_sync": (c_int, [vp]),
         "ccmc_philox_device": (c_int, [c_uint32] * 6 + [c_int64, u32p]),
         "ccmc_selftest_wait": (c_int, [c_uint32]),
+        "ccmc_resident_plan": (c_int, [c_int, c_int, c_int, i64p]),
         "ccmc_peak_smem_read": (c_int, [POINTER(c_double)]),
         "ccmc_peak_l2_read": (c_int, [c_int64, POINTER(c_double)]),
         "ccmc_batch_create": (c_int, [c_int, POINTER(vp), vp, POINTER(vp)]),
@@ -158,6 +159,14 @@ def philox_device(ctr, key, count: int) -> np.ndarray:
                                    *[int(k) & 0xFFFFFFFF for k in key], count,
                                    out.ctypes.data_as(POINTER(c_uint32))), "ccmc_philox_device")
     return out.reshape(count, 4)
+
+
+def resident_plan(Lx: int, Ly: int, max_cluster: int = 16) -> dict:
+    """How Lattice.sweep holds such a lattice in shared memory where clusters of
+    max_cluster CTAs can be placed (ctas 0: it is swept a launch a phase)."""
+    out = (c_int64 * 4)()
+    _check(lib().ccmc_resident_plan(Lx, Ly, max_cluster, out), "ccmc_resident_plan")
+    return dict(zip(("ctas", "rows", "threads_per_word", "smem"), out))
 
 
 def selftest_wait(polls: int = 1 << 16) -> int:

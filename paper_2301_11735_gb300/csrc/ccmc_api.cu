@@ -188,7 +188,8 @@ struct ccmc_lattice {
   bool have_params = false;
   double params[4] = {0, 0, 0, 0};  // beta, Delta, V, J
   LaunchCfg cfg{};
-  bool resident = false;  // may be swept by the resident kernel
+  int max_cluster = 0;    // largest cluster its resident launches may take (0: none runs)
+  bool resident = false;  // swept by the resident kernel
   std::vector<GraphEntry> graphs;
   int32_t *d_maps = nullptr;  // paper-map mode: uploaded pairs
   int64_t map_cap = 0;        // int32 entries held by d_maps
@@ -202,7 +203,14 @@ namespace {
 // further on a launch of a phase's own is as fast (us a sweep resident and with a
 // launch a phase: 64^2 3.5, 16.9; 256^2 7.5, 18.3; 1000^2, ragged, 17.9, 23.6; 1024^2
 // 15.0, 21.4; 1200^2 22.6, 23.4; 1280^2 22.5, 22.1; 1536^2 33.3, 22.9).
-bool resident_default(const Geo &g) { return g.cstride <= 4608 && resident_possible(g); }
+bool resident_default(const Geo &g, int max_cluster) {
+  return g.cstride <= 4608 && resident_possible(g, max_cluster);
+}
+
+// How ccmc_sweep launches a lattice it holds in shared memory.
+ResShape resident_alone(const Geo &g, int max_cluster) {
+  return resident_shape(g, max_cluster, max_cluster, 0.0, kResMaxWorkers, 4);
+}
 
 // The move table, the same for every lattice (built and checked once: 25 us).
 struct MoveTable {
@@ -223,6 +231,19 @@ int validate_shape(int Lx, int Ly) {
   if (Lx < 4 || Ly < 4 || (Lx & 3) || (Ly & 3)) return CCMC_E_INVAL;
   if ((int64_t)Lx * (int64_t)Ly > ((int64_t)1 << 30)) return CCMC_E_INVAL;
   return CCMC_OK;
+}
+
+Geo geometry(int Lx, int Ly) {
+  Geo g{};
+  g.Lx = Lx;
+  g.Ly = Ly;
+  g.Cx = Lx / 4;
+  g.Cy = Ly / 4;
+  g.W = (g.Cx + 15) / 16;
+  g.cstride = (int64_t)g.Cy * g.W;
+  const uint64_t N = (uint64_t)Lx * (uint64_t)Ly;
+  g.rej = (0 - N) % N;
+  return g;
 }
 
 // (a graph that is still running is freed when it has ended)
@@ -322,7 +343,7 @@ ResJob resident_job(const ccmc_lattice *h, int64_t nsweeps, int obs_every, int r
 
 // Sweep one lattice by the resident kernel, a bounded number of sweeps a launch.
 int resident_sweeps(ccmc_lattice *h, int64_t nsweeps, int obs_every) {
-  const ResShape sh = resident_shape(h->g, kResMaxCluster, 0.0, kResMaxWorkers, 4);
+  const ResShape sh = resident_alone(h->g, h->max_cluster);
   for (int64_t s = 0; s < nsweeps; s += kResMaxSweeps) {
     const ResJob j =
         resident_job(h, std::min<int64_t>(nsweeps - s, kResMaxSweeps), obs_every, sh.rows);
@@ -415,18 +436,14 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
   ccmc_lattice *h = new (std::nothrow) ccmc_lattice();
   if (!h) return CCMC_E_NOMEM;
   Geo &g = h->g;
-  g.Lx = Lx;
-  g.Ly = Ly;
-  g.Cx = Lx / 4;
-  g.Cy = Ly / 4;
-  g.W = (g.Cx + 15) / 16;
-  g.cstride = (int64_t)g.Cy * g.W;
+  g = geometry(Lx, Ly);
   const uint64_t N = (uint64_t)Lx * (uint64_t)Ly;
-  g.rej = (0 - N) % N;
   h->cfg.phase_grid_cap = phase_resident_grid((g.Cx & 15) == 0);
   // any of these variables (tests) keeps the lattice on the phase kernels
-  h->resident = resident_default(g) && !std::getenv("CCMC_NO_TILE") &&
-                !std::getenv("CCMC_TILE_GRID") && !std::getenv("CCMC_NO_RESIDENT") && resident_ready();
+  h->max_cluster = resident_cluster_limit();
+  if (h->max_cluster > 1 && fault_injected("cluster")) h->max_cluster = 1;
+  h->resident = resident_default(g, h->max_cluster) && !std::getenv("CCMC_NO_TILE") &&
+                !std::getenv("CCMC_TILE_GRID") && !std::getenv("CCMC_NO_RESIDENT");
   while (((int64_t)1 << (2 * h->h)) < (int64_t)N) ++h->h;
   h->ring_cap = obs_capacity > 0 ? obs_capacity : 4096;
   cudaGetDevice(&h->device);
@@ -594,6 +611,20 @@ int ccmc_threshold_table(double beta, double Delta, double V, double J, uint32_t
       !std::isfinite(J))
     return CCMC_E_INVAL;
   build_thresholds(beta, Delta, V, J, out);
+  return CCMC_OK;
+}
+
+int ccmc_resident_plan(int Lx, int Ly, int max_cluster, int64_t *plan) {
+  if (!plan || max_cluster < 0 || max_cluster > kResMaxCluster ||
+      (max_cluster & (max_cluster - 1)) || validate_shape(Lx, Ly) != CCMC_OK)
+    return CCMC_E_INVAL;
+  const Geo g = geometry(Lx, Ly);
+  const ResShape sh =
+      resident_default(g, max_cluster) ? resident_alone(g, max_cluster) : ResShape{};
+  plan[0] = sh.cluster;
+  plan[1] = sh.rows;
+  plan[2] = sh.cluster ? sh.tpw : 0;
+  plan[3] = sh.smem;
   return CCMC_OK;
 }
 
@@ -925,7 +956,7 @@ namespace {
 // what ccmc_sweep would hold.
 bool batch_resident(const ccmc_batch *b, const ccmc_lattice *h) {
   if (b->resident_max_sites < 0) return h->resident;
-  return 16 * h->g.cstride * 16 <= b->resident_max_sites;
+  return h->max_cluster > 0 && 16 * h->g.cstride * 16 <= b->resident_max_sites;
 }
 
 // A resident launch of a batch: lattices of one shape.
@@ -971,7 +1002,8 @@ int run_resident(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats,
   for (int i : which) {
     const Geo &g = lats[i]->g;
     plans.push_back({i,
-                     resident_shape(g, ctas * (double)g.cstride * (double)nsweeps[i] / work,
+                     resident_shape(g, lats[i]->max_cluster,
+                                    ctas * (double)g.cstride * (double)nsweeps[i] / work,
                                     words / b->sms, b->threads, b->max_tpw),
                      (g.Cx & 15) == 0});
   }
@@ -985,7 +1017,7 @@ int run_resident(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats,
     if (sh.cluster > 1) {
       int n = 0;
       for (const Plan &o : plans) n += same(o.shape, p.shape);
-      sh = resident_fit(h->g, sh, p.aligned, n);
+      sh = resident_fit(h->g, h->max_cluster, sh, p.aligned, n);
     }
     ResGroup *hit = nullptr;
     for (ResGroup &G : groups)
@@ -1292,7 +1324,6 @@ int ccmc::batch_new(int cap, cudaStream_t stream, ccmc_batch **out) {
   b->d_jobs = (ResJob *)b->d_slab;
   b->d_multi = (MultiJob *)((char *)b->d_slab + o_multi);
   b->d_ctls = (int64_t **)((char *)b->d_slab + o_ctls);
-  if (!resident_ready()) return fail(CCMC_E_CUDA);
   if (cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming) != cudaSuccess)
     return fail(CCMC_E_CUDA);
   b->lat_ev.assign(count, nullptr);

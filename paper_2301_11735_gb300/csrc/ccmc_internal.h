@@ -163,21 +163,23 @@ cudaError_t launch_set_ctl(int64_t *ctl, int64_t phase_base, cudaStream_t s);
 cudaError_t launch_gather_status(int64_t *const *ctls, int n, int64_t *out, cudaStream_t s);
 cudaError_t launch_unpack(const Geo &g, uint8_t *out, cudaStream_t s);
 cudaError_t launch_pack(const Geo &g, const uint8_t *in, int *bad, cudaStream_t s);
-// Resident sweeps (ccmc_resident.cu): whether the current device can run them
-// (raises the kernels' limits once per device; call outside a capture), a CTA's
-// shared memory for `rows` rows of every class, and the launch of `one` lattice or
+// Resident sweeps (ccmc_resident.cu): the most CTAs in a cluster (16, 8, 4, 2 or 1)
+// that the current device places for any shape of the kernels, 0 when they cannot run
+// there (raises the kernels' limits once per device; call outside a capture); a CTA's
+// shared memory for `rows` rows of every class; and the launch of `one` lattice or
 // of the njobs lattices of d_jobs (in device memory), all of one shape.
-bool resident_ready();
+int resident_cluster_limit();
 int64_t resident_smem(const Geo &g, int rows);
 // The launch shape of a lattice that may take `ctas` CTAs of the GPU (at least
-// one) while `load` a-words a phase run on an average SM, with at most
-// max_threads workers a CTA and max_tpw threads a word.
-ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads, int max_tpw);
+// one), clusters of max_cluster at most, while `load` a-words a phase run on an
+// average SM, with at most max_threads workers a CTA and max_tpw threads a word.
+ResShape resident_shape(const Geo &g, int max_cluster, double ctas, double load, int max_threads,
+                        int max_tpw);
 // Whether the lattice fits shared memory in some shape.
-bool resident_possible(const Geo &g);
+bool resident_possible(const Geo &g, int max_cluster);
 // The shape for n such lattices in one launch: another one when their clusters
 // would not all fit the GPU at once.
-ResShape resident_fit(const Geo &g, const ResShape &shape, bool aligned, int n);
+ResShape resident_fit(const Geo &g, int max_cluster, const ResShape &shape, bool aligned, int n);
 cudaError_t launch_resident_sweep(const ResJob *one, const ResJob *d_jobs, int njobs,
                                   const ResShape &shape, bool aligned, cudaStream_t s);
 cudaError_t launch_philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,

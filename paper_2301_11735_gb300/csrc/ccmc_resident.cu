@@ -798,7 +798,7 @@ Kernel kernel_of(bool cluster, bool aligned, int tpw) {
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
-bool g_ready[kMaxDevices] = {};
+int g_limit[kMaxDevices] = {};  // resident_cluster_limit + 1, 0: not asked yet
 
 void launch_config(const ResShape &shape, int njobs, cudaStream_t s, cudaLaunchConfig_t &cfg,
                    cudaLaunchAttribute *attr) {
@@ -814,33 +814,53 @@ void launch_config(const ResShape &shape, int njobs, cudaStream_t s, cudaLaunchC
   cfg.numAttrs = shape.cluster > 1 ? 1 : 0;
 }
 
-// Raises every instance's shared-memory limit and allows clusters of 16, once
-// per device (outside any capture: called when a lattice or a batch is created).
-bool prepare_device(int dev) {
-  if (dev < 0 || dev >= kMaxDevices) return false;
-  std::lock_guard<std::mutex> lock(g_mu);
-  if (g_ready[dev]) return true;
+// Raises every instance's shared-memory limit and allows clusters of 16 (outside any
+// capture: called when a lattice is created), then asks for the largest cluster that
+// the device places with the most threads and shared memory a CTA may have: a part of
+// a GPU may have no sixteen SMs side by side, and its lattices then take smaller
+// clusters or a launch a phase.  (A whole GB300 holds seven such clusters of 16.)
+int cluster_limit() {
   for (int c = 0; c < 2; ++c)
     for (int a = 0; a < 2; ++a)
-      for (int t : {1, 2, 4}) {
-        const void *f = reinterpret_cast<const void *>(kernel_of(c, a, t));
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kResMaxSmem) !=
-                cudaSuccess ||
-            (c && cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-                      cudaSuccess)) {
+      for (int t : {1, 2, 4})
+        if (cudaFuncSetAttribute(reinterpret_cast<const void *>(kernel_of(c, a, t)),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kResMaxSmem) != cudaSuccess) {
           cudaGetLastError();
-          return false;
+          return 0;
         }
+  for (int C = kResMaxCluster; C > 1; C /= 2) {
+    bool ok = true;
+    for (int a = 0; a < 2; ++a)
+      for (int t : {1, 2, 4}) {
+        const void *f = reinterpret_cast<const void *>(kernel_of(true, a, t));
+        ResShape most;
+        most.cluster = C;
+        most.threads = kResMaxThreads;
+        most.smem = kResMaxSmem;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr[1];
+        launch_config(most, 1, nullptr, cfg, attr);
+        int n = 0;
+        ok = ok &&
+             cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, C > 8) ==
+                 cudaSuccess &&
+             cudaOccupancyMaxActiveClusters(&n, f, &cfg) == cudaSuccess && n > 0;
       }
-  g_ready[dev] = true;
-  return true;
+    if (ok) return C;
+    cudaGetLastError();
+  }
+  return 1;
 }
 
 }  // namespace
 
-bool resident_ready() {
+int resident_cluster_limit() {
   int dev = 0;
-  return cudaGetDevice(&dev) == cudaSuccess && prepare_device(dev);
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+  std::lock_guard<std::mutex> lock(g_mu);
+  if (!g_limit[dev]) g_limit[dev] = cluster_limit() + 1;
+  return g_limit[dev] - 1;
 }
 
 int64_t resident_smem(const Geo &g, int rows) {
@@ -877,13 +897,14 @@ static ResShape shape_of(const Geo &g, int C, int tpw, int max_workers) {
 // 256^2 and 128 of 64^2 34 against 23; 512 replicas: 28 against 14.7), while a
 // 416-thread CTA finds no room beside another (512 replicas: 18.5 with four lanes for
 // their 128^2 lattices, 14.7 with one thread).
-ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads, int max_tpw) {
+ResShape resident_shape(const Geo &g, int max_cluster, double ctas, double load, int max_threads,
+                        int max_tpw) {
   int C = 1;
   if (g.cstride >= kResClusterWords)
-    while (C < kResMaxCluster && 2 * C <= ctas && g.cstride >= 2 * C * kResMinWords &&
+    while (C < max_cluster && 2 * C <= ctas && g.cstride >= 2 * C * kResMinWords &&
            g.Cy >= 4 * C)  // two rows a CTA at least
       C *= 2;
-  while (C < kResMaxCluster && g.Cy >= 4 * C && resident_smem(g, (g.Cy + C - 1) / C) > kResMaxSmem)
+  while (C < max_cluster && g.Cy >= 4 * C && resident_smem(g, (g.Cy + C - 1) / C) > kResMaxSmem)
     C *= 2;
   const int words = (g.Cy + C - 1) / C * g.W;
   const bool crowded = load > 128.0;
@@ -897,15 +918,16 @@ ResShape resident_shape(const Geo &g, double ctas, double load, int max_threads,
   return shape_of(g, C, tpw, max_threads);
 }
 
-bool resident_possible(const Geo &g) {
-  return resident_shape(g, kResMaxCluster, 0.0, kResMaxWorkers, 1).smem <= kResMaxSmem;
+bool resident_possible(const Geo &g, int max_cluster) {
+  return max_cluster > 0 && resident_shape(g, max_cluster, max_cluster, 0.0, kResMaxWorkers, 1)
+                                    .smem <= kResMaxSmem;
 }
 
 // Clusters of eight full CTAs do not all find eight free SMs of one processing
 // cluster: for 16 lattices of 1024^2 two waited for the others (54 us a sweep).
 // CTAs of 128 workers that take their words in several passes fit four to an SM:
 // 37 us (eight CTAs of 256 workers, two to an SM: 43).
-ResShape resident_fit(const Geo &g, const ResShape &shape, bool aligned, int n) {
+ResShape resident_fit(const Geo &g, int max_cluster, const ResShape &shape, bool aligned, int n) {
   auto fits = [&](const ResShape &sh) {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
@@ -920,7 +942,8 @@ ResShape resident_fit(const Geo &g, const ResShape &shape, bool aligned, int n) 
     return n <= most;
   };
   if (shape.cluster == 1 || fits(shape)) return shape;
-  if (g.cstride >= kResMaxCluster * 128 && g.Cy >= 2 * kResMaxCluster) {
+  if (max_cluster == kResMaxCluster && g.cstride >= kResMaxCluster * 128 &&
+      g.Cy >= 2 * kResMaxCluster) {
     const ResShape wide = shape_of(g, kResMaxCluster, 1, std::min(128, shape.workers));
     if (fits(wide)) return wide;
   }
