@@ -279,7 +279,9 @@ int ccmc_threshold_table(double beta, double Delta, double V, double J, uint32_t
  * CCMC_FAULT (comma-separated): "alloc" makes ccmc_lattice_create and
  * ccmc_batch_create return E_NOMEM before allocating anything, "launch" makes
  * ccmc_sweep, ccmc_phases and ccmc_batch_sweep return E_CUDA before queuing
- * anything (the handle stays usable), "cluster" makes ccmc_lattice_create take
+ * anything (the handle stays usable), "group" makes ccmc_batch_sweep return
+ * E_CUDA at its second resident launch, once what it queued has ended,
+ * "cluster" makes ccmc_lattice_create take
  * the device for one that places no thread-block cluster (the lattice is held by
  * one CTA or swept a launch a phase, with the same results), "admit" makes the
  * server refuse every request at admission (result status E_BUDGET). */

@@ -1051,6 +1051,7 @@ int run_resident(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats,
   for (int k = 0; k < n; ++k) {
     const ResGroup &G = groups[k];
     const int on = k % (side + 1);
+    if (k == 1 && fault_injected("group")) return CCMC_E_CUDA;
     CK(launch_resident_sweep(nullptr, b->d_jobs + off, (int)G.jobs.size(), G.shape, G.aligned,
                              on == 0 ? b->stream : b->side[on - 1]));
     off += (int64_t)G.jobs.size();
@@ -1166,25 +1167,11 @@ int run_multi(ccmc_batch *b, MultiGroup &G, int64_t nsweeps, int obs_every) {
   return CCMC_OK;
 }
 
-}  // namespace
-
-namespace ccmc {
-
-int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int64_t *nsweeps,
-              const double *beta, const double *Delta, const double *V, const double *J,
-              const int *obs_every, bool lockstep) {
+// Queues the sweeps of lattices that batch_run has checked.
+int batch_queue(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int64_t *nsweeps,
+                const double *beta, const double *Delta, const double *V, const double *J,
+                const int *obs_every, bool lockstep) {
   const int n = (int)lats.size();
-  if (n > b->cap) return CCMC_E_INVAL;
-  TraceRange trace("ccmc_batch_run");
-  for (int i = 0; i < n; ++i) {
-    if (nsweeps[i] < 0 || !(beta[i] >= 0.0) || !std::isfinite(Delta[i]) ||
-        !std::isfinite(V[i]) || !std::isfinite(J[i]))
-      return CCMC_E_INVAL;
-    ccmc_lattice *h = lats[i];
-    if (!h || !h->initialised || h->phases_done % 8) return CCMC_E_STATE;
-    for (int k = 0; k < i; ++k)
-      if (lats[k] == h) return CCMC_E_INVAL;  // a lattice may appear once
-  }
   std::vector<int> resident;
   for (int i = 0; i < n; ++i) {
     ccmc_lattice *h = lats[i];
@@ -1266,6 +1253,35 @@ int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int6
     }
   }
   return CCMC_OK;
+}
+
+}  // namespace
+
+namespace ccmc {
+
+int batch_run(ccmc_batch *b, const std::vector<ccmc_lattice *> &lats, const int64_t *nsweeps,
+              const double *beta, const double *Delta, const double *V, const double *J,
+              const int *obs_every, bool lockstep) {
+  const int n = (int)lats.size();
+  if (n > b->cap) return CCMC_E_INVAL;
+  TraceRange trace("ccmc_batch_run");
+  for (int i = 0; i < n; ++i) {
+    if (nsweeps[i] < 0 || !(beta[i] >= 0.0) || !std::isfinite(Delta[i]) ||
+        !std::isfinite(V[i]) || !std::isfinite(J[i]))
+      return CCMC_E_INVAL;
+    ccmc_lattice *h = lats[i];
+    if (!h || !h->initialised || h->phases_done % 8) return CCMC_E_STATE;
+    for (int k = 0; k < i; ++k)
+      if (lats[k] == h) return CCMC_E_INVAL;  // a lattice may appear once
+  }
+  const int rc = batch_queue(b, lats, nsweeps, beta, Delta, V, J, obs_every, lockstep);
+  if (rc != CCMC_OK) {
+    // some launches may be queued that no lattice's stream waits for: they end before
+    // the caller may destroy a lattice and its memory goes to another
+    cudaStreamSynchronize(b->stream);
+    for (cudaStream_t x : b->side) cudaStreamSynchronize(x);
+  }
+  return rc;
 }
 
 }  // namespace ccmc

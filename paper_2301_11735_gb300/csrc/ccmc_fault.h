@@ -5,6 +5,8 @@
 //            before anything is allocated or any CUDA call is made;
 //   launch : sweep calls fail as if a kernel launch failed (CCMC_E_CUDA),
 //            before anything is queued, leaving the handle usable;
+//   group  : a batched sweep's second resident launch fails (CCMC_E_CUDA), the
+//            first having been queued;
 //   cluster: lattices are created as if the device placed no cluster of CTAs;
 //   admit  : the server refuses every request at admission as if it could
 //            never fit the memory budget (result status CCMC_E_BUDGET).
