@@ -119,11 +119,12 @@ void dfree(void *p, int dev) {
 
 // Pinned host buffers through which short results reach the caller: a copy or a
 // kernel writes the buffer, one synchronisation, then a host copy (a copy to
-// pageable memory stages and waits inside the driver: 24 us for a 16 KB state
-// instead of 10).  At most kStages of kStageBytes for the process, lent for the
+// pageable memory stages and waits inside the driver: 15.5 us for a 16 KB state
+// instead of 12.1).  At most kStages of kStageBytes for the process, lent for the
 // length of one call; a caller that finds none takes the pageable path.
 constexpr size_t kStageBytes = (size_t)1 << 20;
-constexpr size_t kStateBytes = (size_t)256 << 10;  // lattice states at most this long
+constexpr size_t kDirectBytes = (size_t)64 << 10;  // lattice states (see read_state)
+constexpr size_t kStateBytes = (size_t)256 << 10;  // and those that nothing waits for
 constexpr int kStages = 8;
 std::mutex g_stage_mu;
 std::vector<void *> g_stage_free;
@@ -834,16 +835,19 @@ int ccmc_hist_get(ccmc_lattice *h, int64_t *out) {
 
 }  // extern "C"
 
-// Hands `n` bytes of state made by `make(device pointer)` to the caller: short ones
-// through a pinned buffer, which the kernel writes itself when its rows are whole
-// 16-byte groups (wide) or there are few of them (1648 x 2048 in single bytes: 80 us
-// more than a copy).
+// Hands `n` bytes of state made by `make(device pointer)` to the caller: at most
+// `direct` of them through a pinned buffer that the kernel writes itself, longer ones by
+// a copy from device memory, which the driver stages.  (us a call, written into a pinned
+// buffer and copied by the driver: 4 KB 11.4 and 15.2, 64 KB 15.2 and 15.6, 96 KB 17.2 and
+// 17.1, 256 KB 26.5 and 17.3; packed rows written in single bytes 12 KB 16.4 and 17.5,
+// 16 KB 17.7 and 18.5, 24 KB 19.4 and 17.3, 64 KB 24.2 and 17.4.  A copy to the pinned
+// buffer and another on the host is never the fastest.)
 template <typename Make>
-static int read_state(ccmc_lattice *h, uint8_t *host_out, size_t n, bool wide, Make make) {
+static int read_state(ccmc_lattice *h, uint8_t *host_out, size_t n, size_t direct, Make make) {
   if (!h || !host_out) return CCMC_E_INVAL;
   if (!h->initialised) return CCMC_E_STATE;
-  Stage st(n <= kStateBytes ? n : kStageBytes + 1);  // longer ones: the driver's own staging
-  if (st && (wide || n <= 4096)) {
+  Stage st(n <= direct ? n : kStageBytes + 1);
+  if (st) {
     CK(make(st.as<uint8_t>()));
     CK(cudaStreamSynchronize(h->stream));
     std::memcpy(host_out, st.as<uint8_t>(), n);
@@ -851,10 +855,8 @@ static int read_state(ccmc_lattice *h, uint8_t *host_out, size_t n, bool wide, M
     const int rc = ensure_bytes(h);
     if (rc) return rc;
     CK(make(h->d_bytes));
-    CK(cudaMemcpyAsync(st ? st.as<uint8_t>() : host_out, h->d_bytes, n, cudaMemcpyDeviceToHost,
-                       h->stream));
+    CK(cudaMemcpyAsync(host_out, h->d_bytes, n, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    if (st) std::memcpy(host_out, st.as<uint8_t>(), n);
   }
   h->queued = false;
   return CCMC_OK;
@@ -863,12 +865,13 @@ static int read_state(ccmc_lattice *h, uint8_t *host_out, size_t n, bool wide, M
 extern "C" {
 
 int ccmc_get_state(ccmc_lattice *h, uint8_t *host_out) {
-  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly : 0, h && h->g.Lx % 16 == 0,
+  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly : 0, kDirectBytes,
                     [&](uint8_t *to) { return launch_unpack(h->g, to, h->stream); });
 }
 
 int ccmc_get_state_packed(ccmc_lattice *h, uint8_t *host_out) {
-  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly / 4 : 0, h && h->g.Lx % 64 == 0,
+  return read_state(h, host_out, h ? (size_t)h->g.Lx * h->g.Ly / 4 : 0,
+                    h && h->g.Lx % 64 ? kDirectBytes / 4 : kDirectBytes,
                     [&](uint8_t *to) { return launch_unpack2(h->g, to, h->stream); });
 }
 
