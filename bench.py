@@ -331,6 +331,7 @@ def measure_batched(cc, nsweeps=5000, plain_per_size=4):
         lats.append(lat)
     with cc.Batch(lats) as b:
         cfg = b.autotune(probe_sweeps=200)
+        configured = b.configured is not None
         b.sweep(3, *cols)
         b.sync()
         torch.cuda.synchronize()
@@ -363,7 +364,7 @@ def measure_batched(cc, nsweeps=5000, plain_per_size=4):
                         "Delta~U{-.5,0,.5}, V=J=1, 5000 sweeps",
             "value": work / dt, "unit": "site-updates/s", "seconds": dt,
             "config": {"threads": cfg[0], "resident_max_sites": cfg[1], "ctas_per_sm": cfg[2],
-                       "max_threads_per_word": cfg[3]},
+                       "max_threads_per_word": cfg[3]} if configured else "library's plan",
             "plain_back_to_back": {"value": plain, "unit": "site-updates/s",
                                    "sample": f"{len(picked)} of the lattices ({plain_per_size} of "
                                              f"each size), the full {nsweeps} sweeps each, one "
@@ -396,7 +397,8 @@ def measure_small(cc, reps=3):
             best = min(best, time.perf_counter() - t0)
         out["plain_us_per_sweep"] = 1e6 * best / nsw
         with cc.Batch([lat]) as b:
-            out["batched_config"] = list(b.autotune(probe_sweeps=200))
+            cfg = b.autotune(probe_sweeps=200)
+            out["batched_config"] = list(cfg) if b.configured else "library's plan"
             cols = ([beta], [c["Delta"]], [c["V"]], [c["J"]])
             b.sweep(20, *cols, obs_every=1)
             b.sync()

@@ -339,25 +339,37 @@ class Batch:
 
     def __init__(self, lattices, stream=None):
         self.lattices = list(lattices)
+        self._stream = stream
+        self._create()
+
+    def _create(self):
         arr = (c_void_p * len(self.lattices))(*[lat.handle.value for lat in self.lattices])
         h = c_void_p()
-        _check(lib().ccmc_batch_create(len(self.lattices), arr, _stream_handle(stream),
+        _check(lib().ccmc_batch_create(len(self.lattices), arr, _stream_handle(self._stream),
                                        ctypes.byref(h)), "ccmc_batch_create")
         self._h = h
+        self.configured = None  # the launch shape given by config(), None: the library's plan
 
     def config(self, threads: int = 256, resident_max_sites: int = 1 << 17, ctas_per_sm: int = 2,
                max_threads_per_word: int = 4):
         _check(lib().ccmc_batch_config(self._h, threads, resident_max_sites, ctas_per_sm,
                                        max_threads_per_word), "ccmc_batch_config")
+        self.configured = (threads, resident_max_sites, ctas_per_sm, max_threads_per_word)
 
     def autotune(self, probe_sweeps: int = 20):
-        """Time the candidate launch shapes on a probe batch of the same shapes
-        (cached per GPU and shape mix) and apply the fastest."""
+        """Time the library's own plan and the candidate launch shapes on a probe batch
+        of the same shapes (cached per GPU and shape mix) and apply the
+        fastest; returns the fastest candidate (`configured` is None when the library's
+        plan was faster)."""
         from . import autotune
 
-        best = autotune.tune([(lat.Lx, lat.Ly) for lat in self.lattices], probe_sweeps)
-        self.config(*best)
-        return best
+        m = autotune.measured([(lat.Lx, lat.Ly) for lat in self.lattices], probe_sweeps)
+        if not m["plan"]:
+            self.config(*m["config"])
+        elif self.configured is not None:  # back to a batch that was never configured
+            self.close()
+            self._create()
+        return tuple(m["config"])
 
     def sweep(self, nsweeps, beta, Delta, V, J, obs_every: int = 0):
         n = len(self.lattices)

@@ -9,9 +9,9 @@ the pairs each thread evaluates, 16, 8 or 4).  None of them changes results -- t
 streams are keyed by (seed, phase, site) -- so the tuner may pick freely.
 
 A probe batch of synthetic lattices with the same shapes is swept for a few
-sweeps under every candidate, twice (the faster probe counts); the fastest
-candidate is cached in a JSON file
-(paper_2301_11735_gb300/_build/autotune.json) keyed by the GPU name and the
+sweeps under the library's own plan (a batch that was never configured) and under
+every candidate, twice each (the faster probe counts).  The times are cached in a
+JSON file (paper_2301_11735_gb300/_build/autotune.json) keyed by the GPU name and the
 batch's shape signature.
 """
 from __future__ import annotations
@@ -69,14 +69,11 @@ def _store(cache):
     os.replace(tmp, _CACHE)
 
 
-def tune(shapes, probe_sweeps: int = 20, params=(1.0, 0.0, 1.0, 1.0), use_cache: bool = True):
-    """Best (threads, resident_max_sites, ctas_per_sm) for a batch of `shapes`."""
+def _probe(shapes, probe_sweeps, params):
+    """Seconds of probe_sweeps sweeps of a batch of `shapes`, by launch shape (None:
+    the library's own plan)."""
     import paper_2301_11735_gb300 as cc
 
-    key = f"{_gpu_name()}|{signature(shapes)}|{len(DEFAULT)}"
-    cache = _load() if use_cache else {}
-    if key in cache:
-        return tuple(cache[key]["config"])
     lats = []
     for i, (Lx, Ly) in enumerate(shapes):
         lat = cc.Lattice(Lx, Ly)
@@ -84,11 +81,12 @@ def tune(shapes, probe_sweeps: int = 20, params=(1.0, 0.0, 1.0, 1.0), use_cache:
         lats.append(lat)
     timings = {}
     with cc.Batch(lats) as b:
-        for cand in CANDIDATES:
-            try:
-                b.config(*cand)
-            except cc.CcmcError:
-                continue
+        for cand in [None] + CANDIDATES:
+            if cand is not None:
+                try:
+                    b.config(*cand)
+                except cc.CcmcError:
+                    continue
             b.sweep(2, *params)  # warm-up
             b.sync()
             best = float("inf")
@@ -100,10 +98,32 @@ def tune(shapes, probe_sweeps: int = 20, params=(1.0, 0.0, 1.0, 1.0), use_cache:
             timings[cand] = best
     for lat in lats:
         lat.close()
-    if not timings:
-        return DEFAULT
-    best = min(timings, key=timings.get)
-    cache[key] = {"config": list(best),
-                  "timings_ms": {str(list(c)): 1e3 * t for c, t in timings.items()}}
-    _store(cache)
-    return best
+    return timings
+
+
+def measured(shapes, probe_sweeps: int = 20, params=(1.0, 0.0, 1.0, 1.0),
+             use_cache: bool = True) -> dict:
+    """What the probes of a batch of `shapes` say: "config", the fastest candidate;
+    "plan", whether a batch that is not configured at all is at least as fast (one with
+    lattices of more than about 360 x 360 is, which no candidate holds in shared memory:
+    20 of 512 x 512 take 15 us a sweep, not 40); "timings_ms"."""
+    key = f"{_gpu_name()}|{signature(shapes)}|{len(DEFAULT)} plan"
+    cache = _load() if use_cache else {}
+    if key not in cache:
+        timings = _probe(shapes, probe_sweeps, params)
+        configs = {c: t for c, t in timings.items() if c is not None}
+        best = min(configs, key=configs.get) if configs else DEFAULT
+        entry = {"config": list(best),
+                 "plan": None in timings and timings[None] <= configs.get(best, float("inf")),
+                 "timings_ms": {str(c and list(c)): 1e3 * t for c, t in timings.items()}}
+        if not configs:
+            return entry
+        cache[key] = entry
+        _store(cache)
+    return cache[key]
+
+
+def tune(shapes, probe_sweeps: int = 20, params=(1.0, 0.0, 1.0, 1.0), use_cache: bool = True):
+    """Best (threads, resident_max_sites, ctas_per_sm, max_threads_per_word) for a batch
+    of `shapes`, of the candidates."""
+    return tuple(measured(shapes, probe_sweeps, params, use_cache)["config"])
