@@ -358,7 +358,7 @@ class Batch:
 
     def autotune(self, probe_sweeps: int = 20):
         """Time the library's own plan and the candidate launch shapes on a probe batch
-        of the same shapes (cached per GPU and shape mix) and apply the
+        of the same shapes (cached per GPU, shape mix and library sources) and apply the
         fastest; returns the fastest candidate (`configured` is None when the library's
         plan was faster)."""
         from . import autotune

@@ -11,8 +11,9 @@ streams are keyed by (seed, phase, site) -- so the tuner may pick freely.
 A probe batch of synthetic lattices with the same shapes is swept for a few
 sweeps under the library's own plan (a batch that was never configured) and under
 every candidate, twice each (the faster probe counts).  The times are cached in a
-JSON file (paper_2301_11735_gb300/_build/autotune.json) keyed by the GPU name and the
-batch's shape signature.
+JSON file (paper_2301_11735_gb300/_build/autotune.json) keyed by the GPU name, the
+batch's shape signature and a digest of the library's sources: times taken with
+other kernels say nothing about these.
 """
 from __future__ import annotations
 
@@ -51,6 +52,17 @@ def signature(shapes) -> str:
         counts[tuple(s)] = counts.get(tuple(s), 0) + 1
     key = ",".join(f"{a}x{b}:{n}" for (a, b), n in sorted(counts.items()))
     return hashlib.sha1(key.encode()).hexdigest()[:16]
+
+
+def _sources() -> str:
+    """Digest of the sources that the library is built from."""
+    h = hashlib.sha1()
+    here = os.path.dirname(os.path.abspath(__file__))
+    for d in (os.path.join(here, "csrc"), os.path.join(os.path.dirname(here), "include")):
+        for name in sorted(os.listdir(d)):
+            with open(os.path.join(d, name), "rb") as f:
+                h.update(name.encode() + b"\0" + f.read())
+    return h.hexdigest()[:16]
 
 
 def _load():
@@ -107,7 +119,7 @@ def measured(shapes, probe_sweeps: int = 20, params=(1.0, 0.0, 1.0, 1.0),
     "plan", whether a batch that is not configured at all is at least as fast (one with
     lattices of more than about 360 x 360 is, which no candidate holds in shared memory:
     20 of 512 x 512 take 15 us a sweep, not 40); "timings_ms"."""
-    key = f"{_gpu_name()}|{signature(shapes)}|{len(DEFAULT)} plan"
+    key = f"{_gpu_name()}|{signature(shapes)}|{len(DEFAULT)}|{_sources()}"
     cache = _load() if use_cache else {}
     if key not in cache:
         timings = _probe(shapes, probe_sweeps, params)

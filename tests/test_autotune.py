@@ -1,7 +1,7 @@
 """What the autotuner makes of its probes (given ones here: no GPU): a batch stays on
-the library's own plan where no candidate is faster, and the fastest candidate is
-returned either way.  On the GPU: batches that stay on the plan, go back to it
-and leave it."""
+the library's own plan where no candidate is faster, the fastest candidate is returned
+either way, and times taken with other kernels are not used again.  On the GPU: batches
+that stay on the plan, go back to it and leave it."""
 import numpy as np
 import pytest
 
@@ -29,6 +29,15 @@ def test_the_plan_competes_with_the_candidates(probes, plan, best):
     m = autotune.measured(SHAPES)
     assert m["plan"] == (plan <= best)
     assert tuple(m["config"]) == autotune.tune(SHAPES) == fast
+
+
+def test_times_of_other_kernels_are_taken_again(probes, monkeypatch):
+    calls = probes({None: 1.0, autotune.DEFAULT: 2.0})
+    for digest, probed in (("a", 1), ("a", 1), ("b", 2), ("a", 2)):
+        monkeypatch.setattr(autotune, "_sources", lambda: digest)
+        assert autotune.tune(SHAPES) == autotune.DEFAULT
+        assert len(calls) == probed
+    assert autotune.measured(SHAPES[:2])["plan"] and len(calls) == 3
 
 
 def test_a_gpu_that_takes_no_candidate_keeps_the_plan(probes):
