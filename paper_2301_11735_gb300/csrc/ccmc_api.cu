@@ -440,6 +440,10 @@ int ccmc::lattice_new(int Lx, int Ly, void *cuda_stream, int64_t obs_capacity, b
   g = geometry(Lx, Ly);
   const uint64_t N = (uint64_t)Lx * (uint64_t)Ly;
   h->cfg.phase_grid_cap = phase_resident_grid((g.Cx & 15) == 0);
+  // CCMC_TILE_GRID=n (tests): at most n CTAs a phase, so that small lattices take
+  // several rounds of words a CTA
+  if (const char *e = std::getenv("CCMC_TILE_GRID"))
+    if (const int n = std::atoi(e); n > 0) h->cfg.phase_grid_cap = std::min(n, h->cfg.phase_grid_cap);
   // any of these variables (tests) keeps the lattice on the phase kernels
   h->max_cluster = resident_cluster_limit();
   if (h->max_cluster > 1 && fault_injected("cluster")) h->max_cluster = 1;
@@ -1129,7 +1133,7 @@ int run_multi_graph(ccmc_batch *b, const MultiGroup &G, int sweeps, int obs_ever
 int run_multi(ccmc_batch *b, MultiGroup &G, int64_t nsweeps, int obs_every) {
   int64_t words = 0;
   for (ccmc_lattice *h : G.m) words += (int64_t)h->g.Cy * h->g.W;
-  const int wave = phase_resident_grid(G.aligned);
+  const int wave = G.m[0]->cfg.phase_grid_cap;  // the same for all of one alignment
   std::vector<MultiJob> jobs;
   int begin = 0;
   for (ccmc_lattice *h : G.m) {
