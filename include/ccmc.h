@@ -148,8 +148,10 @@ int ccmc_batch_sync(ccmc_batch *b);
  * admitted first come first served while fewer than max_active are running and
  * their device memory fits the budget (a request that can never fit finishes
  * with E_BUDGET).  Admitted simulations stay resident on the GPU; a scheduler
- * thread advances all of them in slices of about slice_ms (each slice is one
- * batched launch, ccmc_batch_*), so requests that arrive while others run
+ * thread advances all of them in slices (one batched call each, as
+ * ccmc_batch_sweep): every simulation by as many sweeps as it would make in
+ * slice_ms alone, at least one or one interval of its records, so that a slice
+ * of many simulations takes longer.  Requests that arrive while others run
  * join at the next slice and leave as soon as they are done.  Results equal
  * those of running each request alone.  Times are seconds since the server
  * started (host clock). */

@@ -231,6 +231,9 @@ const MoveTable &move_table() {
 int validate_shape(int Lx, int Ly) {
   if (Lx < 4 || Ly < 4 || (Lx & 3) || (Ly & 3)) return CCMC_E_INVAL;
   if ((int64_t)Lx * (int64_t)Ly > ((int64_t)1 << 30)) return CCMC_E_INVAL;
+  // the phase kernels' byte offsets are 32-bit: 64 bytes a row of a class and block of
+  // 16 columns, at most 2^32 of the sites above (Lx = 4)
+  if (64 * (int64_t)(Ly / 4) * ((Lx / 4 + 15) / 16) > ((int64_t)1 << 32)) return CCMC_E_INVAL;
   return CCMC_OK;
 }
 

@@ -16,12 +16,6 @@
 
 namespace ccmc {
 
-__device__ __forceinline__ int64_t warp_sum(int64_t v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  return v;
-}
-
 // like, unlike, b1, b0, both, and b1, b0 over the sites of even x + y.
 constexpr int kSums = 7;
 

@@ -105,10 +105,6 @@ struct TableKeys {
   }
 };
 
-__device__ __forceinline__ uint32_t *row_ptr(const Geo &g, int cls, int row) {
-  return g.words + (int64_t)cls * g.cstride + (int64_t)row * g.W;
-}
-
 // n (<= 16) consecutive sites of a class row starting at column `start`
 // (periodic in the row), site t at bits 2t .. 2t+1.  Bits beyond 2n are
 // unspecified.

@@ -29,7 +29,7 @@ enum CtlSlot : int {
   kCtlPhaseBase = 0,  // global phase index of the next phase with offset 0
   kCtlObsCount = 1,   // records written to the ring so far
   kCtlTicket = 2,     // arrival counter of the recount's last-block reduction
-  kCtlStatus = 3,     // device-side error flag
+  kCtlStatus = 3,     // device-side error flag (no sweep kernel has a wait that could set it)
   kCtlLatest = 4,     // 8 words: the last recount record
   kCtlWords = 16
 };
@@ -86,7 +86,7 @@ constexpr int kMoveN = 2 * kTransN;  // both kinds
 constexpr int kThrT = (kDevN + 7) / 8 * 8;  // 16-bit levels, padded to 16 bytes
 
 struct LaunchCfg {
-  int phase_grid_cap = 152 * 3;  // one resident wave of phase_kernel (set at create)
+  int phase_grid_cap = 152 * 4;  // one resident wave of phase_kernel (set at create)
 };
 
 // One lattice of a resident launch (ccmc_resident.cu): held in the shared memory
@@ -132,8 +132,9 @@ struct MultiJob {
   int cta_begin, cta_count;
 };
 
-// What ccmc_batch_config's upper limit of resident_max_sites sets aside of a
-// CTA's shared memory (words).
+// ccmc_batch_config takes resident limits of at most four sites for every word of a
+// CTA's shared memory but these and 64 (219,024 sites, 55 KB of packed words, on a
+// GB300): a quarter of what one CTA holds, a limit that callers know.
 constexpr int kConfigTableWords = 3292;
 
 // Host-side table builders (ccmc_tables.cpp): the full table of

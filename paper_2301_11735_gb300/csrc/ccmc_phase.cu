@@ -45,7 +45,8 @@ struct PhaseSmem {
 
 // The direct path's view of a word: row j, word w of the classes in global memory,
 // rows of whole words (kAl) or of any width.  Addresses are 32-bit byte offsets from
-// the lattice's base (at most 2^28 bytes).
+// the lattice's base: its words take at most 2^32 bytes (validate_shape), which a
+// lattice of 4 x 2^28 sites does, with one site a word.
 template <bool kAl>
 struct DirectView {
   const Geo &g;
@@ -291,7 +292,7 @@ int phase_resident_grid(bool aligned) {
   const cudaError_t e =
       aligned ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, phase_kernel<true>, 256, 0)
               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, phase_kernel<false>, 256, 0);
-  if (e != cudaSuccess || per_sm < 1 || sms < 1) return 152 * 3;
+  if (e != cudaSuccess || per_sm < 1 || sms < 1) return 152 * 4;
   return per_sm * sms;
 }
 

@@ -96,7 +96,8 @@ int64_t ring_records(const ccmc_request &r) {
   return r.obs_every > 0 ? std::min<int64_t>(r.nsweeps / r.obs_every + 1, 1 << 16) : 1;
 }
 
-// Estimated wall time of one sweep, for sizing slices (measured: 3.5 us at 64^2, 7.5 at
+// Estimated wall time of one sweep of a lattice that runs alone, for sizing slices: a
+// slice of many lattices takes longer than slice_ms (measured: 3.5 us at 64^2, 7.5 at
 // 256^2, 10.5 at 512^2, 15 to 18 at 1000^2, held in shared memory; 24 at 2048^2, 33 at
 // 4096^2, 213 at 16384^2, a launch a phase).
 double sweep_us(const ccmc_request &r) {

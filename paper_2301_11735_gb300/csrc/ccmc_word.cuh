@@ -271,12 +271,9 @@ __device__ __forceinline__ uint32_t exact_group(const uint2 *trans, const uint32
   return acc;
 }
 
-// The fast path of the pairs of a word one thread evaluates: kTPW threads
-// share a word (1, 2 or 4), thread `sub` of them takes MOVE call(s) and
-// half(s):
-//   kTPW 1: both calls, both halves (all 16 pairs);
-//   kTPW 2: call sub, both halves (8 pairs);
-//   kTPW 4: call sub / 2, half sub mod 2 (4 pairs: group k = sub).
+// The fast path of the pairs of a word one thread evaluates: all 16 (kTPW 1), or with
+// two threads a word (kTPW 2) the eight of MOVE call `sub`.  (Four lanes a word have a
+// path of their own in the resident kernel.)
 // rand(c): the four words of the word's MOVE call c.  Returns the (dA, dB) of the
 // fast decisions and, in z, what needs the exact path (a tie or a field >= 65532,
 // rejected here): bit t for every such pair t (kPairs), or bit c for every call c
@@ -287,25 +284,15 @@ template <int kTPW, bool kPairs, class Rand>
 __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *thrT, int sub,
                                             const WordIn &in, uint32_t near128,
                                             const Rand &rand) {
-  static_assert(kTPW == 1 || kTPW == 2 || kTPW == 4, "one, two or four threads a word");
+  static_assert(kTPW == 1 || kTPW == 2, "one or two threads a word");
   constexpr int kCalls = kTPW == 1 ? 2 : 1;
-  constexpr int kHalves = kTPW == 4 ? 1 : 2;
-  const int c0 = kTPW == 1 ? 0 : (kTPW == 2 ? sub : sub >> 1);
-  const int h0 = kTPW == 4 ? (sub & 1) : 0;
-  Env env[kHalves];
-  uint32_t pcs[kHalves];
+  const int c0 = kTPW == 1 ? 0 : sub;
+  Env env[2];
+  uint32_t pcs[2];
 #pragma unroll
-  for (int hi = 0; hi < kHalves; ++hi) {
-    if constexpr (kTPW == 4) {  // the thread's half moved to half 0's place
-      auto half = [&](const Planes &p) {
-        return Planes{p.O >> (2 * h0), p.T >> (2 * h0), p.F >> (2 * h0)};
-      };
-      env[hi] = half_env(half(in.na), half(in.nb), 0);
-      pcs[hi] = half_pc(in.A >> (2 * h0), in.B >> (2 * h0), 0);
-    } else {
-      env[hi] = half_env(in.na, in.nb, hi);
-      pcs[hi] = half_pc(in.A, in.B, hi);
-    }
+  for (int h = 0; h < 2; ++h) {
+    env[h] = half_env(in.na, in.nb, h);
+    pcs[h] = half_pc(in.A, in.B, h);
   }
   uint32_t dA = 0u, dB = 0u, slow = 0u;
 #pragma unroll
@@ -315,13 +302,12 @@ __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *
     const uint32_t mx = __vmaxu2(__vimax3_u16x2(r.x, r.y, r.z), r.w);
     const bool big = mx >= 0xFFFC0000u || (mx & 0xFFFFu) >= 0xFFFCu;  // a field >= 65532
     uint32_t mn = 0xFFFFFFFFu;  // smallest w - T of the call
-    uint32_t d[kHalves][4];
+    uint32_t d[2][4];
 #pragma unroll
-    for (int hi = 0; hi < kHalves; ++hi) {
-      const int h = h0 + hi;
+    for (int h = 0; h < 2; ++h) {
       const int k = 2 * c + h;
       uint32_t t[4];
-      const uint32_t pc = __funnelshift_l(pcs[hi], pcs[hi], 3 - 4 * c);  // counts modulo 32
+      const uint32_t pc = __funnelshift_l(pcs[h], pcs[h], 3 - 4 * c);  // counts modulo 32
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
@@ -329,15 +315,15 @@ __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *
         const uint32_t wq = div12(v);
         const uint2 e =
             move_entry(trans, entry_offset(pc, q, (v - 12u * wq) * 264u + near128));
-        t[q] = (uint32_t)__dp4a((int)e.y, (int)((env[hi].ev[q] >> (4 * c)) & kEnvMask), (int)e.x);
-        d[hi][q] = wq - level_at(thrT, t[q] & 0xFFFFu);  // negative: accept; zero: a tie
+        t[q] = (uint32_t)__dp4a((int)e.y, (int)((env[h].ev[q] >> (4 * c)) & kEnvMask), (int)e.x);
+        d[h][q] = wq - level_at(thrT, t[q] & 0xFFFFu);  // negative: accept; zero: a tie
       }
-      mn = __vimin3_u32(mn, d[hi][0], d[hi][1]);
-      mn = __vimin3_u32(mn, d[hi][2], d[hi][3]);
+      mn = __vimin3_u32(mn, d[h][0], d[h][1]);
+      mn = __vimin3_u32(mn, d[h][2], d[h][3]);
       // byte q: the accepted move of lane q, i.e. byte 3 of t[q] under the sign
       // of d[q] (byte permutes: bit 3 of a selector replicates a byte's sign)
       const uint32_t acc =
-          prmt(prmt(d[hi][0], d[hi][1], 0x00FBu), prmt(d[hi][2], d[hi][3], 0x00FBu), 0x5410u) &
+          prmt(prmt(d[h][0], d[h][1], 0x00FBu), prmt(d[h][2], d[h][3], 0x00FBu), 0x5410u) &
           prmt(prmt(t[0], t[1], 0x0073u), prmt(t[2], t[3], 0x0073u), 0x5410u);
       // byte q of acc -> site k + 4 q: b bits to 2 (k + 4 q) of dB, a bits of dA
       dB |= (acc & 0x03030303u) << (2 * k);
@@ -346,12 +332,12 @@ __device__ __forceinline__ uint3 fast_moves(const uint2 *trans, const uint16_t *
     if (mn == 0u || big) {
       if constexpr (kPairs) {
 #pragma unroll
-        for (int hi = 0; hi < kHalves; ++hi)
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const uint32_t X = q == 0 ? r.x : q == 1 ? r.y : q == 2 ? r.z : r.w;
-            if (d[hi][q] == 0u || ((X >> (16 * (h0 + hi))) & 0xFFFFu) >= 65532u)
-              slow |= 1u << (2 * c + h0 + hi + 4 * q);
+            if (d[h][q] == 0u || ((X >> (16 * h)) & 0xFFFFu) >= 65532u)
+              slow |= 1u << (2 * c + h + 4 * q);
           }
       } else {
         slow |= 1u << c;

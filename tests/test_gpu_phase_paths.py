@@ -112,3 +112,19 @@ def test_lock_step_groups(cc, shapes, ctas):
         assert np.array_equal(got, st), (Lx, Ly, ctas, first_difference(got, st))
         assert np.array_equal(lat.obs_series(), rec)
         lat.close()
+
+
+def test_largest_lattice_of_one_site_a_word(cc):
+    """4 x 2^28 sites take 2^32 bytes: the phase kernel's byte offsets reach 2^32 - 4."""
+    Lx, Ly, seed = 4, 1 << 28, 9
+    packed = np.random.default_rng(1).integers(0, 256, size=Lx * Ly // 4, dtype=np.uint8)
+    st = np.empty((Ly, Lx), np.uint8)
+    for k in range(4):
+        st[:, k] = (packed >> (2 * k)) & 3
+    with cc.Lattice(Lx, Ly) as lat:
+        lat.set_state_packed(packed, seed, 0)
+        lat.phases(1, *PARAMS)
+        got = lat.get_state_packed()
+    oracle.phase(st, seed, 0, oracle.threshold_table(*PARAMS))
+    assert np.array_equal(got, st[:, 0] | (st[:, 1] << 2) | (st[:, 2] << 4) | (st[:, 3] << 6))
+    assert not np.array_equal(got, packed)
