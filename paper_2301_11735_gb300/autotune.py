@@ -22,7 +22,8 @@ import json
 import os
 import time
 
-_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "autotune.json")
+_HERE = os.path.dirname(os.path.abspath(__file__))
+_CACHE = os.path.join(_HERE, "_build", "autotune.json")
 
 # (threads per CTA, largest resident lattice in sites, CTAs per SM, most
 # threads a word): the argument order of Batch.config
@@ -57,9 +58,8 @@ def signature(shapes) -> str:
 def _sources() -> str:
     """Digest of the sources that the library is built from."""
     h = hashlib.sha1()
-    here = os.path.dirname(os.path.abspath(__file__))
-    for d in (os.path.join(here, "csrc"), os.path.join(os.path.dirname(here), "include")):
-        for name in sorted(os.listdir(d)):
+    for d in (os.path.join(_HERE, "csrc"), os.path.join(os.path.dirname(_HERE), "include")):
+        for name in sorted(os.listdir(d) if os.path.isdir(d) else ()):  # a copy without sources
             with open(os.path.join(d, name), "rb") as f:
                 h.update(name.encode() + b"\0" + f.read())
     return h.hexdigest()[:16]

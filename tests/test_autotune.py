@@ -40,6 +40,13 @@ def test_times_of_other_kernels_are_taken_again(probes, monkeypatch):
     assert autotune.measured(SHAPES[:2])["plan"] and len(calls) == 3
 
 
+def test_a_copy_without_the_sources_tunes_as_well(probes, monkeypatch, tmp_path):
+    here = autotune._sources()
+    monkeypatch.setattr(autotune, "_HERE", str(tmp_path / "elsewhere"))
+    probes({None: 1.0, autotune.DEFAULT: 2.0})
+    assert autotune.tune(SHAPES) == autotune.DEFAULT and autotune._sources() != here
+
+
 def test_a_gpu_that_takes_no_candidate_keeps_the_plan(probes):
     calls = probes({None: 1.0})
     assert autotune.measured(SHAPES)["plan"] and autotune.tune(SHAPES) == autotune.DEFAULT
