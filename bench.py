@@ -315,7 +315,8 @@ def measure_batched(cc, nsweeps=5000, plain_per_size=4):
     call, against the same lattices swept one at a time: a stated subset
     (the first `plain_per_size` lattices of every size), each for the full
     5000 sweeps from the same state, whose final states must equal the
-    batch's bit for bit."""
+    batch's bit for bit.  Both hold a lattice in shared memory: a quarter of the subset
+    is swept again a launch a phase, by other kernels, and compared too."""
     import numpy as np
     import torch
 
@@ -357,6 +358,18 @@ def measure_batched(cc, nsweeps=5000, plain_per_size=4):
             one.sync()
             t_plain += time.perf_counter() - t0
             identical &= bool(np.array_equal(one.get_state(), lats[i].get_state()))
+    independent = True
+    for i in picked[::4]:  # a quarter of them by other kernels: a launch a phase
+        s = sims[i]
+        os.environ["CCMC_NO_RESIDENT"] = "1"
+        try:
+            one = cc.Lattice(s.Lx, s.Ly)
+        finally:
+            del os.environ["CCMC_NO_RESIDENT"]
+        with one:
+            one.init_constrained(s.seed, s.n, s.charged_frac)
+            one.sweep(3 + nsweeps, s.beta, s.Delta, s.V, s.J)
+            independent &= bool(np.array_equal(one.get_state(), lats[i].get_state()))
     plain = sum(sims[i].sites for i in picked) * nsweeps / t_plain
     for lat in lats:
         lat.close()
@@ -369,7 +382,8 @@ def measure_batched(cc, nsweeps=5000, plain_per_size=4):
                                    "sample": f"{len(picked)} of the lattices ({plain_per_size} of "
                                              f"each size), the full {nsweeps} sweeps each, one "
                                              "ccmc_sweep call at a time",
-                                   "identical_final_states": identical},
+                                   "identical_final_states": identical,
+                                   "identical_to_a_launch_a_phase": independent},
             "speedup_vs_plain": (work / dt) / plain}
 
 
